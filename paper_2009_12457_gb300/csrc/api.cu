@@ -492,7 +492,8 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   const bool rebuild =
       !plan_matches(g->plan, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition);
   if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[2], s));
-  BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition));
+  BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
+                      !budgeted));
   if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[3], s));
   g->plan_timed = rebuild;
   const Plan &pl = g->plan;
@@ -532,7 +533,7 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
                        task_cycles, edge_sup, task_mask));
     g->stream_stats_total_ms = -1.0;
   }
-  unsigned long long head[SCR_TASKS] = {0, 0, 0};
+  unsigned long long head[SCR_TASKS] = {0};
   BBTC_CUDA(cudaMemcpyAsync(head, pl.scratch, sizeof(head), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   if ((int32_t)head[SCR_STATUS] != 0) return count_status_error("bbtc_count", (int32_t)head[SCR_STATUS], opts.timeout_ms);

@@ -17,14 +17,13 @@
 
 #include "graph.cuh"
 #include "primitives.cuh"
+#include "stage.cuh"
 
 namespace bbtc {
 
 namespace {
 
 constexpr int CT_NT = 256;
-
-constexpr int32_t STATUS_TIMEOUT = 1, STATUS_COPY_WAIT = 2;
 
 struct CountParams {
   const TaskDesc *desc;  // per task (Alg. 4 order): where its three blocks live
@@ -39,165 +38,12 @@ struct CountParams {
   unsigned *edge_sup;               // per-edge support by position in the block columns (MODE & 4)
   const uint8_t *task_mask;         // nullable: items of tasks whose byte is 0 are skipped
   int32_t *status;
+  const unsigned long long *t0;     // start of the count, when a kernel before this one set it
   uint64_t timeout_ns;
+  int use_core;                     // the dense core's edges are counted by core.cu: skip them
 };
 
 constexpr int MODE_VERTEX = 1, MODE_GRAPH = 2, MODE_EDGE = 4;
-
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Per-warp shared staging area for N(G_jk, v) (int32 slots).
-constexpr int STAGE = 2048;
-static_assert(STAGE % 4 == 0, "the bitmap is cleared with 16-byte stores");
-// largest power of two <= STAGE: the biggest hash table the stage holds
-constexpr int STAGE_POW2 = STAGE >= 2048 ? 2048 : STAGE >= 1024 ? 1024 : STAGE >= 512 ? 512 : 256;
-static_assert(STAGE_POW2 <= STAGE && STAGE >= 256, "stage too small");
-constexpr int MIN_STAGE = 8;
-// lists at least this long are staged through one bulk copy (TMA)
-constexpr int BULK_STAGE_MIN = 64;
-constexpr int ST_NONE = 0, ST_SORTED = 1, ST_HASH = 2, ST_BITMAP = 3, ST_FILTER = 4;
-// ST_FILTER: an open-addressed table of up to FILTER_SLOTS slots in the upper
-// half of the stage, with a bit filter over a second hash of the keys in the
-// lower half. A probe reads one filter word and looks in the table only when
-// its bit is set: for a key not in the list that happens with probability at
-// most blen / FILTER_BITS (below 1/64 for blen <= 512).
-constexpr int FILTER_WORDS = STAGE / 2;
-constexpr int FILTER_BITS_LOG2 = 15;
-constexpr int FILTER_SLOTS = STAGE - FILTER_WORDS;
-static_assert(FILTER_WORDS * 32 == 1 << FILTER_BITS_LOG2, "filter size");
-static_assert((FILTER_SLOTS & (FILTER_SLOTS - 1)) == 0 && FILTER_WORDS % 4 == 0, "filter table");
-constexpr int32_t EMPTY = -1;
-
-__device__ __forceinline__ uint32_t hash_slot(int32_t w, int log2h) {
-  return ((uint32_t)w * 2654435761u) >> (32 - log2h);
-}
-
-__device__ __forceinline__ uint32_t filter_bit(int32_t w) {
-  return ((uint32_t)w * 0x85EBCA6Bu) >> (32 - FILTER_BITS_LOG2);
-}
-
-// Membership of w in the sorted list stage[0, len): lower bound by a fixed
-// number of halvings (the same for every lane, since len is warp-uniform).
-__device__ __forceinline__ bool sorted_contains(const int32_t *stage, int len, int32_t w) {
-  int pos = 0;
-  for (int step = len > 0 ? 1 << (31 - __clz(len)) : 0; step > 0; step >>= 1)
-    if (pos + step <= len && stage[pos + step - 1] < w) pos += step;
-  return pos < len && stage[pos] == w;
-}
-
-// Membership of w in the open-addressed table stage[0, 2^log2h) (linear
-// probing, at most half full). The probe reads four slots per 16-byte load,
-// starting at the 4-slot group of w's hash slot, so nearly every lookup ends
-// after one load and the lanes of a warp stay together.
-__device__ __forceinline__ bool hash_contains(const int32_t *stage, int log2h, int32_t w) {
-  const uint32_t gmask = (1u << (log2h - 2)) - 1u;
-  uint32_t g = hash_slot(w, log2h) >> 2;
-  const int4 *groups = reinterpret_cast<const int4 *>(stage);
-  for (uint32_t n = 0; n <= gmask; ++n) {
-    const int4 q = groups[g];
-    if (q.x == w || q.y == w || q.z == w || q.w == w) return true;
-    if (q.x == EMPTY || q.y == EMPTY || q.z == EMPTY || q.w == EMPTY) return false;
-    g = (g + 1) & gmask;
-  }
-  return false;
-}
-
-// The table half of an ST_FILTER stage, reached only when the filter bit is set.
-__device__ __forceinline__ bool filter_verify(const int32_t *table, int log2h, int32_t w) {
-  return hash_contains(table, log2h, w);
-}
-
-__device__ __forceinline__ uint32_t filter_lookup(const int32_t *stage, int log2h, int32_t w) {
-  const uint32_t h = filter_bit(w);
-  const uint32_t word = reinterpret_cast<const uint32_t *>(stage)[h >> 5];
-  if (((word >> (h & 31u)) & 1u) == 0u) return 0u;
-  return filter_verify(stage + FILTER_WORDS, log2h, w) ? 1u : 0u;
-}
-
-// ------------------------------------------------ bulk copies (TMA, PTX)
-
-__device__ __forceinline__ uint32_t smem_addr(const void *ptr) {
-  return (uint32_t)__cvta_generic_to_shared(ptr);
-}
-__device__ __forceinline__ void mbar_init(unsigned long long *m) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(m)) : "memory");
-}
-// Makes an initialised barrier visible to the bulk-copy unit.
-__device__ __forceinline__ void mbar_init_fence() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-// The one arrival of the barrier's current phase, announcing `bytes` of copies.
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *m, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(m)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *m, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(smem_addr(m)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-// limit of one wait on a bulk copy (copies of valid addresses take microseconds)
-constexpr uint64_t COPY_WAIT_NS = 200ull * 1000 * 1000;
-// Waits for the barrier's phase of the given parity, for at most COPY_WAIT_NS.
-__device__ __noinline__ bool mbar_wait_bounded(unsigned long long *m, uint32_t parity) {
-  if (mbar_try_wait(m, parity)) return true;
-  const uint64_t t0 = global_ns();
-  while (!mbar_try_wait(m, parity))
-    if (global_ns() - t0 > COPY_WAIT_NS) return false;
-  return true;
-}
-// TMA bulk copy global -> shared of `bytes` (a multiple of 16, both addresses
-// 16-byte aligned), completing on barrier m.
-__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes,
-                                          unsigned long long *m) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(m))
-      : "memory");
-}
-// Orders this thread's earlier plain shared-memory accesses before later bulk
-// copies into the same memory.
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Starts one bulk copy of list[e0, e1) into `dst` (e0, e1 multiples of 4:
-// whole 16-byte quads of a 16-byte aligned, quad-padded column array; dst
-// 16-byte aligned), issued by lane 0 on barrier mbar. Warp-uniform call.
-__device__ __forceinline__ void bulk_issue(int32_t *dst, const int32_t *list, int64_t e0,
-                                           int64_t e1, unsigned long long *mbar, unsigned lane) {
-  fence_proxy_async();  // earlier plain accesses to the stage before the copy
-  __syncwarp();
-  if (lane == 0) {
-    const uint32_t bytes = (uint32_t)(4 * (e1 - e0));
-    mbar_expect_tx(mbar, bytes);
-    bulk_copy(dst, list + e0, bytes, mbar);
-  }
-}
-
-// Waits (bounded) for the copy of bulk_issue; true on every lane when it
-// arrived. On false the copy is awaited once more and the caller stops.
-__device__ __forceinline__ bool bulk_wait(unsigned long long *mbar, uint32_t &parity) {
-  const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(mbar, parity));
-  if (!ok) {
-    mbar_wait_bounded(mbar, parity);
-    return false;
-  }
-  parity ^= 1u;
-  return true;
-}
 
 // Per-batch lane records, shared by the warp: where each in-edge's probes
 // start in the flattened probe sequence and where they come from.
@@ -353,7 +199,11 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
   }
   __syncwarp();
   uint32_t mbar_parity = 0;  // parity of rec.mbar's next phase
-  const uint64_t t_start = P.timeout_ns ? global_ns() : 0;
+  uint64_t t_start = 0;
+  if (P.timeout_ns) {
+    t_start = *P.t0;
+    if (t_start == 0) t_start = global_ns();
+  }
   // (task, v) whose N(G_jk, v) is in `stage`, and how it is stored
   unsigned long long staged_tag = ~0ull;
   int staged_len = 0, staged_log2h = 0, staged_mode = ST_NONE, staged_off = 0;
@@ -389,6 +239,9 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
     const int64_t rs_ik = d.rs_ik, rs_jk = d.rs_jk;
     const int32_t c_i = d.c_i, c_j = d.c_j;
     const bool diag = d.diag != 0;
+    const unsigned *__restrict__ core_flags =
+        !PER_VERTEX && !PER_EDGE && P.use_core ? d.core_flags : nullptr;
+    const int32_t core_u0 = d.core_u0, core_v0 = d.core_v0;
     unsigned long long acc = 0;
 
     int64_t base = w.x0;
@@ -422,11 +275,16 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
       const InEdge rn = base + lane < w.x1 ? ie[base + lane - ie_off] : make_int4(0, -1, 0, 0);
       if (base + 32 + lane < w.x1)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(ie + (base + 32 + lane - ie_off)));
-      const bool active = (int)lane < nb;
+      bool active = (int)lane < nb;
       const int32_t u = r.x;
+      if (core_flags && active && v >= core_v0 && u >= core_u0) {
+        const uint32_t x = (uint32_t)(u - core_u0);
+        active = ((core_flags[x >> 5] >> (x & 31u)) & 1u) == 0u;
+      }
       const int64_t e = (int64_t)(uint32_t)r.z;
       const int64_t f = (int64_t)(uint32_t)r.w;
       r = rn;
+      if (core_flags && !__any_sync(0xffffffffu, active)) continue;
       // N(G_jk, v): direct row pointers of block (j, k); [b0, b1) local to ci_jk
       int64_t b0 = 0, b1 = 0;
       if (uniform) {
@@ -828,7 +686,7 @@ bbtc_status count_reset(bbtc_graph *g, const Plan &pl, unsigned long long *verte
 bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t nitems,
                          unsigned long long *vertex_count, bool per_graph, uint32_t timeout_ms,
                          cudaStream_t s, unsigned long long *task_cycles, unsigned *edge_sup,
-                         const uint8_t *task_mask) {
+                         const uint8_t *task_mask, bool use_core) {
   if (nitems <= 0) return BBTC_OK;
   unsigned long long *scr = pl.scratch;
   BBTC_CUDA(cudaMemsetAsync(scr + SCR_HEAD, 0, sizeof(unsigned long long), s));
@@ -842,7 +700,9 @@ bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t n
   P.gid = g->gid;
   P.graph_count = scr + SCR_TASKS + pl.ntasks;
   P.status = reinterpret_cast<int32_t *>(scr + SCR_STATUS);
+  P.t0 = scr + SCR_T0;
   P.timeout_ns = (uint64_t)timeout_ms * 1000000ull;
+  P.use_core = use_core;
   P.task_cycles = task_cycles;
   P.edge_sup = edge_sup;
   P.task_mask = task_mask;
@@ -890,8 +750,18 @@ bbtc_status run_count(bbtc_graph *g, const Plan &pl, unsigned long long *vertex_
                       const uint8_t *task_mask) {
   BBTC_TRY(count_reset(g, pl, vertex_count, per_graph, s));
   if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
-  BBTC_TRY(count_launch(g, pl, 0, pl.nitems, vertex_count, per_graph, timeout_ms, s,
-                        task_cycles, edge_sup, task_mask));
+  // the core's bitmaps count triangles per task and per graph; outputs per
+  // vertex and edge, measured cycles and shares of the tasks go to the lists
+  const bool core = !vertex_count && !edge_sup && !task_cycles && !task_mask && pl.core.bits;
+  if (core)
+    BBTC_TRY(core_launch(core_desc(g, pl, 0, 0), nullptr, 1, pl.core.nitems, pl.core.parts.quads,
+                         pl.scratch + SCR_TASKS, pl.ntasks,
+                         per_graph ? pl.scratch + SCR_TASKS + pl.ntasks : nullptr,
+                         reinterpret_cast<int32_t *>(pl.scratch + SCR_STATUS),
+                         pl.scratch + SCR_T0, timeout_ms, s));
+  if (!(core && pl.core.all))
+    BBTC_TRY(count_launch(g, pl, 0, pl.nitems, vertex_count, per_graph, timeout_ms, s,
+                          task_cycles, edge_sup, task_mask, core));
   if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
   return count_finish(pl, s);
 }
@@ -939,18 +809,26 @@ bbtc_status count_plans(bbtc_graph *const *gs, int32_t ng, uint32_t timeout_ms, 
   });
   std::vector<PlanRef> refs((size_t)ng);
   std::vector<int64_t> task_base((size_t)ng);
-  int64_t ntasks = 0, nitems = 0;
-  int blocks_per_sm = 0;
+  int64_t ntasks = 0, nitems = 0, core_items = 0;
+  int blocks_per_sm = 0, quads_max = 0;
+  std::vector<CoreDesc> cores;
   for (int32_t r = 0; r < ng; ++r) {
     const Plan &pl = gs[order[(size_t)r]]->plan;
     if (pl.streamed || pl.p < 1) {
       set_error("internal: count_plans needs resident plans");
       return BBTC_EINTERNAL;
     }
-    refs[(size_t)r] = PlanRef{pl.desc, pl.items, pl.ntasks, pl.nitems, ntasks, nitems};
+    const bool all_core = pl.core.bits && pl.core.all;
+    refs[(size_t)r] =
+        PlanRef{pl.desc, pl.items, pl.ntasks, all_core ? 0 : pl.nitems, ntasks, nitems};
     task_base[(size_t)order[(size_t)r]] = ntasks;
+    if (pl.core.bits && pl.core.nitems > 0 && ntasks <= INT32_MAX) {
+      cores.push_back(core_desc(gs[order[(size_t)r]], pl, core_items, (int32_t)ntasks));
+      core_items += pl.core.nitems;
+      quads_max = std::max(quads_max, (int)pl.core.parts.quads);
+    }
     ntasks += pl.ntasks;
-    nitems += pl.nitems;
+    if (!all_core) nitems += pl.nitems;
     if (pl.blocks_per_sm[0] > blocks_per_sm) blocks_per_sm = pl.blocks_per_sm[0];
   }
   if (ntasks > INT32_MAX) {
@@ -962,30 +840,45 @@ bbtc_status count_plans(bbtc_graph *const *gs, int32_t ng, uint32_t timeout_ms, 
   PlanRef *d_refs = nullptr;
   TaskDesc *desc = nullptr;
   WorkItem *items = nullptr;
-  unsigned long long *counters = nullptr;  // [0] head, [1] status, [2, 2 + T) per task
+  unsigned long long *counters = nullptr;  // head, status, start time, then per task
+  constexpr int C_HEAD = 0, C_STATUS = 1, C_T0 = 2, C_TASKS = 3;
+  CoreDesc *d_cores = nullptr;
   BBTC_TRY(scratch.get(&d_refs, ng));
   BBTC_TRY(scratch.get(&desc, ntasks));
   BBTC_TRY(scratch.get(&items, nitems));
-  BBTC_TRY(scratch.get(&counters, 2 + ntasks));
+  BBTC_TRY(scratch.get(&counters, C_TASKS + ntasks));
+  if (cores.size() > 1) BBTC_TRY(scratch.get(&d_cores, (int64_t)cores.size()));
   BBTC_CUDA(cudaMemcpyAsync(d_refs, refs.data(), sizeof(PlanRef) * (size_t)ng,
                             cudaMemcpyHostToDevice, s));
-  BBTC_CUDA(cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * (size_t)(2 + ntasks), s));
-  k_gather_plans<<<(unsigned)std::min<int64_t>(ng, 4096), 256, 0, s>>>(d_refs, ng, desc, items);
-  BBTC_LAUNCH_CHECK();
+  BBTC_CUDA(cudaMemsetAsync(counters, 0,
+                            sizeof(unsigned long long) * (size_t)(C_TASKS + ntasks), s));
+  if (!cores.empty()) {
+    if (d_cores)
+      BBTC_CUDA(cudaMemcpyAsync(d_cores, cores.data(), sizeof(CoreDesc) * cores.size(),
+                                cudaMemcpyHostToDevice, s));
+    BBTC_TRY(core_launch(cores[0], d_cores, (int32_t)cores.size(), core_items, quads_max,
+                         counters + C_TASKS, ntasks, nullptr,
+                         reinterpret_cast<int32_t *>(counters + C_STATUS), counters + C_T0,
+                         timeout_ms, s));
+  }
   if (nitems > 0) {
+    k_gather_plans<<<(unsigned)std::min<int64_t>(ng, 4096), 256, 0, s>>>(d_refs, ng, desc, items);
+    BBTC_LAUNCH_CHECK();
     CountParams P;
     P.desc = desc;
     P.items = items;
     P.nitems = nitems;
-    P.head = counters;
-    P.task_count = counters + 2;
+    P.head = counters + C_HEAD;
+    P.task_count = counters + C_TASKS;
+    P.t0 = counters + C_T0;
+    P.use_core = 1;
     P.vcount = nullptr;
     P.gid = nullptr;
     P.graph_count = nullptr;
     P.task_cycles = nullptr;
     P.edge_sup = nullptr;
     P.task_mask = nullptr;
-    P.status = reinterpret_cast<int32_t *>(counters + 1);
+    P.status = reinterpret_cast<int32_t *>(counters + C_STATUS);
     P.timeout_ns = (uint64_t)timeout_ms * 1000000ull;
     if (blocks_per_sm < 1) BBTC_TRY(configure_mode<0>(&blocks_per_sm));
     int64_t blocks = (int64_t)num_sms() * blocks_per_sm;
@@ -994,15 +887,16 @@ bbtc_status count_plans(bbtc_graph *const *gs, int32_t ng, uint32_t timeout_ms, 
     k_count<0><<<(unsigned)blocks, CT_NT, count_smem_bytes(), s>>>(P);
     BBTC_LAUNCH_CHECK();
   }
-  std::vector<unsigned long long> h((size_t)(2 + ntasks));
+  std::vector<unsigned long long> h((size_t)(C_TASKS + ntasks));
   BBTC_CUDA(cudaMemcpyAsync(h.data(), counters, sizeof(unsigned long long) * h.size(),
                             cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
-  if ((int32_t)h[1] != 0) return count_status_error("bbtc_count_batch", (int32_t)h[1], timeout_ms);
+  if ((int32_t)h[C_STATUS] != 0)
+    return count_status_error("bbtc_count_batch", (int32_t)h[C_STATUS], timeout_ms);
   for (int32_t i = 0; i < ng; ++i) {
     uint64_t c = 0;
     const int64_t b = task_base[(size_t)i];
-    for (int64_t t = 0; t < gs[i]->plan.ntasks; ++t) c += h[(size_t)(2 + b + t)];
+    for (int64_t t = 0; t < gs[i]->plan.ntasks; ++t) c += h[(size_t)(C_TASKS + b + t)];
     counts[i] = c;
   }
   return BBTC_OK;
@@ -1098,7 +992,13 @@ extern "C" bbtc_status bbtc_count_noalloc(bbtc_graph_t g, int32_t p, uint64_t *c
       st = BBTC_ECUDA;
       break;
     }
-    if (pl.nitems > 0) {
+    if (pl.core.bits &&
+        (st = core_launch(core_desc(g, pl, 0, 0), nullptr, 1, pl.core.nitems,
+                          pl.core.parts.quads, task_count, nt, nullptr,
+                          reinterpret_cast<int32_t *>(scratch + NOALLOC_STATUS), nullptr, 0, s)) !=
+            BBTC_OK)
+      break;
+    if (pl.nitems > 0 && !(pl.core.bits && pl.core.all)) {
       CountParams P;
       P.desc = pl.desc;
       P.items = pl.items;
@@ -1112,7 +1012,9 @@ extern "C" bbtc_status bbtc_count_noalloc(bbtc_graph_t g, int32_t p, uint64_t *c
       P.edge_sup = nullptr;
       P.task_mask = nullptr;
       P.status = reinterpret_cast<int32_t *>(scratch + NOALLOC_STATUS);
+      P.t0 = nullptr;
       P.timeout_ns = 0;
+      P.use_core = 1;
       const size_t smem = count_smem_bytes();
       int blocks_per_sm = 0;
       if (cudaFuncSetAttribute(k_count<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,

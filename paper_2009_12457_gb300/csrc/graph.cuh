@@ -43,6 +43,10 @@ struct TaskDesc {
   int32_t c_i, c_j;
   int32_t diag;  // k == j
   int32_t task;  // index in Alg. 4 order
+  // in-edges counted by the dense core (core.cu): v >= core_v0, u >= core_u0 and
+  // the flag bit of u - core_u0 set. Resident plans only; nullptr = none
+  const unsigned *core_flags;
+  int32_t core_u0, core_v0;
 };
 
 // One unit of counting work: the in-edges [x0, x1) of block G_ij (grouped by
@@ -51,6 +55,54 @@ struct WorkItem {
   int32_t task;
   int32_t flags;  // bits 0-1: 0 INTERSECT, 1 HASHMAP, 2 AUTO; bits 2..: AUTO hash threshold
   int64_t x0, x1;
+};
+
+// The dense core of a resident plan (core.cu): bitmap rows over the columns of
+// the top positions [v0, n), and the sources whose core neighbours are counted
+// with them. Columns are laid out by part: the core vertices of the q-th part
+// that reaches into the core (number id[q]) are [first[q], first[q + 1]) and
+// their columns start at quad (128 columns) quad0[q]. Rows are stored from the
+// group of 32 quads that holds their vertex: gfirst[g] is the first core vertex
+// of group g, gbase[g] the byte offset of its row.
+struct CoreParts {
+  static constexpr int kGroups = 8;
+  int32_t np = 0;
+  int32_t quads = 0;  // columns / 128, a multiple of 32
+  int32_t first[64] = {0};
+  int32_t quad0[64] = {0};
+  int32_t gfirst[kGroups] = {0};
+  uint32_t gbase[kGroups] = {0};
+  uint8_t id[64] = {0};
+};
+
+struct Core {
+  bool all = false;     // every edge between two sources' lists is in the core: no list is probed
+  int32_t v0 = 0;       // first core vertex
+  int64_t u0 = 0;       // first position that may be a source (a multiple of 32)
+  uint32_t cap = 0;     // room in items
+  int64_t nitems = 0;   // work items
+  CoreParts parts;
+  uint4 *bits = nullptr;       // rows
+  int2 *tab = nullptr;         // per core vertex {row offset from group 0, first quad | part << 16}
+  uint8_t *qpart = nullptr;    // part of each quad
+  int4 *items = nullptr;       // {u, first core edge, first edge of the item, row end}
+  unsigned *flags = nullptr;   // bit u - u0: u is counted here
+  unsigned *count = nullptr;   // number of items (device)
+  uint64_t bytes = 0;
+};
+
+// Where the core's counting kernel finds one plan's core.
+struct CoreDesc {
+  const int4 *items;
+  int64_t item_base;  // items of the descriptors before this one
+  const int32_t *colidx;
+  const uint4 *bits;
+  const int2 *tab;
+  const uint8_t *qpart;
+  const int32_t *cuts;
+  const int32_t *gid;
+  int32_t v0, quads, p, task_base;
+  CoreParts parts;
 };
 
 // Everything bbtc_count builds for one p (Sec. 2 partition, Sec. 4.2 tasks,
@@ -88,9 +140,10 @@ struct Plan {
   int32_t partition = 0;        // bbtc_partition the cuts were built with
   int64_t bstar = -1;           // probe-based partition: the bound B* on every block
   int64_t chunk = 0;            // in-edges per item used
-  // counting scratch owned by the plan: [0] work-stealing head, [1] status,
-  // [2] total, [3, 3+T) per-task counts, [3+T, 3+T+ng) per-graph counts
+  // counting scratch owned by the plan: the SCR_* words, then T per-task
+  // counts, then ng per-graph counts
   unsigned long long *scratch = nullptr;
+  Core core;
   int blocks_per_sm[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // occupancy of each counting-kernel mode
   // streamed mode: the block arrays live in pinned host memory instead
   bool streamed = false;
@@ -100,7 +153,8 @@ struct Plan {
   uint64_t bytes = 0;
 };
 
-constexpr int SCR_HEAD = 0, SCR_STATUS = 1, SCR_TOTAL = 2, SCR_TASKS = 3;
+// work-stealing head, status, total, start time of a count with a time limit
+constexpr int SCR_HEAD = 0, SCR_STATUS = 1, SCR_TOTAL = 2, SCR_T0 = 3, SCR_TASKS = 4;
 
 }  // namespace bbtc
 
@@ -151,8 +205,10 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
 // a5-a8: partition, blocks, tasks, estimate, order and work items for p.
 // partition: 0 = contiguous parts balanced on oriented edges, 1 = probe-based
 // (bounds the largest block).
+// want_core: build the dense core too (resident counts; not for INTERSECT,
+// whose lists are searched sorted by the caller's choice).
 bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold, int chunk,
-                       cudaStream_t s, int partition = 0);
+                       cudaStream_t s, int partition = 0, bool want_core = true);
 inline bool plan_matches(const Plan &pl, int p, int kernel_mode, int hash_threshold, int chunk,
                          int partition = 0) {
   return pl.p == p && pl.kernel_mode == kernel_mode && pl.hash_threshold == hash_threshold &&
@@ -164,6 +220,18 @@ inline bool plan_matches(const Plan &pl, int p, int kernel_mode, int hash_thresh
 bbtc_status pbd_partition(const bbtc_graph *g, int p, int32_t *d_cuts, int64_t *h_bstar,
                           cudaStream_t s);
 void free_plan(Plan *pl, cudaStream_t s);
+
+// The dense core (core.cu). build_core enqueues its construction for the
+// plan's cuts; the number of items lands in core.count. core_launch counts the
+// nd descriptors' items into task_count (each at its task_base) and, when
+// given, graph_count; `descs` is read when nd > 1.
+bbtc_status build_core(const bbtc_graph *g, Plan &pl, cudaStream_t s);
+void free_core(Plan *pl, cudaStream_t s);
+CoreDesc core_desc(const bbtc_graph *g, const Plan &pl, int64_t item_base, int32_t task_base);
+bbtc_status core_launch(const CoreDesc &one, const CoreDesc *descs, int32_t nd, int64_t nitems,
+                        int quads_max, unsigned long long *task_count, int64_t ntasks,
+                        unsigned long long *graph_count, int32_t *status, unsigned long long *t0,
+                        uint32_t timeout_ms, cudaStream_t s);
 void free_plan_host(Plan *pl);  // pinned host copies of a streamed plan
 
 // Occupancy of the counting kernel (set at plan time so that a count only
@@ -189,7 +257,8 @@ bbtc_status count_reset(bbtc_graph *g, const Plan &pl, unsigned long long *verte
 bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t nitems,
                          unsigned long long *vertex_count, bool per_graph, uint32_t timeout_ms,
                          cudaStream_t s, unsigned long long *task_cycles = nullptr,
-                         unsigned *edge_sup = nullptr, const uint8_t *task_mask = nullptr);
+                         unsigned *edge_sup = nullptr, const uint8_t *task_mask = nullptr,
+                         bool use_core = false);
 bbtc_status count_finish(const Plan &pl, cudaStream_t s);
 // The error of a nonzero status word left by the counting kernel: 1 = it
 // passed opts.timeout_ms (ETIMEOUT), 2 = a bulk copy wait ran out (EINTERNAL).

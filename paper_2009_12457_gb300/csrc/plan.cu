@@ -578,6 +578,7 @@ void free_plan(Plan *pl, cudaStream_t s) {
   dfree(pl->ci, s);
   dfree(pl->spl, s);
   dfree(pl->desc, s);
+  free_core(pl, s);
   free_plan_host(pl);
   *pl = Plan();
 }
@@ -597,7 +598,7 @@ int default_p(const bbtc_graph *g, bool budgeted) {
 }
 
 bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold, int chunk_req,
-                       cudaStream_t s, int partition) {
+                       cudaStream_t s, int partition, bool want_core) {
   if (plan_matches(g->plan, p, kernel_mode, hash_threshold, chunk_req, partition)) return BBTC_OK;
   free_plan(&g->plan, s);
   Plan pl;
@@ -765,6 +766,17 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, pl.order);
   PLAN_TRY(launch_status("build_plan"));
 
+  // the dense core (INTERSECT searches every list, as the caller chose)
+  if (want_core && kernel_mode != BBTC_KERNEL_INTERSECT) {
+    const bbtc_status cst = build_core(g, pl, s);
+    if (cst == BBTC_ENOMEM) {  // no room: the lists count everything
+      free_core(&pl, s);
+      clear_error();
+    } else {
+      PLAN_TRY(cst);
+    }
+  }
+
   // task descriptors: every block of the resident BCSR
   {
     TaskDesc *h_desc = new (std::nothrow) TaskDesc[(size_t)nt];
@@ -792,6 +804,9 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
           d.c_j = pl.h_cuts[j];
           d.diag = k == j;
           d.task = (int32_t)t;
+          d.core_flags = pl.core.flags;
+          d.core_u0 = (int32_t)pl.core.u0;
+          d.core_v0 = pl.core.v0;
         }
     bbtc_status dst = dalloc_n(&pl.desc, nt, s);
     if (dst == BBTC_OK &&
@@ -819,14 +834,18 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   PLAN_TRY(launch_status("build_plan"));
   PLAN_TRY(exclusive_scan_u64(first, first, nt + 1, s));
   uint64_t nitems = 0;
+  unsigned core_items = 0;
   if (cudaMemcpyAsync(&nitems, first + nt, sizeof(uint64_t), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
+      (pl.core.count && cudaMemcpyAsync(&core_items, pl.core.count, sizeof(unsigned),
+                                        cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("build_plan: reading the work-item count failed");
     free_plan(&pl, s);
     return BBTC_ECUDA;
   }
   pl.nitems = (int64_t)nitems;
+  pl.core.nitems = (int64_t)core_items;
   PLAN_TRY(dalloc_n(&pl.items, pl.nitems, s));
   if (nitems > 0) {
     k_item_fill<<<grid_for((int64_t)nitems, 256, 8), 256, 0, s>>>(
@@ -839,7 +858,8 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   PLAN_TRY(configure_count_kernels(&pl));
 #undef PLAN_TRY
   pl.bytes = (uint64_t)m * sizeof(InEdge) + (uint64_t)pl.h_spl_off[p] * 4 + (uint64_t)nt * (24 + sizeof(TaskDesc)) +
-             (uint64_t)pl.nitems * sizeof(WorkItem) + (uint64_t)(SCR_TASKS + nt + g->ng) * 8;
+             (uint64_t)pl.nitems * sizeof(WorkItem) + (uint64_t)(SCR_TASKS + nt + g->ng) * 8 +
+             pl.core.bytes;
   g->plan = pl;
   return BBTC_OK;
 }

@@ -119,6 +119,7 @@ bbtc_status plan_to_host(const bbtc_graph *g, Plan &pl, int64_t m, cudaStream_t 
   pl.rp = nullptr;
   pl.ci = nullptr;
   pl.ie = nullptr;
+  free_core(&pl, s);  // streamed counts keep nothing but the pool's blocks
   // work items in Alg. 4 task order (a task's items stay together and keep
   // their order), so that the tasks sharing an in-edge block are consecutive
   if (pl.nitems > 0) {
