@@ -489,11 +489,22 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   // a resident count needs the block arrays on the device: a plan that was
   // streamed (its arrays now in host memory) is rebuilt
   if (!budgeted && g->plan.streamed) free_plan(&g->plan, s);
+  // counted task by task: with a budget, for a share of the tasks and for their cycles
+  const bool by_task = budgeted || opts.per_task_cycles_out || opts.task_mask;
+  const bool detail = !by_task && (opts.per_vertex_out || opts.per_edge_out);
+  const bool tasks = opts.per_task_out && p > 1, per_graph = opts.per_graph_out != nullptr;
+  // (a detail count alone needs neither the core nor the in-edges that it leaves)
+  const bool resident = !by_task && (!detail || tasks || per_graph);
+  const Plan &old = g->plan;
   const bool rebuild =
-      !plan_matches(g->plan, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition);
+      !plan_matches(old, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition) ||
+      (by_task && !old.tasks_ready) || (resident && !old.flat.ready) ||
+      (detail && !old.full.ready && !(old.flat.ready && !old.core.bits));
   if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[2], s));
   BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
-                      !budgeted));
+                      resident));
+  if (by_task) BBTC_TRY(build_tasks(g, s));
+  if (detail) BBTC_TRY(build_full(g, s));
   if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[3], s));
   g->plan_timed = rebuild;
   const Plan &pl = g->plan;
@@ -510,7 +521,6 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
     BBTC_TRY(scratch.get(&edge_sup, g->m > 0 ? g->m : 1));
     BBTC_CUDA(cudaMemsetAsync(edge_sup, 0, sizeof(unsigned) * (size_t)(g->m > 0 ? g->m : 1), s));
   }
-  const bool per_graph = opts.per_graph_out != nullptr;
   uint8_t *task_mask = nullptr;  // this caller's share of the tasks, on the device
   if (opts.task_mask) {
     BBTC_TRY(scratch.get(&task_mask, pl.ntasks));
@@ -529,8 +539,14 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
     g->stream_stats.mode = st.mode;
     g->stream_stats_total_ms = st.total_ms;
   } else {
-    BBTC_TRY(run_count(g, pl, vertex_count, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5],
-                       task_cycles, edge_sup, task_mask));
+    if (by_task)
+      BBTC_TRY(run_count(g, pl, vertex_count, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5],
+                         task_cycles, edge_sup, task_mask));
+    else if (detail)
+      BBTC_TRY(run_detail(g, pl, tasks, per_graph, vertex_count, edge_sup, opts.timeout_ms, s,
+                          g->ev[4], g->ev[5]));
+    else
+      BBTC_TRY(run_flat(g, pl, tasks, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5]));
     g->stream_stats_total_ms = -1.0;
   }
   unsigned long long head[SCR_TASKS] = {0};
@@ -590,7 +606,7 @@ bbtc_status bbtc_count_async(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t 
   cudaStream_t s = opts.stream ? (cudaStream_t)opts.stream : g->stream;
   const Plan &pl = g->plan;
   const bool per_graph = opts.per_graph_out != nullptr;
-  BBTC_TRY(run_count(g, pl, nullptr, per_graph, 0, s, nullptr, nullptr));
+  BBTC_TRY(run_flat(g, pl, opts.per_task_out != nullptr, per_graph, 0, s, nullptr, nullptr));
   BBTC_CUDA(cudaMemcpyAsync(total_dev, pl.scratch + SCR_TOTAL, sizeof(uint64_t),
                             cudaMemcpyDeviceToDevice, s));
   if (opts.per_task_out)
@@ -781,7 +797,7 @@ bbtc_status bbtc_graph_get_timings(bbtc_graph_t g, bbtc_timings *t) {
   t->plan_ms = g->plan_timed ? elapsed(g->ev[2], g->ev[3]) : 0.0;
   t->count_ms = g->stream_stats_total_ms >= 0 ? g->stream_stats_total_ms
                                               : elapsed(g->ev[4], g->ev[5]);
-  t->work_items = g->plan.nitems;
+  t->work_items = g->plan.flat.ready ? g->plan.flat.nitems + g->plan.core.nitems : g->plan.nitems;
   t->stream_rounds = g->stream_stats.rounds;
   t->stream_h2d_bytes = g->stream_stats.h2d_bytes;
   t->stream_copy_ms = g->stream_stats.copy_ms;
@@ -851,6 +867,7 @@ bbtc_status bbtc_graph_get_plan(bbtc_graph_t g, int32_t p, int32_t *cuts, int64_
   const int chunk = g->plan.p == p ? g->plan.chunk_req : 0;
   const int part = g->plan.p == p ? g->plan.partition : BBTC_PARTITION_EDGES;
   BBTC_TRY(build_plan(g, p, kmode, thr, chunk, s, part));
+  BBTC_TRY(build_tasks(g, s));
   const Plan &pl = g->plan;
   if (cuts)
     BBTC_CUDA(cudaMemcpyAsync(cuts, pl.cuts, sizeof(int32_t) * (size_t)(p + 1),

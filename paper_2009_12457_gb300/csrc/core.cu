@@ -35,7 +35,6 @@ constexpr int CORE_MAX_COLS = 8192;  // columns of the core at most
 // a graph of at most so many vertices is all core, and no list is probed: R-MAT
 // scale 14 counts in 27 us where the lists took 117 (latency, not work)
 constexpr int CORE_ALL_COLS = 16384;
-constexpr int CORE_CHUNK = 128;       // core edges of one source per work item
 constexpr int CORE_TABLE = 816;       // task counters kept in shared memory (p <= 16)
 constexpr int CORE_CTAS = 4;          // counting CTAs per SM
 constexpr int32_t CORE_STATUS_TIMEOUT = 1;
@@ -544,12 +543,13 @@ CoreDesc core_desc(const bbtc_graph *g, const Plan &pl, int64_t item_base, int32
   return d;
 }
 
-bbtc_status core_launch(const CoreDesc &one, const CoreDesc *descs, int32_t nd, int64_t nitems,
-                        int quads_max, unsigned long long *task_count, int64_t ntasks,
+bbtc_status core_launch(CoreDesc one, const CoreDesc *descs, int32_t nd, int64_t nitems,
+                        int quads_max, unsigned long long *task_count, int64_t ntasks, bool tasks,
                         unsigned long long *graph_count, int32_t *status, unsigned long long *t0,
                         uint32_t timeout_ms, cudaStream_t s) {
   if (nitems <= 0) return BBTC_OK;
   CoreLaunch P;
+  if (!tasks) one.p = 1;
   P.one = one;
   P.descs = descs;
   P.nd = nd;

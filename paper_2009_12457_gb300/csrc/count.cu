@@ -15,6 +15,7 @@
 #include <mutex>
 #include <vector>
 
+#include "flat.cuh"
 #include "graph.cuh"
 #include "primitives.cuh"
 #include "stage.cuh"
@@ -38,21 +39,18 @@ struct CountParams {
   unsigned *edge_sup;               // per-edge support by position in the block columns (MODE & 4)
   const uint8_t *task_mask;         // nullable: items of tasks whose byte is 0 are skipped
   int32_t *status;
-  const unsigned long long *t0;     // start of the count, when a kernel before this one set it
   uint64_t timeout_ns;
-  int use_core;                     // the dense core's edges are counted by core.cu: skip them
 };
 
 constexpr int MODE_VERTEX = 1, MODE_GRAPH = 2, MODE_EDGE = 4;
 
 // Per-batch lane records, shared by the warp: where each in-edge's probes
 // start in the flattened probe sequence and where they come from.
-struct LaneRec {
+struct alignas(16) LaneRec {
   int64_t b0[32];     // N(G_jk, v) range of each lane (mixed batches only)
   int64_t b1[32];
   uint32_t s0[32];    // first probe element (local column index) of each lane's in-edge
-  uint32_t s1[32];    // one past its last probe element (quad probes only)
-  uint32_t incl[32];  // inclusive prefix of the probe counts (quad counts for quad probes)
+  uint32_t incl[32];  // inclusive prefix of the probe counts
   int32_t u[32];
   int32_t v[32];
   unsigned long long mbar;  // completion of bulk copies into the warp's stage
@@ -122,63 +120,6 @@ __device__ __forceinline__ void probe_batch(const int32_t *__restrict__ ci_ik, c
   }
 }
 
-// Quad probes (plain counts against a bitmap-staged list): the probe range
-// [s0, s1) of each in-edge is widened down to a multiple of four, cut into
-// aligned groups of four columns ("quads"), and the quads of the batch are
-// flattened like single probes: lane l takes quads l, l + 32, ... and loads
-// each with one 16-byte load. A 4-bit mask per quad keeps the columns inside
-// [s0, s1). Column arrays are 16-byte aligned and padded by whole quads, so
-// the widened reads stay inside them. UQ quads per lane are in flight.
-__device__ __forceinline__ uint32_t quad_mask(uint32_t q, uint32_t lo, uint32_t hi) {
-  // columns q + c, 0 <= c < 4, with lo <= q + c < hi (q <= hi - 1, q >= lo - 3)
-  const uint32_t first = lo > q ? lo - q : 0u;
-  const uint32_t last = hi - q < 4u ? hi - q : 4u;
-  return ((1u << last) - 1u) & ~((1u << first) - 1u);
-}
-
-template <int UQ, typename Lookup>
-__device__ __forceinline__ uint32_t probe_quads(const int32_t *__restrict__ ci,
-                                                const LaneRec &rec, uint32_t totalq,
-                                                unsigned lane, Lookup lookup) {
-  uint32_t hits = 0;
-  int o = 0;
-  uint32_t o_end = rec.incl[0];
-  uint32_t lo = rec.s0[0], hi = rec.s1[0];
-  uint32_t base = lo & ~3u;  // column of quad j is base + 4 * j (mod 2^32)
-  uint32_t jb = lane;
-  for (; jb - lane < totalq; jb += 32u * UQ) {
-    int4 wq[UQ];
-    uint32_t msk[UQ];
-#pragma unroll
-    for (int r = 0; r < UQ; ++r) {
-      const uint32_t j = jb + 32u * r;
-      msk[r] = 0u;
-      wq[r] = make_int4(0, 0, 0, 0);
-      if (j < totalq) {
-        while (j >= o_end) {
-          ++o;
-          const uint32_t prev_end = o_end;
-          o_end = rec.incl[o];
-          lo = rec.s0[o];
-          hi = rec.s1[o];
-          base = (lo & ~3u) - 4u * prev_end;
-        }
-        const uint32_t q = base + 4u * j;
-        wq[r] = *reinterpret_cast<const int4 *>(ci + q);
-        msk[r] = quad_mask(q, lo, hi);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < UQ; ++r) {
-      hits += lookup(wq[r].x) & msk[r];
-      hits += lookup(wq[r].y) & (msk[r] >> 1);
-      hits += lookup(wq[r].z) & (msk[r] >> 2);
-      hits += lookup(wq[r].w) & (msk[r] >> 3);
-    }
-  }
-  return hits;
-}
-
 constexpr int UNIFORM_MIN = 4;  // a run of >= 4 in-edges into one v is a uniform batch
 
 template <int MODE>
@@ -199,15 +140,11 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
   }
   __syncwarp();
   uint32_t mbar_parity = 0;  // parity of rec.mbar's next phase
-  uint64_t t_start = 0;
-  if (P.timeout_ns) {
-    t_start = *P.t0;
-    if (t_start == 0) t_start = global_ns();
-  }
+  const uint64_t t_start = P.timeout_ns ? global_ns() : 0;
   // (task, v) whose N(G_jk, v) is in `stage`, and how it is stored
   unsigned long long staged_tag = ~0ull;
   int staged_len = 0, staged_log2h = 0, staged_mode = ST_NONE, staged_off = 0;
-  int32_t staged_first = 0;
+  uint32_t staged_word0 = 0;   // bitmap: first word of its window
   uint32_t staged_gw = STAGE;  // bitmap: index of its zero guard word
   bool failed = false;
 
@@ -239,9 +176,6 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
     const int64_t rs_ik = d.rs_ik, rs_jk = d.rs_jk;
     const int32_t c_i = d.c_i, c_j = d.c_j;
     const bool diag = d.diag != 0;
-    const unsigned *__restrict__ core_flags =
-        !PER_VERTEX && !PER_EDGE && P.use_core ? d.core_flags : nullptr;
-    const int32_t core_u0 = d.core_u0, core_v0 = d.core_v0;
     unsigned long long acc = 0;
 
     int64_t base = w.x0;
@@ -275,16 +209,11 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
       const InEdge rn = base + lane < w.x1 ? ie[base + lane - ie_off] : make_int4(0, -1, 0, 0);
       if (base + 32 + lane < w.x1)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(ie + (base + 32 + lane - ie_off)));
-      bool active = (int)lane < nb;
+      const bool active = (int)lane < nb;
       const int32_t u = r.x;
-      if (core_flags && active && v >= core_v0 && u >= core_u0) {
-        const uint32_t x = (uint32_t)(u - core_u0);
-        active = ((core_flags[x >> 5] >> (x & 31u)) & 1u) == 0u;
-      }
       const int64_t e = (int64_t)(uint32_t)r.z;
       const int64_t f = (int64_t)(uint32_t)r.w;
       r = rn;
-      if (core_flags && !__any_sync(0xffffffffu, active)) continue;
       // N(G_jk, v): direct row pointers of block (j, k); [b0, b1) local to ci_jk
       int64_t b0 = 0, b1 = 0;
       if (uniform) {
@@ -340,11 +269,12 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
           const int32_t first = __shfl_sync(0xffffffffu, x0, 0);
           const int32_t last = blen > 32 ? __shfl_sync(0xffffffffu, lastv, 0)
                                          : __shfl_sync(0xffffffffu, x0, blen - 1);
-          const int64_t span = (int64_t)last - first + 1;
+          const uint32_t word0 = (uint32_t)first >> 5;
+          const uint32_t nw = ((uint32_t)last >> 5) - word0 + 1u;
           int mode = ST_NONE;
           if (kflag == 0) {
             if (blen <= STAGE) mode = ST_SORTED;
-          } else if (span <= (int64_t)STAGE * 32) {
+          } else if (nw <= (uint32_t)STAGE) {
             mode = ST_BITMAP;
           } else if (2 * blen <= FILTER_SLOTS && (kflag == 1 || blen > hash_min)) {
             mode = ST_FILTER;
@@ -366,7 +296,6 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
             if (mode == ST_BITMAP) {
               // words [0, nw) hold the window, word nw is its zero guard; only
               // these are cleared (4-word groups up to `land`)
-              const uint32_t nw = (uint32_t)((span + 31) >> 5);
               const int64_t land = (int64_t)((nw + 4u) & ~3u);
               const bool bulk = long_list && land + (e1 - e0) <= STAGE;
               if (bulk) bulk_issue(stage + land, ci_jk, e0, e1, &rec.mbar, lane);
@@ -379,11 +308,10 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
               __syncwarp();
               if (!failed)
                 for (int i = lane; i < blen; i += 32) {
-                  const uint32_t d = (uint32_t)((i < 32 ? x0 : src[i]) - first);
-                  atomicOr(reinterpret_cast<unsigned *>(stage) + (d >> 5), 1u << (d & 31u));
+                  const uint32_t w = (uint32_t)(i < 32 ? x0 : src[i]);
+                  atomicOr(reinterpret_cast<unsigned *>(stage) + ((w >> 5) - word0), 1u << (w & 31u));
                 }
-              staged_first = first;
-              staged_len = (int)span;
+              staged_word0 = word0;
               staged_gw = nw;
             } else if (mode == ST_FILTER || mode == ST_HASH) {
               int log2h = 5;
@@ -409,8 +337,9 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
                 for (int i = lane; i < blen; i += 32) {
                   const int32_t key = i < 32 ? x0 : src[i];
                   if (mode == ST_FILTER) {
-                    const uint32_t fb = filter_bit(key);
-                    atomicOr(reinterpret_cast<unsigned *>(stage) + (fb >> 5), 1u << (fb & 31u));
+                    const uint32_t h = InFilter::hash(key);
+                    atomicOr(reinterpret_cast<unsigned *>(stage) + InFilter::word_of(h),
+                             InFilter::bits_of(h));
                   }
                   // linear probing from the first slot of the key's 4-slot
                   // group, the order in which hash_contains reads the table
@@ -455,34 +384,30 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
       }
 
       if (MODE == 0 && staged && (staged_mode == ST_BITMAP || staged_mode == ST_FILTER)) {
-        // quad probes (see probe_quads) against a bitmap or a filtered table;
-        // plain hash-table and sorted lookups keep the single-probe loop below,
-        // which measured faster for them
+        // quads (flat.cuh) against a bitmap or a filtered table; plain hash-table
+        // and sorted lookups keep the single-probe loop below
         const uint32_t a0 = (uint32_t)s0 & ~3u;
         const uint32_t nq = len ? ((uint32_t)s1 - a0 + 3u) >> 2 : 0u;
         const uint32_t inclq = warp_inclusive_scan(nq);
         const uint32_t totalq = __shfl_sync(0xffffffffu, inclq, 31);
-        rec.s0[lane] = (uint32_t)s0;
-        rec.s1[lane] = (uint32_t)s1;
-        rec.incl[lane] = inclq;
+        uint4 *q4 = reinterpret_cast<uint4 *>(rec.b0);  // b0 and b1 are for mixed batches
+        const unsigned with = __ballot_sync(0xffffffffu, nq > 0);
+        if (nq > 0)
+          q4[__popc(with & ((1u << lane) - 1u))] =
+              make_uint4((uint32_t)s0, (uint32_t)s1, a0 - 4u * (inclq - nq), 0u);
         __syncwarp();
+        uint32_t hits = 0;
         if (staged_mode == ST_BITMAP) {
-          const unsigned *__restrict__ bm = reinterpret_cast<const unsigned *>(stage);
-          const int32_t first = staged_first;
-          const uint32_t gw = staged_gw;
-          acc += probe_quads<2>(ci_ik, rec, totalq, lane, [&](int32_t w) -> uint32_t {
-            const uint32_t dlt = (uint32_t)(w - first);
-            // values outside the window [first, first + 32 * gw) read the zero
-            // guard word gw
-            const uint32_t word = bm[min(dlt >> 5, gw)];
-            return (word >> (dlt & 31u)) & 1u;
-          });
+          const InBitmap look{reinterpret_cast<const uint32_t *>(stage), staged_word0, staged_gw};
+          flat_rounds<2>(ci_ik, q4, totalq, inclq - nq, nq > 0, lane,
+                         [&](int, const int4 &w, uint32_t m, uint32_t) { hits += look.count(w, m); });
         } else {
-          const int log2h = staged_log2h;
-          acc += probe_quads<2>(ci_ik, rec, totalq, lane, [&](int32_t w) -> uint32_t {
-            return filter_lookup(stage, log2h, w);
-          });
+          const InFilter look{reinterpret_cast<const uint32_t *>(stage), stage + FILTER_WORDS,
+                              staged_log2h};
+          flat_rounds<2>(ci_ik, q4, totalq, inclq - nq, nq > 0, lane,
+                         [&](int, const int4 &w, uint32_t m, uint32_t) { hits += look.count(w, m); });
         }
+        acc += hits;
         __syncwarp();
         continue;
       }
@@ -530,20 +455,15 @@ __global__ void __launch_bounds__(CT_NT, 3) k_count(CountParams P) {
       };
       // the probe loop, specialised by how N(G_jk, v) is looked up
       if (staged && staged_mode == ST_BITMAP) {
-        const unsigned *__restrict__ bm = reinterpret_cast<const unsigned *>(stage);
-        const int32_t first = staged_first;
-        const uint32_t span = (uint32_t)staged_len;
-        probe_batch<4>(ci_ik, rec, total, lane, on_hit, [&](int32_t w, int) {
-          // branch-free: the word index is clamped into the bitmap, and the
-          // range test masks the bit
-          const uint32_t dlt = (uint32_t)(w - first);
-          const uint32_t word = bm[min(dlt >> 5, (uint32_t)(STAGE - 1))];
-          return ((dlt < span) & (word >> (dlt & 31u))) & 1u;
-        });
-      } else if (staged && staged_mode == ST_FILTER) {
-        const int log2h = staged_log2h;
+        const InBitmap look{reinterpret_cast<const uint32_t *>(stage), staged_word0, staged_gw};
         probe_batch<4>(ci_ik, rec, total, lane, on_hit,
-                       [&](int32_t w, int) { return filter_lookup(stage, log2h, w) != 0u; });
+                       [&](int32_t w, int) { return (look.one(w) & 1u) != 0u; });
+      } else if (staged && staged_mode == ST_FILTER) {
+        const InFilter look{reinterpret_cast<const uint32_t *>(stage), stage + FILTER_WORDS,
+                            staged_log2h};
+        probe_batch<4>(ci_ik, rec, total, lane, on_hit, [&](int32_t w, int) {
+          return (look.maybe(w) & 1u) != 0u && hash_contains(look.table, look.log2h, w);
+        });
       } else if (staged && staged_mode == ST_HASH) {
         const int log2h = staged_log2h;
         probe_batch<4>(ci_ik, rec, total, lane, on_hit,
@@ -683,30 +603,33 @@ bbtc_status count_reset(bbtc_graph *g, const Plan &pl, unsigned long long *verte
   return BBTC_OK;
 }
 
-bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t nitems,
-                         unsigned long long *vertex_count, bool per_graph, uint32_t timeout_ms,
-                         cudaStream_t s, unsigned long long *task_cycles, unsigned *edge_sup,
-                         const uint8_t *task_mask, bool use_core) {
+namespace {
+
+// The by-task launch with its counters anywhere: head, status, T task counters
+// and, with per_graph, the graph counters.
+bbtc_status count_launch_at(const bbtc_graph *g, const Plan &pl, int64_t item0, int64_t nitems,
+                            unsigned long long *head, int32_t *status,
+                            unsigned long long *task_count, unsigned long long *graph_count,
+                            unsigned long long *vertex_count, uint32_t timeout_ms, cudaStream_t s,
+                            unsigned long long *task_cycles, unsigned *edge_sup,
+                            const uint8_t *task_mask) {
   if (nitems <= 0) return BBTC_OK;
-  unsigned long long *scr = pl.scratch;
-  BBTC_CUDA(cudaMemsetAsync(scr + SCR_HEAD, 0, sizeof(unsigned long long), s));
+  BBTC_CUDA(cudaMemsetAsync(head, 0, sizeof(unsigned long long), s));
   CountParams P;
   P.desc = pl.desc;
   P.items = pl.items + item0;
   P.nitems = nitems;
-  P.head = scr + SCR_HEAD;
-  P.task_count = scr + SCR_TASKS;
+  P.head = head;
+  P.task_count = task_count;
   P.vcount = vertex_count;
   P.gid = g->gid;
-  P.graph_count = scr + SCR_TASKS + pl.ntasks;
-  P.status = reinterpret_cast<int32_t *>(scr + SCR_STATUS);
-  P.t0 = scr + SCR_T0;
+  P.graph_count = graph_count;
+  P.status = status;
   P.timeout_ns = (uint64_t)timeout_ms * 1000000ull;
-  P.use_core = use_core;
   P.task_cycles = task_cycles;
   P.edge_sup = edge_sup;
   P.task_mask = task_mask;
-  const int mode = (vertex_count ? MODE_VERTEX : 0) | (per_graph ? MODE_GRAPH : 0) |
+  const int mode = (vertex_count ? MODE_VERTEX : 0) | (graph_count ? MODE_GRAPH : 0) |
                    (edge_sup ? MODE_EDGE : 0);
   int64_t blocks = (int64_t)num_sms() * pl.blocks_per_sm[mode];
   const int64_t need = (nitems + CT_NT / 32 - 1) / (CT_NT / 32);
@@ -724,6 +647,19 @@ bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t n
   }
   BBTC_LAUNCH_CHECK();
   return BBTC_OK;
+}
+
+}  // namespace
+
+bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t nitems,
+                         unsigned long long *vertex_count, bool per_graph, uint32_t timeout_ms,
+                         cudaStream_t s, unsigned long long *task_cycles, unsigned *edge_sup,
+                         const uint8_t *task_mask) {
+  unsigned long long *scr = pl.scratch;
+  return count_launch_at(g, pl, item0, nitems, scr + SCR_HEAD,
+                         reinterpret_cast<int32_t *>(scr + SCR_STATUS), scr + SCR_TASKS,
+                         per_graph ? scr + SCR_TASKS + pl.ntasks : nullptr, vertex_count,
+                         timeout_ms, s, task_cycles, edge_sup, task_mask);
 }
 
 bbtc_status count_status_error(const char *where, int32_t status, uint32_t timeout_ms) {
@@ -750,54 +686,71 @@ bbtc_status run_count(bbtc_graph *g, const Plan &pl, unsigned long long *vertex_
                       const uint8_t *task_mask) {
   BBTC_TRY(count_reset(g, pl, vertex_count, per_graph, s));
   if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
-  // the core's bitmaps count triangles per task and per graph; outputs per
-  // vertex and edge, measured cycles and shares of the tasks go to the lists
-  const bool core = !vertex_count && !edge_sup && !task_cycles && !task_mask && pl.core.bits;
-  if (core)
-    BBTC_TRY(core_launch(core_desc(g, pl, 0, 0), nullptr, 1, pl.core.nitems, pl.core.parts.quads,
-                         pl.scratch + SCR_TASKS, pl.ntasks,
-                         per_graph ? pl.scratch + SCR_TASKS + pl.ntasks : nullptr,
-                         reinterpret_cast<int32_t *>(pl.scratch + SCR_STATUS),
-                         pl.scratch + SCR_T0, timeout_ms, s));
-  if (!(core && pl.core.all))
-    BBTC_TRY(count_launch(g, pl, 0, pl.nitems, vertex_count, per_graph, timeout_ms, s,
-                          task_cycles, edge_sup, task_mask, core));
+  BBTC_TRY(count_launch(g, pl, 0, pl.nitems, vertex_count, per_graph, timeout_ms, s,
+                        task_cycles, edge_sup, task_mask));
   if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
   return count_finish(pl, s);
+}
+
+// Counts the handle's graph with what its resident plan holds: the core and
+// the in-edges that it leaves; else all in-edges (a plan built for a detail
+// count); else the tasks' work items (a plan built for a by-task count).
+static bbtc_status count_resident(const bbtc_graph *g, const Plan &pl, bool tasks,
+                                  unsigned long long *head, int32_t *status,
+                                  unsigned long long *t0, unsigned long long *task_count,
+                                  unsigned long long *graph_count, uint32_t timeout_ms,
+                                  cudaStream_t s) {
+  if (!pl.flat.ready && !pl.full.ready)
+    return count_launch_at(g, pl, 0, pl.nitems, head, status, task_count, graph_count, nullptr,
+                           timeout_ms, s, nullptr, nullptr, nullptr);
+  if (pl.flat.ready)
+    BBTC_TRY(core_launch(core_desc(g, pl, 0, 0), nullptr, 1, pl.core.nitems, pl.core.parts.quads,
+                         task_count, pl.ntasks, tasks, graph_count, status, t0, timeout_ms, s));
+  const Flat &f = pl.flat.ready ? pl.flat : pl.full;
+  return flat_launch(flat_desc(g, pl, f, 0, 0), nullptr, 1, f.nitems, head, task_count, pl.ntasks,
+                     tasks, graph_count, status, t0, timeout_ms, pl.flat_blocks_per_sm, s);
+}
+
+bbtc_status run_flat(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
+                     uint32_t timeout_ms, cudaStream_t s, cudaEvent_t ev_begin,
+                     cudaEvent_t ev_end) {
+  BBTC_TRY(count_reset(g, pl, nullptr, per_graph, s));
+  if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
+  unsigned long long *scr = pl.scratch;
+  BBTC_TRY(count_resident(g, pl, tasks, scr + SCR_HEAD,
+                          reinterpret_cast<int32_t *>(scr + SCR_STATUS), scr + SCR_T0,
+                          scr + SCR_TASKS, per_graph ? scr + SCR_TASKS + pl.ntasks : nullptr,
+                          timeout_ms, s));
+  if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
+  return count_finish(pl, s);
+}
+
+bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
+                       unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
+                       cudaStream_t s, cudaEvent_t ev_begin, cudaEvent_t ev_end) {
+  if (vcount)
+    BBTC_CUDA(cudaMemsetAsync(vcount, 0, sizeof(unsigned long long) * (size_t)std::max<int64_t>(g->n, 1),
+                              s));
+  // per task or per graph counts come from a flat count of their own
+  const bool both = tasks || per_graph;
+  if (both) {
+    BBTC_TRY(run_flat(g, pl, tasks, per_graph, timeout_ms, s, ev_begin, nullptr));
+  } else {
+    BBTC_TRY(count_reset(g, pl, nullptr, false, s));
+    if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
+  }
+  BBTC_TRY(detail_launch(g, pl, both ? nullptr : pl.scratch + SCR_TASKS, vcount, edge_sup,
+                         timeout_ms, s));
+  if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
+  return both ? BBTC_OK : count_finish(pl, s);
 }
 
 // --------------------------------------------- several plans, one launch
 //
 // A batch of resident handles is counted without copying them into a union:
-// each handle keeps its own plan, and one persistent launch drains the work
-// items of all of them. The descriptors of the handles' tasks are gathered
-// into one array (a task is found through its descriptor alone), and each
-// handle's items are copied with their task index moved to the handle's
-// first slot in that array.
-
-namespace {
-
-struct PlanRef {
-  const TaskDesc *desc;
-  const WorkItem *items;
-  int64_t ntasks, nitems;
-  int64_t task_base, item_base;
-};
-
-__global__ void k_gather_plans(const PlanRef *__restrict__ refs, int32_t nref,
-                               TaskDesc *__restrict__ desc, WorkItem *__restrict__ items) {
-  for (int32_t r = blockIdx.x; r < nref; r += gridDim.x) {
-    const PlanRef f = refs[r];
-    for (int64_t t = threadIdx.x; t < f.ntasks; t += blockDim.x) desc[f.task_base + t] = f.desc[t];
-    for (int64_t x = threadIdx.x; x < f.nitems; x += blockDim.x) {
-      WorkItem w = f.items[x];
-      w.task += (int32_t)f.task_base;
-      items[f.item_base + x] = w;
-    }
-  }
-}
-
-}  // namespace
+// each handle keeps its own plan, and one launch of each counting kernel (core,
+// flat) drains the work items of all of them, found through the handles'
+// descriptors. Each handle's whole count goes to its own counter.
 
 bbtc_status count_plans(bbtc_graph *const *gs, int32_t ng, uint32_t timeout_ms, cudaStream_t s,
                         uint64_t *counts) {
@@ -805,100 +758,65 @@ bbtc_status count_plans(bbtc_graph *const *gs, int32_t ng, uint32_t timeout_ms, 
   std::vector<int32_t> order((size_t)ng);
   for (int32_t i = 0; i < ng; ++i) order[(size_t)i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-    return gs[a]->plan.nitems > gs[b]->plan.nitems;
+    return gs[a]->plan.flat.nitems > gs[b]->plan.flat.nitems;
   });
-  std::vector<PlanRef> refs((size_t)ng);
-  std::vector<int64_t> task_base((size_t)ng);
-  int64_t ntasks = 0, nitems = 0, core_items = 0;
-  int blocks_per_sm = 0, quads_max = 0;
+  int64_t flat_items = 0, core_items = 0;
+  int quads_max = 0;
   std::vector<CoreDesc> cores;
+  std::vector<FlatDesc> flats;
   for (int32_t r = 0; r < ng; ++r) {
-    const Plan &pl = gs[order[(size_t)r]]->plan;
-    if (pl.streamed || pl.p < 1) {
+    const int32_t h = order[(size_t)r];
+    const Plan &pl = gs[h]->plan;
+    if (pl.streamed || pl.p < 1 || !pl.flat.ready) {
       set_error("internal: count_plans needs resident plans");
       return BBTC_EINTERNAL;
     }
-    const bool all_core = pl.core.bits && pl.core.all;
-    refs[(size_t)r] =
-        PlanRef{pl.desc, pl.items, pl.ntasks, all_core ? 0 : pl.nitems, ntasks, nitems};
-    task_base[(size_t)order[(size_t)r]] = ntasks;
-    if (pl.core.bits && pl.core.nitems > 0 && ntasks <= INT32_MAX) {
-      cores.push_back(core_desc(gs[order[(size_t)r]], pl, core_items, (int32_t)ntasks));
+    if (pl.core.nitems > 0) {
+      cores.push_back(core_desc(gs[h], pl, core_items, h));
+      cores.back().p = 1;
       core_items += pl.core.nitems;
       quads_max = std::max(quads_max, (int)pl.core.parts.quads);
     }
-    ntasks += pl.ntasks;
-    if (!all_core) nitems += pl.nitems;
-    if (pl.blocks_per_sm[0] > blocks_per_sm) blocks_per_sm = pl.blocks_per_sm[0];
-  }
-  if (ntasks > INT32_MAX) {
-    set_error("bbtc_count_batch: %lld tasks in one batch exceed the 32-bit task index",
-              (long long)ntasks);
-    return BBTC_EINVAL;
+    if (pl.flat.nitems > 0) {
+      flats.push_back(flat_desc(gs[h], pl, pl.flat, flat_items, h));
+      flat_items += pl.flat.nitems;
+    }
   }
   Scratch scratch(s);
-  PlanRef *d_refs = nullptr;
-  TaskDesc *desc = nullptr;
-  WorkItem *items = nullptr;
-  unsigned long long *counters = nullptr;  // head, status, start time, then per task
-  constexpr int C_HEAD = 0, C_STATUS = 1, C_T0 = 2, C_TASKS = 3;
+  unsigned long long *counters = nullptr;  // head, status, start time, then one per handle
+  constexpr int C_HEAD = 0, C_STATUS = 1, C_T0 = 2, C_COUNTS = 3;
   CoreDesc *d_cores = nullptr;
-  BBTC_TRY(scratch.get(&d_refs, ng));
-  BBTC_TRY(scratch.get(&desc, ntasks));
-  BBTC_TRY(scratch.get(&items, nitems));
-  BBTC_TRY(scratch.get(&counters, C_TASKS + ntasks));
-  if (cores.size() > 1) BBTC_TRY(scratch.get(&d_cores, (int64_t)cores.size()));
-  BBTC_CUDA(cudaMemcpyAsync(d_refs, refs.data(), sizeof(PlanRef) * (size_t)ng,
-                            cudaMemcpyHostToDevice, s));
-  BBTC_CUDA(cudaMemsetAsync(counters, 0,
-                            sizeof(unsigned long long) * (size_t)(C_TASKS + ntasks), s));
+  FlatDesc *d_flats = nullptr;
+  BBTC_TRY(scratch.get(&counters, C_COUNTS + ng));
+  BBTC_CUDA(cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * (size_t)(C_COUNTS + ng), s));
+  int32_t *status = reinterpret_cast<int32_t *>(counters + C_STATUS);
   if (!cores.empty()) {
-    if (d_cores)
+    if (cores.size() > 1) {
+      BBTC_TRY(scratch.get(&d_cores, (int64_t)cores.size()));
       BBTC_CUDA(cudaMemcpyAsync(d_cores, cores.data(), sizeof(CoreDesc) * cores.size(),
                                 cudaMemcpyHostToDevice, s));
+    }
     BBTC_TRY(core_launch(cores[0], d_cores, (int32_t)cores.size(), core_items, quads_max,
-                         counters + C_TASKS, ntasks, nullptr,
-                         reinterpret_cast<int32_t *>(counters + C_STATUS), counters + C_T0,
+                         counters + C_COUNTS, ng, false, nullptr, status, counters + C_T0,
                          timeout_ms, s));
   }
-  if (nitems > 0) {
-    k_gather_plans<<<(unsigned)std::min<int64_t>(ng, 4096), 256, 0, s>>>(d_refs, ng, desc, items);
-    BBTC_LAUNCH_CHECK();
-    CountParams P;
-    P.desc = desc;
-    P.items = items;
-    P.nitems = nitems;
-    P.head = counters + C_HEAD;
-    P.task_count = counters + C_TASKS;
-    P.t0 = counters + C_T0;
-    P.use_core = 1;
-    P.vcount = nullptr;
-    P.gid = nullptr;
-    P.graph_count = nullptr;
-    P.task_cycles = nullptr;
-    P.edge_sup = nullptr;
-    P.task_mask = nullptr;
-    P.status = reinterpret_cast<int32_t *>(counters + C_STATUS);
-    P.timeout_ns = (uint64_t)timeout_ms * 1000000ull;
-    if (blocks_per_sm < 1) BBTC_TRY(configure_mode<0>(&blocks_per_sm));
-    int64_t blocks = (int64_t)num_sms() * blocks_per_sm;
-    const int64_t need = (nitems + CT_NT / 32 - 1) / (CT_NT / 32);
-    if (blocks > need) blocks = need;
-    k_count<0><<<(unsigned)blocks, CT_NT, count_smem_bytes(), s>>>(P);
-    BBTC_LAUNCH_CHECK();
+  if (!flats.empty()) {
+    if (flats.size() > 1) {
+      BBTC_TRY(scratch.get(&d_flats, (int64_t)flats.size()));
+      BBTC_CUDA(cudaMemcpyAsync(d_flats, flats.data(), sizeof(FlatDesc) * flats.size(),
+                                cudaMemcpyHostToDevice, s));
+    }
+    BBTC_TRY(flat_launch(flats[0], d_flats, (int32_t)flats.size(), flat_items, counters + C_HEAD,
+                         counters + C_COUNTS, ng, false, nullptr, status, counters + C_T0,
+                         timeout_ms, gs[0]->plan.flat_blocks_per_sm, s));
   }
-  std::vector<unsigned long long> h((size_t)(C_TASKS + ntasks));
+  std::vector<unsigned long long> h((size_t)(C_COUNTS + ng));
   BBTC_CUDA(cudaMemcpyAsync(h.data(), counters, sizeof(unsigned long long) * h.size(),
                             cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   if ((int32_t)h[C_STATUS] != 0)
     return count_status_error("bbtc_count_batch", (int32_t)h[C_STATUS], timeout_ms);
-  for (int32_t i = 0; i < ng; ++i) {
-    uint64_t c = 0;
-    const int64_t b = task_base[(size_t)i];
-    for (int64_t t = 0; t < gs[i]->plan.ntasks; ++t) c += h[(size_t)(C_TASKS + b + t)];
-    counts[i] = c;
-  }
+  for (int32_t i = 0; i < ng; ++i) counts[i] = h[(size_t)(C_COUNTS + i)];
   return BBTC_OK;
 }
 
@@ -992,46 +910,11 @@ extern "C" bbtc_status bbtc_count_noalloc(bbtc_graph_t g, int32_t p, uint64_t *c
       st = BBTC_ECUDA;
       break;
     }
-    if (pl.core.bits &&
-        (st = core_launch(core_desc(g, pl, 0, 0), nullptr, 1, pl.core.nitems,
-                          pl.core.parts.quads, task_count, nt, nullptr,
-                          reinterpret_cast<int32_t *>(scratch + NOALLOC_STATUS), nullptr, 0, s)) !=
-            BBTC_OK)
+    int32_t *status = reinterpret_cast<int32_t *>(scratch + NOALLOC_STATUS);
+    const bool tasks = per_task_dev != nullptr;
+    if ((st = count_resident(g, pl, tasks, scratch + NOALLOC_HEAD, status, nullptr, task_count,
+                             nullptr, 0, s)) != BBTC_OK)
       break;
-    if (pl.nitems > 0 && !(pl.core.bits && pl.core.all)) {
-      CountParams P;
-      P.desc = pl.desc;
-      P.items = pl.items;
-      P.nitems = pl.nitems;
-      P.head = scratch + NOALLOC_HEAD;
-      P.task_count = task_count;
-      P.vcount = nullptr;
-      P.gid = nullptr;
-      P.graph_count = nullptr;
-      P.task_cycles = nullptr;
-      P.edge_sup = nullptr;
-      P.task_mask = nullptr;
-      P.status = reinterpret_cast<int32_t *>(scratch + NOALLOC_STATUS);
-      P.t0 = nullptr;
-      P.timeout_ns = 0;
-      P.use_core = 1;
-      const size_t smem = count_smem_bytes();
-      int blocks_per_sm = 0;
-      if (cudaFuncSetAttribute(k_count<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_count<0>, CT_NT,
-                                                        smem) != cudaSuccess) {
-        set_error("bbtc_count_noalloc: kernel configuration failed");
-        st = BBTC_ECUDA;
-        break;
-      }
-      if (blocks_per_sm < 1) blocks_per_sm = 1;
-      int64_t blocks = (int64_t)num_sms() * blocks_per_sm;
-      const int64_t need = (pl.nitems + CT_NT / 32 - 1) / (CT_NT / 32);
-      if (blocks > need) blocks = need;
-      k_count<0><<<(unsigned)blocks, CT_NT, smem, s>>>(P);
-      if ((st = launch_status("bbtc_count_noalloc")) != BBTC_OK) break;
-    }
     k_sum_u64<<<grid_for(nt, 256, 2), 256, 0, s>>>(
         task_count, nt, reinterpret_cast<unsigned long long *>(count_dev));
     if ((st = launch_status("bbtc_count_noalloc")) != BBTC_OK) break;

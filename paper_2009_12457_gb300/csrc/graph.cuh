@@ -43,10 +43,6 @@ struct TaskDesc {
   int32_t c_i, c_j;
   int32_t diag;  // k == j
   int32_t task;  // index in Alg. 4 order
-  // in-edges counted by the dense core (core.cu): v >= core_v0, u >= core_u0 and
-  // the flag bit of u - core_u0 set. Resident plans only; nullptr = none
-  const unsigned *core_flags;
-  int32_t core_u0, core_v0;
 };
 
 // One unit of counting work: the in-edges [x0, x1) of block G_ij (grouped by
@@ -91,6 +87,33 @@ struct Core {
   uint64_t bytes = 0;
 };
 
+// core edges of one source per work item of the core
+constexpr int CORE_CHUNK = 128;
+
+// The in-edges that the lists count (flat.cu), grouped by destination over the
+// whole graph: records {e + 1, f} (the CSR position after (u, v), the end of
+// u's row), destination v's at [inptr[v], inptr[v + 1]); work item k takes the
+// records [k * chunk, (k + 1) * chunk).
+struct Flat {
+  bool ready = false;
+  int64_t records = 0, nitems = 0, chunk = 1;
+  uint2 *rec = nullptr;
+  uint32_t *inptr = nullptr;
+  uint64_t bytes = 0;
+};
+
+struct FlatDesc {
+  const uint2 *rec;
+  const uint32_t *inptr;
+  const int64_t *rowptr;
+  const int32_t *colidx;
+  const int32_t *gid;
+  const int32_t *cuts;
+  int64_t n, records, nitems, item_base, chunk;
+  int32_t flags;  // as WorkItem::flags
+  int32_t p, task_base;
+};
+
 // Where the core's counting kernel finds one plan's core.
 struct CoreDesc {
   const int4 *items;
@@ -106,9 +129,13 @@ struct CoreDesc {
 };
 
 // Everything bbtc_count builds for one p (Sec. 2 partition, Sec. 4.2 tasks,
-// Sec. 5 estimate and order), cached on the handle until p changes.
+// Sec. 5 estimate and order), cached on the handle until p changes. Resident
+// counts use the cuts, the core and the flat in-edges; the tasks' own part
+// (tasks_ready: blocks, in-edges by part, tasks, estimates, work items) is built
+// when a call needs it (build_tasks).
 struct Plan {
   int p = 0;
+  bool tasks_ready = false;
   int64_t ntasks = 0;
   int32_t *cuts = nullptr;      // p+1
   int32_t h_cuts[65] = {0};     // host copy of the cuts
@@ -144,6 +171,9 @@ struct Plan {
   // counts, then ng per-graph counts
   unsigned long long *scratch = nullptr;
   Core core;
+  Flat flat;   // the in-edges that the core leaves
+  Flat full;   // all in-edges (detail.cu), when flat does not hold them
+  int flat_blocks_per_sm[4] = {0, 0, 0, 0};
   int blocks_per_sm[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // occupancy of each counting-kernel mode
   // streamed mode: the block arrays live in pinned host memory instead
   bool streamed = false;
@@ -205,10 +235,14 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
 // a5-a8: partition, blocks, tasks, estimate, order and work items for p.
 // partition: 0 = contiguous parts balanced on oriented edges, 1 = probe-based
 // (bounds the largest block).
-// want_core: build the dense core too (resident counts; not for INTERSECT,
-// whose lists are searched sorted by the caller's choice).
+// resident: build what a resident count uses, too (the dense core, except for
+// INTERSECT, whose lists are searched sorted by the caller's choice, and the
+// flat in-edges).
 bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold, int chunk,
-                       cudaStream_t s, int partition = 0, bool want_core = true);
+                       cudaStream_t s, int partition = 0, bool resident = true);
+// The tasks' own part of the handle's plan: blocks (split table, in-edges by
+// part), tasks, estimates, order, descriptors and work items.
+bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s);
 inline bool plan_matches(const Plan &pl, int p, int kernel_mode, int hash_threshold, int chunk,
                          int partition = 0) {
   return pl.p == p && pl.kernel_mode == kernel_mode && pl.hash_threshold == hash_threshold &&
@@ -223,22 +257,53 @@ void free_plan(Plan *pl, cudaStream_t s);
 
 // The dense core (core.cu). build_core enqueues its construction for the
 // plan's cuts; the number of items lands in core.count. core_launch counts the
-// nd descriptors' items into task_count (each at its task_base) and, when
-// given, graph_count; `descs` is read when nd > 1.
+// nd descriptors' items into task_count (per task when `tasks`, else the whole
+// at each descriptor's task_base) and, when given, graph_count; `descs` is read
+// when nd > 1.
 bbtc_status build_core(const bbtc_graph *g, Plan &pl, cudaStream_t s);
 void free_core(Plan *pl, cudaStream_t s);
 CoreDesc core_desc(const bbtc_graph *g, const Plan &pl, int64_t item_base, int32_t task_base);
-bbtc_status core_launch(const CoreDesc &one, const CoreDesc *descs, int32_t nd, int64_t nitems,
-                        int quads_max, unsigned long long *task_count, int64_t ntasks,
+bbtc_status core_launch(CoreDesc one, const CoreDesc *descs, int32_t nd, int64_t nitems,
+                        int quads_max, unsigned long long *task_count, int64_t ntasks, bool tasks,
                         unsigned long long *graph_count, int32_t *status, unsigned long long *t0,
                         uint32_t timeout_ms, cudaStream_t s);
+
+// The flat in-edges (flat.cu): all of them, or (use_core) those that the core
+// leaves. build_flat synchronises s; with use_core it reads the core's item count.
+bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cudaStream_t s);
+void free_flat(Flat *f, cudaStream_t s);
+FlatDesc flat_desc(const bbtc_graph *g, const Plan &pl, const Flat &f, int64_t item_base,
+                   int32_t task_base);
+bbtc_status configure_flat_kernels(int *blocks_per_sm);
+bbtc_status flat_launch(const FlatDesc &one, const FlatDesc *descs, int32_t nd, int64_t nitems,
+                        unsigned long long *head, unsigned long long *task_count, int64_t ntasks,
+                        bool tasks, unsigned long long *graph_count, int32_t *status,
+                        const unsigned long long *t0, uint32_t timeout_ms,
+                        const int *blocks_per_sm, cudaStream_t s);
 void free_plan_host(Plan *pl);  // pinned host copies of a streamed plan
 
 // Occupancy of the counting kernel (set at plan time so that a count only
 // enqueues work).
 bbtc_status configure_count_kernels(Plan *pl);
 
-// a9-a10: per-task counts (plan scratch, Alg. 4 order), optional per-vertex
+// a9-a10, resident: the total and, with `tasks`, per-task counts (plan scratch,
+// Alg. 4 order) and, with per_graph, per-graph counts (plan scratch), by the
+// core and the flat in-edges. Enqueues only.
+bbtc_status run_flat(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
+                     uint32_t timeout_ms, cudaStream_t s, cudaEvent_t ev_begin,
+                     cudaEvent_t ev_end);
+// a10, resident: per-vertex counts by position (vcount, device, n) and/or the
+// support of each edge by column position (edge_sup, device, m), both zeroed by
+// the caller, over all in-edges (build_full first); total (nullable) receives
+// the number of triangles. Enqueues only.
+bbtc_status build_full(bbtc_graph *g, cudaStream_t s);
+bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, unsigned long long *total,
+                          unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
+                          cudaStream_t s);
+bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
+                       unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
+                       cudaStream_t s, cudaEvent_t ev_begin, cudaEvent_t ev_end);
+// a9-a10, task by task (needs build_tasks): per-task counts, optional per-vertex
 // counts by position (vertex_count, device, n), per-graph counts (plan
 // scratch) and per-edge support by column position (edge_sup, device, m,
 // zeroed by the caller; resident plans index the oriented CSR, so this is the
@@ -257,8 +322,7 @@ bbtc_status count_reset(bbtc_graph *g, const Plan &pl, unsigned long long *verte
 bbtc_status count_launch(bbtc_graph *g, const Plan &pl, int64_t item0, int64_t nitems,
                          unsigned long long *vertex_count, bool per_graph, uint32_t timeout_ms,
                          cudaStream_t s, unsigned long long *task_cycles = nullptr,
-                         unsigned *edge_sup = nullptr, const uint8_t *task_mask = nullptr,
-                         bool use_core = false);
+                         unsigned *edge_sup = nullptr, const uint8_t *task_mask = nullptr);
 bbtc_status count_finish(const Plan &pl, cudaStream_t s);
 // The error of a nonzero status word left by the counting kernel: 1 = it
 // passed opts.timeout_ms (ETIMEOUT), 2 = a bulk copy wait ran out (EINTERNAL).

@@ -579,6 +579,8 @@ void free_plan(Plan *pl, cudaStream_t s) {
   dfree(pl->spl, s);
   dfree(pl->desc, s);
   free_core(pl, s);
+  free_flat(&pl->flat, s);
+  free_flat(&pl->full, s);
   free_plan_host(pl);
   *pl = Plan();
 }
@@ -597,9 +599,32 @@ int default_p(const bbtc_graph *g, bool budgeted) {
   return 8;
 }
 
+// Adds what a resident count uses: the dense core (not for INTERSECT, which
+// searches every list as the caller chose) and the in-edges that it leaves.
+static bbtc_status add_resident(const bbtc_graph *g, Plan &pl, cudaStream_t s) {
+  if (pl.kernel_mode != BBTC_KERNEL_INTERSECT) {
+    const bbtc_status st = build_core(g, pl, s);
+    if (st == BBTC_ENOMEM) {  // no room: the lists count everything
+      free_core(&pl, s);
+      clear_error();
+    } else {
+      BBTC_TRY(st);
+    }
+  }
+  BBTC_TRY(build_flat(g, pl, pl.flat, true, s));
+  BBTC_TRY(configure_flat_kernels(pl.flat_blocks_per_sm));
+  pl.bytes += pl.core.bytes + pl.flat.bytes;
+  return BBTC_OK;
+}
+
 bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold, int chunk_req,
-                       cudaStream_t s, int partition, bool want_core) {
-  if (plan_matches(g->plan, p, kernel_mode, hash_threshold, chunk_req, partition)) return BBTC_OK;
+                       cudaStream_t s, int partition, bool resident) {
+  if (plan_matches(g->plan, p, kernel_mode, hash_threshold, chunk_req, partition)) {
+    if (!resident || g->plan.flat.ready) return BBTC_OK;
+    const bbtc_status st = add_resident(g, g->plan, s);
+    if (st != BBTC_OK) free_plan(&g->plan, s);
+    return st;
+  }
   free_plan(&g->plan, s);
   Plan pl;
   pl.p = p;
@@ -608,8 +633,7 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   pl.chunk_req = chunk_req;
   pl.partition = partition;
   pl.ntasks = (int64_t)p * (p + 1) * (p + 2) / 6;
-  const int64_t n = g->n, m = g->m;
-  Scratch scratch(s);
+  const int64_t n = g->n;
   bbtc_status st = BBTC_OK;
 #define PLAN_TRY(expr)          \
   do {                          \
@@ -628,16 +652,45 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
     k_cuts<<<1, MAXP + 1, 0, s>>>(g->rowptr, n, p, pl.cuts);
     PLAN_TRY(launch_status("build_plan"));
   }
-
-  // a6: the blocks, read in place from the oriented CSR through the split
-  // table (per part a: |V_a| rows of p - a + 1 positions)
-  if (cudaMemcpyAsync(pl.h_cuts, pl.cuts, sizeof(int32_t) * (size_t)(p + 1),
-                      cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess) {
+  pl.h_cuts[0] = 0;
+  pl.h_cuts[p] = (int32_t)n;
+  if (p > 1 && (cudaMemcpyAsync(pl.h_cuts, pl.cuts, sizeof(int32_t) * (size_t)(p + 1),
+                                cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess)) {
     set_error("build_plan: reading the cuts failed");
     free_plan(&pl, s);
     return BBTC_ECUDA;
   }
+
+  // counting scratch, so that a count only enqueues
+  PLAN_TRY(dalloc_n(&pl.scratch, SCR_TASKS + pl.ntasks + g->ng, s));
+  pl.bytes = (uint64_t)(SCR_TASKS + pl.ntasks + g->ng) * 8;
+  if (resident) PLAN_TRY(add_resident(g, pl, s));
+  g->plan = pl;
+  return BBTC_OK;
+}
+
+bbtc_status build_full(bbtc_graph *g, cudaStream_t s) {
+  Plan &pl = g->plan;
+  if (pl.full.ready || (pl.flat.ready && !pl.core.bits)) return BBTC_OK;
+  BBTC_TRY(configure_flat_kernels(pl.flat_blocks_per_sm));
+  const bbtc_status st = build_flat(g, pl, pl.full, false, s);
+  if (st != BBTC_OK) free_flat(&pl.full, s);
+  else pl.bytes += pl.full.bytes;
+  return st;
+}
+
+bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
+  if (g->plan.tasks_ready) return BBTC_OK;
+  Plan &pl = g->plan;
+  const int p = pl.p;
+  const int64_t n = g->n, m = g->m;
+  const int kernel_mode = pl.kernel_mode, hash_threshold = pl.hash_threshold;
+  Scratch scratch(s);
+  bbtc_status st = BBTC_OK;
+
+  // a6: the blocks, read in place from the oriented CSR through the split
+  // table (per part a: |V_a| rows of p - a + 1 positions)
   {
     int64_t off = 0;
     for (int a = 0; a < p; ++a) {
@@ -766,17 +819,6 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, pl.order);
   PLAN_TRY(launch_status("build_plan"));
 
-  // the dense core (INTERSECT searches every list, as the caller chose)
-  if (want_core && kernel_mode != BBTC_KERNEL_INTERSECT) {
-    const bbtc_status cst = build_core(g, pl, s);
-    if (cst == BBTC_ENOMEM) {  // no room: the lists count everything
-      free_core(&pl, s);
-      clear_error();
-    } else {
-      PLAN_TRY(cst);
-    }
-  }
-
   // task descriptors: every block of the resident BCSR
   {
     TaskDesc *h_desc = new (std::nothrow) TaskDesc[(size_t)nt];
@@ -804,9 +846,6 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
           d.c_j = pl.h_cuts[j];
           d.diag = k == j;
           d.task = (int32_t)t;
-          d.core_flags = pl.core.flags;
-          d.core_u0 = (int32_t)pl.core.u0;
-          d.core_v0 = pl.core.v0;
         }
     bbtc_status dst = dalloc_n(&pl.desc, nt, s);
     if (dst == BBTC_OK &&
@@ -825,7 +864,7 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   const int64_t warps = (int64_t)num_sms() * 24;
   int64_t chunk = (m * (int64_t)(p < 3 ? p : 3)) / (warps * 64);
   chunk = chunk < 64 ? 64 : (chunk > 4096 ? 4096 : chunk);
-  if (chunk_req > 0) chunk = chunk_req;
+  if (pl.chunk_req > 0) chunk = pl.chunk_req;
   pl.chunk = chunk;
   uint64_t *first = nullptr;
   PLAN_TRY(scratch.get(&first, nt + 1));
@@ -834,18 +873,14 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   PLAN_TRY(launch_status("build_plan"));
   PLAN_TRY(exclusive_scan_u64(first, first, nt + 1, s));
   uint64_t nitems = 0;
-  unsigned core_items = 0;
   if (cudaMemcpyAsync(&nitems, first + nt, sizeof(uint64_t), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
-      (pl.core.count && cudaMemcpyAsync(&core_items, pl.core.count, sizeof(unsigned),
-                                        cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("build_plan: reading the work-item count failed");
     free_plan(&pl, s);
     return BBTC_ECUDA;
   }
   pl.nitems = (int64_t)nitems;
-  pl.core.nitems = (int64_t)core_items;
   PLAN_TRY(dalloc_n(&pl.items, pl.nitems, s));
   if (nitems > 0) {
     k_item_fill<<<grid_for((int64_t)nitems, 256, 8), 256, 0, s>>>(
@@ -853,14 +888,11 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
         pl.items);
     PLAN_TRY(launch_status("build_plan"));
   }
-  // counting scratch and kernel configuration, so that a count only enqueues
-  PLAN_TRY(dalloc_n(&pl.scratch, SCR_TASKS + nt + g->ng, s));
   PLAN_TRY(configure_count_kernels(&pl));
 #undef PLAN_TRY
-  pl.bytes = (uint64_t)m * sizeof(InEdge) + (uint64_t)pl.h_spl_off[p] * 4 + (uint64_t)nt * (24 + sizeof(TaskDesc)) +
-             (uint64_t)pl.nitems * sizeof(WorkItem) + (uint64_t)(SCR_TASKS + nt + g->ng) * 8 +
-             pl.core.bytes;
-  g->plan = pl;
+  pl.bytes += (uint64_t)m * sizeof(InEdge) + (uint64_t)pl.h_spl_off[p] * 4 +
+              (uint64_t)nt * (24 + sizeof(TaskDesc)) + (uint64_t)pl.nitems * sizeof(WorkItem);
+  pl.tasks_ready = true;
   return BBTC_OK;
 }
 

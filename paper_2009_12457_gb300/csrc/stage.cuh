@@ -27,10 +27,9 @@ constexpr int MIN_STAGE = 8;
 constexpr int BULK_STAGE_MIN = 64;
 constexpr int ST_NONE = 0, ST_SORTED = 1, ST_HASH = 2, ST_BITMAP = 3, ST_FILTER = 4;
 // ST_FILTER: an open-addressed table of up to FILTER_SLOTS slots in the upper
-// half of the stage, with a bit filter over a second hash of the keys in the
-// lower half. A probe reads one filter word and looks in the table only when
-// its bit is set: for a key not in the list that happens with probability at
-// most blen / FILTER_BITS (below 1/64 for blen <= 512).
+// half of the stage, with a filter in the lower half: two bits per key in one
+// word (see InFilter). A probe reads one filter word and looks in the table only
+// when both bits are set.
 constexpr int FILTER_WORDS = STAGE / 2;
 constexpr int FILTER_BITS_LOG2 = 15;
 constexpr int FILTER_SLOTS = STAGE - FILTER_WORDS;
@@ -40,10 +39,6 @@ constexpr int32_t EMPTY = -1;
 
 __device__ __forceinline__ uint32_t hash_slot(int32_t w, int log2h) {
   return ((uint32_t)w * 2654435761u) >> (32 - log2h);
-}
-
-__device__ __forceinline__ uint32_t filter_bit(int32_t w) {
-  return ((uint32_t)w * 0x85EBCA6Bu) >> (32 - FILTER_BITS_LOG2);
 }
 
 // Membership of w in the sorted list stage[0, len): lower bound by a fixed
@@ -72,17 +67,58 @@ __device__ __forceinline__ bool hash_contains(const int32_t *stage, int log2h, i
   return false;
 }
 
-// The table half of an ST_FILTER stage, reached only when the filter bit is set.
-__device__ __forceinline__ bool filter_verify(const int32_t *table, int log2h, int32_t w) {
-  return hash_contains(table, log2h, w);
-}
+// Bit c of the result: column c of the quad is in the list.
+struct InBitmap {  // window of words from `word0` on, zero word at index gw
+  const uint32_t *bm;
+  uint32_t word0, gw;
+  __device__ __forceinline__ uint32_t one(int32_t w) const {
+    const uint32_t word = bm[min(((uint32_t)w >> 5) - word0, gw)];
+    return word >> ((uint32_t)w & 31u);
+  }
+  __device__ __forceinline__ uint32_t count(const int4 &w, uint32_t m) const {
+    return (one(w.x) & m & 1u) + (one(w.y) & (m >> 1) & 1u) + (one(w.z) & (m >> 2) & 1u) +
+           (one(w.w) & (m >> 3) & 1u);
+  }
+  __device__ __forceinline__ uint32_t bits(const int4 &w, uint32_t m) const {
+    return ((one(w.x) & 1u) | ((one(w.y) & 1u) << 1) | ((one(w.z) & 1u) << 2) |
+            ((one(w.w) & 1u) << 3)) & m;
+  }
+};
 
-__device__ __forceinline__ uint32_t filter_lookup(const int32_t *stage, int log2h, int32_t w) {
-  const uint32_t h = filter_bit(w);
-  const uint32_t word = reinterpret_cast<const uint32_t *>(stage)[h >> 5];
-  if (((word >> (h & 31u)) & 1u) == 0u) return 0u;
-  return filter_verify(stage + FILTER_WORDS, log2h, w) ? 1u : 0u;
-}
+// A table behind a filter of one word per key with two bits in it (both from
+// the word's hash), so that one load rejects most keys that are not in the list.
+struct InFilter {
+  const uint32_t *filter;
+  const int32_t *table;
+  int log2h;
+  static __device__ __forceinline__ uint32_t hash(int32_t w) { return (uint32_t)w * 0x85EBCA6Bu; }
+  static __device__ __forceinline__ uint32_t word_of(uint32_t h) {
+    return h >> (32 - (FILTER_BITS_LOG2 - 5));
+  }
+  static __device__ __forceinline__ uint32_t bits_of(uint32_t h) {
+    return (1u << (h & 31u)) | (1u << ((h >> 10) & 31u));
+  }
+  __device__ __forceinline__ uint32_t maybe(int32_t w) const {
+    const uint32_t h = hash(w);
+    const uint32_t word = filter[word_of(h)];
+    return (word >> (h & 31u)) & (word >> ((h >> 10) & 31u));
+  }
+  __device__ __forceinline__ uint32_t bits(const int4 &w, uint32_t m) const {
+    uint32_t cand = ((maybe(w.x) & 1u) | ((maybe(w.y) & 1u) << 1) | ((maybe(w.z) & 1u) << 2) |
+                     ((maybe(w.w) & 1u) << 3)) & m;
+    uint32_t hit = 0;
+    while (cand) {
+      const int c = __ffs(cand) - 1;
+      cand &= cand - 1;
+      const int32_t x = c == 0 ? w.x : c == 1 ? w.y : c == 2 ? w.z : w.w;
+      hit |= (uint32_t)hash_contains(table, log2h, x) << c;
+    }
+    return hit;
+  }
+  __device__ __forceinline__ uint32_t count(const int4 &w, uint32_t m) const {
+    return __popc(bits(w, m));
+  }
+};
 
 // ------------------------------------------------ bulk copies (TMA, PTX)
 

@@ -119,7 +119,11 @@ bbtc_status plan_to_host(const bbtc_graph *g, Plan &pl, int64_t m, cudaStream_t 
   pl.rp = nullptr;
   pl.ci = nullptr;
   pl.ie = nullptr;
-  free_core(&pl, s);  // streamed counts keep nothing but the pool's blocks
+  // streamed counts keep nothing but the pool's blocks
+  pl.bytes -= pl.core.bytes + pl.flat.bytes + pl.full.bytes;
+  free_core(&pl, s);
+  free_flat(&pl.flat, s);
+  free_flat(&pl.full, s);
   // work items in Alg. 4 task order (a task's items stay together and keep
   // their order), so that the tasks sharing an in-edge block are consecutive
   if (pl.nitems > 0) {
