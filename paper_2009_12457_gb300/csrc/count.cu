@@ -507,17 +507,16 @@ __global__ void k_sum_u64(const unsigned long long *__restrict__ in, int64_t cou
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
 }
 
-__global__ void k_wedges(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                         const int32_t *__restrict__ esrc, int64_t m, int64_t n,
+// sum over oriented edges (u, v) of d+(v) = sum over v of (in-degree of v) d+(v), the
+// in-degree being the undirected degree minus d+(v); and sum over u of C(d+(u), 2)
+__global__ void k_wedges(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ perm,
+                         const int32_t *__restrict__ deg, int64_t n,
                          unsigned long long *__restrict__ sums) {
   unsigned long long win = 0, wout = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-    const int32_t v = colidx[e];
-    win += (unsigned long long)(rowptr[v + 1] - rowptr[v]);
-  }
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += stride) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x) {
     const unsigned long long d = (unsigned long long)(rowptr[u + 1] - rowptr[u]);
+    win += ((unsigned long long)deg[perm[u]] - d) * d;
     wout += d * (d > 0 ? d - 1 : 0) / 2;
   }
   win = warp_sum(win);
@@ -578,10 +577,8 @@ bbtc_status wedge_sums(const bbtc_graph *g, uint64_t *in_sum, uint64_t *out_sum,
   unsigned long long *sums = nullptr;
   BBTC_TRY(scratch.get(&sums, 2));
   BBTC_CUDA(cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), s));
-  const int64_t work = g->m > g->n ? g->m : g->n;
-  if (work > 0) {
-    k_wedges<<<grid_for(work, 256, 16), 256, 0, s>>>(g->rowptr, g->colidx, g->esrc, g->m, g->n,
-                                                     sums);
+  if (g->n > 0) {
+    k_wedges<<<grid_for(g->n, 256, 16), 256, 0, s>>>(g->rowptr, g->perm, g->deg, g->n, sums);
     BBTC_LAUNCH_CHECK();
   }
   unsigned long long h[2] = {0, 0};

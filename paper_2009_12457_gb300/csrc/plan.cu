@@ -815,7 +815,14 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
   k_tasks<<<(p * p * p + 127) / 128, 128, 0, s>>>(pl.boff, pl.cuts, p, pl.tasks, pl.est, okeys,
                                                   ovals);
   PLAN_TRY(launch_status("build_plan"));
-  PLAN_TRY(radix_sort(okeys, okeys_alt, ovals, ovals_alt, nt, 0, 64, s, &in_alt));
+  int32_t *serr = nullptr;
+  PLAN_TRY(scratch.get(&serr, 1));
+  if (cudaMemsetAsync(serr, 0, sizeof(int32_t), s) != cudaSuccess) {
+    set_error("build_plan: cudaMemsetAsync failed");
+    free_plan(&pl, s);
+    return BBTC_ECUDA;
+  }
+  PLAN_TRY(radix_sort(okeys, okeys_alt, ovals, ovals_alt, nt, 0, 64, s, serr, &in_alt));
   k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, pl.order);
   PLAN_TRY(launch_status("build_plan"));
 
@@ -873,13 +880,17 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
   PLAN_TRY(launch_status("build_plan"));
   PLAN_TRY(exclusive_scan_u64(first, first, nt + 1, s));
   uint64_t nitems = 0;
+  int32_t sort_err = 0;
   if (cudaMemcpyAsync(&nitems, first + nt, sizeof(uint64_t), cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
+      cudaMemcpyAsync(&sort_err, serr, sizeof(int32_t), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("build_plan: reading the work-item count failed");
     free_plan(&pl, s);
     return BBTC_ECUDA;
   }
+  if (sort_err) PLAN_TRY(sort_failed("build_plan"));
   pl.nitems = (int64_t)nitems;
   PLAN_TRY(dalloc_n(&pl.items, pl.nitems, s));
   if (nitems > 0) {

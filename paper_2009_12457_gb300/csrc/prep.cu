@@ -12,172 +12,94 @@ namespace bbtc {
 
 namespace {
 
-constexpr int EK_NT = 256;
-constexpr int EK_TILE = 2048;
-
-// rowptr[0] == 0 and non-decreasing; error bit 1 otherwise.
+// rowptr[0] == 0 and non-decreasing; error bit 1 otherwise. With deg, also
+// deg[r] = the row's length (pass 0 takes off what is no edge).
 __global__ void k_validate_rowptr(const int64_t *__restrict__ rowptr, int64_t n,
-                                  int32_t *__restrict__ err) {
+                                  int32_t *__restrict__ deg, int32_t *__restrict__ err) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    if (rowptr[i] > rowptr[i + 1]) atomicOr(err, 1);
+    const int64_t b = rowptr[i], e = rowptr[i + 1];
+    if (b > e) atomicOr(err, 1);
+    if (deg) deg[i] = (int32_t)(e - b);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0 && rowptr[0] != 0) atomicOr(err, 1);
-}
-
-// a1: one 64-bit key (min << nb) | max per input entry joining two different
-// vertices. Self-loops (and, for symmetric input, entries with u > v) emit
-// nothing. Two passes over tiles of EK_TILE entries: count the keys of each
-// tile, then (after a scan of the counts) write them compacted. Thread t of a
-// tile owns entries [t*EK_ITEMS, (t+1)*EK_ITEMS) and walks their rows forward
-// from one binary search inside the tile's row window.
-constexpr int EK_ITEMS = EK_TILE / EK_NT;
-
-// For a batch (voff != nullptr), graph g owns rows [voff[g], voff[g+1]) and
-// its entries are local ids in [0, voff[g+1] - voff[g]), shifted by voff[g].
-template <bool WRITE>
-__global__ void __launch_bounds__(EK_NT) k_emit_keys(const int64_t *__restrict__ rowptr,
-                                                     const int32_t *__restrict__ colidx,
-                                                     int64_t n, int64_t nnz, int nb,
-                                                     bool symmetric,
-                                                     const int64_t *__restrict__ voff, int ng,
-                                                     uint64_t *__restrict__ tile_count,
-                                                     uint64_t *__restrict__ keys,
-                                                     int32_t *__restrict__ err) {
-  __shared__ int64_t win[2];
-  __shared__ uint64_t tmp[EK_NT / 32 + 1];
-  const int64_t ntiles = (nnz + EK_TILE - 1) / EK_TILE;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t t0 = tile * EK_TILE;
-    const int64_t t1 = t0 + EK_TILE < nnz ? t0 + EK_TILE : nnz;
-    if (threadIdx.x < 2) {
-      // last row r in [0, n) with rowptr[r] <= target
-      int64_t target = threadIdx.x == 0 ? t0 : t1 - 1;
-      int64_t lo = 0, hi = n;  // invariant: rowptr[lo] <= target
-      while (hi - lo > 1) {
-        int64_t mid = (lo + hi) >> 1;
-        if (rowptr[mid] <= target) lo = mid; else hi = mid;
-      }
-      win[threadIdx.x] = lo;
-    }
-    __syncthreads();
-    const int64_t rlo = win[0], rhi = win[1];
-    const int64_t first = t0 + (int64_t)threadIdx.x * EK_ITEMS;
-    uint64_t key[EK_ITEMS];
-    uint64_t c = 0;
-    int64_t u = rlo;
-    if (first < t1) {
-      int64_t lo = rlo, hi = rhi + 1;
-      while (hi - lo > 1) {
-        int64_t mid = (lo + hi) >> 1;
-        if (rowptr[mid] <= first) lo = mid; else hi = mid;
-      }
-      u = lo;
-    }
-    int gi = 0;
-    int64_t gbase = 0, gend = n;
-    if (voff) {
-      int lo = 0, hi = ng;  // last graph with voff[lo] <= u
-      while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (voff[mid] <= u) lo = mid; else hi = mid;
-      }
-      gi = lo;
-      gbase = voff[gi];
-      gend = voff[gi + 1];
-    }
-#pragma unroll
-    for (int i = 0; i < EK_ITEMS; ++i) {
-      const int64_t idx = first + i;
-      key[i] = ~0ull;
-      if (idx < t1) {
-        while (u < rhi && rowptr[u + 1] <= idx) ++u;
-        if (voff) {
-          while (u >= gend && gi + 1 < ng) {
-            ++gi;
-            gbase = voff[gi];
-            gend = voff[gi + 1];
-          }
-        }
-        int64_t v = colidx[idx];
-        const bool in_range = voff ? (v >= 0 && v < gend - gbase) : (v >= 0 && v < n);
-        v += gbase;
-        if (!in_range) {
-          if (!WRITE) atomicOr(err, 2);
-        } else if (v != u && !(symmetric && u > v)) {
-          uint64_t a = (uint64_t)(u < v ? u : v), b = (uint64_t)(u < v ? v : u);
-          key[i] = (a << nb) | b;
-          ++c;
-        }
-      }
-    }
-    uint64_t total;
-    uint64_t pos = block_exclusive_scan<uint64_t, EK_NT>(c, tmp, &total);
-    if (!WRITE) {
-      if (threadIdx.x == 0) tile_count[tile] = total;
-    } else {
-      pos += tile_count[tile];
-#pragma unroll
-      for (int i = 0; i < EK_ITEMS; ++i)
-        if (key[i] != ~0ull) keys[pos++] = key[i];
-    }
-  }
 }
 
 constexpr int UQ_NT = 512;
 constexpr int UQ_ITEMS = 8;
 constexpr int UQ_TILE = UQ_NT * UQ_ITEMS;
 
-__device__ __forceinline__ bool is_head(const uint64_t *keys, int64_t i, uint64_t sentinel) {
-  uint64_t k = keys[i];
-  return k != sentinel && (i == 0 || keys[i - 1] != k);
-}
-
 __global__ void __launch_bounds__(UQ_NT) k_unique_count(const uint64_t *__restrict__ keys,
                                                         int64_t count, uint64_t sentinel,
+                                                        const int32_t *__restrict__ err,
                                                         uint64_t *__restrict__ block_counts) {
   __shared__ uint64_t tmp[UQ_NT / 32 + 1];
+  if (*err & SORT_FAILED) count = 0;  // the keys are not in order: nothing is read from them
   const int64_t base = (int64_t)blockIdx.x * UQ_TILE + (int64_t)threadIdx.x * UQ_ITEMS;
   uint64_t c = 0;
+  uint64_t k = base > 0 && base < count ? keys[base - 1] : sentinel;
 #pragma unroll
   for (int i = 0; i < UQ_ITEMS; ++i)
-    if (base + i < count && is_head(keys, base + i, sentinel)) ++c;
+    if (base + i < count) {
+      const uint64_t x = keys[base + i];
+      if (x != sentinel && (base + i == 0 || x != k)) ++c;
+      k = x;
+    }
   uint64_t total;
   block_exclusive_scan<uint64_t, UQ_NT>(c, tmp, &total);
   if (threadIdx.x == 0) block_counts[blockIdx.x] = total;
 }
 
-// a1 + a2: compact the distinct keys and count each endpoint's degree. Keys
-// are sorted by their first endpoint, so lanes holding equal endpoints add
-// once per group (match_any) instead of once per edge.
+// a1 + a2: compact the distinct keys and count each endpoint's degree. Keys are
+// sorted by their first endpoint, so a thread adds once per run of equal first
+// endpoints among its eight keys (and a warp within one run once); the second
+// endpoints differ from lane to lane and are added one by one.
 __global__ void __launch_bounds__(UQ_NT) k_unique_write(const uint64_t *__restrict__ keys,
                                                         int64_t count, uint64_t sentinel,
+                                                        const int32_t *__restrict__ err,
                                                         const uint64_t *__restrict__ block_off,
                                                         int nb, uint64_t *__restrict__ ukeys,
                                                         int32_t *__restrict__ deg) {
   __shared__ uint64_t tmp[UQ_NT / 32 + 1];
+  if (*err & SORT_FAILED) count = 0;
   const int64_t base = (int64_t)blockIdx.x * UQ_TILE + (int64_t)threadIdx.x * UQ_ITEMS;
   const unsigned lane = threadIdx.x & 31u;
-  bool head[UQ_ITEMS];
-  uint64_t c = 0;
+  uint64_t k[UQ_ITEMS];
+  unsigned heads = 0;
+  uint64_t prev = base > 0 && base < count ? keys[base - 1] : sentinel;
 #pragma unroll
   for (int i = 0; i < UQ_ITEMS; ++i) {
-    head[i] = base + i < count && is_head(keys, base + i, sentinel);
-    c += head[i];
+    k[i] = base + i < count ? keys[base + i] : sentinel;
+    if (k[i] != sentinel && (base + i == 0 || k[i] != prev)) heads |= 1u << i;
+    prev = k[i];
   }
   uint64_t total;
-  uint64_t pos = block_exclusive_scan<uint64_t, UQ_NT>(c, tmp, &total) + block_off[blockIdx.x];
+  uint64_t pos = block_exclusive_scan<uint64_t, UQ_NT>((uint64_t)__popc(heads), tmp, &total) +
+                 block_off[blockIdx.x];
   const uint64_t mask = (1ull << nb) - 1ull;
+  int64_t cur = -1;
+  int cnt = 0, groups = 0;
 #pragma unroll
   for (int i = 0; i < UQ_ITEMS; ++i) {
-    uint64_t k = head[i] ? keys[base + i] : 0;
-    if (head[i]) ukeys[pos++] = k;
-    const int64_t a = head[i] ? (int64_t)(k >> nb) : -1;
-    const int64_t b = head[i] ? (int64_t)(k & mask) : -1;
-    unsigned peers = __match_any_sync(0xffffffffu, a);
-    if (a >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[a], __popc(peers));
-    peers = __match_any_sync(0xffffffffu, b);
-    if (b >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[b], __popc(peers));
+    if ((heads >> i) & 1u) {
+      ukeys[pos++] = k[i];
+      const int64_t a = (int64_t)(k[i] >> nb);
+      atomicAdd(&deg[k[i] & mask], 1);
+      if (a != cur) {
+        if (cur >= 0) atomicAdd(&deg[cur], cnt);
+        cur = a;
+        cnt = 0;
+        ++groups;
+      }
+      ++cnt;
+    }
+  }
+  const int64_t cur0 = __shfl_sync(0xffffffffu, cur, 0);
+  if (__all_sync(0xffffffffu, groups == 1 && cur == cur0)) {
+    const int tot = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) atomicAdd(&deg[cur0], tot);
+  } else if (cur >= 0) {
+    atomicAdd(&deg[cur], cnt);
   }
 }
 
@@ -190,11 +112,13 @@ __global__ void k_rank_keys(const int32_t *__restrict__ deg, int64_t n, int nb,
 }
 
 __global__ void k_rank_finish(const uint64_t *__restrict__ sorted, int64_t n, int nb,
-                              int32_t *__restrict__ perm, int32_t *__restrict__ rank) {
+                              const int32_t *__restrict__ err, int32_t *__restrict__ perm,
+                              int32_t *__restrict__ rank) {
   const uint64_t mask = (1ull << nb) - 1ull;
+  const bool failed = (*err & SORT_FAILED) != 0;  // then any order: the caller reports it
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n;
        r += (int64_t)gridDim.x * blockDim.x) {
-    int32_t v = (int32_t)(sorted[r] & mask);
+    int32_t v = failed ? (int32_t)r : (int32_t)(sorted[r] & mask);
     perm[r] = v;
     rank[v] = (int32_t)r;
   }
@@ -216,40 +140,31 @@ __global__ void k_graph_of_position(const int32_t *__restrict__ perm, int64_t n,
   }
 }
 
-// a4 keys: each edge {a,b} as (min(rank) << nb) | max(rank).
-__global__ void k_orient_keys(const uint64_t *__restrict__ ukeys, int64_t m, int nb,
-                              const int32_t *__restrict__ rank, uint64_t *__restrict__ okeys) {
+// a4 by counting: each edge's slot within its source's row (the count before it),
+// and the rows' lengths; then the scatter into the rows, which are sorted after.
+__global__ void k_orient_count(const uint64_t *__restrict__ ukeys, int64_t m, int nb,
+                               const int32_t *__restrict__ rank, uint64_t *__restrict__ okeys,
+                               unsigned *__restrict__ slot,
+                               unsigned long long *__restrict__ rowlen) {
   const uint64_t mask = (1ull << nb) - 1ull;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t k = ukeys[e];
-    uint64_t ra = (uint64_t)rank[k >> nb], rb = (uint64_t)rank[k & mask];
-    okeys[e] = ra < rb ? (ra << nb) | rb : (rb << nb) | ra;
+    const uint64_t k = ukeys[e];
+    const uint64_t ra = (uint64_t)rank[k >> nb], rb = (uint64_t)rank[k & mask];
+    const uint64_t lo = ra < rb ? ra : rb, hi = ra < rb ? rb : ra;
+    okeys[e] = (lo << nb) | hi;
+    slot[e] = (unsigned)atomicAdd(&rowlen[lo], 1ull);
   }
 }
 
-// Oriented CSR from the sorted oriented keys: colidx, the source of each
-// edge, and the row lengths (counted into rowptr[src], warp-aggregated; a scan
-// turns them into offsets).
-__global__ void k_csr_finish(const uint64_t *__restrict__ okeys, int64_t m, int nb,
-                             int32_t *__restrict__ colidx, int32_t *__restrict__ esrc,
-                             unsigned long long *__restrict__ rowlen) {
+__global__ void k_orient_scatter(const uint64_t *__restrict__ okeys,
+                                 const unsigned *__restrict__ slot, int64_t m, int nb,
+                                 const int64_t *__restrict__ rowptr, int32_t *__restrict__ colidx) {
   const uint64_t mask = (1ull << nb) - 1ull;
-  const unsigned lane = threadIdx.x & 31u;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < m; base += stride) {
-    const int64_t e = base + threadIdx.x;
-    const bool valid = e < m;
-    int64_t s = -1;
-    if (valid) {
-      uint64_t k = okeys[e];
-      s = (int64_t)(k >> nb);
-      colidx[e] = (int32_t)(k & mask);
-      esrc[e] = (int32_t)s;
-    }
-    unsigned peers = __match_any_sync(0xffffffffu, s);
-    if (valid && lane == (unsigned)(__ffs(peers) - 1))
-      atomicAdd(&rowlen[s], (unsigned long long)__popc(peers));
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t k = okeys[e];
+    colidx[rowptr[k >> nb] + slot[e]] = (int32_t)(k & mask);
   }
 }
 
@@ -285,42 +200,97 @@ __global__ void k_tile_rows(const int64_t *__restrict__ rowptr, int64_t n, int64
   }
 }
 
-// Pass over the entries: thread t of a tile owns entries [t*8, t*8+8) and walks
-// their rows forward from one search inside the tile's row window; the counts
-// of a row are added once per thread. MODE 0:
-// degree of u += first copies of v != u, flag unsorted rows and out-of-range
-// ids. MODE 1: out-degree at rank(u) += first copies with rank(v) > rank(u).
-// MODE 2: scatter rank(v) into row rank(u) (any order; rows are sorted after;
-// the rows' sources are written afterwards by k_fill_esrc, with coalesced stores).
-// When rr is given, MODE 1 also stores each entry's rank(v) when the entry is
-// such an upward first copy (else -1), and MODE 2 reads it back in order
-// instead of gathering rank(v) a second time.
-// For a batch (voff != nullptr), the entries of a row of graph g are local ids
-// in [0, voff[g+1] - voff[g]), shifted here by voff[g].
-template <int MODE>
-__global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ rowptr,
-                                                    const int32_t *__restrict__ colidx, int64_t n,
-                                                    int64_t nnz,
-                                                    const int64_t *__restrict__ tile_rows,
-                                                    int32_t *__restrict__ deg,
-                                                    const int32_t *__restrict__ rank,
-                                                    unsigned long long *__restrict__ dplus,
-                                                    const int64_t *__restrict__ rowptr_o,
-                                                    unsigned int *__restrict__ cursor,
-                                                    int32_t *__restrict__ colidx_o,
-                                                    int32_t *__restrict__ err,
-                                                    const int64_t *__restrict__ voff, int ng,
-                                                    int32_t *__restrict__ rr) {
-  const unsigned lane = threadIdx.x & 31u;
+// The rows of a tile's entries. The starts of the rows inside the tile are marked
+// in a bit mask (and each start's row beside it), so that an entry's row is that of
+// the last mark at or before it: no search and no walk along row pointers, whose
+// dependent loads bounded these passes before (0.38 ms for pass 0 over the 67 M
+// entries of R-MAT scale 21, 1.4 TB/s for a pass that only streams them).
+struct TileRows {
+  uint32_t start[SP_TILE / 32];  // marks
+  unsigned long long words;      // words of `start` with a mark (SP_TILE / 32 = 64)
+  int32_t row[SP_TILE];          // row of each mark
+  int first_is_start;            // the tile's first entry begins its row
+};
+static_assert(SP_TILE / 32 == 64 && SP_ITEMS == 8, "tile layout");
+
+// Marks the tile of entries [t0, t1), whose rows are rlo .. rhi. Block-wide.
+__device__ __forceinline__ void tile_rows_mark(TileRows &tr, const int64_t *__restrict__ rowptr,
+                                               int64_t t0, int64_t t1, int64_t rlo, int64_t rhi) {
+  __syncthreads();  // the tile before this one has been read
+  if (threadIdx.x < 64) tr.start[threadIdx.x] = threadIdx.x == 0 ? 1u : 0u;
+  if (threadIdx.x == 0) {
+    tr.row[0] = (int32_t)rlo;  // the row that holds entry t0
+    tr.first_is_start = rowptr[rlo] == t0;
+  }
+  __syncthreads();
+  for (int64_t r = rlo + 1 + threadIdx.x; r <= rhi; r += SP_NT) {
+    const int64_t b = rowptr[r], e = rowptr[r + 1];
+    if (e > b && b > t0 && b < t1) {  // (row pointers are checked, but only read back later)
+      const int x = (int)(b - t0);
+      atomicOr(&tr.start[x >> 5], 1u << (x & 31));
+      tr.row[x] = (int32_t)r;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const unsigned lo = __ballot_sync(0xffffffffu, tr.start[threadIdx.x] != 0u);
+    const unsigned hi = __ballot_sync(0xffffffffu, tr.start[threadIdx.x + 32] != 0u);
+    if (threadIdx.x == 0) tr.words = ((unsigned long long)hi << 32) | lo;
+  }
+  __syncthreads();
+}
+
+// Row of the tile's entry x (x a multiple of 8), and the marks of x .. x + 7.
+__device__ __forceinline__ int32_t tile_row_at(const TileRows &tr, int x, unsigned *marks) {
+  const int w = x >> 5;
+  const uint32_t word = tr.start[w];
+  *marks = (word >> (x & 31)) & 0xffu;
+  uint32_t below = word & ((2u << (x & 31)) - 1u);  // marks at or before x in its word
+  int at = w;
+  if (!below) {  // word 0 holds mark 0, so an earlier word has one
+    at = 63 - __clzll((long long)(tr.words & ((1ull << w) - 1ull)));
+    below = tr.start[at];
+  }
+  return tr.row[at * 32 + 31 - __clz(below)];
+}
+
+// The eight entries of a thread, by two 16-byte loads where they are aligned.
+__device__ __forceinline__ void load_entries(const int32_t *__restrict__ colidx, int64_t first,
+                                             int64_t t1, bool aligned, int32_t (&v)[SP_ITEMS]) {
+  if (aligned && first + SP_ITEMS <= t1) {
+    const int4 a = *reinterpret_cast<const int4 *>(colidx + first);
+    const int4 b = *reinterpret_cast<const int4 *>(colidx + first + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < SP_ITEMS; ++i) v[i] = first + i < t1 ? colidx[first + i] : -1;
+  }
+}
+
+// a1: one 64-bit key (min << nb) | max per input entry that joins two different
+// vertices; the others (and, for symmetric input, entries with u > v) get the
+// sentinel, which sorts last.
+__global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__ rowptr,
+                                                     const int32_t *__restrict__ colidx, int64_t n,
+                                                     int64_t nnz, int nb, bool symmetric,
+                                                     bool aligned, uint64_t sentinel,
+                                                     const int64_t *__restrict__ tile_rows,
+                                                     const int64_t *__restrict__ voff, int ng,
+                                                     uint64_t *__restrict__ keys,
+                                                     int32_t *__restrict__ err) {
+  __shared__ TileRows tr;
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t t0 = tile * SP_TILE;
     const int64_t t1 = t0 + SP_TILE < nnz ? t0 + SP_TILE : nnz;
-    const int64_t rlo = tile_rows[tile], rhi = tile_rows[tile + 1];
     const int64_t first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
-    int64_t u = first < t1 ? row_of_first(rowptr, n, first, rlo, rhi + 1) : rlo;
-    int64_t row_end = rowptr[u + 1];
-    int32_t ru = MODE > 0 ? rank[u] : 0;
+    int32_t w[SP_ITEMS];
+    if (first < t1) load_entries(colidx, first, t1, aligned, w);
+    tile_rows_mark(tr, rowptr, t0, t1, tile_rows[tile], tile_rows[tile + 1]);
+    if (first >= t1) continue;
+    unsigned marks = 0;
+    int32_t u = tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &marks);
     int gi = 0;
     int64_t gbase = 0, gend = n;
     if (voff) {
@@ -333,33 +303,13 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
       gbase = voff[gi];
       gend = voff[gi + 1];
     }
-    // key of each item: MODE 0 its row u when it is the first copy of a
-    // neighbour != u; MODE 1/2 rank(u) when it is such a copy and points up;
-    // else -1. Keys >= 0 never decrease along a thread's items (rows ascend), so
-    // equal keys form one group per row and each group costs one atomic.
-    int64_t key[SP_ITEMS];
-    int32_t val[SP_ITEMS];  // MODE 2: rank(v)
-    int32_t up[SP_ITEMS];   // MODE 1: the entry's upward rank, else -1 (stored in rr)
+    bool bad = false;
+    uint64_t key[SP_ITEMS];
 #pragma unroll
     for (int i = 0; i < SP_ITEMS; ++i) {
-      const int64_t e = first + i;
-      key[i] = -1;
-      val[i] = 0;
-      up[i] = -1;
-      if (e < t1) {
-        while (e >= row_end) {  // next non-empty row
-          ++u;
-          row_end = rowptr[u + 1];
-          if (MODE > 0) ru = rank[u];
-        }
-        if (MODE == 2 && rr) {  // the upward rank stored by MODE 1
-          const int32_t rv = rr[e];
-          if (rv >= 0) {
-            key[i] = ru;
-            val[i] = rv;
-          }
-          continue;
-        }
+      key[i] = sentinel;
+      if (first + i < t1) {
+        if (i > 0 && ((marks >> i) & 1u)) u = tr.row[(int)threadIdx.x * SP_ITEMS + i];
         if (voff) {
           while (u >= gend && gi + 1 < ng) {
             ++gi;
@@ -367,85 +317,215 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
             gend = voff[gi + 1];
           }
         }
-        const int32_t vl = colidx[e];  // local to the row's graph
-        const bool first_in_row = e == rowptr[u];
-        const int32_t prev = first_in_row ? -1 : colidx[e - 1];
-        const bool in_range = vl >= 0 && (int64_t)vl < gend - gbase;
-        if (MODE == 0) {
-          if (!in_range) atomicOr(err, 2);
-          else if (!first_in_row && prev > vl) atomicOr(err, 4);
-        }
-        const int32_t v = in_range ? (int32_t)(vl + gbase) : 0;
-        const bool head = in_range && v != u && (first_in_row || prev != vl);
-        if (MODE == 0) {
-          key[i] = head ? u : -1;
-        } else {
-          const int32_t rv = head ? rank[v] : -1;
-          if (head && rv > ru) key[i] = ru;
-          val[i] = rv;
-          if (MODE == 1) up[i] = head && rv > ru ? rv : -1;
+        const int64_t v = (int64_t)w[i] + gbase;
+        if (w[i] < 0 || v >= gend) bad = true;
+        else if (v != u && !(symmetric && u > v)) {
+          const uint64_t a = (uint64_t)(u < v ? u : v), b = (uint64_t)(u < v ? v : u);
+          key[i] = (a << nb) | b;
         }
       }
     }
-    if (MODE == 1 && rr) {
-      // rr + first is 32-byte aligned (first is a multiple of 8 entries)
-      if (first + SP_ITEMS <= t1) {
-        int4 *d = reinterpret_cast<int4 *>(rr + first);
-        d[0] = make_int4(up[0], up[1], up[2], up[3]);
-        d[1] = make_int4(up[4], up[5], up[6], up[7]);
-      } else {
+    if (bad) atomicOr(err, 2);
+    if (first + SP_ITEMS <= t1) {  // keys + first is 64-byte aligned
+      ulonglong2 *d = reinterpret_cast<ulonglong2 *>(keys + first);
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; i += 2) d[i / 2] = make_ulonglong2(key[i], key[i + 1]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i)
+        if (first + i < t1) keys[first + i] = key[i];
+    }
+  }
+}
+
+// Passes over the entries of a symmetric CSR, thread t of a tile owning entries
+// [8t, 8t + 8). An entry is an edge's first copy when it differs from its row's
+// vertex and from the entry before it in the row. The next tile's entries are
+// loaded while this one is worked on.
+// MODE 0: degree of u -= entries that are no first copy; flag unsorted rows and
+// out-of-range ids.
+// MODE 1: the ranks of the upward first copies (rank(v) > rank(u)) move to the
+// front of u's own entries in `up` (an array like colidx; any order), and
+// dplus[u] counts them. The rows are picked up in rank order by the row sort, so
+// no second pass over the entries scatters them (it read every entry's stored
+// rank and took 0.32 ms on R-MAT scale 21). When there is no room for `up` (null),
+// the pass only counts, and a second one with `place` (the rows' offsets by rank)
+// writes into the oriented rows themselves.
+// For a batch (voff != nullptr), the entries of a row of graph g are local ids
+// in [0, voff[g+1] - voff[g]), shifted here by voff[g].
+template <int MODE>
+__global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ rowptr,
+                                                    const int32_t *__restrict__ colidx, int64_t n,
+                                                    int64_t nnz, bool aligned,
+                                                    const int64_t *__restrict__ tile_rows,
+                                                    int32_t *__restrict__ deg,
+                                                    const int32_t *__restrict__ rank,
+                                                    unsigned *__restrict__ dplus,
+                                                    int32_t *__restrict__ up,
+                                                    const int64_t *__restrict__ place,
+                                                    int32_t *__restrict__ err,
+                                                    const int64_t *__restrict__ voff, int ng) {
+  __shared__ TileRows tr;
+  const unsigned lane = threadIdx.x & 31u;
+  const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
+  int32_t next[SP_ITEMS];
+  auto load = [&](int64_t tile) {
+    const int64_t t0 = tile * SP_TILE, first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
+    const int64_t t1 = t0 + SP_TILE < nnz ? t0 + SP_TILE : nnz;
+    if (tile < ntiles && first < t1) load_entries(colidx, first, t1, aligned, next);
+  };
+  load(blockIdx.x);
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t t0 = tile * SP_TILE;
+    const int64_t t1 = t0 + SP_TILE < nnz ? t0 + SP_TILE : nnz;
+    const int64_t first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
+    const bool mine = first < t1;
+    int32_t w[SP_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SP_ITEMS; ++i) w[i] = mine ? next[i] : -1;
+    load(tile + gridDim.x);
+    tile_rows_mark(tr, rowptr, t0, t1, tile_rows[tile], tile_rows[tile + 1]);
+    unsigned marks = 0;
+    int32_t u = mine ? tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &marks) : 0;
+    if (threadIdx.x == 0 && !tr.first_is_start) marks &= ~1u;  // t0 goes on with its row
+    int32_t prev = __shfl_up_sync(0xffffffffu, w[SP_ITEMS - 1], 1);
+    if (lane == 0) prev = first > 0 && mine ? colidx[first - 1] : -1;
+    int gi = 0;
+    int64_t gbase = 0, gend = n;
+    if (voff && mine) {
+      int lo = 0, hi = ng;  // last graph with voff[lo] <= u
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (voff[mid] <= u) lo = mid; else hi = mid;
+      }
+      gi = lo;
+      gbase = voff[gi];
+      gend = voff[gi + 1];
+    }
+    // row[i] >= 0: entry i counts for that row (MODE 0: it is no edge; MODE 1: it is an
+    // upward first copy)
+    int32_t row[SP_ITEMS], val[SP_ITEMS];
+    unsigned bad = 0;
+#pragma unroll
+    for (int i = 0; i < SP_ITEMS; ++i) {
+      row[i] = -1;
+      val[i] = -1;
+      if (first + i < t1) {
+        const bool starts = ((marks >> i) & 1u) != 0u;
+        if (i > 0 && starts) u = tr.row[(int)threadIdx.x * SP_ITEMS + i];
+        if (voff && starts) {
+          while (u >= gend && gi + 1 < ng) {
+            ++gi;
+            gbase = voff[gi];
+            gend = voff[gi + 1];
+          }
+        }
+        const int32_t vl = w[i];
+        const bool in_range = vl >= 0 && (int64_t)vl < gend - gbase;
+        const int32_t v = in_range ? (int32_t)(vl + gbase) : 0;
+        const bool head = in_range && v != u && (starts || prev != vl);
+        if (MODE == 0) {
+          if (!in_range) bad |= 2u;
+          else if (!starts && prev > vl) bad |= 4u;
+          row[i] = head ? -1 : u;
+        } else {
+          row[i] = u;
+          val[i] = head ? v : -1;
+        }
+        prev = vl;
+      }
+    }
+    if (MODE == 0 && bad) atomicOr(err, (int)bad);
+    if (MODE == 1) {
+      // the gathers of the eight ranks are in flight together
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i)
+        if (val[i] >= 0) val[i] = rank[val[i]];
+      int32_t cur = -1, ru = 0;
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i) {
+        if (row[i] >= 0 && row[i] != cur) {
+          cur = row[i];
+          ru = rank[cur];
+        }
+        if (val[i] <= ru) row[i] = -1;
+      }
+    }
+    // one addition per thread and row
+    if (MODE == 0) {
+      int32_t cur = -1;
+      int cnt = 0;
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i) {
+        if (row[i] >= 0 && row[i] != cur) {
+          if (cur >= 0) atomicSub(&deg[cur], cnt);
+          cur = row[i];
+          cnt = 0;
+        }
+        if (row[i] >= 0) ++cnt;
+      }
+      if (cur >= 0) atomicSub(&deg[cur], cnt);
+    } else {
+      // a warp inside one long row (a hub's) reserves once for all its lanes
+      int32_t only = -1;
+      unsigned cnt = 0;
+      bool one = true;
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i)
+        if (row[i] >= 0) {
+          if (only >= 0 && row[i] != only) one = false;
+          only = row[i];
+          ++cnt;
+        }
+      const int32_t only0 = __reduce_max_sync(0xffffffffu, only);
+      if (only0 < 0) continue;  // nothing points up in the warp
+      if (__all_sync(0xffffffffu, one && (only < 0 || only == only0))) {
+        const unsigned incl = warp_inclusive_scan(cnt);
+        unsigned at = 0;
+        if (lane == 31) at = atomicAdd(&dplus[only0], incl);
+        if (!up) continue;
+        at = __shfl_sync(0xffffffffu, at, 31);
+        int64_t pos = (place ? place[rank[only0]] : rowptr[only0]) + (int64_t)(at + incl - cnt);
 #pragma unroll
         for (int i = 0; i < SP_ITEMS; ++i)
-          if (first + i < t1) rr[first + i] = up[i];
+          if (row[i] >= 0) up[pos++] = val[i];
+        continue;
       }
-    }
-    if (MODE < 2) {
-      int64_t cur = -1;
-      unsigned cnt = 0;
-      int groups = 0;
+      int32_t cur = -1;
+      int64_t pos = 0;
 #pragma unroll
       for (int i = 0; i < SP_ITEMS; ++i) {
-        if (key[i] >= 0 && key[i] != cur) {
-          if (cur >= 0) {
-            if (MODE == 0) atomicAdd(&deg[cur], (int)cnt);
-            else atomicAdd(&dplus[cur], (unsigned long long)cnt);
-          }
-          cur = key[i];
-          cnt = 0;
-          ++groups;
-        }
-        if (key[i] >= 0) ++cnt;
-      }
-      // a warp inside one long row (a hub's) adds once for all its lanes
-      const int64_t cur0 = __shfl_sync(0xffffffffu, cur, 0);
-      if (__all_sync(0xffffffffu, groups == 1 && cur == cur0)) {
-        const unsigned tot = __reduce_add_sync(0xffffffffu, cnt);
-        if (lane == 0) {
-          if (MODE == 0) atomicAdd(&deg[cur0], (int)tot);
-          else atomicAdd(&dplus[cur0], (unsigned long long)tot);
-        }
-      } else if (cur >= 0) {
-        if (MODE == 0) atomicAdd(&deg[cur], (int)cnt);
-        else atomicAdd(&dplus[cur], (unsigned long long)cnt);
-      }
-    } else {
-      int64_t cur = -1, pos = 0;
-#pragma unroll
-      for (int i = 0; i < SP_ITEMS; ++i) {
-        if (key[i] >= 0) {
-          if (key[i] != cur) {  // first item of a group: reserve the group's slots
-            cur = key[i];
+        if (row[i] >= 0) {
+          if (row[i] != cur) {  // first item of a group: reserve the group's slots
+            cur = row[i];
             unsigned c = 0;
 #pragma unroll
-            for (int j = i; j < SP_ITEMS; ++j) c += key[j] == cur ? 1u : 0u;
-            pos = rowptr_o[cur] + (int64_t)atomicAdd(&cursor[cur], c);
+            for (int j = i; j < SP_ITEMS; ++j) c += row[j] == cur ? 1u : 0u;
+            const unsigned at = atomicAdd(&dplus[cur], c);
+            pos = (place ? place[rank[cur]] : rowptr[cur]) + (int64_t)at;
           }
-          colidx_o[pos] = val[i];
+          if (up) up[pos] = val[i];
           ++pos;
         }
       }
     }
   }
+}
+
+// out-degree by position from the out-degree by vertex, and its maximum
+__global__ void k_rowlen_by_rank(const unsigned *__restrict__ dplus,
+                                 const int32_t *__restrict__ perm, int64_t n,
+                                 uint64_t *__restrict__ rowlen,
+                                 unsigned long long *__restrict__ longest) {
+  unsigned best = 0;
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= n;
+       r += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned d = r < n ? dplus[perm[r]] : 0u;
+    rowlen[r] = d;
+    best = d > best ? d : best;
+  }
+  best = __reduce_max_sync(0xffffffffu, best);
+  if ((threadIdx.x & 31) == 0 && best > 0) atomicMax(longest, (unsigned long long)best);
 }
 
 // esrc[x] = the row of position x, for every position of the oriented CSR.
@@ -485,8 +565,9 @@ __global__ void k_pair_keys(const int32_t *__restrict__ esrc, const int32_t *__r
 }
 
 __global__ void k_pair_unkey(const uint64_t *__restrict__ keys, int64_t m, int nb,
-                             int32_t *__restrict__ colidx) {
+                             const int32_t *__restrict__ err, int32_t *__restrict__ colidx) {
   const uint64_t mask = (1ull << nb) - 1ull;
+  if (*err & SORT_FAILED) return;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x)
     colidx[e] = (int32_t)(keys[e] & mask);
@@ -529,12 +610,13 @@ __device__ __forceinline__ void warp_bitonic(int32_t (&x)[K], unsigned lane) {
 }
 
 template <int K>
-__device__ __forceinline__ void sort_row_regs(int32_t *__restrict__ row, int len, unsigned lane) {
+__device__ __forceinline__ void sort_row_regs(const int32_t *in, int32_t *row, int len,
+                                              unsigned lane) {
   int32_t x[K];
 #pragma unroll
   for (int r = 0; r < K; ++r) {
     const int i = (int)lane + 32 * r;
-    x[r] = i < len ? row[i] : INT_MAX;
+    x[r] = i < len ? in[i] : INT_MAX;
   }
   warp_bitonic<K>(x, lane);
 #pragma unroll
@@ -581,89 +663,186 @@ __device__ __forceinline__ void sort_row_thread(int32_t *__restrict__ row, int l
     if (i < len) row[i] = x[i];
 }
 
-// Sort every oriented row ascending. A warp takes 32 rows at a time: each
-// lane sorts its own row when it has at most 16 entries (a register network
-// of 8 or 16), then the warp sorts the longer rows one at a time: up to 1024
-// in registers (bitonic network over shuffles and register slots, padded to
-// 32 * 2^t), longer ones (up to SEG_CAP) in the warp's shared memory.
-constexpr int SR_WARPS = 4;
+// Sort every oriented row ascending. A warp takes 32 consecutive rows, whose
+// entries are one span of the column array: spans of up to SR_SPAN entries are
+// copied to shared memory and back with coalesced accesses (rows dealt to the
+// lanes one by one, each at its own place in memory, took 264 us for the 32 M
+// entries of R-MAT scale 21); there each lane sorts its own row when it has at
+// most 16 entries (a register network of 8 or 16), then the warp sorts the
+// longer ones. Longer spans (runs of long rows, which the degree order keeps
+// together) are listed for k_sort_long, one warp per row.
+constexpr int SR_WARPS = 8;
 constexpr int SR_SMALL = 16;
+constexpr int SR_SPAN = 1024;
 
+// Sorts one row of up to 1,024 entries (a warp, in registers).
+__device__ __forceinline__ void sort_row_warp(const int32_t *in, int32_t *row, int len,
+                                              unsigned lane) {
+  if (len <= 32) sort_row_regs<1>(in, row, len, lane);
+  else if (len <= 64) sort_row_regs<2>(in, row, len, lane);
+  else if (len <= 128) sort_row_regs<4>(in, row, len, lane);
+  else if (len <= 256) sort_row_regs<8>(in, row, len, lane);
+  else if (len <= 512) sort_row_regs<16>(in, row, len, lane);
+  else sort_row_regs<32>(in, row, len, lane);
+}
+
+// Where row r's unsorted entries lie: in place, or at start[perm[r]] of src.
+struct RowSource {
+  const int32_t *src;
+  const int64_t *start;  // nullptr: in place
+  const int32_t *perm;
+};
+
+// esrc (nullable) receives each entry's row.
 __global__ void __launch_bounds__(SR_WARPS * 32) k_sort_rows(const int64_t *__restrict__ rowptr,
-                                                             int64_t n,
-                                                             int32_t *__restrict__ colidx) {
-  __shared__ int32_t buf[SR_WARPS][SEG_CAP];
+                                                             int64_t n, RowSource from,
+                                                             int32_t *colidx,
+                                                             int32_t *__restrict__ esrc,
+                                                             int32_t *__restrict__ listed,
+                                                             unsigned *__restrict__ nlisted) {
+  __shared__ int32_t buf[SR_WARPS][SR_SPAN];
   const unsigned lane = threadIdx.x & 31u;
-  const int warp = threadIdx.x >> 5;
-  int32_t *sm = buf[warp];
-  // rows are dealt round-robin over the warps (row r to warp r mod W), so that
-  // runs of long rows, which the degree order keeps together, spread evenly
-  const int64_t nwarps = (int64_t)gridDim.x * SR_WARPS;
-  const int64_t gw = (int64_t)blockIdx.x * SR_WARPS + warp;
-  for (int64_t t0 = 0; gw + nwarps * t0 < n; t0 += 32) {
-    const int64_t r = gw + nwarps * (t0 + lane);
-    int64_t b = 0;
-    int len = 0;
-    if (r < n) {
-      b = rowptr[r];
-      len = (int)(rowptr[r + 1] - b);
+  int32_t *sm = buf[threadIdx.x >> 5];
+  const int64_t nblk = (n + 31) >> 5;
+  for (int64_t blk = ((int64_t)blockIdx.x * (SR_WARPS * 32) + threadIdx.x) >> 5; blk < nblk;
+       blk += ((int64_t)gridDim.x * (SR_WARPS * 32)) >> 5) {
+    const int64_t r = blk * 32 + lane;
+    const int64_t b = rowptr[r < n ? r : n], e = rowptr[r + 1 < n ? r + 1 : n];
+    const int len = (int)(e - b);
+    const int64_t s0 = __shfl_sync(0xffffffffu, b, 0), s1 = __shfl_sync(0xffffffffu, e, 31);
+    if (s1 == s0 || (!from.start && !esrc && __all_sync(0xffffffffu, len <= 1))) continue;
+    if (s1 - s0 > SR_SPAN) {
+      if (lane == 0) listed[atomicAdd(nlisted, 1u)] = (int32_t)blk;
+      continue;
     }
-    const bool small = len > 1 && len <= SR_SMALL;
-    const int small_max = __reduce_max_sync(0xffffffffu, small ? len : 0);
-    if (small_max > 0) {
-      if (small_max <= 8) {
-        if (small) sort_row_thread<8>(colidx + b, len);
-      } else {
-        if (small) sort_row_thread<16>(colidx + b, len);
+    const int span = (int)(s1 - s0), at = (int)(b - s0);
+    // offset of the lane's row in the source, from its place in the span
+    const int64_t shift = from.start && len > 0 ? from.start[from.perm[r]] - at : s0;
+    for (int i0 = 0; i0 < span; i0 += 32) {
+      const int i = i0 + (int)lane;
+      int j = 0;  // last lane whose row starts at or before i
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1) {
+        const int aj = __shfl_sync(0xffffffffu, at, j + step);
+        if (aj <= i) j += step;
+      }
+      const int64_t sh = __shfl_sync(0xffffffffu, shift, j);
+      if (i < span) {
+        sm[i] = from.src[sh + i];
+        if (esrc) esrc[s0 + i] = (int32_t)(blk * 32 + j);
       }
     }
+    __syncwarp();
+    const bool small = len > 1 && len <= SR_SMALL;
+    const int small_max = __reduce_max_sync(0xffffffffu, small ? len : 0);
+    if (small_max > 8) {
+      if (small) sort_row_thread<16>(sm + at, len);
+    } else if (small_max > 0) {
+      if (small) sort_row_thread<8>(sm + at, len);
+    }
+    __syncwarp();
     unsigned big = __ballot_sync(0xffffffffu, len > SR_SMALL);
     while (big) {
       const int src = __ffs(big) - 1;
       big &= big - 1;
-      const int64_t bb = __shfl_sync(0xffffffffu, b, src);
-      const int blen = __shfl_sync(0xffffffffu, len, src);
-      int32_t *row = colidx + bb;
-      if (blen <= 32) {
-        sort_row_regs<1>(row, blen, lane);
-      } else if (blen <= 64) {
-        sort_row_regs<2>(row, blen, lane);
-      } else if (blen <= 128) {
-        sort_row_regs<4>(row, blen, lane);
-      } else if (blen <= 256) {
-        sort_row_regs<8>(row, blen, lane);
-      } else if (blen <= 512) {
-        sort_row_regs<16>(row, blen, lane);
-      } else if (blen <= 1024) {
-        sort_row_regs<32>(row, blen, lane);
-      } else {
-        int size = 64;
-        while (size < blen) size <<= 1;
-        for (int i = lane; i < size; i += 32) sm[i] = i < blen ? row[i] : INT_MAX;
-        __syncwarp();
-        for (int k = 2; k <= size; k <<= 1)
-          for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < size; i += 32) {
-              const int l = i ^ j;
-              if (l > i) {
-                const int32_t a = sm[i], c = sm[l];
-                const bool up = (i & k) == 0;
-                if ((a > c) == up) {
-                  sm[i] = c;
-                  sm[l] = a;
-                }
-              }
+      int32_t *row = sm + __shfl_sync(0xffffffffu, at, src);
+      sort_row_warp(row, row, __shfl_sync(0xffffffffu, len, src), lane);
+    }
+    __syncwarp();
+    for (int i = lane; i < span; i += 32) colidx[s0 + i] = sm[i];
+    __syncwarp();
+  }
+}
+
+// The rows of the listed blocks of 32, one warp per row: up to 1,024 entries in
+// registers (bitonic network over shuffles and register slots, padded to
+// 32 * 2^t), longer ones (up to SEG_CAP) in the warp's shared memory.
+constexpr int SL_WARPS = 4;
+__global__ void __launch_bounds__(SL_WARPS * 32) k_sort_long(const int64_t *__restrict__ rowptr,
+                                                             int64_t n, RowSource from,
+                                                             int32_t *colidx,
+                                                             int32_t *__restrict__ esrc,
+                                                             const int32_t *__restrict__ listed,
+                                                             const unsigned *__restrict__ nlisted) {
+  __shared__ int32_t buf[SL_WARPS][SEG_CAP];
+  const unsigned lane = threadIdx.x & 31u;
+  int32_t *sm = buf[threadIdx.x >> 5];
+  const int64_t total = (int64_t)*nlisted * 32;
+  for (int64_t x = (int64_t)blockIdx.x * SL_WARPS + (threadIdx.x >> 5); x < total;
+       x += (int64_t)gridDim.x * SL_WARPS) {
+    const int64_t r = (int64_t)listed[x >> 5] * 32 + (x & 31);
+    if (r >= n) continue;
+    const int64_t b = rowptr[r];
+    const int len = (int)(rowptr[r + 1] - b);
+    if (len <= 0) continue;
+    int32_t *row = colidx + b;
+    const int32_t *in = from.start ? from.src + from.start[from.perm[r]] : row;
+    if (esrc)
+      for (int i = lane; i < len; i += 32) esrc[b + i] = (int32_t)r;
+    if (len <= 1024) {
+      sort_row_warp(in, row, len, lane);
+      continue;
+    }
+    int size = 2048;
+    while (size < len) size <<= 1;
+    for (int i = lane; i < size; i += 32) sm[i] = i < len ? in[i] : INT_MAX;
+    __syncwarp();
+    for (int k = 2; k <= size; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int i = lane; i < size; i += 32) {
+          const int l = i ^ j;
+          if (l > i) {
+            const int32_t a = sm[i], c = sm[l];
+            const bool up = (i & k) == 0;
+            if ((a > c) == up) {
+              sm[i] = c;
+              sm[l] = a;
             }
-            __syncwarp();
           }
-        for (int i = lane; i < blen; i += 32) row[i] = sm[i];
+        }
         __syncwarp();
       }
+    for (int i = lane; i < len; i += 32) row[i] = sm[i];
+    __syncwarp();
+  }
+}
+
+// Rows too long for k_sort_long: entries and their rows moved to their places,
+// unsorted (one warp per row).
+__global__ void k_gather_rows(const int64_t *__restrict__ rowptr, int64_t n, RowSource from,
+                              int32_t *__restrict__ colidx, int32_t *__restrict__ esrc) {
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
+    const int64_t b = rowptr[r], len = rowptr[r + 1] - b;
+    if (len <= 0) continue;
+    const int32_t *in = from.src + from.start[from.perm[r]];
+    for (int64_t i = threadIdx.x & 31; i < len; i += 32) {
+      colidx[b + i] = in[i];
+      esrc[b + i] = (int32_t)r;
     }
   }
 }
 
 }  // namespace
+
+// Sorts every row of an oriented CSR whose rows have at most SEG_CAP entries
+// into colidx, and writes each entry's row.
+static bbtc_status sort_rows(const int64_t *rowptr, int64_t n, const RowSource &from,
+                             int32_t *colidx, int32_t *esrc, cudaStream_t s) {
+  Scratch scratch(s);
+  int32_t *listed = nullptr;
+  unsigned *nlisted = nullptr;
+  BBTC_TRY(scratch.get(&listed, (n + 31) / 32));
+  BBTC_TRY(scratch.get(&nlisted, 1));
+  BBTC_CUDA(cudaMemsetAsync(nlisted, 0, sizeof(unsigned), s));
+  k_sort_rows<<<grid_for((n + 31) / 32, SR_WARPS, 7), SR_WARPS * 32, 0, s>>>(
+      rowptr, n, from, colidx, esrc, listed, nlisted);
+  BBTC_LAUNCH_CHECK();
+  k_sort_long<<<grid_for((n + 31) / 32, 1, 7), SL_WARPS * 32, 0, s>>>(rowptr, n, from, colidx,
+                                                                     esrc, listed, nlisted);
+  BBTC_LAUNCH_CHECK();
+  return BBTC_OK;
+}
 
 // a1-a4 for symmetric input with sorted rows. Sets *applied = false (and does
 // nothing lasting) when some row turns out unsorted.
@@ -677,17 +856,23 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   Scratch scratch(s);
   BBTC_TRY(dalloc_n(&g->deg, n, s));
   g->bytes += (uint64_t)(n > 0 ? n : 1) * sizeof(int32_t);
-  BBTC_CUDA(cudaMemsetAsync(g->deg, 0, sizeof(int32_t) * (size_t)(n > 0 ? n : 1), s));
+  k_validate_rowptr<<<grid_for(n, 256, 8), 256, 0, s>>>(d_rowptr, n, g->deg, err);
+  BBTC_LAUNCH_CHECK();
+  const bool aligned = (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0;  // the caller's array
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
   int64_t *tile_rows = nullptr;
   BBTC_TRY(scratch.get(&tile_rows, ntiles + 1));
   k_tile_rows<<<grid_for(ntiles + 1, 256, 16), 256, 0, s>>>(d_rowptr, n, nnz, ntiles, tile_rows);
   BBTC_LAUNCH_CHECK();
   const unsigned grid = grid_for(ntiles, 1, 32);
-  k_sym_pass<0><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, tile_rows, g->deg, nullptr,
-                                       nullptr, nullptr, nullptr, nullptr, err, g->voff, g->ng,
-                                       nullptr);
+  k_sym_pass<0><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, g->deg,
+                                       nullptr, nullptr, nullptr, nullptr, err, g->voff, g->ng);
   BBTC_LAUNCH_CHECK();
+  int32_t *dmax = nullptr;
+  BBTC_TRY(scratch.get(&dmax, 1));
+  BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
+  int32_t hdmax = 0;
+  BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   int32_t herr = 0;
   BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
@@ -703,25 +888,22 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   *applied = true;
 
   // a3: order by (degree, id)
-  int32_t *rank = nullptr, *dmax = nullptr;
+  int32_t *rank = nullptr;
   uint64_t *rk = nullptr, *rk_alt = nullptr;
   BBTC_TRY(scratch.get(&rank, n));
-  BBTC_TRY(scratch.get(&dmax, 1));
   BBTC_TRY(scratch.get(&rk, n));
   BBTC_TRY(scratch.get(&rk_alt, n));
   BBTC_TRY(dalloc_n(&g->perm, n, s));
   g->bytes += (uint64_t)n * sizeof(int32_t);
-  BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
-  int32_t hdmax = 0;
-  BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaStreamSynchronize(s));
   g->deg_max = hdmax;
   k_rank_keys<<<grid_for(n, 256, 16), 256, 0, s>>>(g->deg, n, nb, rk);
   BBTC_LAUNCH_CHECK();
   bool in_alt = false;
-  BBTC_TRY(radix_sort(rk, rk_alt, nullptr, nullptr, n, 0, nb + ceil_log2_u64((uint64_t)hdmax + 1),
-                      s, &in_alt));
-  k_rank_finish<<<grid_for(n, 256, 16), 256, 0, s>>>(in_alt ? rk_alt : rk, n, nb, g->perm, rank);
+  // the keys start in id order and the sort is stable: only the degree bits are sorted
+  BBTC_TRY(radix_sort(rk, rk_alt, nullptr, nullptr, n, nb, nb + ceil_log2_u64((uint64_t)hdmax + 1),
+                      s, err, &in_alt));
+  k_rank_finish<<<grid_for(n, 256, 16), 256, 0, s>>>(in_alt ? rk_alt : rk, n, nb, err, g->perm,
+                                                      rank);
   BBTC_LAUNCH_CHECK();
   if (g->voff) {
     BBTC_TRY(dalloc_n(&g->gid, n, s));
@@ -730,35 +912,40 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
     BBTC_LAUNCH_CHECK();
   }
 
-  // a4: out-degrees by rank, offsets, scatter, per-row sort
+  // a4: each row's upward entries to its front, out-degrees by rank, offsets, and
+  // the rows picked up in rank order and sorted
   BBTC_TRY(dalloc_n(&g->rowptr, n + 1, s));
   g->bytes += (uint64_t)(n + 1) * 8;
-  BBTC_CUDA(cudaMemsetAsync(g->rowptr, 0, sizeof(int64_t) * (size_t)(n + 1), s));
-  // each entry's upward rank, kept for the scatter pass (it is skipped, and the
-  // scatter gathers the ranks again, when the nnz-entry array does not fit)
-  int32_t *rr = nullptr;
-  if (dalloc_n(&rr, nnz, s) != BBTC_OK) {
+  int32_t *up = nullptr;
+  unsigned *dplus = nullptr;
+  unsigned long long *longest = nullptr;
+  BBTC_TRY(scratch.get(&dplus, n));
+  BBTC_TRY(scratch.get(&longest, 1));
+  if (dalloc_n(&up, nnz, s) != BBTC_OK) {  // no room: the rows are written in a second pass
     clear_error();
-    rr = nullptr;
+    up = nullptr;
   }
-  struct FreeRR {
+  struct FreeUp {
     int32_t *p;
     cudaStream_t s;
-    ~FreeRR() { dfree(p, s); }
-  } free_rr{rr, s};
-  k_sym_pass<1><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, tile_rows, nullptr, rank,
-                                       reinterpret_cast<unsigned long long *>(g->rowptr),
-                                       nullptr, nullptr, nullptr, err, g->voff, g->ng, rr);
+    ~FreeUp() { dfree(p, s); }
+  } free_up{up, s};
+  BBTC_CUDA(cudaMemsetAsync(dplus, 0, sizeof(unsigned) * (size_t)n, s));
+  BBTC_CUDA(cudaMemsetAsync(longest, 0, sizeof(unsigned long long), s));
+  k_sym_pass<1><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, nullptr, rank,
+                                       dplus, up, nullptr, err, g->voff, g->ng);
   BBTC_LAUNCH_CHECK();
-  int64_t *stats = nullptr;
-  BBTC_TRY(scratch.get(&stats, 2));
-  BBTC_TRY(reduce_max_i64(g->rowptr, n, &stats[0], s));
+  k_rowlen_by_rank<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(
+      dplus, g->perm, n, reinterpret_cast<uint64_t *>(g->rowptr), longest);
+  BBTC_LAUNCH_CHECK();
   BBTC_TRY(exclusive_scan_u64(reinterpret_cast<uint64_t *>(g->rowptr),
                               reinterpret_cast<uint64_t *>(g->rowptr), n + 1, s));
   int64_t h[2] = {0, 0};
-  BBTC_CUDA(cudaMemcpyAsync(&h[0], &stats[0], sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaMemcpyAsync(&h[0], longest, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaMemcpyAsync(&h[1], g->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
+  if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
   g->dplus_max = h[0];
   const int64_t m = h[1];
   if (m > 0xFFFFFFFFLL) {
@@ -769,34 +956,32 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   BBTC_TRY(dalloc_n(&g->colidx, padded_columns(m), s));
   BBTC_TRY(dalloc_n(&g->esrc, m, s));
   g->bytes += (uint64_t)(m > 0 ? m : 1) * 8;
-  unsigned int *cursor = nullptr;
-  BBTC_TRY(scratch.get(&cursor, n));
-  BBTC_CUDA(cudaMemsetAsync(cursor, 0, sizeof(unsigned int) * (size_t)(n > 0 ? n : 1), s));
-  k_sym_pass<2><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, tile_rows, nullptr, rank,
-                                       nullptr, g->rowptr, cursor, g->colidx, err, g->voff, g->ng,
-                                       rr);
-  BBTC_LAUNCH_CHECK();
-  if (m > 0) {
-    k_fill_esrc<<<grid_for((n + 31) / 32 * 32, 256, 16), 256, 0, s>>>(g->rowptr, n, g->esrc);
+  if (!up && m > 0) {
+    BBTC_CUDA(cudaMemsetAsync(dplus, 0, sizeof(unsigned) * (size_t)n, s));
+    k_sym_pass<1><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, nullptr,
+                                         rank, dplus, g->colidx, g->rowptr, err, g->voff, g->ng);
     BBTC_LAUNCH_CHECK();
   }
-  if (m > 0) {
-    if (g->dplus_max <= SEG_CAP) {
-      k_sort_rows<<<grid_for((n + 31) / 32, SR_WARPS, 64), SR_WARPS * 32, 0, s>>>(g->rowptr, n,
-                                                                                g->colidx);
-      BBTC_LAUNCH_CHECK();
-    } else {
-      uint64_t *ok = nullptr, *ok_alt = nullptr;
-      BBTC_TRY(scratch.get(&ok, m));
-      BBTC_TRY(scratch.get(&ok_alt, m));
-      k_pair_keys<<<grid_for(m, 256, 32), 256, 0, s>>>(g->esrc, g->colidx, m, nb, ok);
-      BBTC_LAUNCH_CHECK();
-      BBTC_TRY(radix_sort(ok, ok_alt, nullptr, nullptr, m, 0, 2 * nb, s, &in_alt));
-      k_pair_unkey<<<grid_for(m, 256, 32), 256, 0, s>>>(in_alt ? ok_alt : ok, m, nb, g->colidx);
-      BBTC_LAUNCH_CHECK();
-    }
+  const RowSource from = up ? RowSource{up, d_rowptr, g->perm}
+                            : RowSource{g->colidx, nullptr, nullptr};
+  if (m > 0 && g->dplus_max <= SEG_CAP) {
+    BBTC_TRY(sort_rows(g->rowptr, n, from, g->colidx, g->esrc, s));
+  } else if (m > 0) {
+    if (up) k_gather_rows<<<grid_for(n * 32, 256, 16), 256, 0, s>>>(g->rowptr, n, from, g->colidx, g->esrc);
+    else k_fill_esrc<<<grid_for((n + 31) / 32 * 32, 256, 16), 256, 0, s>>>(g->rowptr, n, g->esrc);
+    BBTC_LAUNCH_CHECK();
+    uint64_t *ok = nullptr, *ok_alt = nullptr;
+    BBTC_TRY(scratch.get(&ok, m));
+    BBTC_TRY(scratch.get(&ok_alt, m));
+    k_pair_keys<<<grid_for(m, 256, 32), 256, 0, s>>>(g->esrc, g->colidx, m, nb, ok);
+    BBTC_LAUNCH_CHECK();
+    BBTC_TRY(radix_sort(ok, ok_alt, nullptr, nullptr, m, 0, 2 * nb, s, err, &in_alt));
+    k_pair_unkey<<<grid_for(m, 256, 32), 256, 0, s>>>(in_alt ? ok_alt : ok, m, nb, err, g->colidx);
+    BBTC_LAUNCH_CHECK();
+    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaStreamSynchronize(s));
+    if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
   }
-  BBTC_CUDA(cudaStreamSynchronize(s));
   return BBTC_OK;
 }
 
@@ -813,69 +998,42 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
   BBTC_TRY(scratch.get(&hstats, 3));
   BBTC_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
 
-  // ---- validation of rowptr (colidx range is checked while emitting keys)
-  if (n > 0) {
-    k_validate_rowptr<<<grid_for(n, 256, 8), 256, 0, s>>>(d_rowptr, n, err);
-    BBTC_LAUNCH_CHECK();
-  }
-
   // ---- symmetric input with sorted rows: per-row path, no global sort
-  if (symmetric && nnz > 0) {
+  if (symmetric && nnz > 0 && n > 0) {
     bool applied = false;
     BBTC_TRY(prepare_sym_sorted(g, d_rowptr, d_colidx, nnz, err, &applied));
     if (applied) return BBTC_OK;
     BBTC_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));  // fall through: general path
   }
 
-  // ---- a1: canonical keys (compacted), sort, unique; a2: degree
+  // ---- validation of rowptr (colidx range is checked while emitting keys)
+  if (n > 0) {
+    k_validate_rowptr<<<grid_for(n, 256, 8), 256, 0, s>>>(d_rowptr, n, nullptr, err);
+    BBTC_LAUNCH_CHECK();
+  }
+
+  // ---- a1: canonical keys, sort, unique; a2: degree
   // (no key equals the all-ones value: it would need min == max)
   const uint64_t sentinel = (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
   uint64_t *ka = nullptr, *kb = nullptr;
-  int64_t nkeys = 0;
+  const int64_t nkeys = nnz;
+  const int64_t kcap = nkeys > n ? nkeys : n;  // the buffers also take the n rank keys
+  BBTC_TRY(scratch.get(&ka, kcap));
+  BBTC_TRY(scratch.get(&kb, kcap));
   if (nnz > 0) {
-    const int64_t ntiles = (nnz + EK_TILE - 1) / EK_TILE;
-    uint64_t *tile_count = nullptr;
-    BBTC_TRY(scratch.get(&tile_count, ntiles + 1));
-    const unsigned grid = grid_for(ntiles, 1, 64);
-    k_emit_keys<false><<<grid, EK_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, nb, symmetric,
-                                               g->voff, g->ng, tile_count, nullptr, err);
+    const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
+    int64_t *tile_rows = nullptr;
+    BBTC_TRY(scratch.get(&tile_rows, ntiles + 1));
+    k_tile_rows<<<grid_for(ntiles + 1, 256, 16), 256, 0, s>>>(d_rowptr, n, nnz, ntiles, tile_rows);
     BBTC_LAUNCH_CHECK();
-    BBTC_TRY(exclusive_scan_u64(tile_count, tile_count, ntiles + 1, s));
-    BBTC_CUDA(cudaMemcpyAsync(&hstats[0], &tile_count[ntiles], sizeof(int64_t),
-                              cudaMemcpyDeviceToDevice, s));
-    int64_t h[1] = {0};
-    int32_t herr = 0;
-    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    BBTC_CUDA(cudaMemcpyAsync(h, &hstats[0], sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    BBTC_CUDA(cudaStreamSynchronize(s));
-    if (herr & 1) {
-      set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
-      return BBTC_EINVAL;
-    }
-    if (herr & 2) {
-      set_error("bbtc_graph_create: colidx entry outside [0, n)");
-      return BBTC_EINVAL;
-    }
-    nkeys = h[0];
-    const int64_t kcap = nkeys > n ? nkeys : n;  // the buffers also take the n rank keys
-    BBTC_TRY(scratch.get(&ka, kcap));
-    BBTC_TRY(scratch.get(&kb, kcap));
-    k_emit_keys<true><<<grid, EK_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, nb, symmetric,
-                                              g->voff, g->ng, tile_count, ka, err);
+    k_emit_keys<<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
+        d_rowptr, d_colidx, n, nnz, nb, symmetric,
+        (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0, sentinel, tile_rows, g->voff, g->ng, ka,
+        err);
     BBTC_LAUNCH_CHECK();
-  } else {
-    int32_t herr = 0;
-    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    BBTC_CUDA(cudaStreamSynchronize(s));
-    if (herr & 1) {
-      set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
-      return BBTC_EINVAL;
-    }
-    BBTC_TRY(scratch.get(&ka, n));
-    BBTC_TRY(scratch.get(&kb, n));
   }
   bool in_alt = false;
-  BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, &in_alt));
+  BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
   uint64_t *sorted = in_alt ? kb : ka;
   uint64_t *ukeys = in_alt ? ka : kb;
 
@@ -889,10 +1047,10 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
     const int64_t nblk = (nkeys + UQ_TILE - 1) / UQ_TILE;
     uint64_t *boff = nullptr;
     BBTC_TRY(scratch.get(&boff, nblk + 1));
-    k_unique_count<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, boff);
+    k_unique_count<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff);
     BBTC_LAUNCH_CHECK();
     BBTC_TRY(exclusive_scan_u64(boff, boff, nblk + 1, s));  // boff[nblk] = total
-    k_unique_write<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, boff, nb, ukeys,
+    k_unique_write<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff, nb, ukeys,
                                                      g->deg);
     BBTC_LAUNCH_CHECK();
     BBTC_CUDA(cudaMemcpyAsync(&hstats[0], &boff[nblk], sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
@@ -903,10 +1061,20 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
   BBTC_TRY(scratch.get(&dmax, 1));
   BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
   int64_t stats[2] = {0, 0};
-  int32_t hdmax = 0;
+  int32_t hdmax = 0, herr = 0;
+  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaMemcpyAsync(&stats[0], &hstats[0], sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
+  if (herr & 1) {
+    set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
+    return BBTC_EINVAL;
+  }
+  if (herr & 2) {
+    set_error("bbtc_graph_create: colidx entry outside [0, n)");
+    return BBTC_EINVAL;
+  }
+  if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
   m = stats[0];
   if (m > 0xFFFFFFFFLL) {
     set_error("bbtc_graph_create: %lld simple edges exceed 2^32 - 1", (long long)m);
@@ -929,8 +1097,8 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
     k_rank_keys<<<grid_for(n, 256, 16), 256, 0, s>>>(g->deg, n, nb, rk);
     BBTC_LAUNCH_CHECK();
     int dbits = ceil_log2_u64((uint64_t)hdmax + 1);
-    BBTC_TRY(radix_sort(rk, rk_alt, nullptr, nullptr, n, 0, nb + dbits, s, &in_alt));
-    k_rank_finish<<<grid_for(n, 256, 16), 256, 0, s>>>(in_alt ? rk_alt : rk, n, nb, g->perm,
+    BBTC_TRY(radix_sort(rk, rk_alt, nullptr, nullptr, n, nb, nb + dbits, s, err, &in_alt));
+    k_rank_finish<<<grid_for(n, 256, 16), 256, 0, s>>>(in_alt ? rk_alt : rk, n, nb, err, g->perm,
                                                         rank);
     BBTC_LAUNCH_CHECK();
     if (g->voff) {
@@ -942,31 +1110,47 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
     }
   }
 
-  // ---- a4: orient and build the oriented CSR
+  // ---- a4: orient and build the oriented CSR: row lengths and each edge's slot by
+  // counting, offsets, scatter, per-row sort
   BBTC_TRY(dalloc_n(&g->rowptr, n + 1, s));
   BBTC_TRY(dalloc_n(&g->colidx, padded_columns(m), s));
   BBTC_TRY(dalloc_n(&g->esrc, m, s));
   g->bytes += (uint64_t)(n + 1) * 8 + (uint64_t)(m > 0 ? m : 1) * 8;
   BBTC_CUDA(cudaMemsetAsync(g->rowptr, 0, sizeof(int64_t) * (size_t)(n + 1), s));
+  uint64_t *ok = sorted;  // rank keys are consumed; reuse
+  unsigned *slot = nullptr;
   if (m > 0) {
-    uint64_t *ok = sorted;  // rank keys are consumed; reuse
-    uint64_t *ok_alt = nullptr;
-    BBTC_TRY(scratch.get(&ok_alt, m));
-    k_orient_keys<<<grid_for(m, 256, 32), 256, 0, s>>>(ukeys, m, nb, rank, ok);
-    BBTC_LAUNCH_CHECK();
-    BBTC_TRY(radix_sort(ok, ok_alt, nullptr, nullptr, m, 0, 2 * nb, s, &in_alt));
-    k_csr_finish<<<grid_for(m, 256, 32), 256, 0, s>>>(
-        in_alt ? ok_alt : ok, m, nb, g->colidx, g->esrc,
-        reinterpret_cast<unsigned long long *>(g->rowptr));
+    BBTC_TRY(scratch.get(&slot, m));
+    k_orient_count<<<grid_for(m, 256, 32), 256, 0, s>>>(
+        ukeys, m, nb, rank, ok, slot, reinterpret_cast<unsigned long long *>(g->rowptr));
     BBTC_LAUNCH_CHECK();
   }
   // rowptr holds the row lengths: their maximum is d+_max, their scan the offsets
   BBTC_TRY(reduce_max_i64(g->rowptr, n, &hstats[1], s));
   BBTC_CUDA(cudaMemcpyAsync(&stats[1], &hstats[1], sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   BBTC_TRY(exclusive_scan_u64(reinterpret_cast<uint64_t *>(g->rowptr),
                               reinterpret_cast<uint64_t *>(g->rowptr), n + 1, s));
+  if (m > 0) {
+    k_orient_scatter<<<grid_for(m, 256, 32), 256, 0, s>>>(ok, slot, m, nb, g->rowptr, g->colidx);
+    BBTC_LAUNCH_CHECK();
+  }
   BBTC_CUDA(cudaStreamSynchronize(s));
+  if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
   g->dplus_max = n > 0 ? stats[1] : 0;
+  if (m > 0 && g->dplus_max <= SEG_CAP) {
+    BBTC_TRY(sort_rows(g->rowptr, n, RowSource{g->colidx, nullptr, nullptr}, g->colidx, g->esrc, s));
+  } else if (m > 0) {
+    k_fill_esrc<<<grid_for((n + 31) / 32 * 32, 256, 16), 256, 0, s>>>(g->rowptr, n, g->esrc);
+    BBTC_LAUNCH_CHECK();
+    uint64_t *ok_alt = ukeys;
+    BBTC_TRY(radix_sort(ok, ok_alt, nullptr, nullptr, m, 0, 2 * nb, s, err, &in_alt));
+    k_pair_unkey<<<grid_for(m, 256, 32), 256, 0, s>>>(in_alt ? ok_alt : ok, m, nb, err, g->colidx);
+    BBTC_LAUNCH_CHECK();
+    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaStreamSynchronize(s));
+    if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
+  }
   return BBTC_OK;
 }
 
