@@ -492,7 +492,7 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   // counted task by task: with a budget, for a share of the tasks and for their cycles
   const bool by_task = budgeted || opts.per_task_cycles_out || opts.task_mask;
   const bool detail = !by_task && (opts.per_vertex_out || opts.per_edge_out);
-  const bool tasks = opts.per_task_out && p > 1, per_graph = opts.per_graph_out != nullptr;
+  const bool tasks = opts.per_task_out != nullptr, per_graph = opts.per_graph_out != nullptr;
   // (a detail count alone needs neither the core nor the in-edges that it leaves)
   const bool resident = !by_task && (!detail || tasks || per_graph);
   const Plan &old = g->plan;
@@ -553,6 +553,10 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   BBTC_CUDA(cudaMemcpyAsync(head, pl.scratch, sizeof(head), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   if ((int32_t)head[SCR_STATUS] != 0) return count_status_error("bbtc_count", (int32_t)head[SCR_STATUS], opts.timeout_ms);
+  if (!opts.per_task_out && !per_graph && !task_cycles && !edge_sup && !opts.per_vertex_out) {
+    *count = head[SCR_TOTAL];
+    return BBTC_OK;
+  }
   const bool out_dev = (opts.flags & BBTC_OUT_DEVICE) != 0;
   const cudaMemcpyKind kind = out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   if (opts.per_task_out)

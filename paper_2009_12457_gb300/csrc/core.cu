@@ -31,11 +31,12 @@ namespace {
 
 constexpr int CORE_NT = 256;
 constexpr int CORE_WARPS = CORE_NT / 32;
-constexpr int CORE_MAX_COLS = 8192;  // columns of the core at most
+constexpr int CORE_MAX_COLS = 12288;  // columns of the core at most
 // a graph of at most so many vertices is all core, and no list is probed: R-MAT
 // scale 14 counts in 27 us where the lists took 117 (latency, not work)
 constexpr int CORE_ALL_COLS = 16384;
 constexpr int CORE_TABLE = 816;       // task counters kept in shared memory (p <= 16)
+constexpr int64_t CORE_WIDE_EDGES = 1 << 23;  // fewer edges: 8,192 columns
 constexpr int CORE_CTAS = 4;          // counting CTAs per SM
 constexpr int32_t CORE_STATUS_TIMEOUT = 1;
 
@@ -250,9 +251,10 @@ __device__ __forceinline__ int core_steps(ColumnSums &cols, const uint4 &m,
 // matrix of a few MB). Four CTAs of 64 registers (0.44 ms on R-MAT scale 20)
 // beat three of 80 (0.53): the loads' latency needs the warps. Rows that start
 // in the last half or quarter of the top group are read two or four side by
-// side, since the lanes below them would only read zeros. 8,192 columns beat
-// 16,384 there (1.26 against 1.32 ms for the whole count): the lower columns
-// are too thin for words. ONE: a single descriptor with p = 1 and no per-graph counts, where a
+// side, since the lanes below them would only read zeros. Columns: 8,192 beat
+// 12,288 on R-MAT scale 18 (0.165 against 0.173 ms for the whole count), they tie
+// on scale 20 (0.745, 0.740), and 12,288 win on scale 22 (4.91, 4.66) and on the
+// 1/16 Friendster-shaped graph (7.43, 7.32): hence CORE_WIDE_EDGES. ONE: a single descriptor with p = 1 and no per-graph counts, where a
 // lane keeps its sum to the end.
 template <bool ONE>
 __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P) {
@@ -444,7 +446,8 @@ bbtc_status build_core(const bbtc_graph *g, Plan &pl, cudaStream_t s) {
   if (m < 3 || n < 3) return BBTC_OK;
   // columns: all of a small graph, else the top CORE_MAX_COLS; the packed rows
   // take K^2 / 16 bytes, which is kept to about 96 bytes per edge
-  int64_t K = n <= CORE_ALL_COLS ? CORE_ALL_COLS : CORE_MAX_COLS;
+  int64_t K = n <= CORE_ALL_COLS ? CORE_ALL_COLS : m < CORE_WIDE_EDGES ? 8192 : CORE_MAX_COLS;
+  const int max_quads = (int)(K / 128);
   while (K > 256 && K * K / 16 > 96 * m) K = K * 7 / 8;
   const bool all = n <= K;
   // the graphs of a union interleave in the degree order, so that its top
@@ -469,8 +472,8 @@ bbtc_status build_core(const bbtc_graph *g, Plan &pl, cudaStream_t s) {
     const int room = (quads + 31) / 32 * 32;
     // parts that start on a quad can push the columns into one more group of 32
     // quads; a core of the top positions gives up a few columns instead
-    if (!all && quads > CORE_MAX_COLS / 128 && tries < 64) {
-      K -= 128 * (quads - CORE_MAX_COLS / 128);
+    if (!all && quads > max_quads && tries < 64) {
+      K -= 128 * (quads - max_quads);
       if (K < 1024) return BBTC_OK;
       continue;
     }

@@ -702,24 +702,27 @@ static bbtc_status count_resident(const bbtc_graph *g, const Plan &pl, bool task
                            timeout_ms, s, nullptr, nullptr, nullptr);
   if (pl.flat.ready)
     BBTC_TRY(core_launch(core_desc(g, pl, 0, 0), nullptr, 1, pl.core.nitems, pl.core.parts.quads,
-                         task_count, pl.ntasks, tasks, graph_count, status, t0, timeout_ms, s));
+                         task_count, tasks ? pl.ntasks : 1, tasks, graph_count, status, t0,
+                         timeout_ms, s));
   const Flat &f = pl.flat.ready ? pl.flat : pl.full;
-  return flat_launch(flat_desc(g, pl, f, 0, 0), nullptr, 1, f.nitems, head, task_count, pl.ntasks,
-                     tasks, graph_count, status, t0, timeout_ms, pl.flat_blocks_per_sm, s);
+  return flat_launch(flat_desc(g, pl, f, 0, 0), nullptr, 1, f.nitems, head, task_count,
+                     tasks ? pl.ntasks : 1, tasks, graph_count, status, t0, timeout_ms, pl.flat_blocks_per_sm, s);
 }
 
 bbtc_status run_flat(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
                      uint32_t timeout_ms, cudaStream_t s, cudaEvent_t ev_begin,
                      cudaEvent_t ev_end) {
+  // without per-task counts the kernels add to the total itself, which saves the sum
+  const bool sum = tasks || (!pl.flat.ready && !pl.full.ready);
   BBTC_TRY(count_reset(g, pl, nullptr, per_graph, s));
   if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
   unsigned long long *scr = pl.scratch;
   BBTC_TRY(count_resident(g, pl, tasks, scr + SCR_HEAD,
                           reinterpret_cast<int32_t *>(scr + SCR_STATUS), scr + SCR_T0,
-                          scr + SCR_TASKS, per_graph ? scr + SCR_TASKS + pl.ntasks : nullptr,
-                          timeout_ms, s));
+                          sum ? scr + SCR_TASKS : scr + SCR_TOTAL,
+                          per_graph ? scr + SCR_TASKS + pl.ntasks : nullptr, timeout_ms, s));
   if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
-  return count_finish(pl, s);
+  return sum ? count_finish(pl, s) : BBTC_OK;
 }
 
 bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
@@ -736,10 +739,10 @@ bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph
     BBTC_TRY(count_reset(g, pl, nullptr, false, s));
     if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
   }
-  BBTC_TRY(detail_launch(g, pl, both ? nullptr : pl.scratch + SCR_TASKS, vcount, edge_sup,
+  BBTC_TRY(detail_launch(g, pl, both ? nullptr : pl.scratch + SCR_TOTAL, vcount, edge_sup,
                          timeout_ms, s));
   if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
-  return both ? BBTC_OK : count_finish(pl, s);
+  return BBTC_OK;
 }
 
 // --------------------------------------------- several plans, one launch

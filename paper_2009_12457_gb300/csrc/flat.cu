@@ -14,6 +14,7 @@
 // so [e + 1, f) is the probe run, and v is the column just before it.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "flat.cuh"
 #include "graph.cuh"
@@ -24,9 +25,10 @@ namespace bbtc {
 
 namespace {
 
-constexpr int FL_NT = 256;
+constexpr int FL_NT = 128;
+constexpr int FL_CTAS = 6;        // per SM: 24 warps, whose stages fill the shared memory
 constexpr int FL_WARPS = FL_NT / 32;
-constexpr int FL_RUN_MIN = 4;     // in-edges of one v that make a batch of their own
+constexpr int FL_RUN_MIN = 8;     // in-edges of one v that make a batch of their own
 constexpr int FL_TABLE = 816;     // task counters kept in shared memory (p <= 16)
 constexpr int FL_MODE_GRAPH = 1, FL_MODE_TASK = 2;
 
@@ -72,23 +74,39 @@ struct InHash {
   }
 };
 
-// The sorted copy, searched by halving.
+// The sorted copy, searched by halving inside the key's bucket. Keys are bucketed
+// by the exponent and three more bits of their distance to the list's last entry
+// (in degree order lists crowd towards the hubs, at the end), so a bucket holds a
+// few entries and a search takes `steps` halvings, the same for every lane: three
+// or four where the whole list takes nine or ten. index[b] = first position of
+// bucket b | end << 16; without an index (log2 steps of the length) the whole
+// list is one bucket.
+constexpr int SI_BUCKETS = 256;
 struct InSorted {
   const int32_t *list;
-  int len;
-  __device__ __forceinline__ uint32_t bits(const int4 &w, uint32_t m) const {
-    int p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-    for (int step = len > 0 ? 1 << (31 - __clz(len)) : 0; step > 0; step >>= 1) {
-      if (p0 + step <= len && list[p0 + step - 1] < w.x) p0 += step;
-      if (p1 + step <= len && list[p1 + step - 1] < w.y) p1 += step;
-      if (p2 + step <= len && list[p2 + step - 1] < w.z) p2 += step;
-      if (p3 + step <= len && list[p3 + step - 1] < w.w) p3 += step;
+  const uint32_t *index;  // nullptr: none
+  int len, steps;
+  uint32_t last, bucket0;
+  static __device__ __forceinline__ uint32_t bucket_of(uint32_t distance) {
+    return __float_as_uint((float)(distance + 1u)) >> 20;  // does not decrease with the distance
+  }
+  __device__ __forceinline__ bool one(int32_t w) const {
+    int at = 0, end = len;
+    if (index) {
+      const uint32_t b = bucket_of(last - (uint32_t)w) - bucket0;  // (a key past the end: a far bucket)
+      const uint32_t r = index[min(b, (uint32_t)SI_BUCKETS)];
+      at = (int)(r & 0xffffu);
+      end = (int)(r >> 16);
     }
-    const uint32_t h = (uint32_t)(p0 < len && list[p0] == w.x) |
-                       ((uint32_t)(p1 < len && list[p1] == w.y) << 1) |
-                       ((uint32_t)(p2 < len && list[p2] == w.z) << 2) |
-                       ((uint32_t)(p3 < len && list[p3] == w.w) << 3);
-    return h & m;
+    for (int step = 1 << steps; step > 1;) {
+      step >>= 1;
+      if (at + step <= end && list[at + step - 1] < w) at += step;
+    }
+    return at < end && list[at] == w;
+  }
+  __device__ __forceinline__ uint32_t bits(const int4 &w, uint32_t m) const {
+    return ((uint32_t)one(w.x) | ((uint32_t)one(w.y) << 1) | ((uint32_t)one(w.z) << 2) |
+            ((uint32_t)one(w.w) << 3)) & m;
   }
   __device__ __forceinline__ uint32_t count(const int4 &w, uint32_t m) const {
     return __popc(bits(w, m));
@@ -115,12 +133,20 @@ struct InPlace {
   }
 };
 
+constexpr size_t flat_smem_bytes() {
+  return (size_t)FL_WARPS * ((STAGE + 4) * sizeof(int32_t) + sizeof(FlatSmem));
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
+__global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
   constexpr bool GRAPH = (MODE & FL_MODE_GRAPH) != 0;
   constexpr bool TASK = (MODE & FL_MODE_TASK) != 0;
+  // quads in flight per lane against a bitmap or a filter: 2, 3 and 4 gave 4.91,
+  // 4.38 and 4.19 ms on R-MAT scale 22 and 7.43, 6.84 and 6.87 ms on the 1/16
+  // Friendster-shaped graph; attribution to tasks, which keeps more registers
+  // live, 3.84, 4.06 and 4.30 ms on its 1/64 size at p = 16
+  constexpr int FL_QUADS = TASK ? 2 : 4;
   extern __shared__ __align__(16) unsigned char flat_smem[];
-  __shared__ unsigned long long table[TASK ? FL_TABLE : 1];
   __shared__ int32_t cuts_s[TASK ? 65 : 1];
   __shared__ uint32_t ecut_s[TASK ? 65 : 1];
   const unsigned lane = threadIdx.x & 31u;
@@ -128,6 +154,8 @@ __global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
   int32_t *stage = reinterpret_cast<int32_t *>(flat_smem) + warp * (STAGE + 4);
   FlatSmem &sm = reinterpret_cast<FlatSmem *>(flat_smem + (size_t)FL_WARPS * (STAGE + 4) *
                                                               sizeof(int32_t))[warp];
+  // task counters behind the warps' areas
+  unsigned long long *table = reinterpret_cast<unsigned long long *>(flat_smem + flat_smem_bytes());
   const bool in_table = TASK && P.ntasks <= FL_TABLE;
   const int p = P.one.p;
   if (TASK) {
@@ -211,6 +239,9 @@ __global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
     int32_t vl = -1;              // the lane's own destination (set when a run begins)
     int staged_mode = ST_NONE, staged_log2h = 0, staged_len = 0;
     const int32_t *staged_list = stage;
+    const uint32_t *staged_index = nullptr;
+    int staged_steps = 0;
+    uint32_t staged_last = 0, staged_bucket0 = 0;
     uint32_t staged_word0 = 0, staged_gw = STAGE;
     bool staged = false;
     int j_part = 0;
@@ -364,6 +395,37 @@ __global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
               for (int i = lane; i < blen; i += 32) stage[i] = i < 32 ? x0 : ci[b0 + i];
             }
             staged_len = blen;
+            staged_index = nullptr;
+            staged_steps = 32 - __clz(blen);
+            // the index goes behind the list
+            const int behind = (int)((span4 + 3) & ~int64_t(3));
+            if (!failed && behind + SI_BUCKETS + 1 <= STAGE) {
+              uint32_t *index = reinterpret_cast<uint32_t *>(stage + behind);
+              __syncwarp();
+              for (int i = lane; i <= SI_BUCKETS; i += 32) index[i] = 0u;
+              staged_last = (uint32_t)last;
+              staged_bucket0 = InSorted::bucket_of(0u);
+              __syncwarp();
+              int most = 0;
+              for (int i0 = 0; i0 < blen; i0 += 32) {
+                const int i = i0 + (int)lane;
+                if (i < blen) {
+                  // the first entry of a bucket finds its end and writes both
+                  const uint32_t b = InSorted::bucket_of(staged_last - (uint32_t)staged_list[i]);
+                  if (i == 0 || InSorted::bucket_of(staged_last - (uint32_t)staged_list[i - 1]) != b) {
+                    int e = i + 1;
+                    while (e < blen &&
+                           InSorted::bucket_of(staged_last - (uint32_t)staged_list[e]) == b)
+                      ++e;
+                    index[b - staged_bucket0] = (uint32_t)i | ((uint32_t)e << 16);
+                    most = max(most, e - i);
+                  }
+                }
+              }
+              most = __reduce_max_sync(0xffffffffu, most);
+              staged_index = index;
+              staged_steps = 32 - __clz(most);
+            }
           }
           __syncwarp();
           staged_mode = mode;
@@ -410,8 +472,8 @@ __global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
       __syncwarp();
       unsigned long long packed = 0;
       uint32_t hits = 0;
-      auto probe = [&](auto make) {
-        flat_rounds<2>(ci, sm.rec, total, first, has, lane, [&](int own, const int4 &w, uint32_t m, uint32_t) {
+      auto probe = [&](auto quads, auto make) {
+        flat_rounds<decltype(quads)::value>(ci, sm.rec, total, first, has, lane, [&](int own, const int4 &w, uint32_t m, uint32_t) {
           if (!TASK && (!GRAPH || uniform)) {
             hits += make(own).count(w, m);
             return;
@@ -465,22 +527,23 @@ __global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
       };
       if (uniform && staged && staged_mode == ST_BITMAP) {
         const InBitmap look{reinterpret_cast<const uint32_t *>(stage), staged_word0, staged_gw};
-        probe([&](int) { return look; });
+        probe(std::integral_constant<int, FL_QUADS>(), [&](int) { return look; });
       } else if (uniform && staged && staged_mode == ST_FILTER) {
         const InFilter look{reinterpret_cast<const uint32_t *>(stage), stage + FILTER_WORDS,
                             staged_log2h};
-        probe([&](int) { return look; });
+        probe(std::integral_constant<int, FL_QUADS>(), [&](int) { return look; });
       } else if (uniform && staged && staged_mode == ST_HASH) {
         const InHash look{stage, staged_log2h};
-        probe([&](int) { return look; });
+        probe(std::integral_constant<int, 1>(), [&](int) { return look; });
       } else if (uniform && staged) {
-        const InSorted look{staged_list, staged_len};
-        probe([&](int) { return look; });
+        const InSorted look{staged_list, staged_index, staged_len, staged_steps, staged_last,
+                            staged_bucket0};
+        probe(std::integral_constant<int, 1>(), [&](int) { return look; });
       } else if (uniform) {
         const InPlace look{ci, b0, b1};
-        probe([&](int) { return look; });
+        probe(std::integral_constant<int, 1>(), [&](int) { return look; });
       } else {
-        probe([&](int own) {
+        probe(std::integral_constant<int, 1>(), [&](int own) {
           const uint2 b = sm.rng[max(own, 0)];
           return InPlace{ci, b.x, b.y};
         });
@@ -519,13 +582,9 @@ __global__ void __launch_bounds__(FL_NT, 3) k_flat(FlatLaunch P) {
   }
 }
 
-size_t flat_smem_bytes() {
-  return (size_t)FL_WARPS * ((STAGE + 4) * sizeof(int32_t) + sizeof(FlatSmem));
-}
-
 template <int MODE>
 bbtc_status flat_configure(int *blocks_per_sm) {
-  const size_t smem = flat_smem_bytes();
+  const size_t smem = flat_smem_bytes() + (MODE & FL_MODE_TASK ? 8 * FL_TABLE : 0);
   BBTC_CUDA(cudaFuncSetAttribute(k_flat<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
   BBTC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_flat<MODE>, FL_NT, smem));
@@ -850,9 +909,11 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
   f.records = records;
   if (core.bits) pl.core.nitems = (int64_t)items;
   BBTC_TRY(dalloc_n(&f.rec, f.records, s));
-  // about 64 items per resident warp, 64 to 4,096 in-edges each (or the caller's choice)
+  // about 32 items per resident warp, 64 to 4,096 in-edges each (or the caller's
+  // choice); 64 and 128 items staged each list more often (R-MAT scale 21 at p = 4,
+  // per task: 3.16, 3.36 and 3.36 ms; scale 22: 4.86, 4.91 and 5.12 ms)
   const int64_t warps = (int64_t)num_sms() * 24;
-  int64_t chunk = f.records / (warps * 64);
+  int64_t chunk = f.records / (warps * 32);
   chunk = chunk < 64 ? 64 : (chunk > 4096 ? 4096 : chunk);
   if (pl.chunk_req > 0) chunk = pl.chunk_req;
   f.chunk = chunk;
@@ -956,9 +1017,11 @@ bbtc_status flat_launch(const FlatDesc &one, const FlatDesc *descs, int32_t nd, 
   P.t0 = t0;
   P.timeout_ns = (uint64_t)timeout_ms * 1000000ull;
   const int mode = (graph_count ? FL_MODE_GRAPH : 0) | (tasks && one.p > 1 ? FL_MODE_TASK : 0);
-  int64_t blocks = (int64_t)num_sms() * blocks_per_sm[mode];
+  // (a launch with fewer task counters than configured for may hold more blocks)
+  int64_t blocks = (int64_t)num_sms() * (mode & FL_MODE_TASK ? FL_CTAS : blocks_per_sm[mode]);
   blocks = std::min<int64_t>(blocks, (nitems + FL_WARPS - 1) / FL_WARPS);
-  const size_t smem = flat_smem_bytes();
+  const bool table = (mode & FL_MODE_TASK) != 0 && ntasks <= FL_TABLE;
+  const size_t smem = flat_smem_bytes() + (table ? 8 * (size_t)ntasks : 0);
   switch (mode) {
     case 0: k_flat<0><<<(unsigned)blocks, FL_NT, smem, s>>>(P); break;
     case 1: k_flat<1><<<(unsigned)blocks, FL_NT, smem, s>>>(P); break;
