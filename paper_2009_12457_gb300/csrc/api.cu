@@ -489,16 +489,16 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   // a resident count needs the block arrays on the device: a plan that was
   // streamed (its arrays now in host memory) is rebuilt
   if (!budgeted && g->plan.streamed) free_plan(&g->plan, s);
-  // counted task by task: with a budget, for a share of the tasks and for their cycles
-  const bool by_task = budgeted || opts.per_task_cycles_out || opts.task_mask;
-  const bool detail = !by_task && (opts.per_vertex_out || opts.per_edge_out);
+  // counted task by task: a share of the tasks, and their cycles
+  const bool by_task = opts.per_task_cycles_out || opts.task_mask;
+  const bool detail = !budgeted && !by_task && (opts.per_vertex_out || opts.per_edge_out);
   const bool tasks = opts.per_task_out != nullptr, per_graph = opts.per_graph_out != nullptr;
   // (a detail count alone needs neither the core nor the in-edges that it leaves)
-  const bool resident = !by_task && (!detail || tasks || per_graph);
+  const bool resident = !budgeted && !by_task && (!detail || tasks || per_graph);
   const Plan &old = g->plan;
   const bool rebuild =
       !plan_matches(old, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition) ||
-      (by_task && !old.tasks_ready) || (resident && !old.flat.ready) ||
+      (by_task && !old.tasks_ready) || (budgeted && !by_task && !old.h_rec) || (resident && !old.flat.ready) ||
       (detail && !old.full.ready && !(old.flat.ready && !old.core.bits));
   if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[2], s));
   BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
@@ -529,8 +529,12 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   }
   if (budgeted) {
     StreamStats st;
-    BBTC_TRY(run_count_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, per_graph,
-                                opts.timeout_ms, s, &st, task_cycles, task_mask));
+    if (by_task)
+      BBTC_TRY(run_count_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, per_graph,
+                                  opts.timeout_ms, s, &st, task_cycles, task_mask));
+    else
+      BBTC_TRY(run_flat_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, tasks,
+                                 per_graph, opts.timeout_ms, s, &st));
     g->stream_stats.rounds = st.rounds;
     g->stream_stats.h2d_bytes = st.h2d_bytes;
     g->stream_stats.copy_ms = st.copy_ms;
@@ -870,7 +874,7 @@ bbtc_status bbtc_graph_get_plan(bbtc_graph_t g, int32_t p, int32_t *cuts, int64_
   const int thr = g->plan.p == p ? g->plan.hash_threshold : 16;
   const int chunk = g->plan.p == p ? g->plan.chunk_req : 0;
   const int part = g->plan.p == p ? g->plan.partition : BBTC_PARTITION_EDGES;
-  BBTC_TRY(build_plan(g, p, kmode, thr, chunk, s, part));
+  BBTC_TRY(build_plan(g, p, kmode, thr, chunk, s, part, !g->plan.streamed));
   BBTC_TRY(build_tasks(g, s));
   const Plan &pl = g->plan;
   if (cuts)

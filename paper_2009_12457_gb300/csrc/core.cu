@@ -254,10 +254,14 @@ __device__ __forceinline__ int core_steps(ColumnSums &cols, const uint4 &m,
 // side, since the lanes below them would only read zeros. Columns: 8,192 beat
 // 12,288 on R-MAT scale 18 (0.165 against 0.173 ms for the whole count), they tie
 // on scale 20 (0.745, 0.740), and 12,288 win on scale 22 (4.91, 4.66) and on the
-// 1/16 Friendster-shaped graph (7.43, 7.32): hence CORE_WIDE_EDGES. ONE: a single descriptor with p = 1 and no per-graph counts, where a
-// lane keeps its sum to the end.
-template <bool ONE>
+// 1/16 Friendster-shaped graph (7.43, 7.32): hence CORE_WIDE_EDGES.
+// MODE 0: totals of one descriptor, where a lane keeps its sum to the end; 1:
+// totals of several, where it keeps it to the warp's last item of a descriptor
+// (64 handles: 0.82 ms; through mode 2 1.13); 2: per task or per graph.
+template <int MODE>
 __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P) {
+  constexpr bool ONE = MODE < 2;  // totals
+  constexpr bool MULTI = MODE == 1;
   extern __shared__ __align__(16) unsigned char core_smem[];
   __shared__ unsigned long long table[ONE ? 1 : CORE_TABLE];
   __shared__ uint32_t rows_s[CORE_WARPS][CORE_ROWS];
@@ -277,6 +281,7 @@ __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P)
     if (lane == 0) atomicCAS(P.t0, 0ull, (unsigned long long)t_start);
   }
   unsigned long long acc = 0;
+  int cur_desc = 0;
   const int64_t nw = (int64_t)gridDim.x * CORE_WARPS;
   for (int64_t item = (int64_t)blockIdx.x * CORE_WARPS + warp; item < P.nitems; item += nw) {
     if (P.timeout_ns && core_ns() - t_start > P.timeout_ns) {
@@ -284,13 +289,19 @@ __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P)
       break;
     }
     const CoreDesc *dp = &P.one;
-    if (!ONE && P.nd > 1) {
+    if (MULTI || (!ONE && P.nd > 1)) {
       int lo = 0, hi = P.nd;  // last descriptor with item_base <= item
       while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (P.descs[mid].item_base <= item) lo = mid; else hi = mid;
       }
       dp = &P.descs[lo];
+      if (MULTI && lo != cur_desc) {
+        acc = warp_sum(acc);
+        if (lane == 0 && acc) atomicAdd(&P.task_count[P.descs[cur_desc].task_base], acc);
+        acc = 0;
+        cur_desc = lo;
+      }
     }
     const CoreDesc &d = *dp;
     const int4 it = d.items[item - d.item_base];
@@ -413,7 +424,7 @@ __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P)
   }
   if (ONE) {
     acc = warp_sum(acc);
-    if (lane == 0 && acc) atomicAdd(&P.task_count[0], acc);
+    if (lane == 0 && acc) atomicAdd(&P.task_count[MULTI ? P.descs[cur_desc].task_base : 0], acc);
   } else if (in_table) {
     __syncthreads();
     for (int i = threadIdx.x; i < (int)P.ntasks; i += CORE_NT)
@@ -566,10 +577,12 @@ bbtc_status core_launch(CoreDesc one, const CoreDesc *descs, int32_t nd, int64_t
   P.timeout_ns = (uint64_t)timeout_ms * 1000000ull;
   const size_t smem = sizeof(uint4) * (size_t)quads_max * CORE_WARPS;
   const unsigned grid = grid_for(nitems, CORE_WARPS, 4);
-  if (nd == 1 && one.p == 1 && !graph_count)
-    k_core_count<true><<<grid, CORE_NT, smem, s>>>(P);
+  if (tasks || graph_count)
+    k_core_count<2><<<grid, CORE_NT, smem, s>>>(P);
+  else if (nd > 1)
+    k_core_count<1><<<grid, CORE_NT, smem, s>>>(P);
   else
-    k_core_count<false><<<grid, CORE_NT, smem, s>>>(P);
+    k_core_count<0><<<grid, CORE_NT, smem, s>>>(P);
   BBTC_LAUNCH_CHECK();
   return BBTC_OK;
 }

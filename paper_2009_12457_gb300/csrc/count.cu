@@ -739,7 +739,8 @@ bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph
     BBTC_TRY(count_reset(g, pl, nullptr, false, s));
     if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
   }
-  BBTC_TRY(detail_launch(g, pl, both ? nullptr : pl.scratch + SCR_TOTAL, vcount, edge_sup,
+  const Flat &f = pl.full.ready ? pl.full : pl.flat;
+  BBTC_TRY(detail_launch(g, pl, flat_desc(g, pl, f, 0, 0), both ? nullptr : pl.scratch + SCR_TOTAL, vcount, edge_sup,
                          timeout_ms, s));
   if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));
   return BBTC_OK;

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(DT_NT, 3) k_detail(DetailLaunch P) {
       if (lane == 0) atomicExch(P.status, STATUS_TIMEOUT);
       break;
     }
-    const int64_t k = d.nitems - 1 - (int64_t)it;
+    const int64_t k = d.item0 + d.nitems - 1 - (int64_t)it;
     uint32_t base = (uint32_t)(k * d.chunk);
     const uint32_t x1 = (uint32_t)min((int64_t)d.records, (k + 1) * d.chunk);
     uint32_t v = 0, vend = base, b0 = 0, b1 = 0;
@@ -313,13 +313,12 @@ bbtc_status detail_configure(int *blocks_per_sm) {
 
 }  // namespace
 
-bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, unsigned long long *total,
-                          unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
-                          cudaStream_t s) {
-  const Flat &f = pl.full.ready ? pl.full : pl.flat;
-  if (f.nitems <= 0) return BBTC_OK;
+bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, const FlatDesc &d,
+                          unsigned long long *total, unsigned long long *vcount,
+                          unsigned *edge_sup, uint32_t timeout_ms, cudaStream_t s) {
+  if (d.nitems <= 0) return BBTC_OK;
   DetailLaunch P;
-  P.d = flat_desc(g, pl, f, 0, 0);
+  P.d = d;
   P.esrc = g->esrc;
   P.head = pl.scratch + SCR_HEAD;
   P.total = total;
@@ -333,7 +332,7 @@ bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, unsigned long lon
   else if (vcount) BBTC_TRY(detail_configure<1>(&per_sm));
   else BBTC_TRY(detail_configure<2>(&per_sm));
   const int64_t blocks = std::min<int64_t>((int64_t)num_sms() * per_sm,
-                                           (f.nitems + DT_WARPS - 1) / DT_WARPS);
+                                           (d.nitems + DT_WARPS - 1) / DT_WARPS);
   const size_t smem = sizeof(DetailSmem) * DT_WARPS;
   BBTC_CUDA(cudaMemsetAsync(P.head, 0, sizeof(unsigned long long), s));
   if (vcount && edge_sup) k_detail<3><<<(unsigned)blocks, DT_NT, smem, s>>>(P);

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
     const int32_t *__restrict__ ci = d.colidx;
     const int kflag = d.flags & 3, hash_min = d.flags >> 2;
     // items run from the last destinations down, so that the light ones end the launch
-    const int64_t k = d.nitems - 1 - ((int64_t)it - d.item_base);
+    const int64_t k = d.item0 + d.nitems - 1 - ((int64_t)it - d.item_base);
     uint32_t base = (uint32_t)(k * d.chunk);
     const uint32_t x1 = (uint32_t)min((int64_t)d.records, (k + 1) * d.chunk);
     uint32_t v = 0, vend = base;  // the run at hand: its destination and end
@@ -842,6 +842,24 @@ __global__ void k_flat_indegree(const int64_t *__restrict__ rowptr, const int32_
     hist[r] = r < n ? (unsigned)(deg[perm[r]] - (int32_t)(rowptr[r + 1] - rowptr[r])) : 0u;
 }
 
+// the same by counting the edges (a union of handles has no degrees); the top
+// positions, which receive most edges of a skewed graph, are counted per CTA
+__global__ void __launch_bounds__(512) k_flat_count(const int32_t *__restrict__ colidx, int64_t m,
+                                                    int64_t n, unsigned *__restrict__ hist) {
+  __shared__ unsigned cnt[FC_COLS];
+  const int64_t first = n > FC_COLS ? n - FC_COLS : 0;
+  for (int i = threadIdx.x; i < FC_COLS; i += 512) cnt[i] = 0;
+  __syncthreads();
+  for (int64_t e = (int64_t)blockIdx.x * 512 + threadIdx.x; e < m; e += (int64_t)gridDim.x * 512) {
+    const int64_t v = colidx[e];
+    if (v >= first) atomicAdd(&cnt[v - first], 1u);
+    else atomicAdd(&hist[v], 1u);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < FC_COLS; i += 512)
+    if (cnt[i]) atomicAdd(&hist[first + i], cnt[i]);
+}
+
 __global__ void k_flat_widen(const unsigned *__restrict__ in, int64_t count,
                              uint64_t *__restrict__ out) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
@@ -888,7 +906,12 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
   BBTC_TRY(scratch.get(&hist, n + 1));
   BBTC_TRY(scratch.get(&scan, n + 1));
   BBTC_TRY(dalloc_n(&f.inptr, n + 1, s));
-  k_flat_indegree<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(g->rowptr, g->perm, g->deg, n, hist);
+  if (g->deg && g->perm) {
+    k_flat_indegree<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(g->rowptr, g->perm, g->deg, n, hist);
+  } else {
+    BBTC_CUDA(cudaMemsetAsync(hist, 0, sizeof(unsigned) * (size_t)(n + 1), s));
+    k_flat_count<<<grid_for(m, 512 * 16, 2), 512, 0, s>>>(g->colidx, m, n, hist);
+  }
   BBTC_LAUNCH_CHECK();
   if (core.bits) {
     k_flat_minus_core<<<(unsigned)num_sms() * 2, 512, 0, s>>>(core.items, core.count, CORE_CHUNK,
@@ -966,6 +989,7 @@ FlatDesc flat_desc(const bbtc_graph *g, const Plan &pl, const Flat &f, int64_t i
   d.records = f.records;
   d.nitems = f.nitems;
   d.item_base = item_base;
+  d.item0 = 0;
   d.chunk = f.chunk;
   d.flags = pl.kernel_mode == BBTC_KERNEL_HASHMAP     ? 1
             : pl.kernel_mode == BBTC_KERNEL_INTERSECT ? 0

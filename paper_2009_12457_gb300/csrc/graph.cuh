@@ -110,6 +110,7 @@ struct FlatDesc {
   const int32_t *gid;
   const int32_t *cuts;
   int64_t n, records, nitems, item_base, chunk;
+  int64_t item0;  // the nitems items counted start here (0, or a streamed round's first)
   int32_t flags;  // as WorkItem::flags
   int32_t p, task_base;
 };
@@ -177,9 +178,16 @@ struct Plan {
   int blocks_per_sm[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // occupancy of each counting-kernel mode
   // streamed mode: the block arrays live in pinned host memory instead
   bool streamed = false;
+  // (by task: h_rp, h_ci, h_ie; else the flat in-edges: h_rec)
   uint32_t *h_rp = nullptr;
   int32_t *h_ci = nullptr;
   InEdge *h_ie = nullptr;
+  uint2 *h_rec = nullptr;
+  // what a budget has to hold: every block CSR and two in-edge blocks (need_all), or
+  // else the three blocks of task need_task; any_task: some task's blocks hold edges
+  uint64_t need_all = 0, need_one = 0;
+  int32_t need_task[3] = {0, 0, 0};
+  bool any_task = false;
   uint64_t bytes = 0;
 };
 
@@ -297,8 +305,8 @@ bbtc_status run_flat(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
 // the caller, over all in-edges (build_full first); total (nullable) receives
 // the number of triangles. Enqueues only.
 bbtc_status build_full(bbtc_graph *g, cudaStream_t s);
-bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, unsigned long long *total,
-                          unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
+bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, const FlatDesc &d,
+                          unsigned long long *total, unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
                           cudaStream_t s);
 bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
                        unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
@@ -354,6 +362,16 @@ bbtc_status run_count_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
                                uint32_t timeout_ms, cudaStream_t s, StreamStats *stats,
                                unsigned long long *task_cycles = nullptr,
                                const uint8_t *task_mask = nullptr);
+
+// As above without a task mask or measured cycles: only the flat in-edges are
+// streamed, and every list is read in place in the oriented CSR, which the handle
+// keeps on the device in any case.
+bbtc_status run_flat_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
+                              unsigned long long *vertex_count, bool tasks, bool per_graph,
+                              uint32_t timeout_ms, cudaStream_t s, StreamStats *stats);
+
+// |G_ab| of every block (p * p, row-major) to the host. Synchronises s.
+bbtc_status block_sizes(const bbtc_graph *g, const Plan &pl, int64_t *nnz, cudaStream_t s);
 
 // Work figures of the oriented graph (device): sum_{(u,v)} d+(v) and
 // sum_u d+(u)(d+(u)-1)/2.

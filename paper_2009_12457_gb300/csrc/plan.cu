@@ -471,6 +471,32 @@ __global__ void k_bcsr_rowptr(const uint64_t *__restrict__ pos, int64_t total,
     rp[i] = (uint32_t)pos[i];
 }
 
+// nnz[a * p + b] += entries of row u of part a in part b (one thread per row).
+__global__ void k_block_sizes(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                              int64_t n, const int32_t *__restrict__ cuts_g, int p,
+                              unsigned long long *__restrict__ nnz) {
+  __shared__ int32_t cuts[MAXP + 1];
+  extern __shared__ unsigned long long block_cnt[];  // p * p
+  for (int i = threadIdx.x; i <= p; i += blockDim.x) cuts[i] = cuts_g[i];
+  for (int i = threadIdx.x; i < p * p; i += blockDim.x) block_cnt[i] = 0;
+  __syncthreads();
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r1 = rowptr[u + 1];
+    int64_t lo = rowptr[u];
+    if (lo == r1) continue;
+    const int a = part_of_dev(cuts, p, (int32_t)u);
+    for (int b = a; b < p && lo < r1; ++b) {
+      const int64_t hi = b + 1 < p ? lower_bound_dev<int32_t, int64_t>(colidx, lo, r1, cuts[b + 1]) : r1;
+      if (hi > lo) atomicAdd(&block_cnt[a * p + b], (unsigned long long)(hi - lo));
+      lo = hi;
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < p * p; i += blockDim.x)
+    if (block_cnt[i]) atomicAdd(&nnz[i], block_cnt[i]);
+}
+
 __device__ __forceinline__ int64_t block_nnz(const int64_t *boff, int p, int i, int j) {
   return boff[i * (p + 1) + j + 1] - boff[i * (p + 1) + j];
 }
@@ -667,6 +693,22 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   pl.bytes = (uint64_t)(SCR_TASKS + pl.ntasks + g->ng) * 8;
   if (resident) PLAN_TRY(add_resident(g, pl, s));
   g->plan = pl;
+  return BBTC_OK;
+}
+
+bbtc_status block_sizes(const bbtc_graph *g, const Plan &pl, int64_t *nnz, cudaStream_t s) {
+  const int p = pl.p;
+  Scratch scratch(s);
+  unsigned long long *d = nullptr;
+  BBTC_TRY(scratch.get(&d, (int64_t)p * p));
+  BBTC_CUDA(cudaMemsetAsync(d, 0, sizeof(uint64_t) * (size_t)p * p, s));
+  if (g->n > 0) {
+    k_block_sizes<<<grid_for(g->n, 256, 4), 256, sizeof(uint64_t) * (size_t)p * p, s>>>(
+        g->rowptr, g->colidx, g->n, pl.cuts, p, d);
+    BBTC_LAUNCH_CHECK();
+  }
+  BBTC_CUDA(cudaMemcpyAsync(nnz, d, sizeof(uint64_t) * (size_t)p * p, cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaStreamSynchronize(s));
   return BBTC_OK;
 }
 

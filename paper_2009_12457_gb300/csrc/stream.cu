@@ -107,7 +107,7 @@ bbtc_status to_pinned(T **host, T **dev, int64_t count, cudaStream_t s) {
 // Moves the block arrays of a resident plan to pinned host memory, as
 // physical per-block copies.
 bbtc_status plan_to_host(const bbtc_graph *g, Plan &pl, int64_t m, cudaStream_t s) {
-  if (pl.streamed) return BBTC_OK;
+  if (pl.h_ie) return BBTC_OK;
   BBTC_TRY(plan_physical_blocks(g, pl, s));
   BBTC_TRY(to_pinned(&pl.h_rp, &pl.rp, pl.total_rp, s));
   BBTC_TRY(to_pinned(&pl.h_ci, &pl.ci, m, s));
@@ -124,6 +124,8 @@ bbtc_status plan_to_host(const bbtc_graph *g, Plan &pl, int64_t m, cudaStream_t 
   free_core(&pl, s);
   free_flat(&pl.flat, s);
   free_flat(&pl.full, s);
+  pinned_release(pl.h_rec);
+  pl.h_rec = nullptr;
   // work items in Alg. 4 task order (a task's items stay together and keep
   // their order), so that the tasks sharing an in-edge block are consecutive
   if (pl.nitems > 0) {
@@ -161,6 +163,8 @@ void free_plan_host(Plan *pl) {
   pinned_release(pl->h_rp);
   pinned_release(pl->h_ci);
   pinned_release(pl->h_ie);
+  pinned_release(pl->h_rec);
+  pl->h_rec = nullptr;
   pl->h_rp = nullptr;
   pl->h_ci = nullptr;
   pl->h_ie = nullptr;
@@ -586,6 +590,211 @@ bbtc_status run_count_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
   for (cudaEvent_t e : {copy_done[0], copy_done[1], kern_done[0], kern_done[1], t_begin, t_end})
     if (e) cudaEventDestroy(e);
   for (TaskDesc *d : stage) pinned_release(d);
+  return st;
+}
+
+
+// What a budget has to hold for the plan's blocks (16-byte in-edges, block CSRs).
+static bbtc_status budget_needs(const bbtc_graph *g, Plan &pl, cudaStream_t s) {
+  const int p = pl.p;
+  std::vector<int64_t> nnz((size_t)p * p);
+  BBTC_TRY(block_sizes(g, pl, nnz.data(), s));
+  auto edges = [&](int a, int b) { return (size_t)nnz[(size_t)(a * p + b)]; };
+  auto csr = [&](int a, int b) {
+    return align_up(4 * (size_t)(pl.h_cuts[a + 1] - pl.h_cuts[a] + 1)) + align_up(4 * edges(a, b));
+  };
+  auto ie = [&](int a, int b) { return align_up(sizeof(InEdge) * edges(a, b)); };
+  size_t all = 0, ie_max = 0;
+  for (int a = 0; a < p; ++a)
+    for (int b = a; b < p; ++b) {
+      all += csr(a, b);
+      ie_max = std::max(ie_max, ie(a, b));
+    }
+  pl.need_all = all + 2 * ie_max;
+  pl.need_one = 0;
+  pl.any_task = false;
+  for (int i = 0; i < p; ++i)
+    for (int j = i; j < p; ++j)
+      for (int k = j; k < p; ++k) {
+        if (!edges(i, j) || !edges(i, k) || !edges(j, k)) continue;
+        pl.any_task = true;
+        const size_t need = ie(i, j) + csr(i, k) + (i == j ? 0 : csr(j, k));
+        if (need > pl.need_one) {
+          pl.need_one = need;
+          pl.need_task[0] = i;
+          pl.need_task[1] = j;
+          pl.need_task[2] = k;
+        }
+      }
+  return BBTC_OK;
+}
+
+// The flat in-edges in pinned host memory, in rounds of whole work items through
+// the two halves of the pool: the next round's copy runs while this one counts.
+// The pool is allocated, and budgets are refused, as in run_count_streamed:
+// when neither every block CSR and two in-edge blocks nor the three blocks of
+// each task fit. R-MAT scale 20 at p = 8 in
+// 192 MB: 1.8 ms, 126 MB copied; block by block and task by task (36 rounds,
+// 346 MB) 10.0 ms.
+bbtc_status run_flat_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
+                              unsigned long long *vertex_count, bool tasks, bool per_graph,
+                              uint32_t timeout_ms, cudaStream_t s, StreamStats *stats) {
+  const size_t pool_bytes = (size_t)budget & ~(ALIGN - 1);
+  if (!pl.h_rec) BBTC_TRY(budget_needs(g, pl, s));
+  if (pl.need_all > pool_bytes && pl.need_one > pool_bytes) {
+    set_error("streamed count: the blocks of task (%d,%d,%d) do not fit in a %llu-byte "
+              "device budget", pl.need_task[0], pl.need_task[1], pl.need_task[2],
+              (unsigned long long)budget);
+    return BBTC_ENOMEM;
+  }
+  // (any task's blocks take more than 512 bytes, so each half of the pool holds a record)
+  // ---- the in-edges to pinned host memory, once per plan
+  Flat &f = pl.full;
+  if (!pl.h_rec) {
+    BBTC_TRY(build_full(g, s));
+    if (!f.ready) std::swap(pl.full, pl.flat);  // an INTERSECT plan's flat in-edges are all of them
+    BBTC_TRY(to_pinned(&pl.h_rec, &f.rec, f.records, s));
+    BBTC_CUDA(cudaStreamSynchronize(s));
+    dfree(f.rec, s);
+    f.rec = nullptr;
+    pl.bytes -= pl.core.bytes + pl.flat.bytes + (uint64_t)f.records * 8;
+    f.bytes -= (uint64_t)f.records * 8;
+    free_core(&pl, s);
+    free_flat(&pl.flat, s);
+    pl.streamed = true;
+  }
+  release_cached_blocks(g->device, s);
+  Scratch scratch(s);
+  unsigned char *pool = nullptr;
+  BBTC_TRY(scratch.get(&pool, (int64_t)pool_bytes));
+  const uint64_t total_bytes = (uint64_t)f.records * sizeof(uint2);
+  stats->block_bytes = total_bytes;
+  stats->mode = 1;
+  cudaMemPool_t mem_pool = nullptr;
+  {
+    int dev = 0;
+    uint64_t zero = 0;  // resets the high-water mark to the memory in use now
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetDefaultMemPool(&mem_pool, dev) == cudaSuccess)
+      cudaMemPoolSetAttribute(mem_pool, cudaMemPoolAttrUsedMemHigh, &zero);
+    else
+      mem_pool = nullptr;
+  }
+  // records of a round: half the pool at most; about an eighth of the whole, so that
+  // the first copy, which nothing overlaps, is short (but 4 MB, so that launches are
+  // few); whole work items
+  const size_t half = (pool_bytes / 2) & ~(ALIGN - 1);
+  const uint64_t wish = std::max<uint64_t>(total_bytes / 8, 4ull << 20);
+  int64_t per_round = (int64_t)(std::min<uint64_t>(half, wish) / sizeof(uint2)) / f.chunk;
+  // (an item larger than half the pool: the caller's chunk; items are re-cut)
+  int64_t chunk = f.chunk;
+  if (per_round < 1) {
+    chunk = std::max<int64_t>((int64_t)(half / sizeof(uint2)), 1);
+    per_round = 1;
+  }
+  const int64_t nitems = (f.records + chunk - 1) / chunk;
+  cudaStream_t cs = nullptr;
+  cudaEvent_t copied[2] = {nullptr, nullptr}, counted[2] = {nullptr, nullptr};
+  cudaEvent_t t_begin = nullptr, t_end = nullptr;
+  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> copy_ev;
+  bbtc_status st = BBTC_OK;
+  unsigned long long *scr = pl.scratch;
+  unsigned long long *graphs = per_graph ? scr + SCR_TASKS + pl.ntasks : nullptr;
+  int32_t *status = reinterpret_cast<int32_t *>(scr + SCR_STATUS);
+  // per-task and per-graph counts come from the flat kernel; per-vertex counts from the
+  // detail kernel, which gives the total too when it runs alone
+  const bool flat_too = !vertex_count || tasks || per_graph;
+  do {
+    bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreate(&t_begin) == cudaSuccess && cudaEventCreate(&t_end) == cudaSuccess;
+    for (int h = 0; h < 2 && ok; ++h)
+      ok = cudaEventCreateWithFlags(&copied[h], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&counted[h], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+      set_error("streamed count: creating streams or events failed");
+      st = BBTC_ECUDA;
+      break;
+    }
+    if ((st = count_reset(g, pl, vertex_count, per_graph, s)) != BBTC_OK) break;
+    if (cudaEventRecord(t_begin, s) != cudaSuccess ||
+        cudaStreamWaitEvent(cs, t_begin, 0) != cudaSuccess) {
+      set_error("streamed count: recording events failed");
+      st = BBTC_ECUDA;
+      break;
+    }
+    int64_t round = 0;
+    // items from the last destinations down, as the resident count takes them
+    for (int64_t end = pl.any_task ? nitems : 0; end > 0 && st == BBTC_OK; end -= per_round, ++round) {
+      const int64_t item0 = std::max<int64_t>(end - per_round, 0);
+      const int64_t x0 = item0 * chunk, x1 = std::min(f.records, end * chunk);
+      const int h = (int)(round & 1);
+      unsigned char *slot = pool + (size_t)h * half;
+      cudaEvent_t c0 = nullptr, c1 = nullptr;
+      cudaEventCreate(&c0);
+      cudaEventCreate(&c1);
+      copy_ev.emplace_back(c0, c1);
+      bool good = round < 2 || cudaStreamWaitEvent(cs, counted[h], 0) == cudaSuccess;
+      cudaEventRecord(c0, cs);
+      good = good && cudaMemcpyAsync(slot, pl.h_rec + x0, sizeof(uint2) * (size_t)(x1 - x0),
+                                     cudaMemcpyHostToDevice, cs) == cudaSuccess;
+      cudaEventRecord(c1, cs);
+      good = good && cudaEventRecord(copied[h], cs) == cudaSuccess &&
+             cudaStreamWaitEvent(s, copied[h], 0) == cudaSuccess;
+      if (!good) {
+        set_error("streamed count: host-to-device block copy failed");
+        st = BBTC_ECUDA;
+        break;
+      }
+      stats->h2d_bytes += sizeof(uint2) * (uint64_t)(x1 - x0);
+      FlatDesc d = flat_desc(g, pl, f, 0, 0);
+      d.rec = reinterpret_cast<const uint2 *>(slot) - x0;  // record x of the plan at rec[x]
+      d.chunk = chunk;
+      d.item0 = item0;
+      d.nitems = end - item0;
+      if (flat_too) {
+        if (cudaMemsetAsync(scr + SCR_HEAD, 0, sizeof(unsigned long long), s) != cudaSuccess) {
+          set_error("streamed count: cudaMemsetAsync failed");
+          st = BBTC_ECUDA;
+          break;
+        }
+        st = flat_launch(d, nullptr, 1, d.nitems, scr + SCR_HEAD,
+                         tasks ? scr + SCR_TASKS : scr + SCR_TOTAL, tasks ? pl.ntasks : 1, tasks,
+                         graphs, status, scr + SCR_T0, timeout_ms, pl.flat_blocks_per_sm, s);
+      }
+      if (st == BBTC_OK && vertex_count)
+        st = detail_launch(g, pl, d, flat_too ? nullptr : scr + SCR_TOTAL, vertex_count, nullptr,
+                           timeout_ms, s);
+      if (st == BBTC_OK && cudaEventRecord(counted[h], s) != cudaSuccess) {
+        set_error("streamed count: recording events failed");
+        st = BBTC_ECUDA;
+      }
+    }
+    stats->rounds = round;
+    if (st != BBTC_OK) break;
+    if (tasks) st = count_finish(pl, s);
+    if (st == BBTC_OK && cudaEventRecord(t_end, s) != cudaSuccess) st = BBTC_ECUDA;
+  } while (0);
+  cudaStreamSynchronize(s);
+  if (cs) {
+    cudaStreamSynchronize(cs);
+    cudaStreamDestroy(cs);
+  }
+  float ms = 0.f;
+  if (st == BBTC_OK && cudaEventElapsedTime(&ms, t_begin, t_end) == cudaSuccess)
+    stats->total_ms = ms;
+  for (auto &ev : copy_ev) {
+    if (cudaEventElapsedTime(&ms, ev.first, ev.second) == cudaSuccess) stats->copy_ms += ms;
+    cudaEventDestroy(ev.first);
+    cudaEventDestroy(ev.second);
+  }
+  cudaGetLastError();
+  if (mem_pool) {
+    uint64_t peak = 0;
+    if (cudaMemPoolGetAttribute(mem_pool, cudaMemPoolAttrUsedMemHigh, &peak) == cudaSuccess)
+      stats->device_peak = peak;
+  }
+  for (cudaEvent_t e : {copied[0], copied[1], counted[0], counted[1], t_begin, t_end})
+    if (e) cudaEventDestroy(e);
   return st;
 }
 
