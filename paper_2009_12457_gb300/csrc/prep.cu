@@ -823,6 +823,157 @@ __global__ void k_gather_rows(const int64_t *__restrict__ rowptr, int64_t n, Row
   }
 }
 
+// ------------------------------------------------------------------------
+// Graphs of up to 1,024 vertices: the whole preparation in one CTA, whose shared
+// memory holds the adjacency matrix as bits. Setting bits takes any input form
+// (one or both directions, any order, duplicates) and removes duplicates by
+// itself, degrees are population counts, and a row's upward neighbours, set
+// again by rank, come out sorted. What bounds such a graph is launches and
+// round trips to the host, not work: R-MAT scale 10 took 13 kernels and 4
+// synchronisations here (about 180 us), and takes one of each.
+constexpr int SG_N = 1024;
+constexpr int64_t SG_ENTRIES = 1 << 17;  // input entries of one CTA at most
+constexpr int SG_NT = 1024;
+
+struct SmallSmem {
+  uint32_t bits[SG_N][SG_N / 32 + 1];  // (rows of 33 words: a column's words lie in 32 banks)
+  uint32_t row[SG_N + 1];     // input row pointers
+  int32_t rank[SG_N];
+  uint32_t sort[SG_N];        // exchange buffer of the sort, then out-degrees by rank
+  uint32_t scan_tmp[SG_NT / 32 + 1];
+  int32_t err, dmax, dpmax;
+};
+
+// stats: {m, largest out-degree, largest degree, error bits as in the passes above}
+__global__ void __launch_bounds__(SG_NT) k_small_graph(const int64_t *__restrict__ rowptr,
+                                                       const int32_t *__restrict__ colidx, int n,
+                                                       int nnz, bool symmetric,
+                                                       int32_t *__restrict__ deg,
+                                                       int32_t *__restrict__ perm,
+                                                       int64_t *__restrict__ rowptr_o,
+                                                       int32_t *__restrict__ colidx_o,
+                                                       int32_t *__restrict__ esrc,
+                                                       int64_t *__restrict__ stats) {
+  extern __shared__ __align__(16) unsigned char small_smem[];
+  SmallSmem &sm = *reinterpret_cast<SmallSmem *>(small_smem);
+  const int t = threadIdx.x, warp = t >> 5;
+  const unsigned lane = t & 31u;
+  if (t == 0) sm.err = sm.dmax = sm.dpmax = 0;
+  auto clear = [&]() {
+    for (int i = t; i < SG_N * (SG_N / 32 + 1); i += SG_NT) (&sm.bits[0][0])[i] = 0;
+  };
+  clear();
+  __syncthreads();
+  {
+    // row pointers, checked and clamped into the entries
+    const int64_t b = t < n ? rowptr[t] : 0, e = t < n ? rowptr[t + 1] : 0;
+    if (b > e || (t == 0 && b != 0)) atomicOr(&sm.err, 1);
+    if (t < n) sm.row[t] = (uint32_t)(b < 0 ? 0 : b > nnz ? nnz : b);
+    if (t == n - 1) sm.row[n] = (uint32_t)nnz;
+  }
+  __syncthreads();
+  // every entry (u, v) that may be an edge
+  auto entries = [&](auto edge) {
+    for (int e0 = t; e0 < nnz; e0 += 4 * SG_NT) {
+      int32_t v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = e0 + i * SG_NT < nnz ? colidx[e0 + i * SG_NT] : -1;
+      int lo[4] = {0, 0, 0, 0};  // last row that starts at or before the entry
+      for (int step = SG_N / 2; step > 0; step >>= 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (lo[i] + step < n && sm.row[lo[i] + step] <= (uint32_t)(e0 + i * SG_NT)) lo[i] += step;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (e0 + i * SG_NT < nnz) {
+          if (v[i] < 0 || v[i] >= n) atomicOr(&sm.err, 2);
+          else if (v[i] != lo[i] && (!symmetric || lo[i] < v[i])) edge(lo[i], v[i]);
+        }
+    }
+  };
+  entries([&](int u, int v) {
+    atomicOr(&sm.bits[u][v >> 5], 1u << (v & 31));
+    atomicOr(&sm.bits[v][u >> 5], 1u << (u & 31));
+  });
+  __syncthreads();
+  for (int u = warp; u < SG_N; u += SG_NT / 32) {
+    const int d = __reduce_add_sync(0xffffffffu, __popc(sm.bits[u][lane]));
+    if (lane == 0) {
+      sm.sort[u] = u < n ? ((uint32_t)d << 10) | (uint32_t)u : 0xffffffffu;
+      if (u < n) deg[u] = d;
+      if (d > 0) atomicMax(&sm.dmax, d);
+    }
+  }
+  __syncthreads();
+  // order by (degree, id): bitonic sort, one key per thread
+  uint32_t x = sm.sort[t];
+  for (int k = 2; k <= SG_N; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      uint32_t y;
+      if (j >= 32) {
+        __syncthreads();
+        sm.sort[t] = x;
+        __syncthreads();
+        y = sm.sort[t ^ j];
+      } else {
+        y = __shfl_xor_sync(0xffffffffu, x, j);
+      }
+      const bool up = (t & k) == 0, lower = (t & j) == 0;
+      x = (lower == up) ? min(x, y) : max(x, y);
+    }
+  __syncthreads();
+  if (t < n) {
+    const int32_t v = (int32_t)(x & 1023u);
+    sm.rank[v] = t;
+    perm[t] = v;
+  }
+  __syncthreads();
+  // the same entries again, as upward neighbours by rank
+  clear();
+  __syncthreads();
+  entries([&](int u, int v) {
+    const int ru = sm.rank[u], rv = sm.rank[v];
+    const int a = min(ru, rv), b = max(ru, rv);
+    atomicOr(&sm.bits[a][b >> 5], 1u << (b & 31));
+  });
+  __syncthreads();
+  for (int r = warp; r < SG_N; r += SG_NT / 32) {
+    const int d = __reduce_add_sync(0xffffffffu, __popc(sm.bits[r][lane]));
+    if (lane == 0) {
+      sm.sort[r] = (uint32_t)d;
+      if (d > 0) atomicMax(&sm.dpmax, d);
+    }
+  }
+  __syncthreads();
+  uint32_t m = 0;
+  const uint32_t at = block_exclusive_scan<uint32_t, SG_NT>(sm.sort[t], sm.scan_tmp, &m);
+  sm.sort[t] = at;
+  if (t < n) rowptr_o[t] = (int64_t)at;
+  if (t == 0) {
+    rowptr_o[n] = (int64_t)m;
+    stats[0] = (int64_t)m;
+    stats[1] = sm.dpmax;
+    stats[2] = sm.dmax;
+    stats[3] = sm.err;
+  }
+  __syncthreads();
+  for (int r = warp; r < n; r += SG_NT / 32) {
+    const uint32_t word = sm.bits[r][lane];
+    uint32_t pos = sm.sort[r];
+    // one word at a time, a lane per bit
+    for (unsigned left = __ballot_sync(0xffffffffu, word != 0u); left; left &= left - 1) {
+      const int w = __ffs(left) - 1;
+      const uint32_t x = __shfl_sync(0xffffffffu, word, w);
+      if ((x >> lane) & 1u) {
+        const uint32_t o = pos + __popc(x & ((1u << lane) - 1u));
+        colidx_o[o] = w * 32 + (int)lane;
+        esrc[o] = r;
+      }
+      pos += __popc(x);
+    }
+  }
+}
+
 }  // namespace
 
 // Sorts every row of an oriented CSR whose rows have at most SEG_CAP entries
@@ -985,12 +1136,53 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   return BBTC_OK;
 }
 
+// a1-a4 of a small graph in one kernel.
+static bbtc_status prepare_small(bbtc_graph *g, const int64_t *d_rowptr, const int32_t *d_colidx,
+                                 int64_t nnz, bool symmetric) {
+  cudaStream_t s = g->stream;
+  const int64_t n = g->n;
+  // an entry gives at most one edge
+  const int64_t room = nnz < n * (n - 1) / 2 ? nnz : n * (n - 1) / 2;
+  Scratch scratch(s);
+  int64_t *stats = nullptr;
+  BBTC_TRY(scratch.get(&stats, 4));
+  BBTC_TRY(dalloc_n(&g->deg, n, s));
+  BBTC_TRY(dalloc_n(&g->perm, n, s));
+  BBTC_TRY(dalloc_n(&g->rowptr, n + 1, s));
+  BBTC_TRY(dalloc_n(&g->colidx, padded_columns(room), s));
+  BBTC_TRY(dalloc_n(&g->esrc, room, s));
+  g->bytes += (uint64_t)n * 8 + (uint64_t)(n + 1) * 8 + (uint64_t)room * 8;
+  BBTC_CUDA(cudaFuncSetAttribute(k_small_graph, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(SmallSmem)));
+  k_small_graph<<<1, SG_NT, sizeof(SmallSmem), s>>>(d_rowptr, d_colidx, (int)n, (int)nnz, symmetric,
+                                                    g->deg, g->perm, g->rowptr, g->colidx, g->esrc,
+                                                    stats);
+  BBTC_LAUNCH_CHECK();
+  int64_t h[4] = {0, 0, 0, 0};
+  BBTC_CUDA(cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaStreamSynchronize(s));
+  if (h[3] & 1) {
+    set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
+    return BBTC_EINVAL;
+  }
+  if (h[3] & 2) {
+    set_error("bbtc_graph_create: colidx entry outside [0, n)");
+    return BBTC_EINVAL;
+  }
+  g->m = h[0];
+  g->dplus_max = h[1];
+  g->deg_max = h[2];
+  return BBTC_OK;
+}
+
 bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t *d_colidx,
                           int64_t nnz, bool symmetric) {
   cudaStream_t s = g->stream;
   const int64_t n = g->n;
   const int nb = ceil_log2_u64((uint64_t)n) < 1 ? 1 : ceil_log2_u64((uint64_t)n);
   g->nb = nb;
+  if (n > 0 && n <= SG_N && nnz > 0 && nnz <= SG_ENTRIES && !g->voff)
+    return prepare_small(g, d_rowptr, d_colidx, nnz, symmetric);
   Scratch scratch(s);
   int32_t *err = nullptr;
   int64_t *hstats = nullptr;  // device: [0]=m, [1]=deg_max, [2]=err

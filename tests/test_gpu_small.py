@@ -1,0 +1,53 @@
+"""Graphs prepared in one kernel (up to 1,024 vertices) against the oracle: every
+input form, the sizes around its limits, and its error cases."""
+import numpy as np
+import pytest
+
+import graphgen
+import oracle
+import paper_2009_12457_gb300 as bb
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
+
+
+def one_sided(n, src, dst):
+    order = np.argsort(src, kind="stable")
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(src, minlength=n), out=rowptr[1:])
+    return n, rowptr, dst[order].astype(np.int32)
+
+
+@pytest.mark.parametrize("n,pairs", [(1, 3), (2, 5), (31, 60), (33, 400), (1000, 20_000),
+                                     (1023, 900), (1024, 30_000), (1024, 65_536), (1024, 65_537),
+                                     (1025, 30_000)])
+def test_small_graph_matches_oracle(n, pairs):
+    _, src, dst = graphgen.gnm_pairs(n, pairs, n + pairs)
+    sym = graphgen.pairs_to_csr(n, src, dst)  # duplicates and self-loops as drawn
+    ref = oracle.bbtc(*sym, p=3, want_per_vertex=True)
+    for graph, symmetric in ((sym, True), (sym, False), (one_sided(n, src, dst), False)):
+        with bb.Graph(*graph, symmetric=symmetric) as g:
+            o = g.oriented()
+            assert np.array_equal(o["rowptr"], ref["rowptr"])
+            assert np.array_equal(o["colidx"], ref["colidx"])
+            assert np.array_equal(o["perm"], ref["perm"])
+            i = g.info()
+            assert i["m"] == len(ref["colidx"])
+            assert i["dplus_max"] == int(np.diff(ref["rowptr"]).max())
+            out = g.count(p=3, per_task=True, per_vertex=True)
+            assert out["total"] == ref["total"]
+            assert np.array_equal(out["per_task"], ref["per_task"])
+            assert np.array_equal(out["per_vertex"], ref["per_vertex"])
+
+
+def test_small_graph_rejects_malformed_input():
+    rp = np.array([0, 2, 4, 6], dtype=np.int64)
+    ci = np.array([1, 2, 0, 2, 0, 1], dtype=np.int32)
+    for bad_rp, bad_ci in (([0, 4, 2, 6], ci), ([1, 2, 4, 6], ci), (rp, [1, 2, 0, 3, 0, 1]),
+                           (rp, [1, 2, 0, -1, 0, 1])):
+        for symmetric in (False, True):
+            with pytest.raises(bb.BbtcError) as e:
+                bb.Graph(3, np.asarray(bad_rp, dtype=np.int64), np.asarray(bad_ci, dtype=np.int32),
+                         symmetric=symmetric)
+            assert e.value.status == 1
