@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(UQ_NT) k_unique_write(const uint64_t *__restri
                                                         int nb, uint64_t *__restrict__ ukeys,
                                                         int32_t *__restrict__ deg) {
   __shared__ uint64_t tmp[UQ_NT / 32 + 1];
+  __shared__ uint64_t out[UQ_TILE];  // the tile's distinct keys, written with coalesced stores
   if (*err & SORT_FAILED) count = 0;
   const int64_t base = (int64_t)blockIdx.x * UQ_TILE + (int64_t)threadIdx.x * UQ_ITEMS;
   const unsigned lane = threadIdx.x & 31u;
@@ -74,15 +75,14 @@ __global__ void __launch_bounds__(UQ_NT) k_unique_write(const uint64_t *__restri
     prev = k[i];
   }
   uint64_t total;
-  uint64_t pos = block_exclusive_scan<uint64_t, UQ_NT>((uint64_t)__popc(heads), tmp, &total) +
-                 block_off[blockIdx.x];
+  uint64_t pos = block_exclusive_scan<uint64_t, UQ_NT>((uint64_t)__popc(heads), tmp, &total);
   const uint64_t mask = (1ull << nb) - 1ull;
   int64_t cur = -1;
   int cnt = 0, groups = 0;
 #pragma unroll
   for (int i = 0; i < UQ_ITEMS; ++i) {
     if ((heads >> i) & 1u) {
-      ukeys[pos++] = k[i];
+      out[pos++] = k[i];
       const int64_t a = (int64_t)(k[i] >> nb);
       atomicAdd(&deg[k[i] & mask], 1);
       if (a != cur) {
@@ -101,6 +101,9 @@ __global__ void __launch_bounds__(UQ_NT) k_unique_write(const uint64_t *__restri
   } else if (cur >= 0) {
     atomicAdd(&deg[cur], cnt);
   }
+  __syncthreads();
+  const uint64_t off = block_off[blockIdx.x];
+  for (int i = threadIdx.x; i < (int)total; i += UQ_NT) ukeys[off + i] = out[i];
 }
 
 // a3 keys: (degree << nb) | id, so ascending order is (degree, id).
@@ -213,18 +216,64 @@ struct TileRows {
 };
 static_assert(SP_TILE / 32 == 64 && SP_ITEMS == 8, "tile layout");
 
-// Marks the tile of entries [t0, t1), whose rows are rlo .. rhi. Block-wide.
+// What a block needs of a tile, loaded while it works on the tile before it (the
+// rows of the tile's ends, two tiles ahead): row pointers of up to SP_NT rows, the
+// thread's eight entries and the one before them.
+struct TileAhead {
+  int64_t rlo, rhi;      // rows of the tile's first entry and of the next tile's
+  int64_t begin, end;    // row rlo + 1 + threadIdx.x
+  int64_t start;         // of row rlo
+  int32_t w[SP_ITEMS];
+  int32_t prev;
+};
+
+__device__ __forceinline__ void load_entries(const int32_t *__restrict__ colidx, int64_t first,
+                                             int64_t t1, bool aligned, int32_t (&v)[SP_ITEMS]);
+
+__device__ __forceinline__ void tile_ends(TileAhead &a, const int64_t *__restrict__ tile_rows,
+                                          int64_t tile, int64_t ntiles) {
+  if (tile < ntiles) {
+    a.rlo = tile_rows[tile];
+    a.rhi = tile_rows[tile + 1];
+  }
+}
+
+__device__ __forceinline__ void tile_load(TileAhead &a, const int64_t *__restrict__ rowptr,
+                                          const int32_t *__restrict__ colidx, int64_t nnz,
+                                          int64_t tile, int64_t ntiles, bool aligned) {
+  if (tile >= ntiles) return;
+  const int64_t first = tile * SP_TILE + (int64_t)threadIdx.x * SP_ITEMS;
+  const int64_t t1 = (tile + 1) * SP_TILE < nnz ? (tile + 1) * SP_TILE : nnz;
+  const int64_t r = a.rlo + 1 + threadIdx.x;
+  a.begin = a.end = 0;
+  if (r <= a.rhi) {
+    a.begin = rowptr[r];
+    a.end = rowptr[r + 1];
+  }
+  a.start = rowptr[a.rlo];
+  a.prev = -1;
+  if (first < t1) {
+    load_entries(colidx, first, t1, aligned, a.w);
+    if ((threadIdx.x & 31) == 0 && first > 0) a.prev = colidx[first - 1];
+  } else {
+#pragma unroll
+    for (int i = 0; i < SP_ITEMS; ++i) a.w[i] = -1;
+  }
+}
+
+// Marks the tile of entries [t0, t1). Block-wide.
 __device__ __forceinline__ void tile_rows_mark(TileRows &tr, const int64_t *__restrict__ rowptr,
-                                               int64_t t0, int64_t t1, int64_t rlo, int64_t rhi) {
+                                               int64_t t0, int64_t t1, const TileAhead &a) {
   __syncthreads();  // the tile before this one has been read
   if (threadIdx.x < 64) tr.start[threadIdx.x] = threadIdx.x == 0 ? 1u : 0u;
   if (threadIdx.x == 0) {
-    tr.row[0] = (int32_t)rlo;  // the row that holds entry t0
-    tr.first_is_start = rowptr[rlo] == t0;
+    tr.row[0] = (int32_t)a.rlo;  // the row that holds entry t0
+    tr.first_is_start = a.start == t0;
   }
   __syncthreads();
-  for (int64_t r = rlo + 1 + threadIdx.x; r <= rhi; r += SP_NT) {
-    const int64_t b = rowptr[r], e = rowptr[r + 1];
+  for (int64_t r = a.rlo + 1 + threadIdx.x; r <= a.rhi; r += SP_NT) {
+    const bool ahead = r == a.rlo + 1 + threadIdx.x;
+    const int64_t b = ahead ? a.begin : rowptr[r], e = ahead ? a.end : rowptr[r + 1];
     if (e > b && b > t0 && b < t1) {  // (row pointers are checked, but only read back later)
       const int x = (int)(b - t0);
       atomicOr(&tr.start[x >> 5], 1u << (x & 31));
@@ -281,13 +330,20 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
                                                      int32_t *__restrict__ err) {
   __shared__ TileRows tr;
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
+  TileAhead next, after;
+  tile_ends(next, tile_rows, blockIdx.x, ntiles);
+  tile_load(next, rowptr, colidx, nnz, blockIdx.x, ntiles, aligned);
+  tile_ends(after, tile_rows, (int64_t)blockIdx.x + gridDim.x, ntiles);
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const TileAhead here = next;
+    next = after;
+    tile_load(next, rowptr, colidx, nnz, tile + gridDim.x, ntiles, aligned);
+    tile_ends(after, tile_rows, tile + 2 * (int64_t)gridDim.x, ntiles);
     const int64_t t0 = tile * SP_TILE;
     const int64_t t1 = t0 + SP_TILE < nnz ? t0 + SP_TILE : nnz;
     const int64_t first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
-    int32_t w[SP_ITEMS];
-    if (first < t1) load_entries(colidx, first, t1, aligned, w);
-    tile_rows_mark(tr, rowptr, t0, t1, tile_rows[tile], tile_rows[tile + 1]);
+    const int32_t(&w)[SP_ITEMS] = here.w;
+    tile_rows_mark(tr, rowptr, t0, t1, here);
     if (first >= t1) continue;
     unsigned marks = 0;
     int32_t u = tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &marks);
@@ -368,28 +424,26 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
   __shared__ TileRows tr;
   const unsigned lane = threadIdx.x & 31u;
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
-  int32_t next[SP_ITEMS];
-  auto load = [&](int64_t tile) {
-    const int64_t t0 = tile * SP_TILE, first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
-    const int64_t t1 = t0 + SP_TILE < nnz ? t0 + SP_TILE : nnz;
-    if (tile < ntiles && first < t1) load_entries(colidx, first, t1, aligned, next);
-  };
-  load(blockIdx.x);
+  TileAhead next, after;
+  tile_ends(next, tile_rows, blockIdx.x, ntiles);
+  tile_load(next, rowptr, colidx, nnz, blockIdx.x, ntiles, aligned);
+  tile_ends(after, tile_rows, (int64_t)blockIdx.x + gridDim.x, ntiles);
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const TileAhead here = next;
+    next = after;
+    tile_load(next, rowptr, colidx, nnz, tile + gridDim.x, ntiles, aligned);
+    tile_ends(after, tile_rows, tile + 2 * (int64_t)gridDim.x, ntiles);
     const int64_t t0 = tile * SP_TILE;
     const int64_t t1 = t0 + SP_TILE < nnz ? t0 + SP_TILE : nnz;
     const int64_t first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
     const bool mine = first < t1;
-    int32_t w[SP_ITEMS];
-#pragma unroll
-    for (int i = 0; i < SP_ITEMS; ++i) w[i] = mine ? next[i] : -1;
-    load(tile + gridDim.x);
-    tile_rows_mark(tr, rowptr, t0, t1, tile_rows[tile], tile_rows[tile + 1]);
+    const int32_t(&w)[SP_ITEMS] = here.w;
+    tile_rows_mark(tr, rowptr, t0, t1, here);
     unsigned marks = 0;
     int32_t u = mine ? tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &marks) : 0;
     if (threadIdx.x == 0 && !tr.first_is_start) marks &= ~1u;  // t0 goes on with its row
     int32_t prev = __shfl_up_sync(0xffffffffu, w[SP_ITEMS - 1], 1);
-    if (lane == 0) prev = first > 0 && mine ? colidx[first - 1] : -1;
+    if (lane == 0) prev = here.prev;
     int gi = 0;
     int64_t gbase = 0, gend = n;
     if (voff && mine) {
@@ -402,111 +456,109 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
       gbase = voff[gi];
       gend = voff[gi + 1];
     }
-    // row[i] >= 0: entry i counts for that row (MODE 0: it is no edge; MODE 1: it is an
-    // upward first copy)
-    int32_t row[SP_ITEMS], val[SP_ITEMS];
-    unsigned bad = 0;
+    // bit i: entry i is a first copy; by then its row's vertex (as a local id) is ul
+    const int32_t size = (int32_t)(gend - gbase);
+    int32_t ul = u - (int32_t)gbase;
+    unsigned heads = 0, valid = 0, bad = 0;
+    int32_t val[SP_ITEMS];
 #pragma unroll
     for (int i = 0; i < SP_ITEMS; ++i) {
-      row[i] = -1;
-      val[i] = -1;
-      if (first + i < t1) {
-        const bool starts = ((marks >> i) & 1u) != 0u;
-        if (i > 0 && starts) u = tr.row[(int)threadIdx.x * SP_ITEMS + i];
-        if (voff && starts) {
+      const bool starts = ((marks >> i) & 1u) != 0u;
+      if (i > 0 && starts) {
+        u = tr.row[(int)threadIdx.x * SP_ITEMS + i];
+        if (voff) {
           while (u >= gend && gi + 1 < ng) {
             ++gi;
             gbase = voff[gi];
             gend = voff[gi + 1];
           }
         }
-        const int32_t vl = w[i];
-        const bool in_range = vl >= 0 && (int64_t)vl < gend - gbase;
-        const int32_t v = in_range ? (int32_t)(vl + gbase) : 0;
-        const bool head = in_range && v != u && (starts || prev != vl);
-        if (MODE == 0) {
-          if (!in_range) bad |= 2u;
-          else if (!starts && prev > vl) bad |= 4u;
-          row[i] = head ? -1 : u;
-        } else {
-          row[i] = u;
-          val[i] = head ? v : -1;
-        }
-        prev = vl;
+        ul = u - (int32_t)gbase;
       }
-    }
-    if (MODE == 0 && bad) atomicOr(err, (int)bad);
-    if (MODE == 1) {
-      // the gathers of the eight ranks are in flight together
-#pragma unroll
-      for (int i = 0; i < SP_ITEMS; ++i)
-        if (val[i] >= 0) val[i] = rank[val[i]];
-      int32_t cur = -1, ru = 0;
-#pragma unroll
-      for (int i = 0; i < SP_ITEMS; ++i) {
-        if (row[i] >= 0 && row[i] != cur) {
-          cur = row[i];
-          ru = rank[cur];
-        }
-        if (val[i] <= ru) row[i] = -1;
+      const int32_t v = w[i];
+      const bool in = first + i < t1;
+      const bool in_range = (uint32_t)v < (uint32_t)(voff ? (int32_t)(gend - gbase) : size);
+      if (MODE == 0 && in) {
+        if (!in_range) bad |= 2u;
+        if (!starts && prev > v) bad |= 4u;
       }
+      const bool head = in && in_range && v != ul && (starts || prev != v);
+      heads |= head ? 1u << i : 0u;
+      valid |= in ? 1u << i : 0u;
+      if (MODE == 1) val[i] = head ? rank[v + (int32_t)gbase] : -1;
+      prev = v;
     }
-    // one addition per thread and row
     if (MODE == 0) {
-      int32_t cur = -1;
-      int cnt = 0;
-#pragma unroll
-      for (int i = 0; i < SP_ITEMS; ++i) {
-        if (row[i] >= 0 && row[i] != cur) {
-          if (cur >= 0) atomicSub(&deg[cur], cnt);
-          cur = row[i];
-          cnt = 0;
-        }
-        if (row[i] >= 0) ++cnt;
-      }
-      if (cur >= 0) atomicSub(&deg[cur], cnt);
-    } else {
-      // a warp inside one long row (a hub's) reserves once for all its lanes
-      int32_t only = -1;
-      unsigned cnt = 0;
-      bool one = true;
-#pragma unroll
-      for (int i = 0; i < SP_ITEMS; ++i)
-        if (row[i] >= 0) {
-          if (only >= 0 && row[i] != only) one = false;
-          only = row[i];
-          ++cnt;
-        }
-      const int32_t only0 = __reduce_max_sync(0xffffffffu, only);
-      if (only0 < 0) continue;  // nothing points up in the warp
-      if (__all_sync(0xffffffffu, one && (only < 0 || only == only0))) {
-        const unsigned incl = warp_inclusive_scan(cnt);
-        unsigned at = 0;
-        if (lane == 31) at = atomicAdd(&dplus[only0], incl);
-        if (!up) continue;
-        at = __shfl_sync(0xffffffffu, at, 31);
-        int64_t pos = (place ? place[rank[only0]] : rowptr[only0]) + (int64_t)(at + incl - cnt);
-#pragma unroll
-        for (int i = 0; i < SP_ITEMS; ++i)
-          if (row[i] >= 0) up[pos++] = val[i];
+      if (bad) atomicOr(err, (int)bad);
+      // a warp inside one long row (a hub's, where most duplicates are) subtracts once
+      const int32_t row0 = mine ? tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &bad) : -1;
+      const int32_t rowx = __shfl_sync(0xffffffffu, row0, 0);
+      if (__all_sync(0xffffffffu, !mine || (row0 == rowx && !(marks & ~1u)))) {
+        const int none = __reduce_add_sync(0xffffffffu, __popc(valid & ~heads));
+        if (lane == 0 && none) atomicSub(&deg[rowx], none);
         continue;
       }
-      int32_t cur = -1;
-      int64_t pos = 0;
+      // entries that are no edge are few: their rows are looked up again
+      for (unsigned left = valid & ~heads; left;) {
+        const int i = __ffs(left) - 1;
+        unsigned unused;
+        const int x = (int)threadIdx.x * SP_ITEMS;
+        const unsigned before = marks & ((2u << i) - 1u);  // starts up to entry i
+        const int32_t r = before && (31 - __clz(before)) > 0
+                              ? tr.row[x + 31 - __clz(before)]
+                              : tile_row_at(tr, x, &unused);
+        // with all others of the same row
+        const unsigned later = marks & ~((2u << i) - 1u);
+        const unsigned seg = later ? (1u << (__ffs(later) - 1)) - 1u : 0xffu;
+        atomicSub(&deg[r], __popc(left & seg));
+        left &= ~seg;
+      }
+      continue;
+    }
+    // MODE 1: bit i: entry i points up (its row's rank: of the row at hand)
+    unsigned ups = 0;
+    int32_t urow = mine ? tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &valid) : 0;
+    int32_t ru = mine ? rank[urow] : 0;
+    const int32_t row0 = urow;
 #pragma unroll
-      for (int i = 0; i < SP_ITEMS; ++i) {
-        if (row[i] >= 0) {
-          if (row[i] != cur) {  // first item of a group: reserve the group's slots
-            cur = row[i];
-            unsigned c = 0;
+    for (int i = 0; i < SP_ITEMS; ++i) {
+      if (i > 0 && ((marks >> i) & 1u)) ru = rank[tr.row[(int)threadIdx.x * SP_ITEMS + i]];
+      if (val[i] > ru) ups |= 1u << i;
+    }
+    const unsigned later0 = marks & ~1u;  // rows that start after the thread's first entry
+    // a warp inside one long row (a hub's) reserves once for all its lanes
+    const int32_t rowx = __shfl_sync(0xffffffffu, row0, 0);
+    if (__all_sync(0xffffffffu, !mine || (row0 == rowx && !later0))) {
+      const unsigned cnt = __popc(ups);
+      const unsigned incl = warp_inclusive_scan(cnt);
+      const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+      if (!total) continue;
+      unsigned at = 0;
+      if (lane == 0) at = atomicAdd(&dplus[rowx], total);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (!up) continue;
+      int64_t pos = (place ? place[rank[rowx]] : rowptr[rowx]) + (int64_t)(at + incl - cnt);
 #pragma unroll
-            for (int j = i; j < SP_ITEMS; ++j) c += row[j] == cur ? 1u : 0u;
-            const unsigned at = atomicAdd(&dplus[cur], c);
-            pos = (place ? place[rank[cur]] : rowptr[cur]) + (int64_t)at;
-          }
-          if (up) up[pos] = val[i];
-          ++pos;
+      for (int i = 0; i < SP_ITEMS; ++i)
+        if ((ups >> i) & 1u) up[pos++] = val[i];
+      continue;
+    }
+    int64_t pos = 0;
+#pragma unroll
+    for (int i = 0; i < SP_ITEMS; ++i) {
+      if (i == 0 || ((marks >> i) & 1u)) {  // a row's first entry here: reserve its slots
+        const unsigned later = marks & ~((2u << i) - 1u);
+        const unsigned seg = ((later ? (1u << (__ffs(later) - 1)) - 1u : 0xffu)) & ~((1u << i) - 1u);
+        const unsigned c = __popc(ups & seg);
+        if (c) {
+          const int32_t r = i == 0 ? row0 : tr.row[(int)threadIdx.x * SP_ITEMS + i];
+          const unsigned at = atomicAdd(&dplus[r], c);
+          pos = (place ? place[rank[r]] : rowptr[r]) + (int64_t)at;
         }
+      }
+      if ((ups >> i) & 1u) {
+        if (up) up[pos] = val[i];
+        ++pos;
       }
     }
   }

@@ -7,12 +7,12 @@ namespace bbtc {
 
 namespace {
 
-constexpr int RS_NT = 256;                 // threads per tile
-constexpr int RS_ITEMS = 16;               // keys per thread
+constexpr int RS_NT = 512;                 // threads per tile (256 threads of 16 keys held
+constexpr int RS_ITEMS = 8;                // 101 registers each: 16 warps per SM)
 constexpr int RS_TILE = RS_NT * RS_ITEMS;  // 4096 keys per tile
 constexpr int RS_WARPS = RS_NT / 32;
 constexpr int RS_BINS = 256;
-constexpr int RS_WARP_SPAN = RS_TILE / RS_WARPS;  // 512 consecutive tile positions per warp
+constexpr int RS_WARP_SPAN = RS_TILE / RS_WARPS;  // consecutive tile positions per warp
 
 // Digit counts of every pass at once (one read of the keys): hist[pass][256].
 __global__ void __launch_bounds__(RS_NT) k_rs_hist(const uint64_t *__restrict__ keys,
@@ -37,12 +37,12 @@ __global__ void __launch_bounds__(RS_NT) k_rs_hist(const uint64_t *__restrict__ 
 }
 
 // The first output position of every digit of every pass (one block per pass).
-__global__ void __launch_bounds__(RS_NT) k_rs_digits(unsigned long long *__restrict__ hist) {
-  __shared__ unsigned long long tmp[RS_NT / 32 + 1];
+__global__ void __launch_bounds__(RS_BINS) k_rs_digits(unsigned long long *__restrict__ hist) {
+  __shared__ unsigned long long tmp[RS_BINS / 32 + 1];
   unsigned long long total;
   unsigned long long *h = hist + (int64_t)blockIdx.x * RS_BINS;
   const unsigned long long c = h[threadIdx.x];
-  h[threadIdx.x] = block_exclusive_scan<unsigned long long, RS_NT>(c, tmp, &total);
+  h[threadIdx.x] = block_exclusive_scan<unsigned long long, RS_BINS>(c, tmp, &total);
 }
 
 // Shared memory layout of a tile's sort (dynamic).
@@ -57,7 +57,7 @@ struct RsSmem {
   uint32_t tile;
 };
 
-// Ranks a tile's keys (thread-owned positions warp * 512 + 32 i + lane) by digit,
+// Ranks a tile's keys (thread-owned positions warp * RS_WARP_SPAN + 32 i + lane) by digit,
 // stably: keys with equal digits in one group of 32 are ranked by lane
 // (match_any), groups in order, warps in order -- the tile's own order.
 // Positions past the end take the largest digit; being last in the tile they
@@ -84,16 +84,19 @@ __device__ __forceinline__ uint32_t rs_rank(RsSmem<HAS_VALS> &sm, const uint64_t
   }
   __syncthreads();
   // per digit: exclusive prefix over warps, and the tile's bucket starts
-  const int d = threadIdx.x;  // RS_NT == RS_BINS
+  const int d = threadIdx.x;  // the first RS_BINS threads
   uint32_t run = 0;
+  if (d < RS_BINS) {
 #pragma unroll
-  for (int w = 0; w < RS_WARPS; ++w) {
-    const uint32_t c = sm.whist[w][d];
-    sm.whist[w][d] = run;
-    run += c;
+    for (int w = 0; w < RS_WARPS; ++w) {
+      const uint32_t c = sm.whist[w][d];
+      sm.whist[w][d] = run;
+      run += c;
+    }
   }
   uint32_t total;
-  sm.bstart[d] = block_exclusive_scan<uint32_t, RS_NT>(run, sm.scan_tmp, &total);
+  const uint32_t start = block_exclusive_scan<uint32_t, RS_NT>(run, sm.scan_tmp, &total);
+  if (d < RS_BINS) sm.bstart[d] = start;
   return run;
 }
 
@@ -109,6 +112,7 @@ __device__ __forceinline__ uint32_t rs_rank(RsSmem<HAS_VALS> &sm, const uint64_t
 // tile's own count) and 2q + 2 (the count up to and with the tile).
 constexpr uint64_t RS_POISON = 0xffull << 56;
 constexpr uint64_t RS_COUNT = (1ull << 56) - 1ull;
+constexpr int RS_BACK = 8;
 constexpr int RS_SPIN_LIMIT = 1 << 22;  // polls of one word (seconds)
 
 template <bool HAS_VALS>
@@ -143,37 +147,52 @@ __global__ void __launch_bounds__(RS_NT) k_rs_pass(
   volatile unsigned long long *st = status + tile * RS_BINS + d;
   uint64_t before = 0;
   bool failed = false;
-  if (tile == 0) {
+  if (d >= RS_BINS) {
+    // no digit
+  } else if (tile == 0) {
     *st = upto | mine;
   } else {
     *st = own | mine;
-    const volatile unsigned long long *p = st - RS_BINS;
+    // RS_BACK tiles are read at a time: the loads' latency, not their number, is what
+    // a walk over the many tiles in flight costs
+    const volatile unsigned long long *p = status + d;
+    int64_t t = tile - 1;  // next tile to add
     int spins = 0;
-    for (;;) {
-      const uint64_t x = *p;
-      const uint64_t code = x & ~RS_COUNT;
-      if (code == upto) {
-        before += x & RS_COUNT;
-        break;
+    for (bool done = false; !done && !failed;) {
+      uint64_t x[RS_BACK];
+#pragma unroll
+      for (int i = 0; i < RS_BACK; ++i) x[i] = t >= i ? p[(t - i) * RS_BINS] : 0ull;
+      int taken = 0;
+#pragma unroll
+      for (int i = 0; i < RS_BACK; ++i) {
+        const uint64_t code = x[i] & ~RS_COUNT;
+        if (!done && !failed && taken == i) {
+          if (code == upto) {
+            before += x[i] & RS_COUNT;
+            done = true;
+          } else if (code == own) {
+            before += x[i] & RS_COUNT;
+            ++taken;
+          } else if (code == RS_POISON) {
+            failed = true;
+          }
+        }
       }
-      if (code == own) {
-        before += x & RS_COUNT;
-        p -= RS_BINS;
-        spins = 0;
-      } else if (code == RS_POISON || ++spins > RS_SPIN_LIMIT) {
-        failed = true;
-        break;
-      }
+      t -= taken;
+      spins = taken ? 0 : spins + 1;
+      if (spins > RS_SPIN_LIMIT) failed = true;
     }
   }
   failed = __syncthreads_or(failed);
   if (failed) {
-    *st = RS_POISON;
+    if (d < RS_BINS) *st = RS_POISON;
     if (threadIdx.x == 0) atomicOr(err, 8);
     return;
   }
-  if (tile > 0) *st = upto | (before + mine);
-  sm.goff[d] = digit_start[d] + before;
+  if (d < RS_BINS) {
+    if (tile > 0) *st = upto | (before + mine);
+    sm.goff[d] = digit_start[d] + before;
+  }
 #pragma unroll
   for (int i = 0; i < RS_ITEMS; ++i) {
     const int pos = warp * RS_WARP_SPAN + i * 32 + (int)lane;
@@ -353,7 +372,7 @@ bbtc_status rs_sort(uint64_t *keys, uint64_t *alt, uint32_t *vals, uint32_t *val
   const int passes = (bit_hi - bit_lo + 7) / 8;
   k_rs_hist<<<grid_for(count, RS_NT * 16, 8), RS_NT, 0, s>>>(keys, count, bit_lo, bit_hi, hist);
   BBTC_LAUNCH_CHECK();
-  k_rs_digits<<<(unsigned)passes, RS_NT, 0, s>>>(hist);
+  k_rs_digits<<<(unsigned)passes, RS_BINS, 0, s>>>(hist);
   BBTC_LAUNCH_CHECK();
   uint64_t *kin = keys, *kout = alt;
   uint32_t *vin = vals, *vout = vals_alt;
