@@ -237,6 +237,13 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
     uint32_t v = 0, vend = base;  // the run at hand: its destination and end
     uint32_t b0 = 0, b1 = 0;      // N(v)
     int32_t vl = -1;              // the lane's own destination (set when a run begins)
+    int32_t run_graph = -1;       // GRAPH: the run's graph, and its hits so far
+    uint32_t run_hits = 0;
+    auto flush_graph = [&]() {
+      const uint32_t sum = __reduce_add_sync(0xffffffffu, run_hits);
+      if (lane == 0 && sum) atomicAdd(&P.graph_count[run_graph], (unsigned long long)sum);
+      run_hits = 0;
+    };
     int staged_mode = ST_NONE, staged_log2h = 0, staged_len = 0;
     const int32_t *staged_list = stage;
     const uint32_t *staged_index = nullptr;
@@ -260,6 +267,12 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
         vend = inptr[v + 1];
         b0 = (uint32_t)rowptr[v];
         b1 = (uint32_t)rowptr[v + 1];
+        if (GRAPH) {
+          // (loaded with the bounds: looked up at each batch's end, it stalled the warp)
+          const int32_t graph = d.gid[v];
+          if (graph != run_graph) flush_graph();
+          run_graph = graph;
+        }
         staged = false;
         if (TASK) {
           const int j = part_of_dev(cuts_s, p, (int32_t)v);
@@ -557,13 +570,11 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
           if ((int)lane == x) field_sum += sum;
         }
       }
-      if (GRAPH && uniform) {
-        const uint32_t s = __reduce_add_sync(0xffffffffu, hits);
-        if (lane == 0 && s) atomicAdd(&P.graph_count[d.gid[v]], (unsigned long long)s);
-      }
+      if (GRAPH && uniform) run_hits += hits;
       __syncwarp();
     }
     if (TASK) flush_fields();
+    if (GRAPH) flush_graph();
     if (failed) break;
     it = __shfl_sync(0xffffffffu, it_next, 0);
   }
@@ -695,7 +706,8 @@ __global__ void __launch_bounds__(FS_NT) k_flat_scatter(const int64_t *__restric
 // a temporary array (records and destinations, coalesced runs), then place
 // them; see plan.cu, which does the same for the per-part records.
 constexpr int FB_T = 4096, FB_NT = 512, FB_B = 512, FB_LUT = 4096;
-constexpr int64_t FB_MIN_EDGES = 16ll << 20;
+// (26 M records of R-MAT scale 21: direct 0.39 ms, two phases 0.62)
+constexpr int64_t FB_MIN_EDGES = 48ll << 20;
 static_assert(FB_NT == FB_B && FB_T == 8 * FB_NT, "partition layout");
 
 __global__ void k_flat_bounds(const uint32_t *__restrict__ inptr, int64_t n,
@@ -860,21 +872,6 @@ __global__ void __launch_bounds__(512) k_flat_count(const int32_t *__restrict__ 
     if (cnt[i]) atomicAdd(&hist[first + i], cnt[i]);
 }
 
-__global__ void k_flat_widen(const unsigned *__restrict__ in, int64_t count,
-                             uint64_t *__restrict__ out) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = in[i];
-}
-__global__ void k_flat_narrow(const uint64_t *__restrict__ in, int64_t count,
-                              uint32_t *__restrict__ inptr, unsigned *__restrict__ cursor) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    inptr[i] = (uint32_t)in[i];
-    cursor[i] = (unsigned)in[i];
-  }
-}
-
 }  // namespace
 
 void free_flat(Flat *f, cudaStream_t s) {
@@ -902,9 +899,7 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
   }
   Scratch scratch(s);
   unsigned *hist = nullptr;
-  uint64_t *scan = nullptr;
   BBTC_TRY(scratch.get(&hist, n + 1));
-  BBTC_TRY(scratch.get(&scan, n + 1));
   BBTC_TRY(dalloc_n(&f.inptr, n + 1, s));
   if (g->deg && g->perm) {
     k_flat_indegree<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(g->rowptr, g->perm, g->deg, n, hist);
@@ -918,11 +913,7 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
                                                              g->colidx, n, hist);
     BBTC_LAUNCH_CHECK();
   }
-  k_flat_widen<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(hist, n + 1, scan);
-  BBTC_LAUNCH_CHECK();
-  BBTC_TRY(exclusive_scan_u64(scan, scan, n + 1, s));
-  k_flat_narrow<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(scan, n + 1, f.inptr, hist);
-  BBTC_LAUNCH_CHECK();
+  BBTC_TRY(exclusive_scan_u32(hist, f.inptr, hist, n + 1, s));  // hist: the cursors
   uint32_t records = 0;
   unsigned items = 0;
   BBTC_CUDA(cudaMemcpyAsync(&records, f.inptr + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));

@@ -177,6 +177,7 @@ __global__ void k_orient_scatter(const uint64_t *__restrict__ okeys,
 // each counted once, so no global sort is needed.
 
 constexpr int SEG_CAP = 2048;  // longest oriented row sorted in shared memory
+constexpr int64_t SYM_ASK_N = 1 << 18;  // vertices from which the largest degree is asked for
 
 __device__ __forceinline__ int64_t row_of_first(const int64_t *rowptr, int64_t n, int64_t target,
                                                 int64_t lo_hint, int64_t hi_hint) {
@@ -538,6 +539,7 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
       at = __shfl_sync(0xffffffffu, at, 0);
       if (!up) continue;
       int64_t pos = (place ? place[rank[rowx]] : rowptr[rowx]) + (int64_t)(at + incl - cnt);
+      if (!place && (uint64_t)pos + cnt > (uint64_t)nnz) continue;  // (see below)
 #pragma unroll
       for (int i = 0; i < SP_ITEMS; ++i)
         if ((ups >> i) & 1u) up[pos++] = val[i];
@@ -557,7 +559,8 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
         }
       }
       if ((ups >> i) & 1u) {
-        if (up) up[pos] = val[i];
+        // (row pointers that decrease are found by the host only after this pass)
+        if (up && (place || (uint64_t)pos < (uint64_t)nnz)) up[pos] = val[i];
         ++pos;
       }
     }
@@ -578,6 +581,17 @@ __global__ void k_rowlen_by_rank(const unsigned *__restrict__ dplus,
   }
   best = __reduce_max_sync(0xffffffffu, best);
   if ((threadIdx.x & 31) == 0 && best > 0) atomicMax(longest, (unsigned long long)best);
+}
+
+// {largest out-degree, edges, largest degree (that of the last position), error bits}
+__global__ void k_sym_stats(const unsigned long long *__restrict__ longest,
+                            const int64_t *__restrict__ rowptr, const int32_t *__restrict__ deg,
+                            const int32_t *__restrict__ perm, int64_t n,
+                            const int32_t *__restrict__ err, int64_t *__restrict__ stats) {
+  stats[0] = (int64_t)*longest;
+  stats[1] = rowptr[n];
+  stats[2] = deg[perm[n - 1]];
+  stats[3] = *err;
 }
 
 // esrc[x] = the row of position x, for every position of the oriented CSR.
@@ -1071,24 +1085,37 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   k_sym_pass<0><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, g->deg,
                                        nullptr, nullptr, nullptr, nullptr, err, g->voff, g->ng);
   BBTC_LAUNCH_CHECK();
-  int32_t *dmax = nullptr;
-  BBTC_TRY(scratch.get(&dmax, 1));
-  BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
-  int32_t hdmax = 0;
-  BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  int32_t herr = 0;
-  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaStreamSynchronize(s));
-  if (herr & 1) {
-    set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
-    return BBTC_EINVAL;
+  int32_t herr = 0, hdmax = 0;
+  // what pass 0 found in the input: BBTC_OK and *sorted, or the error
+  auto check = [&](bool *sorted) -> bbtc_status {
+    if (herr & 1) {
+      set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
+      return BBTC_EINVAL;
+    }
+    if (herr & 2) {
+      set_error("bbtc_graph_create: colidx entry outside [0, n)");
+      return BBTC_EINVAL;
+    }
+    *sorted = (herr & 4) == 0;
+    return BBTC_OK;
+  };
+  bool sorted_rows = true;
+  // The sort of the ranks needs as many bits as the largest degree has. A graph of
+  // many vertices asks the device; for the others sorting the bits of n costs less
+  // than the round trip (about 25 us), and what pass 0 found is read with the sizes.
+  int degree_bits = nb;
+  const bool ask = n > SYM_ASK_N;
+  if (ask) {
+    int32_t *dmax = nullptr;
+    BBTC_TRY(scratch.get(&dmax, 1));
+    BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
+    BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaStreamSynchronize(s));
+    BBTC_TRY(check(&sorted_rows));
+    if (!sorted_rows) return BBTC_OK;  // the general path takes over
+    degree_bits = ceil_log2_u64((uint64_t)hdmax + 1);
   }
-  if (herr & 2) {
-    set_error("bbtc_graph_create: colidx entry outside [0, n)");
-    return BBTC_EINVAL;
-  }
-  if (herr & 4) return BBTC_OK;  // unsorted rows: the general path takes over
-  *applied = true;
 
   // a3: order by (degree, id)
   int32_t *rank = nullptr;
@@ -1098,13 +1125,11 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   BBTC_TRY(scratch.get(&rk_alt, n));
   BBTC_TRY(dalloc_n(&g->perm, n, s));
   g->bytes += (uint64_t)n * sizeof(int32_t);
-  g->deg_max = hdmax;
   k_rank_keys<<<grid_for(n, 256, 16), 256, 0, s>>>(g->deg, n, nb, rk);
   BBTC_LAUNCH_CHECK();
   bool in_alt = false;
   // the keys start in id order and the sort is stable: only the degree bits are sorted
-  BBTC_TRY(radix_sort(rk, rk_alt, nullptr, nullptr, n, nb, nb + ceil_log2_u64((uint64_t)hdmax + 1),
-                      s, err, &in_alt));
+  BBTC_TRY(radix_sort(rk, rk_alt, nullptr, nullptr, n, nb, nb + degree_bits, s, err, &in_alt));
   k_rank_finish<<<grid_for(n, 256, 16), 256, 0, s>>>(in_alt ? rk_alt : rk, n, nb, err, g->perm,
                                                       rank);
   BBTC_LAUNCH_CHECK();
@@ -1143,12 +1168,29 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   BBTC_LAUNCH_CHECK();
   BBTC_TRY(exclusive_scan_u64(reinterpret_cast<uint64_t *>(g->rowptr),
                               reinterpret_cast<uint64_t *>(g->rowptr), n + 1, s));
-  int64_t h[2] = {0, 0};
-  BBTC_CUDA(cudaMemcpyAsync(&h[0], longest, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaMemcpyAsync(&h[1], g->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  int64_t *stats = nullptr;
+  BBTC_TRY(scratch.get(&stats, 4));
+  k_sym_stats<<<1, 1, 0, s>>>(longest, g->rowptr, g->deg, g->perm, n, err, stats);
+  BBTC_LAUNCH_CHECK();
+  int64_t h[4] = {0, 0, 0, 0};
+  BBTC_CUDA(cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
+  herr = (int32_t)h[3];
+  BBTC_TRY(check(&sorted_rows));
   if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
+  if (!sorted_rows) {  // the general path takes over
+    dfree(g->perm, s);
+    dfree(g->rowptr, s);
+    dfree(g->gid, s);
+    g->perm = nullptr;
+    g->rowptr = nullptr;
+    if (g->gid) g->bytes -= (uint64_t)n * sizeof(int32_t);
+    g->gid = nullptr;
+    g->bytes -= (uint64_t)n * sizeof(int32_t) + (uint64_t)(n + 1) * 8;
+    return BBTC_OK;
+  }
+  *applied = true;
+  g->deg_max = h[2];
   g->dplus_max = h[0];
   const int64_t m = h[1];
   if (m > 0xFFFFFFFFLL) {

@@ -331,6 +331,69 @@ __global__ void __launch_bounds__(SC_NT) k_scan_down(const uint64_t *in, uint64_
   }
 }
 
+// 32-bit counts to offsets: the tiles' sums, then the tiles (out and, when given, a
+// copy of it); sums beyond 32 bits wrap, as the offsets' users keep them below.
+__global__ void __launch_bounds__(SC_NT) k_scan32_reduce(const uint32_t *__restrict__ in,
+                                                         int64_t count,
+                                                         uint64_t *__restrict__ partial) {
+  __shared__ uint64_t tmp[SC_NT / 32 + 1];
+  const int64_t base = (int64_t)blockIdx.x * SC_TILE;
+  uint64_t s = 0;
+#pragma unroll
+  for (int i = 0; i < SC_ITEMS; ++i) {
+    const int64_t idx = base + (int64_t)i * SC_NT + threadIdx.x;
+    if (idx < count) s += in[idx];
+  }
+  uint64_t total;
+  block_exclusive_scan<uint64_t, SC_NT>(s, tmp, &total);
+  if (threadIdx.x == 0) partial[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(SC_NT) k_scan32_down(const uint32_t *in, uint32_t *out,
+                                                       uint32_t *copy, int64_t count,
+                                                       const uint64_t *__restrict__ partial,
+                                                       bool sums) {
+  __shared__ uint32_t tile[SC_TILE];
+  __shared__ uint32_t tmp[SC_NT / 32 + 1];
+  __shared__ uint64_t tmp64[SC_NT / 32 + 1];
+  const int64_t base = (int64_t)blockIdx.x * SC_TILE;
+  uint64_t start = 0;
+  if (partial && sums) {
+    uint64_t x = 0;
+    for (int i = threadIdx.x; i < (int)blockIdx.x; i += SC_NT) x += partial[i];
+    block_exclusive_scan<uint64_t, SC_NT>(x, tmp64, &start);
+  } else if (partial) {
+    start = partial[blockIdx.x];
+  }
+#pragma unroll
+  for (int i = 0; i < SC_ITEMS; ++i) {
+    const int64_t idx = base + (int64_t)i * SC_NT + threadIdx.x;
+    tile[i * SC_NT + threadIdx.x] = idx < count ? in[idx] : 0;
+  }
+  __syncthreads();
+  uint32_t local[SC_ITEMS], s = 0, total;
+#pragma unroll
+  for (int i = 0; i < SC_ITEMS; ++i) {
+    local[i] = tile[threadIdx.x * SC_ITEMS + i];
+    s += local[i];
+  }
+  uint32_t run = block_exclusive_scan<uint32_t, SC_NT>(s, tmp, &total) + (uint32_t)start;
+#pragma unroll
+  for (int i = 0; i < SC_ITEMS; ++i) {
+    tile[threadIdx.x * SC_ITEMS + i] = run;
+    run += local[i];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < SC_ITEMS; ++i) {
+    const int64_t idx = base + (int64_t)i * SC_NT + threadIdx.x;
+    if (idx < count) {
+      out[idx] = tile[i * SC_NT + threadIdx.x];
+      if (copy) copy[idx] = tile[i * SC_NT + threadIdx.x];
+    }
+  }
+}
+
 template <typename T>
 __global__ void k_reduce_max(const T *__restrict__ in, int64_t count,
                              unsigned long long *__restrict__ out) {
@@ -421,6 +484,27 @@ bbtc_status exclusive_scan_u64(const uint64_t *in, uint64_t *out, int64_t count,
   const bool sums = nblocks <= SC_DIRECT;
   if (!sums) BBTC_TRY(exclusive_scan_u64(partial, partial, nblocks, s));
   k_scan_down<<<(unsigned)nblocks, SC_NT, 0, s>>>(in, out, count, partial, sums);
+  BBTC_LAUNCH_CHECK();
+  return BBTC_OK;
+}
+
+bbtc_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, uint32_t *copy, int64_t count,
+                               cudaStream_t s) {
+  if (count <= 0) return BBTC_OK;
+  const int64_t nblocks = (count + SC_TILE - 1) / SC_TILE;
+  if (nblocks == 1) {
+    k_scan32_down<<<1, SC_NT, 0, s>>>(in, out, copy, count, nullptr, false);
+    BBTC_LAUNCH_CHECK();
+    return BBTC_OK;
+  }
+  Scratch scratch(s);
+  uint64_t *partial = nullptr;
+  BBTC_TRY(scratch.get(&partial, nblocks));
+  k_scan32_reduce<<<(unsigned)nblocks, SC_NT, 0, s>>>(in, count, partial);
+  BBTC_LAUNCH_CHECK();
+  const bool sums = nblocks <= SC_DIRECT;
+  if (!sums) BBTC_TRY(exclusive_scan_u64(partial, partial, nblocks, s));
+  k_scan32_down<<<(unsigned)nblocks, SC_NT, 0, s>>>(in, out, copy, count, partial, sums);
   BBTC_LAUNCH_CHECK();
   return BBTC_OK;
 }

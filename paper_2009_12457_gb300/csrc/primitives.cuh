@@ -26,6 +26,11 @@ inline bbtc_status sort_failed(const char *where) {
 bbtc_status exclusive_scan_u64(const uint64_t *in, uint64_t *out, int64_t count,
                                cudaStream_t s);
 
+// The same of 32-bit counts whose sum fits 32 bits; copy (nullable) receives the
+// result too, and may alias in.
+bbtc_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, uint32_t *copy, int64_t count,
+                               cudaStream_t s);
+
 // *out (device) = max(in[0..count)) (0 for count == 0).
 bbtc_status reduce_max_i64(const int64_t *in, int64_t count, int64_t *out, cudaStream_t s);
 bbtc_status reduce_max_i32(const int32_t *in, int64_t count, int32_t *out, cudaStream_t s);
