@@ -25,6 +25,82 @@ __global__ void k_validate_rowptr(const int64_t *__restrict__ rowptr, int64_t n,
   if (blockIdx.x == 0 && threadIdx.x == 0 && rowptr[0] != 0) atomicOr(err, 1);
 }
 
+// Distinct edges by hashing instead of sorting: the steps after need the distinct
+// keys in no particular order. A key is stored times an odd factor, a bijection of
+// 64-bit words whose top bits are its slot; EMPTY, all ones, is the image of no key
+// (its preimage is above 2^62).
+constexpr uint64_t HASH_FACTOR = 0xBF58476D1CE4E5B9ull, HASH_INVERSE = 0x96DE1B173F119089ull;
+static_assert(HASH_FACTOR * HASH_INVERSE == 1ull, "inverse of the hash factor");
+static_assert(~0ull * HASH_INVERSE > (1ull << 62), "EMPTY is no key");
+constexpr uint64_t HASH_EMPTY = ~0ull;
+// More keys are sorted instead: preparation by hashing and by sorting took 0.26 and
+// 0.30 ms for 131 K entries (R-MAT scale 13), 0.55 and 0.72 for 4 M, 1.92 and 2.01
+// for 17 M, but 2.68 and 2.46 for 21 M of a G(n, m) without duplicates (2.36 and
+// 2.93 for 34 M with each edge listed twice). Splitting the keys by their top hash
+// bits first cost more than it saved (2.12 ms for the 17 M).
+constexpr int64_t HASH_MAX = 16 << 20;
+constexpr int HI_NT = 256, HI_ITEMS = 8, HI_TILE = HI_NT * HI_ITEMS;
+
+// a1 + a2: inserts the keys into the table of 2^logt slots (at most 2/3 full);
+// the first of equal keys goes to ukeys and counts towards its endpoints'
+// degrees. Lanes that add to one vertex (a hub's edges) add once.
+__global__ void __launch_bounds__(HI_NT) k_hash_unique(const uint64_t *__restrict__ keys,
+                                                       int64_t count, int nb,
+                                                       const int32_t *__restrict__ err, int logt,
+                                                       unsigned long long *__restrict__ table,
+                                                       uint64_t *__restrict__ ukeys,
+                                                       unsigned long long *__restrict__ nunique,
+                                                       int32_t *__restrict__ deg) {
+  __shared__ uint32_t tmp[HI_NT / 32 + 1];
+  __shared__ unsigned long long base_s;
+  if (*err & SORT_FAILED) return;
+  const unsigned lane = threadIdx.x & 31u;
+  const uint64_t mask = (1ull << nb) - 1ull, slots = (1ull << logt) - 1ull;
+  const int64_t ntiles = (count + HI_TILE - 1) / HI_TILE;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    uint64_t k[HI_ITEMS];
+    unsigned long long old[HI_ITEMS];
+    unsigned fresh = 0;
+#pragma unroll
+    for (int i = 0; i < HI_ITEMS; ++i) {
+      const int64_t x = tile * HI_TILE + i * HI_NT + threadIdx.x;
+      k[i] = x < count ? keys[x] : HASH_EMPTY;
+    }
+    // the first probes are in flight together
+#pragma unroll
+    for (int i = 0; i < HI_ITEMS; ++i)
+      old[i] = k[i] != HASH_EMPTY
+                   ? atomicCAS(&table[k[i] >> (64 - logt)], HASH_EMPTY, (unsigned long long)k[i])
+                   : k[i];
+#pragma unroll
+    for (int i = 0; i < HI_ITEMS; ++i) {
+      uint64_t slot = k[i] >> (64 - logt);
+      while (old[i] != HASH_EMPTY && old[i] != k[i]) {  // taken by another key
+        slot = (slot + 1) & slots;
+        old[i] = atomicCAS(&table[slot], HASH_EMPTY, (unsigned long long)k[i]);
+      }
+      if (k[i] != HASH_EMPTY && old[i] == HASH_EMPTY) fresh |= 1u << i;
+    }
+    uint32_t total;
+    uint32_t at = block_exclusive_scan<uint32_t, HI_NT>((uint32_t)__popc(fresh), tmp, &total);
+    if (threadIdx.x == 0) base_s = total ? atomicAdd(nunique, (unsigned long long)total) : 0ull;
+    __syncthreads();
+    const uint64_t base = base_s;
+#pragma unroll
+    for (int i = 0; i < HI_ITEMS; ++i) {
+      const bool is_new = ((fresh >> i) & 1u) != 0u;
+      const uint64_t key = k[i] * HASH_INVERSE;
+      const int32_t a = is_new ? (int32_t)(key >> nb) : -1, b = is_new ? (int32_t)(key & mask) : -1;
+      if (is_new) ukeys[base + at++] = key;
+      unsigned peers = __match_any_sync(0xffffffffu, a);
+      if (a >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[a], __popc(peers));
+      peers = __match_any_sync(0xffffffffu, b);
+      if (b >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[b], __popc(peers));
+    }
+    __syncthreads();  // base_s has been read
+  }
+}
+
 constexpr int UQ_NT = 512;
 constexpr int UQ_ITEMS = 8;
 constexpr int UQ_TILE = UQ_NT * UQ_ITEMS;
@@ -320,11 +396,13 @@ __device__ __forceinline__ void load_entries(const int32_t *__restrict__ colidx,
 
 // a1: one 64-bit key (min << nb) | max per input entry that joins two different
 // vertices; the others (and, for symmetric input, entries with u > v) get the
-// sentinel, which sorts last.
+// sentinel, which sorts last. Keys are multiplied by `factor` (1, or the hash
+// factor below).
 __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__ rowptr,
                                                      const int32_t *__restrict__ colidx, int64_t n,
                                                      int64_t nnz, int nb, bool symmetric,
                                                      bool aligned, uint64_t sentinel,
+                                                     uint64_t factor,
                                                      const int64_t *__restrict__ tile_rows,
                                                      const int64_t *__restrict__ voff, int ng,
                                                      uint64_t *__restrict__ keys,
@@ -378,7 +456,7 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
         if (w[i] < 0 || v >= gend) bad = true;
         else if (v != u && !(symmetric && u > v)) {
           const uint64_t a = (uint64_t)(u < v ? u : v), b = (uint64_t)(u < v ? v : u);
-          key[i] = (a << nb) | b;
+          key[i] = ((a << nb) | b) * factor;
         }
       }
     }
@@ -1298,14 +1376,23 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
     BBTC_LAUNCH_CHECK();
   }
 
-  // ---- a1: canonical keys, sort, unique; a2: degree
+  // ---- a1: canonical keys, the distinct ones; a2: degree
   // (no key equals the all-ones value: it would need min == max)
-  const uint64_t sentinel = (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
   uint64_t *ka = nullptr, *kb = nullptr;
   const int64_t nkeys = nnz;
   const int64_t kcap = nkeys > n ? nkeys : n;  // the buffers also take the n rank keys
   BBTC_TRY(scratch.get(&ka, kcap));
   BBTC_TRY(scratch.get(&kb, kcap));
+  // few keys by hashing (a table of 12 to 24 bytes an entry), many by sorting
+  int logt = 8;
+  while ((2ull << logt) < 3 * (uint64_t)nkeys) ++logt;
+  unsigned long long *table = nullptr;
+  if (nkeys > 0 && nkeys <= HASH_MAX && scratch.get(&table, 1ll << logt) != BBTC_OK) {
+    clear_error();
+    table = nullptr;
+  }
+  const uint64_t sentinel = table ? HASH_EMPTY
+                            : (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
   if (nnz > 0) {
     const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
     int64_t *tile_rows = nullptr;
@@ -1314,22 +1401,31 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
     BBTC_LAUNCH_CHECK();
     k_emit_keys<<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
         d_rowptr, d_colidx, n, nnz, nb, symmetric,
-        (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0, sentinel, tile_rows, g->voff, g->ng, ka,
-        err);
+        (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0, sentinel, table ? HASH_FACTOR : 1ull,
+        tile_rows, g->voff, g->ng, ka, err);
     BBTC_LAUNCH_CHECK();
   }
-  bool in_alt = false;
-  BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
-  uint64_t *sorted = in_alt ? kb : ka;
-  uint64_t *ukeys = in_alt ? ka : kb;
-
   if (!g->deg) {
     BBTC_TRY(dalloc_n(&g->deg, n, s));
     g->bytes += (uint64_t)(n > 0 ? n : 1) * sizeof(int32_t);
   }
   BBTC_CUDA(cudaMemsetAsync(g->deg, 0, sizeof(int32_t) * (size_t)(n > 0 ? n : 1), s));
+  BBTC_CUDA(cudaMemsetAsync(&hstats[0], 0, sizeof(int64_t), s));
+  bool in_alt = false;
   int64_t m = 0;
-  if (nkeys > 0) {
+  if (table) {
+    BBTC_CUDA(cudaMemsetAsync(table, 0xff, sizeof(uint64_t) << logt, s));
+  } else {
+    BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
+  }
+  uint64_t *sorted = in_alt ? kb : ka;
+  uint64_t *ukeys = in_alt ? ka : kb;
+  if (table) {
+    k_hash_unique<<<grid_for(nkeys, HI_TILE, 8), HI_NT, 0, s>>>(
+        sorted, nkeys, nb, err, logt, table, ukeys,
+        reinterpret_cast<unsigned long long *>(&hstats[0]), g->deg);
+    BBTC_LAUNCH_CHECK();
+  } else if (nkeys > 0) {
     const int64_t nblk = (nkeys + UQ_TILE - 1) / UQ_TILE;
     uint64_t *boff = nullptr;
     BBTC_TRY(scratch.get(&boff, nblk + 1));
@@ -1340,8 +1436,6 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
                                                      g->deg);
     BBTC_LAUNCH_CHECK();
     BBTC_CUDA(cudaMemcpyAsync(&hstats[0], &boff[nblk], sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-  } else {
-    BBTC_CUDA(cudaMemsetAsync(&hstats[0], 0, sizeof(int64_t), s));
   }
   int32_t *dmax = nullptr;
   BBTC_TRY(scratch.get(&dmax, 1));

@@ -51,3 +51,29 @@ def test_small_graph_rejects_malformed_input():
                 bb.Graph(3, np.asarray(bad_rp, dtype=np.int64), np.asarray(bad_ci, dtype=np.int32),
                          symmetric=symmetric)
             assert e.value.status == 1
+
+
+@pytest.mark.parametrize("n,pairs", [(1025, 40_000), (5000, 3), (70_000, 300_000)])
+def test_general_input_with_duplicates(n, pairs):
+    # beyond one CTA: distinct edges by hashing; every entry listed up to four times
+    _, src, dst = graphgen.gnm_pairs(n, pairs, 3 * n + pairs)
+    src, dst = np.concatenate([src, dst, src]), np.concatenate([dst, src, dst])
+    graph = one_sided(n, src, dst)
+    ref = oracle.bbtc(*graphgen.pairs_to_csr(n, src, dst), p=1)
+    with bb.Graph(*graph) as g:
+        o = g.oriented()
+        assert np.array_equal(o["rowptr"], ref["rowptr"])
+        assert np.array_equal(o["colidx"], ref["colidx"])
+        assert np.array_equal(o["perm"], ref["perm"])
+        assert g.count() == ref["total"]
+
+
+def test_a_vertex_joined_to_all_others():
+    # every key shares one endpoint, and every degree addition one counter
+    n = 200_000
+    rp = np.zeros(n + 1, dtype=np.int64)
+    rp[1:] = n - 1
+    with bb.Graph(n, rp, np.arange(1, n, dtype=np.int32)) as g:
+        i = g.info()
+        assert i["m"] == n - 1 and i["deg_max"] == n - 1 and i["dplus_max"] == 1
+        assert g.count() == 0
