@@ -27,77 +27,106 @@ __global__ void k_validate_rowptr(const int64_t *__restrict__ rowptr, int64_t n,
 
 // Distinct edges by hashing instead of sorting: the steps after need the distinct
 // keys in no particular order. A key is stored times an odd factor, a bijection of
-// 64-bit words whose top bits are its slot; EMPTY, all ones, is the image of no key
-// (its preimage is above 2^62).
+// 64-bit words: its top bits choose one of 2^lb buckets of at most BK_CAP keys (half
+// to three quarters full on average), the next ones its slot in a table in shared
+// memory. EMPTY, all ones, is the image of no key (its preimage is above 2^62). A
+// bucket overflows only when an edge is listed some hundred times or the keys were
+// chosen to collide (random keys spread by 40 around 1,536; paths, grids, bands,
+// stars and bipartite graphs less); the keys are then sorted. What bounds it is the
+// random additions: one to a bucket's cursor and two to degrees per key. Preparation
+// by hashing and by sorting took 0.26 and 0.30 ms for 131 K entries (R-MAT scale
+// 13), 0.54 and 0.72 for 4 M, 1.38 and 2.02 for 17 M, 1.69 and 2.47 for 21 M of a
+// G(n, m), 13.9 and 17.8 for 134 M (one table in device memory instead of buckets:
+// 1.92 for the 17 M); for an edge listed 4 M times, which overflows, 0.72 and 0.55.
 constexpr uint64_t HASH_FACTOR = 0xBF58476D1CE4E5B9ull, HASH_INVERSE = 0x96DE1B173F119089ull;
 static_assert(HASH_FACTOR * HASH_INVERSE == 1ull, "inverse of the hash factor");
 static_assert(~0ull * HASH_INVERSE > (1ull << 62), "EMPTY is no key");
 constexpr uint64_t HASH_EMPTY = ~0ull;
-// More keys are sorted instead: preparation by hashing and by sorting took 0.26 and
-// 0.30 ms for 131 K entries (R-MAT scale 13), 0.55 and 0.72 for 4 M, 1.92 and 2.01
-// for 17 M, but 2.68 and 2.46 for 21 M of a G(n, m) without duplicates (2.36 and
-// 2.93 for 34 M with each edge listed twice). Splitting the keys by their top hash
-// bits first cost more than it saved (2.12 ms for the 17 M).
-constexpr int64_t HASH_MAX = 16 << 20;
-constexpr int HI_NT = 256, HI_ITEMS = 8, HI_TILE = HI_NT * HI_ITEMS;
+constexpr unsigned long long HASH_FAILED = 1ull << 62;
+constexpr int64_t HASH_MAX = 1ll << 28;  // entries (buckets of 2.7 GB to 4.3 GB); more are sorted
+// cursors lie a sector apart: side by side, 1 M keys (1,024 buckets) took 0.387 ms
+// instead of 0.336 (one sector takes one addition at a time)
+constexpr int BK_PAD = 8;
+constexpr int BK_NT = 256, BK_ITEMS = 8, BK_CAP = BK_NT * BK_ITEMS, BK_MEAN = BK_CAP * 3 / 4;
+static_assert((BK_CAP & (BK_CAP - 1)) == 0, "the table holds any bucket twice over");
 
-// a1 + a2: inserts the keys into the table of 2^logt slots (at most 2/3 full);
-// the first of equal keys goes to ukeys and counts towards its endpoints'
-// degrees. Lanes that add to one vertex (a hub's edges) add once.
-__global__ void __launch_bounds__(HI_NT) k_hash_unique(const uint64_t *__restrict__ keys,
-                                                       int64_t count, int nb,
-                                                       const int32_t *__restrict__ err, int logt,
-                                                       unsigned long long *__restrict__ table,
-                                                       uint64_t *__restrict__ ukeys,
-                                                       unsigned long long *__restrict__ nunique,
-                                                       int32_t *__restrict__ deg) {
-  __shared__ uint32_t tmp[HI_NT / 32 + 1];
+// a1 + a2: one CTA per bucket inserts its keys into a table of at least twice their
+// number; the first of equal keys goes to ukeys and counts towards its endpoints'
+// degrees, lanes that add to one vertex (a hub's edges) adding once. *nunique gets
+// HASH_FAILED when a bucket has overflowed; the results are then void.
+__global__ void __launch_bounds__(BK_NT) k_bucket_unique(const uint64_t *__restrict__ keys,
+                                                         const unsigned *__restrict__ fill,
+                                                         int lb, int nb,
+                                                         uint64_t *__restrict__ ukeys,
+                                                         unsigned long long *__restrict__ nunique,
+                                                         int32_t *__restrict__ deg) {
+  __shared__ unsigned long long table[2 * BK_CAP];
+  __shared__ unsigned fresh_of[BK_NT / 32];
   __shared__ unsigned long long base_s;
-  if (*err & SORT_FAILED) return;
-  const unsigned lane = threadIdx.x & 31u;
-  const uint64_t mask = (1ull << nb) - 1ull, slots = (1ull << logt) - 1ull;
-  const int64_t ntiles = (count + HI_TILE - 1) / HI_TILE;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    uint64_t k[HI_ITEMS];
-    unsigned long long old[HI_ITEMS];
-    unsigned fresh = 0;
+  const unsigned count = fill[blockIdx.x * BK_PAD];
+  if (count == 0 || count > BK_CAP) {
+    if (count && threadIdx.x == 0) atomicOr(nunique, HASH_FAILED);
+    return;
+  }
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const int ls = 32 - __clz((int)(2 * count - 1));  // 2 * count <= 2^ls <= 2 * BK_CAP
+  const unsigned slots = 1u << ls;
+  uint64_t k[BK_ITEMS];
 #pragma unroll
-    for (int i = 0; i < HI_ITEMS; ++i) {
-      const int64_t x = tile * HI_TILE + i * HI_NT + threadIdx.x;
-      k[i] = x < count ? keys[x] : HASH_EMPTY;
-    }
-    // the first probes are in flight together
+  for (int i = 0; i < BK_ITEMS; ++i) {
+    const unsigned x = (unsigned)(i * BK_NT) + threadIdx.x;
+    k[i] = x < count ? keys[(int64_t)blockIdx.x * BK_CAP + x] : HASH_EMPTY;
+  }
+  for (unsigned x = threadIdx.x; x < slots; x += BK_NT) table[x] = HASH_EMPTY;
+  __syncthreads();
+  unsigned fresh[BK_ITEMS], mine = 0;
 #pragma unroll
-    for (int i = 0; i < HI_ITEMS; ++i)
-      old[i] = k[i] != HASH_EMPTY
-                   ? atomicCAS(&table[k[i] >> (64 - logt)], HASH_EMPTY, (unsigned long long)k[i])
-                   : k[i];
-#pragma unroll
-    for (int i = 0; i < HI_ITEMS; ++i) {
-      uint64_t slot = k[i] >> (64 - logt);
-      while (old[i] != HASH_EMPTY && old[i] != k[i]) {  // taken by another key
-        slot = (slot + 1) & slots;
-        old[i] = atomicCAS(&table[slot], HASH_EMPTY, (unsigned long long)k[i]);
+  for (int i = 0; i < BK_ITEMS; ++i) {
+    bool is_new = false;
+    if (k[i] != HASH_EMPTY) {
+      unsigned slot = (unsigned)((k[i] << lb) >> (64 - ls));
+      for (;;) {  // the table is at most half full: a free slot is found
+        unsigned long long old = *(volatile unsigned long long *)&table[slot];
+        if (old == HASH_EMPTY) {
+          old = atomicCAS(&table[slot], HASH_EMPTY, (unsigned long long)k[i]);
+          if (old == HASH_EMPTY) {
+            is_new = true;
+            break;
+          }
+        }
+        if (old == k[i]) break;
+        slot = (slot + 1) & (slots - 1);
       }
-      if (k[i] != HASH_EMPTY && old[i] == HASH_EMPTY) fresh |= 1u << i;
     }
-    uint32_t total;
-    uint32_t at = block_exclusive_scan<uint32_t, HI_NT>((uint32_t)__popc(fresh), tmp, &total);
-    if (threadIdx.x == 0) base_s = total ? atomicAdd(nunique, (unsigned long long)total) : 0ull;
-    __syncthreads();
-    const uint64_t base = base_s;
+    fresh[i] = __ballot_sync(0xffffffffu, is_new);
+    mine += __popc(fresh[i]);
+  }
+  if (lane == 0) fresh_of[warp] = mine;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned total = 0;
+    for (int x = 0; x < BK_NT / 32; ++x) {
+      const unsigned c = fresh_of[x];
+      fresh_of[x] = total;
+      total += c;
+    }
+    base_s = atomicAdd(nunique, (unsigned long long)total) & (HASH_FAILED - 1);
+  }
+  __syncthreads();
+  int64_t at = (int64_t)base_s + fresh_of[warp];
+  const uint64_t mask = (1ull << nb) - 1ull;
 #pragma unroll
-    for (int i = 0; i < HI_ITEMS; ++i) {
-      const bool is_new = ((fresh >> i) & 1u) != 0u;
-      const uint64_t key = k[i] * HASH_INVERSE;
-      const int32_t a = is_new ? (int32_t)(key >> nb) : -1, b = is_new ? (int32_t)(key & mask) : -1;
-      if (is_new) ukeys[base + at++] = key;
-      unsigned peers = __match_any_sync(0xffffffffu, a);
-      if (a >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[a], __popc(peers));
-      peers = __match_any_sync(0xffffffffu, b);
-      if (b >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[b], __popc(peers));
-    }
-    __syncthreads();  // base_s has been read
+  for (int i = 0; i < BK_ITEMS; ++i) {
+    if (!fresh[i]) continue;
+    const bool is_new = ((fresh[i] >> lane) & 1u) != 0u;
+    const uint64_t key = k[i] * HASH_INVERSE;
+    const int32_t a = is_new ? (int32_t)(key >> nb) : -1, b = is_new ? (int32_t)(key & mask) : -1;
+    if (is_new) ukeys[at + __popc(fresh[i] & ((1u << lane) - 1u))] = key;
+    at += __popc(fresh[i]);
+    unsigned peers = __match_any_sync(0xffffffffu, a);
+    if (a >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[a], __popc(peers));
+    peers = __match_any_sync(0xffffffffu, b);
+    if (b >= 0 && lane == (unsigned)(__ffs(peers) - 1)) atomicAdd(&deg[b], __popc(peers));
   }
 }
 
@@ -396,13 +425,15 @@ __device__ __forceinline__ void load_entries(const int32_t *__restrict__ colidx,
 
 // a1: one 64-bit key (min << nb) | max per input entry that joins two different
 // vertices; the others (and, for symmetric input, entries with u > v) get the
-// sentinel, which sorts last. Keys are multiplied by `factor` (1, or the hash
-// factor below).
+// sentinel, which sorts last. With BUCKETS, keys times the hash factor go to their
+// buckets (see above), whose cursors are `fill`, and the others nowhere.
+template <bool BUCKETS>
 __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__ rowptr,
                                                      const int32_t *__restrict__ colidx, int64_t n,
                                                      int64_t nnz, int nb, bool symmetric,
                                                      bool aligned, uint64_t sentinel,
-                                                     uint64_t factor,
+                                                     int lb, unsigned *__restrict__ fill,
+                                                     unsigned long long *__restrict__ nunique,
                                                      const int64_t *__restrict__ tile_rows,
                                                      const int64_t *__restrict__ voff, int ng,
                                                      uint64_t *__restrict__ keys,
@@ -424,6 +455,9 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
     const int32_t(&w)[SP_ITEMS] = here.w;
     tile_rows_mark(tr, rowptr, t0, t1, here);
     if (first >= t1) continue;
+    // (a bucket has overflowed: only the checks go on)
+    const bool given_up =
+        BUCKETS && (*reinterpret_cast<volatile unsigned long long *>(nunique) & HASH_FAILED) != 0;
     unsigned marks = 0;
     int32_t u = tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &marks);
     int gi = 0;
@@ -456,11 +490,27 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
         if (w[i] < 0 || v >= gend) bad = true;
         else if (v != u && !(symmetric && u > v)) {
           const uint64_t a = (uint64_t)(u < v ? u : v), b = (uint64_t)(u < v ? v : u);
-          key[i] = ((a << nb) | b) * factor;
+          key[i] = ((a << nb) | b) * (BUCKETS ? HASH_FACTOR : 1ull);
         }
       }
     }
     if (bad) atomicOr(err, 2);
+    if (BUCKETS) {
+      if (given_up) continue;
+#pragma unroll
+      for (int i = SP_ITEMS - 1; i > 0; --i)  // copies side by side are dropped here
+        if (key[i] == key[i - 1]) key[i] = sentinel;
+      unsigned pos[SP_ITEMS];
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i)
+        pos[i] = key[i] != sentinel ? atomicAdd(&fill[(key[i] >> (64 - lb)) * BK_PAD], 1u) : ~0u;
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i) {
+        if (pos[i] < (unsigned)BK_CAP) keys[(key[i] >> (64 - lb)) * BK_CAP + pos[i]] = key[i];
+        else if (pos[i] == (unsigned)BK_CAP) atomicOr(nunique, HASH_FAILED);
+      }
+      continue;
+    }
     if (first + SP_ITEMS <= t1) {  // keys + first is 64-byte aligned
       ulonglong2 *d = reinterpret_cast<ulonglong2 *>(keys + first);
 #pragma unroll
@@ -1379,83 +1429,94 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
   // ---- a1: canonical keys, the distinct ones; a2: degree
   // (no key equals the all-ones value: it would need min == max)
   uint64_t *ka = nullptr, *kb = nullptr;
+  unsigned *fill = nullptr;  // set: by hashing
   const int64_t nkeys = nnz;
   const int64_t kcap = nkeys > n ? nkeys : n;  // the buffers also take the n rank keys
-  BBTC_TRY(scratch.get(&ka, kcap));
   BBTC_TRY(scratch.get(&kb, kcap));
-  // few keys by hashing (a table of 12 to 24 bytes an entry), many by sorting
-  int logt = 8;
-  while ((2ull << logt) < 3 * (uint64_t)nkeys) ++logt;
-  unsigned long long *table = nullptr;
-  if (nkeys > 0 && nkeys <= HASH_MAX && scratch.get(&table, 1ll << logt) != BBTC_OK) {
-    clear_error();
-    table = nullptr;
+  int lb = 1;
+  while ((nkeys >> lb) > BK_MEAN) ++lb;
+  if (nkeys > 0 && nkeys <= HASH_MAX) {
+    const int64_t cap = (int64_t)BK_CAP << lb;
+    if (scratch.get(&fill, (int64_t)BK_PAD << lb) != BBTC_OK ||
+        scratch.get(&ka, cap > kcap ? cap : kcap) != BBTC_OK) {
+      clear_error();
+      fill = nullptr;
+      ka = nullptr;
+    }
   }
-  const uint64_t sentinel = table ? HASH_EMPTY
-                            : (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
+  if (!ka) BBTC_TRY(scratch.get(&ka, kcap));
+  const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
+  int64_t *tile_rows = nullptr;
   if (nnz > 0) {
-    const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
-    int64_t *tile_rows = nullptr;
     BBTC_TRY(scratch.get(&tile_rows, ntiles + 1));
     k_tile_rows<<<grid_for(ntiles + 1, 256, 16), 256, 0, s>>>(d_rowptr, n, nnz, ntiles, tile_rows);
-    BBTC_LAUNCH_CHECK();
-    k_emit_keys<<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
-        d_rowptr, d_colidx, n, nnz, nb, symmetric,
-        (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0, sentinel, table ? HASH_FACTOR : 1ull,
-        tile_rows, g->voff, g->ng, ka, err);
     BBTC_LAUNCH_CHECK();
   }
   if (!g->deg) {
     BBTC_TRY(dalloc_n(&g->deg, n, s));
     g->bytes += (uint64_t)(n > 0 ? n : 1) * sizeof(int32_t);
   }
-  BBTC_CUDA(cudaMemsetAsync(g->deg, 0, sizeof(int32_t) * (size_t)(n > 0 ? n : 1), s));
-  BBTC_CUDA(cudaMemsetAsync(&hstats[0], 0, sizeof(int64_t), s));
-  bool in_alt = false;
-  int64_t m = 0;
-  if (table) {
-    BBTC_CUDA(cudaMemsetAsync(table, 0xff, sizeof(uint64_t) << logt, s));
-  } else {
-    BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
-  }
-  uint64_t *sorted = in_alt ? kb : ka;
-  uint64_t *ukeys = in_alt ? ka : kb;
-  if (table) {
-    k_hash_unique<<<grid_for(nkeys, HI_TILE, 8), HI_NT, 0, s>>>(
-        sorted, nkeys, nb, err, logt, table, ukeys,
-        reinterpret_cast<unsigned long long *>(&hstats[0]), g->deg);
-    BBTC_LAUNCH_CHECK();
-  } else if (nkeys > 0) {
-    const int64_t nblk = (nkeys + UQ_TILE - 1) / UQ_TILE;
-    uint64_t *boff = nullptr;
-    BBTC_TRY(scratch.get(&boff, nblk + 1));
-    k_unique_count<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff);
-    BBTC_LAUNCH_CHECK();
-    BBTC_TRY(exclusive_scan_u64(boff, boff, nblk + 1, s));  // boff[nblk] = total
-    k_unique_write<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff, nb, ukeys,
-                                                     g->deg);
-    BBTC_LAUNCH_CHECK();
-    BBTC_CUDA(cudaMemcpyAsync(&hstats[0], &boff[nblk], sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-  }
   int32_t *dmax = nullptr;
   BBTC_TRY(scratch.get(&dmax, 1));
-  BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
+  uint64_t *sorted = nullptr, *ukeys = nullptr;
+  unsigned long long *nunique = reinterpret_cast<unsigned long long *>(&hstats[0]);
+  bool in_alt = false;
   int64_t stats[2] = {0, 0};
   int32_t hdmax = 0, herr = 0;
-  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaMemcpyAsync(&stats[0], &hstats[0], sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaStreamSynchronize(s));
-  if (herr & 1) {
-    set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
-    return BBTC_EINVAL;
+  for (;;) {  // once, or again by sorting when a bucket overflows
+    BBTC_CUDA(cudaMemsetAsync(g->deg, 0, sizeof(int32_t) * (size_t)(n > 0 ? n : 1), s));
+    BBTC_CUDA(cudaMemsetAsync(nunique, 0, sizeof(*nunique), s));
+    const bool aligned = (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0;
+    if (fill) {
+      BBTC_CUDA(cudaMemsetAsync(fill, 0, (sizeof(unsigned) * BK_PAD) << lb, s));
+      k_emit_keys<true><<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
+          d_rowptr, d_colidx, n, nnz, nb, symmetric, aligned, HASH_EMPTY, lb, fill, nunique,
+          tile_rows, g->voff, g->ng, ka, err);
+      BBTC_LAUNCH_CHECK();
+      k_bucket_unique<<<1u << lb, BK_NT, 0, s>>>(ka, fill, lb, nb, kb, nunique, g->deg);
+      BBTC_LAUNCH_CHECK();
+    } else if (nkeys > 0) {
+      const uint64_t sentinel = (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
+      k_emit_keys<false><<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
+          d_rowptr, d_colidx, n, nnz, nb, symmetric, aligned, sentinel, 0, nullptr, nullptr,
+          tile_rows, g->voff, g->ng, ka, err);
+      BBTC_LAUNCH_CHECK();
+      BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
+    }
+    sorted = in_alt ? kb : ka;
+    ukeys = in_alt ? ka : kb;
+    if (!fill && nkeys > 0) {
+      const int64_t nblk = (nkeys + UQ_TILE - 1) / UQ_TILE;
+      const uint64_t sentinel = (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
+      uint64_t *boff = nullptr;
+      BBTC_TRY(scratch.get(&boff, nblk + 1));
+      k_unique_count<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff);
+      BBTC_LAUNCH_CHECK();
+      BBTC_TRY(exclusive_scan_u64(boff, boff, nblk + 1, s));  // boff[nblk] = total
+      k_unique_write<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff, nb,
+                                                       ukeys, g->deg);
+      BBTC_LAUNCH_CHECK();
+      BBTC_CUDA(
+          cudaMemcpyAsync(nunique, &boff[nblk], sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    }
+    BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
+    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaMemcpyAsync(&stats[0], nunique, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaStreamSynchronize(s));
+    if (herr & 1) {
+      set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
+      return BBTC_EINVAL;
+    }
+    if (herr & 2) {
+      set_error("bbtc_graph_create: colidx entry outside [0, n)");
+      return BBTC_EINVAL;
+    }
+    if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
+    if (!((unsigned long long)stats[0] & HASH_FAILED)) break;
+    fill = nullptr;
   }
-  if (herr & 2) {
-    set_error("bbtc_graph_create: colidx entry outside [0, n)");
-    return BBTC_EINVAL;
-  }
-  if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
-  m = stats[0];
+  const int64_t m = stats[0];
   if (m > 0xFFFFFFFFLL) {
     set_error("bbtc_graph_create: %lld simple edges exceed 2^32 - 1", (long long)m);
     return BBTC_EINVAL;

@@ -77,3 +77,18 @@ def test_a_vertex_joined_to_all_others():
         i = g.info()
         assert i["m"] == n - 1 and i["deg_max"] == n - 1 and i["dplus_max"] == 1
         assert g.count() == 0
+
+
+def test_an_edge_listed_too_often_for_its_bucket():
+    # its copies share one bucket of 2,048: the keys are sorted instead
+    n = 3000
+    _, src, dst = graphgen.gnm_pairs(n, 20_000, 77)
+    src = np.concatenate([src, np.full(100_000, src[0])])
+    dst = np.concatenate([dst, np.full(100_000, dst[0])])
+    graph = one_sided(n, src, dst)
+    ref = oracle.bbtc(*graphgen.pairs_to_csr(n, src, dst), p=1)
+    with bb.Graph(*graph) as g:
+        o = g.oriented()
+        assert np.array_equal(o["rowptr"], ref["rowptr"])
+        assert np.array_equal(o["colidx"], ref["colidx"])
+        assert g.count() == ref["total"]
