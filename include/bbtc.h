@@ -51,10 +51,12 @@ typedef enum {
 typedef enum {
   BBTC_KERNEL_AUTO = 0,      /* choose per staged list N(G_jk, v): bitmap when its value
                                 range fits on chip, else hash table or sorted search by
-                                its length (hash_threshold) */
+                                its length (hash_threshold); edges between the hubs at
+                                the top of the degree order by whole bitmap rows */
   BBTC_KERNEL_INTERSECT = 1, /* bbTC-Intersect (Alg. 5): sorted-list search */
   BBTC_KERNEL_HASHMAP = 2    /* bbTC-HMap (Alg. 6): direct-address bitmap over the list's
-                                value range when it fits on chip, else hash table */
+                                value range when it fits on chip, else hash table; hubs
+                                by bitmap rows as in AUTO */
 } bbtc_kernel;
 
 /* Symmetric partition of the degree order into p parts (Sec. 2 V^p, Sec. 4.1). */
@@ -82,10 +84,11 @@ typedef struct {
   uint32_t timeout_ms;          /* 0 = no limit on the counting kernel's bounded waits */
   uint64_t device_budget_bytes; /* 0 = blocks resident; else the counting step keeps at most
                                    this many bytes of blocks on the device, streaming them
-                                   from pinned host memory (the plan's block arrays move
-                                   there; their pinned buffers are kept for reuse by later
-                                   streamed plans, up to 64 GiB, until the process exits);
-                                   preparation itself still uses device memory */
+                                   from pinned host memory (the plan's in-edge records move
+                                   there, and with task_mask or per_task_cycles_out its
+                                   block arrays too; the pinned buffers are kept for reuse
+                                   by later streamed plans, up to 64 GiB, until the process
+                                   exits); preparation itself still uses device memory */
   uint64_t *per_vertex_out;     /* NULL, or n uint64 (ORIGINAL ids): triangles at each vertex */
   uint64_t *per_task_out;       /* NULL, or bbtc_num_tasks(p) uint64 in Alg. 4 order */
   void *stream;                 /* cudaStream_t to run on; NULL = the handle's own stream */
@@ -96,7 +99,8 @@ typedef struct {
                                    at most 2^28 */
   uint64_t *per_graph_out;      /* NULL, or one uint64 per graph of a batch handle
                                    (bbtc_graph_create_batch / bbtc_count_batch) */
-  int32_t chunk;                /* in-edges per work item of the counting kernel; 0 = auto */
+  int32_t chunk;                /* in-edges per work item of the counting kernels that walk
+                                   in-edges; 0 = auto */
   int32_t partition;            /* bbtc_partition; part of the plan's identity like p */
   uint64_t *per_task_cycles_out; /* NULL, or bbtc_num_tasks(p) uint64 in Alg. 4 order: SM
                                     clock cycles the counting kernel's warps spent on each
@@ -178,9 +182,13 @@ bbtc_status bbtc_graph_create_batch(int32_t ng, const int64_t *vertex_offsets,
  * Count the triangles of the handle's graph with bbTC at p x p blocks:
  * contiguous symmetric partition of the degree order (opts->partition:
  * balanced on oriented edges, or probe-based to bound the largest block),
- * tasks (i,j,k), i <= j <= k (Alg. 4), ordered by the Sec. 5 estimate
- * and drained by a persistent work-stealing kernel, each task counted as
+ * tasks (i,j,k), i <= j <= k (Alg. 4), each task's count being the
  * sum over (u,v) in G_ij of |N(G_ik,u) ∩ N(G_jk,v)| (Alg. 5 / Alg. 6).
+ * A triangle u < v < w belongs to the task of its vertices' parts in whatever
+ * order it is found, so the in-edges are walked once for all tasks by
+ * persistent work-stealing kernels, and hits are attributed to tasks when
+ * per_task_out asks for them. With task_mask or per_task_cycles_out the tasks
+ * are drained one by one in the order of the Sec. 5 estimate.
  *
  *   count  receives the exact total (host uint64)
  *   opts   NULL = defaults; see bbtc_opts for the optional outputs
@@ -203,13 +211,13 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts, uint64_t *count);
 bbtc_status bbtc_graph_plan(bbtc_graph_t g, const bbtc_opts *opts);
 
 /*
- * Count ng independent handles in one persistent launch (Sec. 4.2 tasks of
- * all of them drained together).
+ * Count ng independent handles together: the work items of all of them are
+ * drained by the same few persistent launches (Sec. 4.2: independent tasks).
  *
  * Resident (device_budget_bytes = 0): each handle keeps its own plan for
  * (p, kernel, hash_threshold, chunk, partition) -- built first, on the handle, when it
- * does not match -- and one counting launch takes the work items of all the
- * handles, largest handles first. p = 0 picks p per handle from its size.
+ * does not match -- and one launch of each counting kernel takes the work items
+ * of all the handles. p = 0 picks p per handle from its size.
  * Handles that already hold a matching resident plan are only read, so
  * concurrent calls on other streams may share them.
  * Under a device budget: the handles' oriented CSRs are gathered into one
@@ -238,7 +246,7 @@ bbtc_status bbtc_count_batch(const bbtc_graph_t *gs, int32_t ng, const bbtc_opts
  * manager (a framework's caching allocator) owns the free device memory, and
  * hooks invoked from inside an allocator, where cudaMalloc would re-enter it.
  *
- * It runs the same counting kernel as bbtc_count on the plan that an earlier
+ * It runs the same counting kernels as bbtc_count on the plan that an earlier
  * bbtc_count or bbtc_graph_get_plan call built for the same p on this handle.
  * Its scratch (work-stealing counter, status, per-task accumulators) is a
  * fixed 8 KiB device array inside the library, which every GPU that loads the
@@ -312,9 +320,9 @@ bbtc_status bbtc_graph_get_info(bbtc_graph_t g, bbtc_graph_info *info);
 typedef struct {
   double prep_ms;      /* bbtc_graph_create: a1-a4 (after any host-to-device copy) */
   double plan_ms;      /* last bbtc_count: a5-a8 (0 when the plan was reused) */
-  double count_ms;     /* last bbtc_count: the counting kernel (a9); with a device
+  double count_ms;     /* last bbtc_count: the counting kernels (a9); with a device
                           budget, the whole streamed count (copies included) */
-  int64_t work_items;  /* work items drained by that kernel */
+  int64_t work_items;  /* work items of the in-edges drained by those kernels */
   int64_t stream_rounds;      /* last budgeted count: rounds of block copies */
   uint64_t stream_h2d_bytes;  /* last budgeted count: block bytes copied to the device */
   double stream_copy_ms;      /* last budgeted count: device time of those copies */
@@ -326,9 +334,11 @@ typedef struct {
                                         plus the block pool of at most the budget); the
                                         library's idle cached blocks are released before
                                         a budgeted count */
-  int32_t stream_mode;        /* last budgeted count: 1 = every block CSR kept on the device
-                                 and each in-edge block copied once; 2 = blocks placed round
-                                 by round in the pool and re-copied when evicted */
+  int32_t stream_mode;        /* last budgeted count: 1 = each in-edge copied once, the lists
+                                 read on the device (in the handle's oriented CSR; with
+                                 task_mask or per_task_cycles_out in block CSRs copied to
+                                 the pool once); 2 = blocks placed round by round in the
+                                 pool and re-copied when evicted */
 } bbtc_timings;
 
 bbtc_status bbtc_graph_get_timings(bbtc_graph_t g, bbtc_timings *t);

@@ -11,8 +11,10 @@
 // the columns above v contribute: exactly Alg. 5's |N(u) ∩ N(v)|). A word
 // covers 32 columns, where a probe of a list covers one entry, so the bitmap
 // form is cheaper as soon as a row holds more than a few entries per group of
-// 32 columns; sources below that ("CORE_MIN_ROW" core neighbours) stay with
-// the lists (count.cu skips the edges that are counted here).
+// 32 columns; sources below that (CORE_MIN_ROW core neighbours) stay with the
+// lists (the flat in-edges leave out the edges that are counted here). Of R-MAT
+// scale 20's count of 0.74 ms, 0.30 are spent here; a count of scale 14, all core,
+// takes 35 us where the lists took 142.
 //
 // Layout: columns are cut into groups of 4,096, one 16-byte quad (128 columns)
 // per lane of a warp. Core vertex v's row is stored from the group that holds v

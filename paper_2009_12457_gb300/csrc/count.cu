@@ -1,5 +1,9 @@
-// count.cu -- per-task triangle counting (a9) and the reduction of the
-// per-task counts (a10).
+// count.cu -- triangle counting task by task (a9), the reduction of the per-task
+// counts (a10), and the host side of all resident counts.
+//
+// k_count serves the calls that need the tasks one by one: a share of them
+// (task_mask), their cycles, and block-wise streaming. All other counts walk the
+// in-edges once for all tasks (flat.cu) and the hubs as bitmaps (core.cu).
 //
 // A task t = (i, j, k) counts, for every edge (u, v) of G_ij, the common
 // elements of N(G_ik, u) and N(G_jk, v) (Sec. 4.3, Alg. 5 / Alg. 6). The

@@ -8,7 +8,12 @@
 // found, so the resident count does not visit the tasks one by one: it walks
 // the in-edges once, with the longest runs and lists the graph has, and
 // attributes hits to tasks only when the caller asks for per-task counts.
-// (R-MAT scale 22 at p = 4, one pass per task: 14.8 ms; see run_flat.)
+// (R-MAT scale 22 at p = 4 with per-task counts: 15.1 ms with a pass per task,
+// 6.2 ms so, of which the dense core takes 1.5.)
+//
+// What bounds it: on R-MAT graphs issue slots (about one warp instruction for each
+// column of a quad), on Chung-Lu graphs the latency of the probe rows, which lie
+// anywhere in the column array (30.6 ms for 18 G probes of a 451 M edge one).
 //
 // A record is {e + 1, f}: the CSR position after (u, v) and the end of u's row,
 // so [e + 1, f) is the probe run, and v is the column just before it.
@@ -929,6 +934,11 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
   const int64_t warps = (int64_t)num_sms() * 24;
   int64_t chunk = f.records / (warps * 32);
   chunk = chunk < 64 ? 64 : (chunk > 4096 ? 4096 : chunk);
+  // too few records for every warp to get an item: the time is one item's chain of
+  // loads, so items are shorter. A G(n, m) of 27 K edges by sorted search with
+  // per-task counts took 145, 103, 85 and 73 us with items of 64, 32, 16 and 8;
+  // R-MAT scale 15 at p = 8 78, 71, 71 and 81
+  if (f.records < warps * 64) chunk = 16;
   if (pl.chunk_req > 0) chunk = pl.chunk_req;
   f.chunk = chunk;
   f.nitems = (f.records + chunk - 1) / chunk;

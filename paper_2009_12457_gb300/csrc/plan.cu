@@ -2,6 +2,8 @@
 //   a5 partition: contiguous cuts of the degree order balanced on oriented
 //      edges (Sec. 2 vertex partition V^p; Sec. 4.1 symmetric partition),
 //      or the probe-based partition of partition.cu
+//   the dense core and the flat in-edges that resident counts walk (core.cu,
+//      flat.cu); the rest only for the calls that need the tasks one by one:
 //   a6 blocks G_ij = {(u,v) : u in V_i, v in V_j} (Sec. 2), materialised as
 //      the in-edges of each v grouped by the part of their source, so that a
 //      block's edges are one contiguous, destination-ordered range

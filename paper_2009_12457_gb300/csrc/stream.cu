@@ -1,12 +1,17 @@
 // stream.cu -- a11: counting with the blocks streamed from pinned host memory.
 //
-// When a caller gives bbtc_count a device budget, the plan's block arrays
-// (each block G_ab's row pointers and columns, and each block's in-edge
-// records) move to pinned host memory, and the plan's work items are put in
-// Alg. 4's task order, so that the tasks (i, j, k), k >= j, which share the
-// in-edge block of G_ij, are consecutive. The counting step then holds at
-// most `budget` bytes of blocks on the device, in one pool, in one of two
-// ways:
+// When a caller gives bbtc_count a device budget, the plan's flat in-edges move
+// to pinned host memory and cross to the device once each, in rounds of whole
+// work items through the two halves of one pool of `budget` bytes
+// (run_flat_streamed); the lists are read in the handle's oriented CSR, which
+// stays on the device.
+//
+// A share of the tasks (task_mask) and cycles per task are counted task by task
+// (run_count_streamed): the block arrays (each block G_ab's row pointers and
+// columns, and each block's in-edge records) move to pinned host memory, and
+// the plan's work items are put in Alg. 4's task order, so that the tasks
+// (i, j, k), k >= j, which share the in-edge block of G_ij, are consecutive.
+// The pool then holds blocks in one of two ways:
 //  1. When every block CSR fits in the pool beside two in-edge buffers, the
 //     block CSRs are copied once and stay, and the in-edge blocks are copied
 //     once each, group by group (one group = the tasks of one G_ij): the next
