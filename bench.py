@@ -116,16 +116,19 @@ def replica_throughput(units_per_rank: int, world: int, ms: float) -> float:
 
 
 def kernel_source_hash() -> str:
-    """sha256 of the counting kernel's source (a changed kernel voids old counters)."""
+    """sha256 of the counting kernels' sources (a changed kernel voids old counters)."""
     import hashlib
-    path = os.path.join(ROOT, "paper_2009_12457_gb300", "csrc", "count.cu")
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()
+    h = hashlib.sha256()
+    for name in ("core.cu", "flat.cu", "flat.cuh", "stage.cuh"):
+        with open(os.path.join(ROOT, "paper_2009_12457_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
 
 
 def recorded_traffic(workload: str, p: int, kernel: str):
-    """DRAM bytes per counting-kernel launch from the committed ncu record, when it
-    was taken on this kernel source and this workload; else None."""
+    """DRAM bytes of one count (the launches of its counting kernels) from the
+    committed ncu record, when it was taken on these kernels' sources and this
+    workload; else None."""
     path = os.path.join(ROOT, "profiles", "k_count_traffic.json")
     if not os.path.exists(path):
         return None
@@ -680,13 +683,14 @@ def measure(args, workload: str, p: int, budget_gb: float, env, with_cpu: bool):
 
     peak, peak_kind = measured_peaks()
     kms = sum(count_ms) / len(count_ms)
-    # bytes the destination-grouped counting kernel reads: the 16-byte in-edge
-    # records, each N(v) staged once (4 B per oriented edge), and the part of each
-    # N(u) above v (sum over u of d+(u)(d+(u)-1)/2 elements, 4 B each)
-    own = 4 * (5 * m + info["wedges_out"])
+    # bytes that destination-grouped counting reads: the 8-byte in-edge records,
+    # each N(v) staged once (4 B per oriented edge), and the part of each N(u) above
+    # v (sum over u of d+(u)(d+(u)-1)/2 elements, 4 B each; the hubs' share is read
+    # as bits instead)
+    own = 4 * (3 * m + info["wedges_out"])
     achieved = own / (kms / 1000.0) / 1e9
-    # W_min: every edge's N(v) read once per in-edge of v; this kernel
-    # never makes those reads, so it is reported for context, not as its roofline
+    # W_min: every edge's N(v) read once per in-edge of v; these kernels
+    # never make those reads, so it is reported for context, not as its roofline
     wmin = 4 * (m + info["wedges_in"])
     # bytes a merge-based intersection of both full lists would read:
     # 4 * sum over (u,v) of (d+(u) + d+(v)), with sum_(u,v) d+(u) = sum_u d+(u)^2
@@ -739,18 +743,20 @@ def measure(args, workload: str, p: int, budget_gb: float, env, with_cpu: bool):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak,
                      "traffic": traffic,
-                     "traffic_source": ("committed ncu record of this kernel source and "
+                     "traffic_source": ("committed ncu record of these kernels' sources and "
                                         "workload (profiles/k_count_traffic.json), not "
                                         "measured in this run" if traffic is not None else
-                                        "no ncu record for this kernel source and workload"),
-                     "kernel": "k_count (per-task counting, a9)",
+                                        "no ncu record for these kernels' sources and workload"),
+                     "kernel": "k_flat and k_core_count (counting, a9)",
                      "algorithmic_bytes": own,
-                     "bytes_formula": "4*(5m + sum over u of d+(u)(d+(u)-1)/2): 16-byte "
+                     "bytes_formula": "4*(3m + sum over u of d+(u)(d+(u)-1)/2): 8-byte "
                                       "in-edge records, each N(v) staged once, the probed "
-                                      "part of each N(u) above v",
+                                      "part of each N(u) above v (the hubs' share is read "
+                                      "as fewer bytes of bitmap rows, so that a skewed "
+                                      "graph can come out above 1)",
                      "w_min_bytes": wmin,
                      "w_min_formula": "4*(m + sum over oriented edges (u,v) of d+(v)); reads "
-                                      "N(v) once per in-edge, which this kernel does not do",
+                                      "N(v) once per in-edge, which these kernels do not do",
                      "w_min_over_time_per_peak": wmin / (kms / 1000.0) / 1e9 / peak,
                      "w_merge_bytes": wmerge,
                      "peak_source": f"{peak_kind} hbm_gbs"},
