@@ -11,9 +11,10 @@
 // (R-MAT scale 22 at p = 4 with per-task counts: 15.1 ms with a pass per task,
 // 6.2 ms so, of which the dense core takes 1.5.)
 //
-// What bounds it: on R-MAT graphs issue slots (about one warp instruction for each
-// column of a quad), on Chung-Lu graphs the latency of the probe rows, which lie
-// anywhere in the column array (30.6 ms for 18 G probes of a 451 M edge one).
+// What bounds it: waits on loads with 24 warps per SM, which the warps' staging
+// areas limit (issue active 55% on R-MAT scale 20, DRAM at 4%); on Chung-Lu graphs the
+// probe rows lie anywhere in the column array (30.6 ms for 18 G probes of a 451 M
+// edge one; 1.8 G edges: 136 ms, 3.9 TB/s from DRAM).
 //
 // A record is {e + 1, f}: the CSR position after (u, v) and the end of u's row,
 // so [e + 1, f) is the probe run, and v is the column just before it.
