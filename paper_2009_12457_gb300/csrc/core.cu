@@ -426,7 +426,8 @@ __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P)
   }
   if (ONE) {
     acc = warp_sum(acc);
-    if (lane == 0 && acc) atomicAdd(&P.task_count[MULTI ? P.descs[cur_desc].task_base : 0], acc);
+    const int32_t tb = MULTI ? P.descs[cur_desc].task_base : P.one.task_base;
+    if (lane == 0 && acc) atomicAdd(&P.task_count[tb], acc);
   } else if (in_table) {
     __syncthreads();
     for (int i = threadIdx.x; i < (int)P.ntasks; i += CORE_NT)

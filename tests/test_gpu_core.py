@@ -53,3 +53,32 @@ def test_core_of_a_batch_per_graph_and_of_handles():
     finally:
         for h in hs:
             h.close()
+
+
+def test_core_items_of_only_one_handle_of_a_batch():
+    # a handle's core triangles are its own, also when no other handle has a core
+    def complete(n):
+        rp = np.arange(n + 1, dtype=np.int64) * (n - 1)
+        ci = np.array([[v for v in range(n) if v != u] for u in range(n)], dtype=np.int32).ravel()
+        return n, rp, ci
+
+    edgeless = (7, np.zeros(8, dtype=np.int64), np.zeros(0, dtype=np.int32))
+    two_edges = (3, np.array([0, 1, 3, 4], dtype=np.int64), np.array([1, 0, 2, 1], dtype=np.int32))
+    sparse = graphgen.gnm(20_000, 60_000, 41)  # lists alone: no source has 64 core neighbours
+    hubs = graphgen.rmat(15, 16, 33)
+    for graphs in ([edgeless, complete(100)], [complete(100), edgeless],
+                   [two_edges, edgeless, complete(65)], [sparse, hubs], [hubs, sparse, two_edges]):
+        want = np.array([oracle.bbtc(*g, p=1)["total"] for g in graphs], dtype=np.uint64)
+        hs = [bb.Graph(*g, symmetric=True) for g in graphs]
+        try:
+            handles = [h.handle for h in hs]
+            for p in (0, 3):
+                counts, stats = bb.bbtc_count_batch(handles, bb.make_opts(p=p))
+                assert not np.any(stats) and np.array_equal(counts, want), p
+                counts, stats = bb.bbtc_count_batch(handles[:1] + [None] + handles[1:],
+                                                    bb.make_opts(p=p))
+                assert stats[1] == 1 and not np.any(np.delete(stats, 1))
+                assert np.array_equal(np.delete(counts, 1), want), p
+        finally:
+            for h in hs:
+                h.close()
