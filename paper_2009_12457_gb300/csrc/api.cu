@@ -599,7 +599,7 @@ bbtc_status bbtc_count_async(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t 
   BBTC_TRY(check_opts(opts_in, &opts));
   const int p = opts.p == 0 ? default_p(g) : opts.p;
   if (!plan_matches(g->plan, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition) ||
-      g->plan.streamed) {
+      !plan_countable(g->plan)) {
     set_error("bbtc_count_async: no resident plan for these options on the handle; build it "
               "with bbtc_count (without a device budget) or bbtc_graph_get_plan first");
     return BBTC_EINVAL;

@@ -892,7 +892,7 @@ extern "C" bbtc_status bbtc_count_noalloc(bbtc_graph_t g, int32_t p, uint64_t *c
     return BBTC_EINVAL;
   }
   const Plan &pl = g->plan;
-  if (pl.p != p || pl.streamed) {
+  if (pl.p != p || !plan_countable(pl)) {
     set_error("bbtc_count_noalloc: no plan for p = %d on this handle; call bbtc_count or "
               "bbtc_graph_get_plan with that p first", p);
     return BBTC_EINVAL;

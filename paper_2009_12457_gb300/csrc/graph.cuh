@@ -257,6 +257,12 @@ inline bool plan_matches(const Plan &pl, int p, int kernel_mode, int hash_thresh
          pl.chunk_req == chunk && pl.partition == partition;
 }
 
+// Whether a count can run on the plan as it stands. A plan holds only its cuts when
+// a budget was refused or memory ran out before any form of the in-edges was built.
+inline bool plan_countable(const Plan &pl) {
+  return !pl.streamed && (pl.flat.ready || pl.full.ready || pl.tasks_ready);
+}
+
 // a5, probe-based: cuts (device, p+1) of the partition that bounds the largest
 // block load by B* (returned on the host). Synchronises s.
 bbtc_status pbd_partition(const bbtc_graph *g, int p, int32_t *d_cuts, int64_t *h_bstar,

@@ -74,3 +74,27 @@ def test_async_refuses_a_streamed_plan():
         total = torch.zeros(1, dtype=torch.int64, device="cuda")
         with pytest.raises(bb.BbtcError):
             bb.bbtc_count_async(g.handle, bb.make_opts(p=2), total)
+
+
+def test_a_refused_budget_leaves_no_plan_to_count_with():
+    n, rp, ci = graphgen.rmat(15, 16, 4)
+    with bb.Graph(n, rp, ci) as g:
+        with pytest.raises(bb.BbtcError) as e:
+            g.count(p=8, device_budget_bytes=4096)
+        assert e.value.status == 2
+        total = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+        for call in (lambda: bb.bbtc_count_async(g.handle, bb.make_opts(p=8), total),
+                     lambda: bb.bbtc_count_noalloc(g.handle, 8, total)):
+            with pytest.raises(bb.BbtcError) as e:
+                call()
+            assert e.value.status == 1
+            torch.cuda.synchronize()
+            assert int(total.item()) == -1  # outputs are left untouched
+        want = g.count(p=8)
+        for call in (lambda: bb.bbtc_count_async(g.handle, bb.make_opts(p=8), total),
+                     lambda: bb.bbtc_count_noalloc(g.handle, 8, total)):
+            total.fill_(-1)
+            torch.cuda.synchronize()  # the handle counts on a stream of its own
+            call()
+            torch.cuda.synchronize()
+            assert int(total.item()) == want
