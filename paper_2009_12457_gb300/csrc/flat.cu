@@ -243,11 +243,13 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
     uint32_t v = 0, vend = base;  // the run at hand: its destination and end
     uint32_t b0 = 0, b1 = 0;      // N(v)
     int32_t vl = -1;              // the lane's own destination (set when a run begins)
-    int32_t run_graph = -1;       // GRAPH: the run's graph, and its hits so far
-    uint32_t run_hits = 0;
+    // GRAPH: the run's graph, and its hits so far (an item's length is the caller's
+    // choice, so they may pass 32 bits)
+    int32_t run_graph = -1;
+    unsigned long long run_hits = 0;
     auto flush_graph = [&]() {
-      const uint32_t sum = __reduce_add_sync(0xffffffffu, run_hits);
-      if (lane == 0 && sum) atomicAdd(&P.graph_count[run_graph], (unsigned long long)sum);
+      const unsigned long long sum = warp_sum(run_hits);
+      if (lane == 0 && sum) atomicAdd(&P.graph_count[run_graph], sum);
       run_hits = 0;
     };
     int staged_mode = ST_NONE, staged_log2h = 0, staged_len = 0;

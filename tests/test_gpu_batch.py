@@ -241,3 +241,19 @@ def test_symmetric_batch_fast_path_matches_oracle():
     with pytest.raises(bb.BbtcError) as e:
         bb.bbtc_graph_create_batch(voff, rowptr, colidx, bb.INPUT_SYMMETRIC)
     assert e.value.status == 1
+
+
+def test_per_graph_count_beyond_32_bits_within_one_work_item():
+    # one graph of the batch holds more than 2^32 triangles, all in one work item of
+    # the caller's choice; the other vertices keep the union out of the all-core form
+    k, rest = 2955, 14_000
+    ci = np.broadcast_to(np.arange(k, dtype=np.int32), (k, k))[~np.eye(k, dtype=bool)]
+    clique = (k, np.arange(k + 1, dtype=np.int64) * (k - 1), ci)
+    edgeless = (rest, np.zeros(rest + 1, dtype=np.int64), np.zeros(0, dtype=np.int32))
+    triangle = (3, np.array([0, 2, 4, 6], dtype=np.int64), np.array([1, 2, 0, 2, 0, 1], np.int32))
+    want = [k * (k - 1) * (k - 2) // 6, 0, 1]
+    assert want[0] > 1 << 32
+    with bb.BatchGraph([clique, edgeless, triangle], symmetric=True) as u:
+        out = u.count(p=1, per_graph=True, chunk=1 << 30)
+        assert out["total"] == sum(want)
+        assert out["per_graph"].tolist() == want
