@@ -108,7 +108,11 @@ __global__ void __launch_bounds__(CORE_NT) k_core_bits(const int64_t *__restrict
 // least min_row core neighbours, as work items {u, first core edge, first edge
 // of the item, end of the row} of at most CORE_CHUNK core edges, and one flag
 // bit per position. Sources that find no room in the item list keep a clear
-// flag (the lists count them). One thread per position, highest first.
+// flag (the lists count them). Room is only ever taken, never given back: what was
+// taken past it by one reservation would else be handed out again while an earlier
+// gap stayed unwritten. So the reservation that crosses the end is the only one
+// that leaves entries below it, which become empty items, and the number of items
+// is the smaller of *nitems and cap. One thread per position, highest first.
 __global__ void __launch_bounds__(CORE_NT) k_core_rows(const int64_t *__restrict__ rowptr,
                                                        const int32_t *__restrict__ colidx,
                                                        int64_t n, int64_t u0, int32_t v0,
@@ -135,12 +139,11 @@ __global__ void __launch_bounds__(CORE_NT) k_core_rows(const int64_t *__restrict
     const uint32_t incl = warp_inclusive_scan(cnt);
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     uint32_t at = 0;
-    if (lane == 0 && total) {
-      at = atomicAdd(nitems, total);
-      if (at + total > cap) atomicSub(nitems, total);  // no room: the whole word stays with the lists
-    }
+    if (lane == 0 && total) at = atomicAdd(nitems, total);
     at = __shfl_sync(0xffffffffu, at, 0);
-    const bool room = total > 0 && at + total <= cap;
+    const bool room = total > 0 && at + total <= cap;  // else the whole word stays with the lists
+    if (total && !room)
+      for (uint32_t o = at + lane; o < cap; o += 32) items[o] = make_int4((int32_t)(u0 + word * 32), 0, 0, 0);
     const unsigned flag = __ballot_sync(0xffffffffu, room && cnt > 0);
     if (lane == 0) flags[word] = flag;
     if (room) {

@@ -623,6 +623,7 @@ namespace {
 constexpr int FC_COLS = 8192;  // core destinations counted on chip: the top ones
 __global__ void __launch_bounds__(512) k_flat_minus_core(const int4 *__restrict__ items,
                                                          const unsigned *__restrict__ count,
+                                                         unsigned cap,
                                                          int32_t chunk,
                                                          const int32_t *__restrict__ colidx,
                                                          int64_t n, unsigned *__restrict__ hist) {
@@ -631,7 +632,7 @@ __global__ void __launch_bounds__(512) k_flat_minus_core(const int4 *__restrict_
   for (int i = threadIdx.x; i < FC_COLS; i += 512) cnt[i] = 0;
   __syncthreads();
   const int64_t nw = (int64_t)gridDim.x * 16;
-  const int64_t total = *count;
+  const int64_t total = *count < cap ? *count : cap;
   for (int64_t x = (int64_t)blockIdx.x * 16 + (threadIdx.x >> 5); x < total; x += nw) {
     const int4 it = items[x];
     const uint32_t x0 = (uint32_t)it.z, re = (uint32_t)it.w;
@@ -897,7 +898,7 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
     unsigned items = 0;
     BBTC_CUDA(cudaMemcpyAsync(&items, core.count, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     BBTC_CUDA(cudaStreamSynchronize(s));
-    pl.core.nitems = (int64_t)items;
+    pl.core.nitems = std::min<int64_t>(items, core.cap);
     f.ready = true;
     return BBTC_OK;
   }
@@ -917,8 +918,8 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
   }
   BBTC_LAUNCH_CHECK();
   if (core.bits) {
-    k_flat_minus_core<<<(unsigned)num_sms() * 2, 512, 0, s>>>(core.items, core.count, CORE_CHUNK,
-                                                             g->colidx, n, hist);
+    k_flat_minus_core<<<(unsigned)num_sms() * 2, 512, 0, s>>>(core.items, core.count, core.cap,
+                                                             CORE_CHUNK, g->colidx, n, hist);
     BBTC_LAUNCH_CHECK();
   }
   BBTC_TRY(exclusive_scan_u32(hist, f.inptr, hist, n + 1, s));  // hist: the cursors
@@ -929,7 +930,7 @@ bbtc_status build_flat(const bbtc_graph *g, Plan &pl, Flat &f, bool use_core, cu
     BBTC_CUDA(cudaMemcpyAsync(&items, core.count, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   f.records = records;
-  if (core.bits) pl.core.nitems = (int64_t)items;
+  if (core.bits) pl.core.nitems = std::min<int64_t>(items, core.cap);
   BBTC_TRY(dalloc_n(&f.rec, f.records, s));
   // about 32 items per resident warp, 64 to 4,096 in-edges each (or the caller's
   // choice); 64 and 128 items staged each list more often (R-MAT scale 21 at p = 4,

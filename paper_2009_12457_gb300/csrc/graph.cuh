@@ -83,7 +83,7 @@ struct Core {
   uint8_t *qpart = nullptr;    // part of each quad
   int4 *items = nullptr;       // {u, first core edge, first edge of the item, row end}
   unsigned *flags = nullptr;   // bit u - u0: u is counted here
-  unsigned *count = nullptr;   // number of items (device)
+  unsigned *count = nullptr;   // items asked for (device); there are at most cap
   uint64_t bytes = 0;
 };
 

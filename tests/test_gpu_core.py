@@ -82,3 +82,18 @@ def test_core_items_of_only_one_handle_of_a_batch():
         finally:
             for h in hs:
                 h.close()
+
+
+def test_a_core_with_more_items_than_its_list_holds():
+    # the complete graph of 20,000 vertices has 1.33 M core items, the list room for 2^20:
+    # the sources without room are counted by lists. Rows of every length, made on the device
+    n = 20_000
+    ids = torch.arange(n, dtype=torch.int32, device="cuda")
+    ci = ids[None, :].expand(n, n)[ids[None, :] != ids[:, None]]
+    rp = torch.arange(n + 1, dtype=torch.int64, device="cuda") * (n - 1)
+    torch.cuda.synchronize()  # the library reads them on its own stream
+    with bb.Graph(n, rp, ci, symmetric=True) as g:
+        del ids, ci, rp
+        assert g.count(p=1) == n * (n - 1) * (n - 2) // 6
+        assert g.count(p=1, per_task=True)["per_task"].tolist() == [n * (n - 1) * (n - 2) // 6]
+    torch.cuda.empty_cache()
