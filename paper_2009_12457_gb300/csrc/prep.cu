@@ -5,6 +5,7 @@
 //   a4 orientation                (Sec. 2: N(G,u) = {v : (u,v) in E, u < v})
 #include <limits.h>
 
+#include "bounds.cuh"
 #include "graph.cuh"
 #include "primitives.cuh"
 
@@ -668,7 +669,8 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
       at = __shfl_sync(0xffffffffu, at, 0);
       if (!up) continue;
       int64_t pos = (place ? place[rank[rowx]] : rowptr[rowx]) + (int64_t)(at + incl - cnt);
-      if (!place && (uint64_t)pos + cnt > (uint64_t)nnz) continue;  // (see below)
+      // (row pointers that decrease are found by the host only after this pass)
+      if (!place && !span_inside(pos, cnt, nnz)) continue;
 #pragma unroll
       for (int i = 0; i < SP_ITEMS; ++i)
         if ((ups >> i) & 1u) up[pos++] = val[i];
@@ -688,8 +690,7 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
         }
       }
       if ((ups >> i) & 1u) {
-        // (row pointers that decrease are found by the host only after this pass)
-        if (up && (place || (uint64_t)pos < (uint64_t)nnz)) up[pos] = val[i];
+        if (up && (place || (uint64_t)pos < (uint64_t)nnz)) up[pos] = val[i];  // (as above)
         ++pos;
       }
     }

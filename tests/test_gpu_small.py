@@ -92,3 +92,18 @@ def test_an_edge_listed_too_often_for_its_bucket():
         assert np.array_equal(o["rowptr"], ref["rowptr"])
         assert np.array_equal(o["colidx"], ref["colidx"])
         assert g.count() == ref["total"]
+
+
+@pytest.mark.parametrize("row,value", [(1024, -1), (1024, -5), (1, -8), (2047, -(1 << 40)),
+                                       (1500, 1 << 40)])
+def test_interior_row_pointers_out_of_range_are_refused(row, value):
+    # beyond one CTA; the error is known to the host only after the entries have been moved
+    n, rp, ci = graphgen.gnm(2048, 30_000, 5)
+    rp = rp.copy()
+    rp[row] = value
+    for symmetric in (True, False):
+        with pytest.raises(bb.BbtcError) as e:
+            bb.Graph(n, rp, ci, symmetric=symmetric)
+        assert e.value.status == 1
+    with bb.Graph(*graphgen.gnm(2048, 30_000, 5), symmetric=True) as g:  # all is well after
+        assert g.count() == oracle.bbtc(*graphgen.gnm(2048, 30_000, 5), p=1)["total"]
