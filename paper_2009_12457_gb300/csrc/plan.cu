@@ -537,10 +537,11 @@ __global__ void k_tasks(const int64_t *__restrict__ boff, const int32_t *__restr
 }
 
 __global__ void k_order_finish(const uint32_t *__restrict__ vals, int64_t nt,
-                               int32_t *__restrict__ order) {
+                               const int32_t *__restrict__ err, int32_t *__restrict__ order) {
+  const bool failed = (*err & SORT_FAILED) != 0;  // then any order: the caller reports it
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nt;
        x += (int64_t)gridDim.x * blockDim.x)
-    order[x] = (int32_t)vals[x];
+    order[x] = failed ? (int32_t)x : (int32_t)vals[x];
 }
 
 // Number of work items of the task at each position of the order. A task
@@ -867,7 +868,7 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
     return BBTC_ECUDA;
   }
   PLAN_TRY(radix_sort(okeys, okeys_alt, ovals, ovals_alt, nt, 0, 64, s, serr, &in_alt));
-  k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, pl.order);
+  k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, serr, pl.order);
   PLAN_TRY(launch_status("build_plan"));
 
   // task descriptors: every block of the resident BCSR

@@ -55,6 +55,7 @@ struct RsSmem {
   uint64_t goff[RS_BINS];             // global start of this tile's part of each bucket
   uint32_t scan_tmp[RS_WARPS + 1];
   uint32_t tile;
+  int32_t failed;  // an earlier pass or tile gave up
 };
 
 // Ranks a tile's keys (thread-owned positions warp * RS_WARP_SPAN + 32 i + lane) by digit,
@@ -107,7 +108,9 @@ __device__ __forceinline__ uint32_t rs_rank(RsSmem<HAS_VALS> &sm, const uint64_t
 // 2.4 ms of passes in R-MAT scale 20's general preparation). Tiles are taken in
 // ticket order, so the tiles waited for are running or done; every wait is
 // bounded all the same, and a tile that gives up poisons its own entry, so that
-// the ones after it stop, writes nothing and sets bit 3 of *err.
+// the ones after it stop, writes nothing and sets bit 3 of *err. The passes after a
+// failed one find the bit and move no key: those that the failed pass left unwritten
+// would not match the digit counts, and could be sent past the end of the output.
 // Word of (tile, digit): code << 56 | count; pass q uses the codes 2q + 1 (the
 // tile's own count) and 2q + 2 (the count up to and with the tile).
 constexpr uint64_t RS_POISON = 0xffull << 56;
@@ -125,9 +128,16 @@ __global__ void __launch_bounds__(RS_NT) k_rs_pass(
   RsSmem<HAS_VALS> &sm = *reinterpret_cast<RsSmem<HAS_VALS> *>(rs_smem_raw);
   const int warp = threadIdx.x >> 5;
   const unsigned lane = threadIdx.x & 31u;
-  if (threadIdx.x == 0) sm.tile = atomicAdd(ticket, 1u);
+  if (threadIdx.x == 0) {
+    sm.tile = atomicAdd(ticket, 1u);
+    sm.failed = *(volatile int32_t *)err & SORT_FAILED;
+  }
   __syncthreads();
   const int64_t tile = sm.tile;
+  if (sm.failed) {
+    if (threadIdx.x < RS_BINS) *(volatile unsigned long long *)(status + tile * RS_BINS + threadIdx.x) = RS_POISON;
+    return;
+  }
   const int64_t base = tile * RS_TILE;
   const int nvalid = (int)(count - base < RS_TILE ? count - base : RS_TILE);
   uint64_t k[RS_ITEMS];
@@ -186,7 +196,7 @@ __global__ void __launch_bounds__(RS_NT) k_rs_pass(
   failed = __syncthreads_or(failed);
   if (failed) {
     if (d < RS_BINS) *st = RS_POISON;
-    if (threadIdx.x == 0) atomicOr(err, 8);
+    if (threadIdx.x == 0) atomicOr(err, SORT_FAILED);
     return;
   }
   if (d < RS_BINS) {
