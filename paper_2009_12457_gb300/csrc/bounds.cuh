@@ -18,4 +18,8 @@ BBTC_HD bool span_inside(int64_t at, uint32_t count, int64_t size) {
   return at >= 0 && at <= size && (int64_t)count <= size - at;
 }
 
+// Whether record base + i lies before `end` (base <= end): positions reach 2^32 - 1,
+// where base + i would wrap to the front of the array.
+BBTC_HD bool window_holds(uint32_t base, uint32_t i, uint32_t end) { return i < end - base; }
+
 }  // namespace bbtc

@@ -344,8 +344,8 @@ __global__ void __launch_bounds__(CORE_NT, CORE_CTAS) k_core_count(CoreLaunch P)
       for (int q = lane; q < nq; q += 32) mask4[q] = make_uint4(0, 0, 0, 0);
       __syncwarp();
       unsigned *mk = reinterpret_cast<unsigned *>(mask4);
-      for (uint32_t e = cs + lane; e < re; e += 32) {
-        const int32_t w = ci[e];
+      for (uint32_t x = lane; x < re - cs; x += 32) {
+        const int32_t w = ci[cs + x];
         const int kw = d.parts.np == 1 ? 0 : core_part(d.parts, w);
         const unsigned col = (unsigned)(d.parts.quad0[kw] * 128 + (w - d.parts.first[kw]));
         atomicOr(&mk[col >> 5], 1u << (col & 31u));

@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "bounds.cuh"
 #include "flat.cuh"
 #include "graph.cuh"
 #include "stage.cuh"
@@ -117,13 +118,13 @@ __global__ void __launch_bounds__(DT_NT, 3) k_detail(DetailLaunch P) {
       }
       since = 0;
     };
-    uint2 r = base + lane < x1 ? rec[base + lane] : make_uint2(0, 0);
+    uint2 r = window_holds(base, lane, x1) ? rec[base + lane] : make_uint2(0, 0);
     while (base < x1) {
       const bool begins = vend <= base;
       if (begins) {
         flush(false);
         staged = ST_NONE;
-        vl = base + lane < x1 ? ci[r.x - 1] : -1;
+        vl = window_holds(base, lane, x1) ? ci[r.x - 1] : -1;
         v = (uint32_t)__shfl_sync(0xffffffffu, vl, 0);
         vend = inptr[v + 1];
         b0 = (uint32_t)rowptr[v];
@@ -133,14 +134,14 @@ __global__ void __launch_bounds__(DT_NT, 3) k_detail(DetailLaunch P) {
       const bool uniform = !begins || run >= (uint32_t)DT_RUN_MIN || run == x1 - base;
       if (uniform && b1 == b0) {
         base += run;
-        r = base + lane < x1 ? rec[base + lane] : make_uint2(0, 0);
+        r = window_holds(base, lane, x1) ? rec[base + lane] : make_uint2(0, 0);
         continue;
       }
       int nb = (int)min(run, 32u);
       uint32_t vb0 = b0, vb1 = b1;
       if (!uniform) {  // short runs share the window (see flat.cu)
         const unsigned same = __match_any_sync(0xffffffffu, vl);
-        const bool lengthy = __popc(same) >= DT_RUN_MIN || ((same >> 31) && base + 32 < x1);
+        const bool lengthy = __popc(same) >= DT_RUN_MIN || ((same >> 31) && window_holds(base, 32u, x1));
         const unsigned stop = __ballot_sync(0xffffffffu, vl < 0 || (lengthy && vl != (int32_t)v));
         nb = stop ? __ffs(stop) - 1 : 32;
         if ((int)lane < nb) {
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(DT_NT, 3) k_detail(DetailLaunch P) {
         vend = base + (uint32_t)nb;
       }
       base += (uint32_t)nb;
-      const uint2 rn = base + lane < x1 ? rec[base + lane] : make_uint2(0, 0);
+      const uint2 rn = window_holds(base, lane, x1) ? rec[base + lane] : make_uint2(0, 0);
       const bool active = (int)lane < nb && vb1 > vb0;
       const uint32_t s0 = r.x, s1 = r.y;
       r = rn;

@@ -22,6 +22,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "bounds.cuh"
 #include "flat.cuh"
 #include "graph.cuh"
 #include "primitives.cuh"
@@ -266,11 +267,11 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
       if (field_sum) add_task((int)lane / nk, j_part, j_part + (int)lane % nk, field_sum);
       field_sum = 0;
     };
-    uint2 r = base + lane < x1 ? rec[base + lane] : make_uint2(0, 0);
+    uint2 r = window_holds(base, lane, x1) ? rec[base + lane] : make_uint2(0, 0);
     while (base < x1) {
       const bool begins = vend <= base;
       if (begins) {  // a new run: (u, v) sits just below its probe run in u's row
-        vl = base + lane < x1 ? ci[r.x - 1] : -1;
+        vl = window_holds(base, lane, x1) ? ci[r.x - 1] : -1;
         v = (uint32_t)__shfl_sync(0xffffffffu, vl, 0);
         vend = inptr[v + 1];
         b0 = (uint32_t)rowptr[v];
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
       const bool uniform = !begins || run >= (uint32_t)FL_RUN_MIN || run == x1 - base;
       if (uniform && b1 == b0) {  // nothing to find in an empty list
         base += run;
-        r = base + lane < x1 ? rec[base + lane] : make_uint2(0, 0);
+        r = window_holds(base, lane, x1) ? rec[base + lane] : make_uint2(0, 0);
         continue;
       }
       int nb = (int)min(run, 32u);
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
         // short runs share the window, up to a run that makes a batch of its own or
         // that may go on past the window
         const unsigned same = __match_any_sync(0xffffffffu, vl);
-        const bool lengthy = __popc(same) >= FL_RUN_MIN || ((same >> 31) && base + 32 < x1);
+        const bool lengthy = __popc(same) >= FL_RUN_MIN || ((same >> 31) && window_holds(base, 32u, x1));
         const unsigned stop = __ballot_sync(0xffffffffu, vl < 0 || (lengthy && vl != (int32_t)v));
         nb = stop ? __ffs(stop) - 1 : 32;
         if ((int)lane < nb) {
@@ -312,8 +313,8 @@ __global__ void __launch_bounds__(FL_NT, FL_CTAS) k_flat(FlatLaunch P) {
         vend = base + (uint32_t)nb;  // the next window begins a new run
       }
       base += (uint32_t)nb;
-      const uint2 rn = base + lane < x1 ? rec[base + lane] : make_uint2(0, 0);
-      if (base + 32 + lane < x1)
+      const uint2 rn = window_holds(base, lane, x1) ? rec[base + lane] : make_uint2(0, 0);
+      if (window_holds(base, 32u + lane, x1))
         asm volatile("prefetch.global.L2 [%0];" ::"l"(rec + base + 32 + lane));
       const bool active = (int)lane < nb && vb1 > vb0;
       const uint32_t s0 = r.x, s1 = r.y;
@@ -636,9 +637,9 @@ __global__ void __launch_bounds__(512) k_flat_minus_core(const int4 *__restrict_
   for (int64_t x = (int64_t)blockIdx.x * 16 + (threadIdx.x >> 5); x < total; x += nw) {
     const int4 it = items[x];
     const uint32_t x0 = (uint32_t)it.z, re = (uint32_t)it.w;
-    const uint32_t x1 = re - x0 < (uint32_t)chunk ? re : x0 + (uint32_t)chunk;
-    for (uint32_t e = x0 + lane_id(); e < x1; e += 32) {
-      const int64_t v = colidx[e];
+    const uint32_t len = re - x0 < (uint32_t)chunk ? re - x0 : (uint32_t)chunk;
+    for (uint32_t i = lane_id(); i < len; i += 32) {
+      const int64_t v = colidx[x0 + i];
       if (v >= first) atomicAdd(&cnt[v - first], 1u);
       else atomicSub(&hist[v], 1u);
     }

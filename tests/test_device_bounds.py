@@ -27,3 +27,15 @@ def test_span_inside(tmp_path):
     body = "\n".join(f'printf("%d\\n", (int)span_inside({a}ll, {c}u, {s}ll));'
                      for a, c, s, _ in cases)
     assert run(tmp_path, body) == [str(w) for *_, w in cases]
+
+
+def test_window_holds(tmp_path):
+    top = (1 << 32) - 1
+    cases = [(0, 0, 0, 0), (0, 31, 32, 1), (0, 32, 32, 0), (100, 0, 100, 0), (100, 5, 106, 1),
+             # windows at the last positions of the largest graph: base + i passes 2^32
+             (top - 16, 15, top, 1), (top - 16, 16, top, 0), (top - 16, 17, top, 0),
+             (top - 16, 31, top, 0), (top - 40, 32, top, 1), (top - 40, 63, top, 0),
+             (top, 1, top, 0)]
+    body = "\n".join(f'printf("%d\\n", (int)window_holds({b}u, {i}u, {e}u));'
+                     for b, i, e, _ in cases)
+    assert run(tmp_path, body) == [str(w) for *_, w in cases]
