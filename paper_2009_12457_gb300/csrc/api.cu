@@ -542,6 +542,7 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
     g->stream_stats.device_peak = st.device_peak;
     g->stream_stats.mode = st.mode;
     g->stream_stats_total_ms = st.total_ms;
+    g->counted_items = st.items;
   } else {
     if (by_task)
       BBTC_TRY(run_count(g, pl, vertex_count, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5],
@@ -552,6 +553,9 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
     else
       BBTC_TRY(run_flat(g, pl, tasks, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5]));
     g->stream_stats_total_ms = -1.0;
+    g->counted_items = by_task ? pl.nitems
+                               : (resident ? pl.core.nitems + pl.flat.nitems : 0) +
+                                     (detail ? detail_flat(pl).nitems : 0);
   }
   unsigned long long head[SCR_TASKS] = {0};
   BBTC_CUDA(cudaMemcpyAsync(head, pl.scratch, sizeof(head), cudaMemcpyDeviceToHost, s));
@@ -805,7 +809,9 @@ bbtc_status bbtc_graph_get_timings(bbtc_graph_t g, bbtc_timings *t) {
   t->plan_ms = g->plan_timed ? elapsed(g->ev[2], g->ev[3]) : 0.0;
   t->count_ms = g->stream_stats_total_ms >= 0 ? g->stream_stats_total_ms
                                               : elapsed(g->ev[4], g->ev[5]);
-  t->work_items = g->plan.flat.ready ? g->plan.flat.nitems + g->plan.core.nitems : g->plan.nitems;
+  t->work_items = g->counted_items >= 0  ? g->counted_items
+                  : g->plan.flat.ready ? g->plan.flat.nitems + g->plan.core.nitems
+                                       : g->plan.nitems;
   t->stream_rounds = g->stream_stats.rounds;
   t->stream_h2d_bytes = g->stream_stats.h2d_bytes;
   t->stream_copy_ms = g->stream_stats.copy_ms;

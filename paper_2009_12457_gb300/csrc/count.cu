@@ -743,7 +743,7 @@ bbtc_status run_detail(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph
     BBTC_TRY(count_reset(g, pl, nullptr, false, s));
     if (ev_begin) BBTC_CUDA(cudaEventRecord(ev_begin, s));
   }
-  const Flat &f = pl.full.ready ? pl.full : pl.flat;
+  const Flat &f = detail_flat(pl);
   BBTC_TRY(detail_launch(g, pl, flat_desc(g, pl, f, 0, 0), both ? nullptr : pl.scratch + SCR_TOTAL, vcount, edge_sup,
                          timeout_ms, s));
   if (ev_end) BBTC_CUDA(cudaEventRecord(ev_end, s));

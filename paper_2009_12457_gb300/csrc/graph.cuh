@@ -226,6 +226,7 @@ struct bbtc_graph {
   bbtc::Plan plan;
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   bool plan_timed = false;
+  int64_t counted_items = -1;  // work items of the last bbtc_count on the plan (-1: none yet)
   StreamStatsLite stream_stats;
   double stream_stats_total_ms = -1.0;  // >= 0 when the last count was streamed
   bool wedges_known = false;
@@ -311,6 +312,7 @@ bbtc_status run_flat(bbtc_graph *g, const Plan &pl, bool tasks, bool per_graph,
 // the caller, over all in-edges (build_full first); total (nullable) receives
 // the number of triangles. Enqueues only.
 bbtc_status build_full(bbtc_graph *g, cudaStream_t s);
+inline const Flat &detail_flat(const Plan &pl) { return pl.full.ready ? pl.full : pl.flat; }
 bbtc_status detail_launch(const bbtc_graph *g, const Plan &pl, const FlatDesc &d,
                           unsigned long long *total, unsigned long long *vcount, unsigned *edge_sup, uint32_t timeout_ms,
                           cudaStream_t s);
@@ -362,6 +364,7 @@ struct StreamStats {
   uint64_t block_bytes = 0;  // every streamed block once
   uint64_t device_peak = 0;  // pool high-water mark during the count
   int32_t mode = 0;          // 1: block CSRs resident, in-edge blocks once; 2: general
+  int64_t items = 0;         // work items drained
 };
 bbtc_status run_count_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
                                unsigned long long *vertex_count, bool per_graph,

@@ -696,6 +696,7 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   pl.bytes = (uint64_t)(SCR_TASKS + pl.ntasks + g->ng) * 8;
   if (resident) PLAN_TRY(add_resident(g, pl, s));
   g->plan = pl;
+  g->counted_items = -1;
   return BBTC_OK;
 }
 

@@ -586,6 +586,7 @@ bbtc_status run_count_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
     if (cudaEventElapsedTime(&ms, t_begin, t_end) == cudaSuccess) stats->total_ms = ms;
   }
   stats->rounds = round;
+  stats->items = pl.nitems;
   stats->copy_ms = copy_ms_total;
   if (mem_pool) {
     uint64_t peak = 0;
@@ -775,6 +776,7 @@ bbtc_status run_flat_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
       }
     }
     stats->rounds = round;
+    stats->items = (pl.any_task ? nitems : 0) * ((flat_too ? 1 : 0) + (vertex_count ? 1 : 0));
     if (st != BBTC_OK) break;
     if (tasks) st = count_finish(pl, s);
     if (st == BBTC_OK && cudaEventRecord(t_end, s) != cudaSuccess) st = BBTC_ECUDA;

@@ -81,3 +81,21 @@ def test_one_destination_with_more_in_edges_than_a_counter_holds():
         assert int(out["per_vertex"][k]) == k and int(out["per_vertex"][k + 1]) == k
         sup = g.count(p=1, per_edge=True, chunk=100_000)["per_edge"]
         assert int(sup.max()) == k and int((sup == 1).sum()) == 2 * k
+
+
+def test_work_items_of_every_kind_of_count():
+    # without a core (INTERSECT) every in-edge is in a work item of `chunk` of them
+    n, rp, ci = graphgen.rmat(14, 16, 15)
+    with bb.Graph(n, rp, ci, symmetric=True) as g:
+        m, chunk = g.info()["m"], 64
+        items = -(-m // chunk)
+        kw = dict(p=3, kernel="intersect", chunk=chunk)
+        for more, want in (({"per_vertex": True}, items), ({}, items), ({"per_edge": True}, items),
+                           ({"per_vertex": True, "per_task": True}, 2 * items),
+                           ({"device_budget_bytes": 64 << 20}, items), ({}, items)):
+            g.count(**kw, **more)
+            assert g.timings()["work_items"] == want, more
+        g.count(**kw, per_task_cycles=True)  # task by task: every task's in-edges
+        assert g.timings()["work_items"] >= items
+        g.count(p=3)
+        assert g.timings()["work_items"] > 0
