@@ -202,9 +202,10 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts, uint64_t *count);
 
 /*
  * Build the resident plan of the handle for opts' p (0 = automatic), kernel,
- * hash_threshold, chunk and partition -- partition, blocks, tasks, estimates and work
- * items (Sec. 2, Sec. 4.1-4.2, Sec. 5) -- without counting; keep it when it
- * already matches. Later counts with the same options only read the plan.
+ * hash_threshold, chunk and partition (Sec. 2, Sec. 4.1-4.2, Sec. 5) without
+ * counting; keep it when it already matches. Later counts with the same options only
+ * read the plan: totals, per-task and per-graph counts; with task_mask or
+ * per_task_cycles_out given (their contents are not read), counts with those.
  * Other options are ignored. Synchronous.
  * Errors: EINVAL (NULL handle, bad options); ENOMEM; ECUDA.
  */
@@ -372,7 +373,8 @@ bbtc_status bbtc_graph_get_oriented(bbtc_graph_t g, int64_t *rowptr, int32_t *co
 /*
  * The plan bbtc_count builds for p (Sec. 2, Sec. 4.2, Sec. 5), as host copies
  * (any output may be NULL); the handle's current plan when it has this p
- * (whatever its partition), else a new one with the edge-balanced partition: cuts p+1 int32 (c_0 = 0, c_p = n), block_nnz p*p
+ * (whatever its partition), else a new one with the edge-balanced partition, ready
+ * for counts as bbtc_graph_plan leaves it: cuts p+1 int32 (c_0 = 0, c_p = n), block_nnz p*p
  * int64 (|G_ij|, row-major), tasks 3*|T| int32 ((i,j,k) in Alg. 4 order),
  * estimate |T| double (ExecTime in Alg. 4 order), order |T| int32 (task
  * indices, non-increasing estimate, ties in Alg. 4 order).

@@ -295,7 +295,8 @@ def bbtc_count_noalloc(handle: int, p: int, count_dev, per_task_dev=None, stream
 
 
 def bbtc_graph_plan(handle: int, opts: bbtc_opts | None = None) -> None:
-    """Build (or keep) the handle's resident plan for the options, without counting."""
+    """Build (or keep) the handle's resident plan for the options, without counting (with a
+    task_mask, the form that counts of a share use)."""
     _check(load().bbtc_graph_plan(handle, ctypes.byref(opts) if opts is not None else None))
 
 

@@ -642,7 +642,10 @@ bbtc_status bbtc_graph_plan(bbtc_graph_t g, const bbtc_opts *opts_in) {
   const int p = opts.p == 0 ? default_p(g) : opts.p;
   cudaStream_t s = opts.stream ? (cudaStream_t)opts.stream : g->stream;
   if (g->plan.streamed) free_plan(&g->plan, s);
-  BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition));
+  const bool by_task = opts.per_task_cycles_out || opts.task_mask;
+  BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
+                      !by_task));
+  if (by_task) BBTC_TRY(build_tasks(g, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   return BBTC_OK;
 }
@@ -880,8 +883,11 @@ bbtc_status bbtc_graph_get_plan(bbtc_graph_t g, int32_t p, int32_t *cuts, int64_
   const int thr = g->plan.p == p ? g->plan.hash_threshold : 16;
   const int chunk = g->plan.p == p ? g->plan.chunk_req : 0;
   const int part = g->plan.p == p ? g->plan.partition : BBTC_PARTITION_EDGES;
-  BBTC_TRY(build_plan(g, p, kmode, thr, chunk, s, part, !g->plan.streamed));
-  BBTC_TRY(build_tasks(g, s));
+  // a plan that can count, or is streamed, is only inspected; a new one gets the form
+  // that resident counts use
+  const bool kept = g->plan.p == p && (g->plan.streamed || plan_countable(g->plan));
+  BBTC_TRY(build_plan(g, p, kmode, thr, chunk, s, part, !kept));
+  BBTC_TRY(build_order(g, s));
   const Plan &pl = g->plan;
   if (cuts)
     BBTC_CUDA(cudaMemcpyAsync(cuts, pl.cuts, sizeof(int32_t) * (size_t)(p + 1),

@@ -131,9 +131,10 @@ struct CoreDesc {
 
 // Everything bbtc_count builds for one p (Sec. 2 partition, Sec. 4.2 tasks,
 // Sec. 5 estimate and order), cached on the handle until p changes. Resident
-// counts use the cuts, the core and the flat in-edges; the tasks' own part
-// (tasks_ready: blocks, in-edges by part, tasks, estimates, work items) is built
-// when a call needs it (build_tasks).
+// counts use the cuts, the core and the flat in-edges; the tasks with their
+// estimates and order (build_order), and what counting them one by one needs beside
+// them (tasks_ready: blocks, in-edges by part, work items; build_tasks), are built
+// when a call needs them.
 struct Plan {
   int p = 0;
   bool tasks_ready = false;
@@ -249,8 +250,11 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
 // flat in-edges).
 bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold, int chunk,
                        cudaStream_t s, int partition = 0, bool resident = true);
-// The tasks' own part of the handle's plan: blocks (split table, in-edges by
-// part), tasks, estimates, order, descriptors and work items.
+// The tasks of the handle's plan, their estimates and order, from the blocks' sizes.
+// Synchronises s.
+bbtc_status build_order(bbtc_graph *g, cudaStream_t s);
+// What counting the tasks one by one needs beside them: blocks (split table,
+// in-edges by part), descriptors and work items.
 bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s);
 inline bool plan_matches(const Plan &pl, int p, int kernel_mode, int hash_threshold, int chunk,
                          int partition = 0) {

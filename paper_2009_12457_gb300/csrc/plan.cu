@@ -3,13 +3,15 @@
 //      edges (Sec. 2 vertex partition V^p; Sec. 4.1 symmetric partition),
 //      or the probe-based partition of partition.cu
 //   the dense core and the flat in-edges that resident counts walk (core.cu,
-//      flat.cu); the rest only for the calls that need the tasks one by one:
+//      flat.cu); the rest only for the calls that ask for the tasks (build_order)
+//      or need them one by one (build_tasks):
 //   a6 blocks G_ij = {(u,v) : u in V_i, v in V_j} (Sec. 2), materialised as
 //      the in-edges of each v grouped by the part of their source, so that a
 //      block's edges are one contiguous, destination-ordered range
 //   a7 task composition: all (i,j,k), i <= j <= k (Sec. 4.2, Alg. 4)
-//   a8 ExecTime estimate and non-increasing order (Sec. 5), split into work
-//      items of at most `chunk` in-edges each
+//   a8 ExecTime estimate and non-increasing order (Sec. 5), for which the blocks'
+//      sizes are enough; the tasks split into work items of at most `chunk`
+//      in-edges each
 #include <new>
 
 #include "graph.cuh"
@@ -109,27 +111,7 @@ __global__ void k_narrow(const uint64_t *__restrict__ in, int64_t count, unsigne
     out[i] = (unsigned)in[i];
 }
 
-// Step 2 (after an exclusive scan of the counts): the block offsets of part a,
-// boff[a*(p+1)+j] = first in-edge of part a whose destination is >= c_j.
-__global__ void k_inedge_offsets(const int64_t *__restrict__ rowptr,
-                                 const int32_t *__restrict__ cuts, int a, int p,
-                                 const unsigned long long *__restrict__ scan, int64_t bins,
-                                 int64_t *__restrict__ boff) {
-  const int j = threadIdx.x;
-  if (j > p) return;
-  const int32_t c_a = cuts[a];
-  const int64_t e0 = rowptr[c_a], e1 = rowptr[cuts[a + 1]];
-  int64_t off;
-  if (j <= a) {
-    off = e0;
-  } else {
-    const int64_t idx = (int64_t)cuts[j] - c_a;  // scan has bins = n - c_a entries
-    off = idx < bins ? e0 + (int64_t)scan[idx] : e1;
-  }
-  boff[a * (p + 1) + j] = off;
-}
-
-// Step 3: scatter each edge of part a whose destination lies in the slab
+// Step 2 (after an exclusive scan of the counts): scatter each edge of part a whose destination lies in the slab
 // [v_lo, v_hi) to its destination's run, as one 16-byte record (source u,
 // destination v, CSR position e, end f of u's run in v's block, from the
 // split table row of u) so that each random write touches one sector; within
@@ -473,7 +455,8 @@ __global__ void k_bcsr_rowptr(const uint64_t *__restrict__ pos, int64_t total,
     rp[i] = (uint32_t)pos[i];
 }
 
-// nnz[a * p + b] += entries of row u of part a in part b (one thread per row).
+// nnz[a * p + b] += entries of row u of part a in part b (one thread per row). The
+// rows of a warp mostly lie in one part, and then add once for each block.
 __global__ void k_block_sizes(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                               int64_t n, const int32_t *__restrict__ cuts_g, int p,
                               unsigned long long *__restrict__ nnz) {
@@ -482,21 +465,49 @@ __global__ void k_block_sizes(const int64_t *__restrict__ rowptr, const int32_t 
   for (int i = threadIdx.x; i <= p; i += blockDim.x) cuts[i] = cuts_g[i];
   for (int i = threadIdx.x; i < p * p; i += blockDim.x) block_cnt[i] = 0;
   __syncthreads();
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r1 = rowptr[u + 1];
-    int64_t lo = rowptr[u];
-    if (lo == r1) continue;
-    const int a = part_of_dev(cuts, p, (int32_t)u);
-    for (int b = a; b < p && lo < r1; ++b) {
-      const int64_t hi = b + 1 < p ? lower_bound_dev<int32_t, int64_t>(colidx, lo, r1, cuts[b + 1]) : r1;
-      if (hi > lo) atomicAdd(&block_cnt[a * p + b], (unsigned long long)(hi - lo));
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
+    const int64_t u = base + threadIdx.x;
+    int64_t lo = 0, r1 = 0;
+    int a = p - 1;  // (a position past n has an empty row)
+    if (u < n) {
+      lo = rowptr[u];
+      r1 = rowptr[u + 1];
+      a = part_of_dev(cuts, p, (int32_t)u);
+    }
+    const int first = __reduce_min_sync(0xffffffffu, a);
+    const bool together = first == __reduce_max_sync(0xffffffffu, a);
+    for (int b = first; b < p && __any_sync(0xffffffffu, lo < r1); ++b) {
+      int64_t hi = lo;
+      if (lo < r1 && b >= a)
+        hi = b + 1 < p ? lower_bound_dev<int32_t, int64_t>(colidx, lo, r1, cuts[b + 1]) : r1;
+      const unsigned long long c = (unsigned long long)(hi - lo);
+      if (together) {
+        const unsigned long long sum = warp_sum(c);
+        if (lane_id() == 0 && sum) atomicAdd(&block_cnt[a * p + b], sum);
+      } else if (c) {
+        atomicAdd(&block_cnt[a * p + b], c);
+      }
       lo = hi;
     }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < p * p; i += blockDim.x)
     if (block_cnt[i]) atomicAdd(&nnz[i], block_cnt[i]);
+}
+
+// boff[a*(p+1)+j] = first in-edge of part a whose destination is >= c_j
+__global__ void k_block_offsets(const int64_t *__restrict__ rowptr,
+                                const int32_t *__restrict__ cuts, int p,
+                                const unsigned long long *__restrict__ nnz,
+                                int64_t *__restrict__ boff) {
+  const int a = threadIdx.x;
+  if (a >= p) return;
+  int64_t off = rowptr[cuts[a]];
+  for (int j = 0; j <= p; ++j) {
+    boff[a * (p + 1) + j] = off;
+    if (j >= a && j < p) off += (int64_t)nnz[a * p + j];
+  }
 }
 
 __device__ __forceinline__ int64_t block_nnz(const int64_t *boff, int p, int i, int j) {
@@ -700,17 +711,25 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   return BBTC_OK;
 }
 
+// |G_ab| of every block into d (device, p * p)
+static bbtc_status block_sizes_dev(const bbtc_graph *g, const Plan &pl, unsigned long long *d,
+                                   cudaStream_t s) {
+  const size_t bytes = sizeof(uint64_t) * (size_t)pl.p * pl.p;
+  BBTC_CUDA(cudaMemsetAsync(d, 0, bytes, s));
+  if (g->n > 0) {
+    k_block_sizes<<<grid_for(g->n, 256, 4), 256, bytes, s>>>(g->rowptr, g->colidx, g->n, pl.cuts,
+                                                            pl.p, d);
+    BBTC_LAUNCH_CHECK();
+  }
+  return BBTC_OK;
+}
+
 bbtc_status block_sizes(const bbtc_graph *g, const Plan &pl, int64_t *nnz, cudaStream_t s) {
   const int p = pl.p;
   Scratch scratch(s);
   unsigned long long *d = nullptr;
   BBTC_TRY(scratch.get(&d, (int64_t)p * p));
-  BBTC_CUDA(cudaMemsetAsync(d, 0, sizeof(uint64_t) * (size_t)p * p, s));
-  if (g->n > 0) {
-    k_block_sizes<<<grid_for(g->n, 256, 4), 256, sizeof(uint64_t) * (size_t)p * p, s>>>(
-        g->rowptr, g->colidx, g->n, pl.cuts, p, d);
-    BBTC_LAUNCH_CHECK();
-  }
+  BBTC_TRY(block_sizes_dev(g, pl, d, s));
   BBTC_CUDA(cudaMemcpyAsync(nnz, d, sizeof(uint64_t) * (size_t)p * p, cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   return BBTC_OK;
@@ -726,11 +745,59 @@ bbtc_status build_full(bbtc_graph *g, cudaStream_t s) {
   return st;
 }
 
+bbtc_status build_order(bbtc_graph *g, cudaStream_t s) {
+  Plan &pl = g->plan;
+  if (pl.order) return BBTC_OK;
+  const int p = pl.p;
+  const int64_t nt = pl.ntasks;
+  Scratch scratch(s);
+  unsigned long long *nnz = nullptr;
+  uint64_t *okeys = nullptr, *okeys_alt = nullptr;
+  uint32_t *ovals = nullptr, *ovals_alt = nullptr;
+  int32_t *serr = nullptr;
+  bbtc_status st = BBTC_OK;
+  PLAN_TRY(scratch.get(&nnz, (int64_t)p * p));
+  PLAN_TRY(scratch.get(&okeys, nt));
+  PLAN_TRY(scratch.get(&okeys_alt, nt));
+  PLAN_TRY(scratch.get(&ovals, nt));
+  PLAN_TRY(scratch.get(&ovals_alt, nt));
+  PLAN_TRY(scratch.get(&serr, 1));
+  PLAN_TRY(dalloc_n(&pl.boff, (int64_t)p * (p + 1), s));
+  PLAN_TRY(dalloc_n(&pl.tasks, 3 * nt, s));
+  PLAN_TRY(dalloc_n(&pl.est, nt, s));
+  PLAN_TRY(dalloc_n(&pl.order, nt, s));
+  PLAN_TRY(block_sizes_dev(g, pl, nnz, s));
+  k_block_offsets<<<1, MAXP, 0, s>>>(g->rowptr, pl.cuts, p, nnz, pl.boff);
+  PLAN_TRY(launch_status("build_plan"));
+  k_tasks<<<(p * p * p + 127) / 128, 128, 0, s>>>(pl.boff, pl.cuts, p, pl.tasks, pl.est, okeys,
+                                                  ovals);
+  PLAN_TRY(launch_status("build_plan"));
+  if (cudaMemsetAsync(serr, 0, sizeof(int32_t), s) != cudaSuccess) {
+    set_error("build_plan: cudaMemsetAsync failed");
+    PLAN_TRY(BBTC_ECUDA);
+  }
+  bool in_alt = false;
+  PLAN_TRY(radix_sort(okeys, okeys_alt, ovals, ovals_alt, nt, 0, 64, s, serr, &in_alt));
+  k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, serr,
+                                                      pl.order);
+  PLAN_TRY(launch_status("build_plan"));
+  int32_t sort_err = 0;
+  if (cudaMemcpyAsync(&sort_err, serr, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess) {
+    set_error("build_plan: reading the sort's status failed");
+    PLAN_TRY(BBTC_ECUDA);
+  }
+  if (sort_err) PLAN_TRY(sort_failed("build_plan"));
+  pl.bytes += (uint64_t)p * (p + 1) * 8 + (uint64_t)nt * 24;
+  return BBTC_OK;
+}
+
 bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
   if (g->plan.tasks_ready) return BBTC_OK;
+  BBTC_TRY(build_order(g, s));
   Plan &pl = g->plan;
   const int p = pl.p;
-  const int64_t n = g->n, m = g->m;
+  const int64_t n = g->n, m = g->m, nt = pl.ntasks;
   const int kernel_mode = pl.kernel_mode, hash_threshold = pl.hash_threshold;
   Scratch scratch(s);
   bbtc_status st = BBTC_OK;
@@ -760,10 +827,8 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
     PLAN_TRY(launch_status("build_plan"));
   }
 
-  // in-edges grouped by (part(u), v), and the block offsets: one counting
-  // sort on the destination per part
+  // in-edges grouped by (part(u), v): one counting sort on the destination per part
   PLAN_TRY(dalloc_n(&pl.ie, m, s));
-  PLAN_TRY(dalloc_n(&pl.boff, (int64_t)p * (p + 1), s));
   {
     unsigned *hist = nullptr;  // counts, then the scatter's cursors
     uint64_t *scan = nullptr;
@@ -800,10 +865,6 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
         k_narrow<<<grid_for(bins, 256, 16), 256, 0, s>>>(scan, bins, hist);
         PLAN_TRY(launch_status("build_plan"));
       }
-      k_inedge_offsets<<<1, MAXP + 1, 0, s>>>(g->rowptr, pl.cuts, a, p,
-                                               reinterpret_cast<const unsigned long long *>(scan),
-                                               bins, pl.boff);
-      PLAN_TRY(launch_status("build_plan"));
       // large parts: partition into destination buckets, then place (the
       // temporary array takes 16 bytes per edge of the part); else, or when it
       // does not fit, one direct scatter
@@ -845,32 +906,6 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
       }
     }
   }
-
-  // a7 + a8: tasks, estimates, order
-  const int64_t nt = pl.ntasks;
-  PLAN_TRY(dalloc_n(&pl.tasks, 3 * nt, s));
-  PLAN_TRY(dalloc_n(&pl.est, nt, s));
-  PLAN_TRY(dalloc_n(&pl.order, nt, s));
-  uint64_t *okeys = nullptr, *okeys_alt = nullptr;
-  uint32_t *ovals = nullptr, *ovals_alt = nullptr;
-  PLAN_TRY(scratch.get(&okeys, nt));
-  PLAN_TRY(scratch.get(&okeys_alt, nt));
-  PLAN_TRY(scratch.get(&ovals, nt));
-  PLAN_TRY(scratch.get(&ovals_alt, nt));
-  bool in_alt = false;
-  k_tasks<<<(p * p * p + 127) / 128, 128, 0, s>>>(pl.boff, pl.cuts, p, pl.tasks, pl.est, okeys,
-                                                  ovals);
-  PLAN_TRY(launch_status("build_plan"));
-  int32_t *serr = nullptr;
-  PLAN_TRY(scratch.get(&serr, 1));
-  if (cudaMemsetAsync(serr, 0, sizeof(int32_t), s) != cudaSuccess) {
-    set_error("build_plan: cudaMemsetAsync failed");
-    free_plan(&pl, s);
-    return BBTC_ECUDA;
-  }
-  PLAN_TRY(radix_sort(okeys, okeys_alt, ovals, ovals_alt, nt, 0, 64, s, serr, &in_alt));
-  k_order_finish<<<grid_for(nt, 256, 4), 256, 0, s>>>(in_alt ? ovals_alt : ovals, nt, serr, pl.order);
-  PLAN_TRY(launch_status("build_plan"));
 
   // task descriptors: every block of the resident BCSR
   {
@@ -926,17 +961,13 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
   PLAN_TRY(launch_status("build_plan"));
   PLAN_TRY(exclusive_scan_u64(first, first, nt + 1, s));
   uint64_t nitems = 0;
-  int32_t sort_err = 0;
   if (cudaMemcpyAsync(&nitems, first + nt, sizeof(uint64_t), cudaMemcpyDeviceToHost, s) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(&sort_err, serr, sizeof(int32_t), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("build_plan: reading the work-item count failed");
     free_plan(&pl, s);
     return BBTC_ECUDA;
   }
-  if (sort_err) PLAN_TRY(sort_failed("build_plan"));
   pl.nitems = (int64_t)nitems;
   PLAN_TRY(dalloc_n(&pl.items, pl.nitems, s));
   if (nitems > 0) {
@@ -948,7 +979,7 @@ bbtc_status build_tasks(bbtc_graph *g, cudaStream_t s) {
   PLAN_TRY(configure_count_kernels(&pl));
 #undef PLAN_TRY
   pl.bytes += (uint64_t)m * sizeof(InEdge) + (uint64_t)pl.h_spl_off[p] * 4 +
-              (uint64_t)nt * (24 + sizeof(TaskDesc)) + (uint64_t)pl.nitems * sizeof(WorkItem);
+              (uint64_t)nt * sizeof(TaskDesc) + (uint64_t)pl.nitems * sizeof(WorkItem);
   pl.tasks_ready = true;
   return BBTC_OK;
 }

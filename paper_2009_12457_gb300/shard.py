@@ -45,7 +45,9 @@ def shard_count(handle: int, p: int, rank: int, world: int, dist=None, device=No
 
     from . import bbtc_count, bbtc_graph_get_plan, bbtc_graph_plan, make_opts
 
-    bbtc_graph_plan(handle, make_opts(p=p, **count_opts))  # the plan the count will use
+    # the plan that the count will use, which takes the tasks one by one
+    every = np.ones(p * (p + 1) * (p + 2) // 6, dtype=np.uint8)
+    bbtc_graph_plan(handle, make_opts(p=p, task_mask=every, **count_opts))
     est = bbtc_graph_get_plan(handle, p)["exec_time"]
     mask = lpt_masks(est, world)[rank]
     local = bbtc_count(handle, make_opts(p=p, task_mask=mask, **count_opts))

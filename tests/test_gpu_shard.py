@@ -55,3 +55,32 @@ def test_async_refuses_a_task_mask():
         with pytest.raises(bb.BbtcError):
             bb.bbtc_count_async(g.handle, bb.make_opts(p=2, task_mask=np.ones(4, np.uint8)),
                                 total)
+
+
+def test_memory_of_an_inspected_plan_and_of_a_share():
+    n, rp, ci = graphgen.rmat(16, 32, 5)
+    p = 3
+    ref = oracle.bbtc(n, rp, ci, p=p)
+    with bb.Graph(n, rp, ci, symmetric=True) as g:
+        m, bare = g.info()["m"], g.info()["device_bytes"]
+        plan = g.plan(p)
+        assert np.array_equal(plan["exec_time"], ref["exec_time"])
+        fresh = g.info()["device_bytes"] - bare
+        assert fresh < 14 * m  # 8 bytes an in-edge and the core: not the tasks' records too
+        total = torch.zeros(1, dtype=torch.int64, device="cuda")
+        bb.bbtc_count_async(g.handle, bb.make_opts(p=p), total)  # it counts with what it has
+        torch.cuda.synchronize()
+        assert int(total.item()) == ref["total"]
+    with bb.Graph(n, rp, ci, symmetric=True) as g:  # a new p after a streamed plan: the same form
+        g.count(p=2, device_budget_bytes=1 << 30)
+        g.plan(p)
+        assert g.info()["device_bytes"] - bare == fresh
+        bb.bbtc_count_async(g.handle, bb.make_opts(p=p), total)
+        torch.cuda.synchronize()
+        assert int(total.item()) == ref["total"]
+    with bb.Graph(n, rp, ci, symmetric=True) as g:  # a share: the tasks' records alone
+        assert shard.shard_count(g.handle, p, 0, 1) == ref["total"]
+        assert g.info()["device_bytes"] - bare < 20 * m
+        bb.bbtc_count_async(g.handle, bb.make_opts(p=p), total)
+        torch.cuda.synchronize()
+        assert int(total.item()) == ref["total"]
