@@ -206,7 +206,9 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts, uint64_t *count);
  * counting; keep it when it already matches. Later counts with the same options only
  * read the plan: totals, per-task and per-graph counts; with task_mask or
  * per_task_cycles_out given (their contents are not read), counts with those.
- * Other options are ignored. Synchronous.
+ * Other options are ignored. A plan keeps what it has built for other options until
+ * it is replaced or device memory runs out: a call that then finds no room frees the
+ * plan and builds only what it needs itself. Synchronous.
  * Errors: EINVAL (NULL handle, bad options); ENOMEM; ECUDA.
  */
 bbtc_status bbtc_graph_plan(bbtc_graph_t g, const bbtc_opts *opts);

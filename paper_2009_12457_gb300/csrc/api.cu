@@ -427,6 +427,130 @@ bbtc_status create_common(int64_t n, const int64_t *rowptr, const int32_t *colid
   return BBTC_OK;
 }
 
+// bbtc_count after the checks of its arguments. lean: a count with per-vertex or
+// per-edge outputs builds the in-edges of all lists alone and counts everything with
+// them. *refused: the budget cannot hold what it has to.
+bbtc_status count_once(bbtc_graph_t g, const bbtc_opts &opts, bool lean, bool *refused,
+                       uint64_t *count) {
+  const bool budgeted = opts.device_budget_bytes != 0;
+  const int p = opts.p == 0 ? default_p(g, budgeted) : opts.p;
+  cudaStream_t s = opts.stream ? (cudaStream_t)opts.stream : g->stream;
+  if (budgeted && opts.per_edge_out) {
+    set_error("bbtc_count: per_edge_out needs a resident count (device_budget_bytes = 0)");
+    return BBTC_EINVAL;
+  }
+  // a resident count needs the block arrays on the device: a plan that was
+  // streamed (its arrays now in host memory) is rebuilt
+  if (!budgeted && g->plan.streamed) free_plan(&g->plan, s);
+  // counted task by task: a share of the tasks, and their cycles
+  const bool by_task = opts.per_task_cycles_out || opts.task_mask;
+  const bool detail = !budgeted && !by_task && (opts.per_vertex_out || opts.per_edge_out);
+  const bool tasks = opts.per_task_out != nullptr, per_graph = opts.per_graph_out != nullptr;
+  // (a detail count alone needs neither the core nor the in-edges that it leaves)
+  const bool resident = !budgeted && !by_task && (!detail || ((tasks || per_graph) && !lean));
+  const Plan &old = g->plan;
+  const bool rebuild =
+      !plan_matches(old, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition) ||
+      (by_task && !old.tasks_ready) || (budgeted && !by_task && !old.h_rec) || (resident && !old.flat.ready) ||
+      (detail && !old.full.ready && !(old.flat.ready && !old.core.bits));
+  if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[2], s));
+  BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
+                      resident));
+  if (by_task) BBTC_TRY(build_tasks(g, s));
+  if (detail) BBTC_TRY(build_full(g, s));
+  if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[3], s));
+  g->plan_timed = rebuild;
+  const Plan &pl = g->plan;
+  Scratch scratch(s);
+  unsigned long long *vertex_count = nullptr;
+  if (opts.per_vertex_out) BBTC_TRY(scratch.get(&vertex_count, g->n));
+  unsigned long long *task_cycles = nullptr;
+  if (opts.per_task_cycles_out) {
+    BBTC_TRY(scratch.get(&task_cycles, pl.ntasks));
+    BBTC_CUDA(cudaMemsetAsync(task_cycles, 0, sizeof(uint64_t) * (size_t)pl.ntasks, s));
+  }
+  unsigned *edge_sup = nullptr;
+  if (opts.per_edge_out) {
+    BBTC_TRY(scratch.get(&edge_sup, g->m > 0 ? g->m : 1));
+    BBTC_CUDA(cudaMemsetAsync(edge_sup, 0, sizeof(unsigned) * (size_t)(g->m > 0 ? g->m : 1), s));
+  }
+  uint8_t *task_mask = nullptr;  // this caller's share of the tasks, on the device
+  if (opts.task_mask) {
+    BBTC_TRY(scratch.get(&task_mask, pl.ntasks));
+    BBTC_CUDA(cudaMemcpyAsync(task_mask, opts.task_mask, (size_t)pl.ntasks,
+                              cudaMemcpyHostToDevice, s));
+  }
+  if (budgeted) {
+    StreamStats st;
+    bbtc_status run = BBTC_OK;
+    if (by_task)
+      run = run_count_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, per_graph,
+                               opts.timeout_ms, s, &st, task_cycles, task_mask);
+    else
+      run = run_flat_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, tasks,
+                              per_graph, opts.timeout_ms, s, &st);
+    *refused = st.refused;
+    BBTC_TRY(run);
+    g->stream_stats.rounds = st.rounds;
+    g->stream_stats.h2d_bytes = st.h2d_bytes;
+    g->stream_stats.copy_ms = st.copy_ms;
+    g->stream_stats.block_bytes = st.block_bytes;
+    g->stream_stats.device_peak = st.device_peak;
+    g->stream_stats.mode = st.mode;
+    g->stream_stats_total_ms = st.total_ms;
+    g->counted_items = st.items;
+  } else {
+    if (by_task)
+      BBTC_TRY(run_count(g, pl, vertex_count, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5],
+                         task_cycles, edge_sup, task_mask));
+    else if (detail)
+      BBTC_TRY(run_detail(g, pl, tasks, per_graph, vertex_count, edge_sup, opts.timeout_ms, s,
+                          g->ev[4], g->ev[5]));
+    else
+      BBTC_TRY(run_flat(g, pl, tasks, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5]));
+    g->stream_stats_total_ms = -1.0;
+    g->counted_items = by_task ? pl.nitems
+                               : (detail ? detail_flat(pl).nitems : 0) +
+                                     (detail && !tasks && !per_graph ? 0
+                                      : pl.flat.ready ? pl.core.nitems + pl.flat.nitems
+                                                      : pl.full.nitems);
+  }
+  unsigned long long head[SCR_TASKS] = {0};
+  BBTC_CUDA(cudaMemcpyAsync(head, pl.scratch, sizeof(head), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaStreamSynchronize(s));
+  if ((int32_t)head[SCR_STATUS] != 0) return count_status_error("bbtc_count", (int32_t)head[SCR_STATUS], opts.timeout_ms);
+  if (!opts.per_task_out && !per_graph && !task_cycles && !edge_sup && !opts.per_vertex_out) {
+    *count = head[SCR_TOTAL];
+    return BBTC_OK;
+  }
+  const bool out_dev = (opts.flags & BBTC_OUT_DEVICE) != 0;
+  const cudaMemcpyKind kind = out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+  if (opts.per_task_out)
+    BBTC_CUDA(cudaMemcpyAsync(opts.per_task_out, pl.scratch + SCR_TASKS,
+                              sizeof(uint64_t) * (size_t)pl.ntasks, kind, s));
+  if (per_graph)
+    BBTC_CUDA(cudaMemcpyAsync(opts.per_graph_out, pl.scratch + SCR_TASKS + pl.ntasks,
+                              sizeof(uint64_t) * (size_t)g->ng, kind, s));
+  if (task_cycles)
+    BBTC_CUDA(cudaMemcpyAsync(opts.per_task_cycles_out, task_cycles,
+                              sizeof(uint64_t) * (size_t)pl.ntasks, kind, s));
+  if (edge_sup && g->m > 0)  // resident plans index the oriented CSR directly
+    BBTC_CUDA(cudaMemcpyAsync(opts.per_edge_out, edge_sup, sizeof(uint32_t) * (size_t)g->m, kind,
+                              s));
+  if (opts.per_vertex_out && g->n > 0) {
+    unsigned long long *by_id = nullptr;
+    BBTC_TRY(scratch.get(&by_id, g->n));
+    k_scatter_by_perm<<<grid_for(g->n, 256, 16), 256, 0, s>>>(vertex_count, g->perm, g->n,
+                                                              by_id);
+    BBTC_LAUNCH_CHECK();
+    BBTC_CUDA(cudaMemcpyAsync(opts.per_vertex_out, by_id, sizeof(uint64_t) * (size_t)g->n, kind,
+                              s));
+  }
+  BBTC_CUDA(cudaStreamSynchronize(s));
+  *count = head[SCR_TOTAL];
+  return BBTC_OK;
+}
+
 }  // namespace
 }  // namespace bbtc
 
@@ -479,118 +603,17 @@ bbtc_status bbtc_count(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *count
   bbtc_opts opts;
   BBTC_TRY(check_opts(opts_in, &opts));
   DeviceGuard dg(g->device);
-  const bool budgeted = opts.device_budget_bytes != 0;
-  const int p = opts.p == 0 ? default_p(g, budgeted) : opts.p;
-  cudaStream_t s = opts.stream ? (cudaStream_t)opts.stream : g->stream;
-  if (budgeted && opts.per_edge_out) {
-    set_error("bbtc_count: per_edge_out needs a resident count (device_budget_bytes = 0)");
-    return BBTC_EINVAL;
-  }
-  // a resident count needs the block arrays on the device: a plan that was
-  // streamed (its arrays now in host memory) is rebuilt
-  if (!budgeted && g->plan.streamed) free_plan(&g->plan, s);
-  // counted task by task: a share of the tasks, and their cycles
-  const bool by_task = opts.per_task_cycles_out || opts.task_mask;
-  const bool detail = !budgeted && !by_task && (opts.per_vertex_out || opts.per_edge_out);
-  const bool tasks = opts.per_task_out != nullptr, per_graph = opts.per_graph_out != nullptr;
-  // (a detail count alone needs neither the core nor the in-edges that it leaves)
-  const bool resident = !budgeted && !by_task && (!detail || tasks || per_graph);
-  const Plan &old = g->plan;
-  const bool rebuild =
-      !plan_matches(old, p, opts.kernel, opts.hash_threshold, opts.chunk, opts.partition) ||
-      (by_task && !old.tasks_ready) || (budgeted && !by_task && !old.h_rec) || (resident && !old.flat.ready) ||
-      (detail && !old.full.ready && !(old.flat.ready && !old.core.bits));
-  if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[2], s));
-  BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
-                      resident));
-  if (by_task) BBTC_TRY(build_tasks(g, s));
-  if (detail) BBTC_TRY(build_full(g, s));
-  if (rebuild) BBTC_CUDA(cudaEventRecord(g->ev[3], s));
-  g->plan_timed = rebuild;
-  const Plan &pl = g->plan;
-  Scratch scratch(s);
-  unsigned long long *vertex_count = nullptr;
-  if (opts.per_vertex_out) BBTC_TRY(scratch.get(&vertex_count, g->n));
-  unsigned long long *task_cycles = nullptr;
-  if (opts.per_task_cycles_out) {
-    BBTC_TRY(scratch.get(&task_cycles, pl.ntasks));
-    BBTC_CUDA(cudaMemsetAsync(task_cycles, 0, sizeof(uint64_t) * (size_t)pl.ntasks, s));
-  }
-  unsigned *edge_sup = nullptr;
-  if (opts.per_edge_out) {
-    BBTC_TRY(scratch.get(&edge_sup, g->m > 0 ? g->m : 1));
-    BBTC_CUDA(cudaMemsetAsync(edge_sup, 0, sizeof(unsigned) * (size_t)(g->m > 0 ? g->m : 1), s));
-  }
-  uint8_t *task_mask = nullptr;  // this caller's share of the tasks, on the device
-  if (opts.task_mask) {
-    BBTC_TRY(scratch.get(&task_mask, pl.ntasks));
-    BBTC_CUDA(cudaMemcpyAsync(task_mask, opts.task_mask, (size_t)pl.ntasks,
-                              cudaMemcpyHostToDevice, s));
-  }
-  if (budgeted) {
-    StreamStats st;
-    if (by_task)
-      BBTC_TRY(run_count_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, per_graph,
-                                  opts.timeout_ms, s, &st, task_cycles, task_mask));
-    else
-      BBTC_TRY(run_flat_streamed(g, g->plan, opts.device_budget_bytes, vertex_count, tasks,
-                                 per_graph, opts.timeout_ms, s, &st));
-    g->stream_stats.rounds = st.rounds;
-    g->stream_stats.h2d_bytes = st.h2d_bytes;
-    g->stream_stats.copy_ms = st.copy_ms;
-    g->stream_stats.block_bytes = st.block_bytes;
-    g->stream_stats.device_peak = st.device_peak;
-    g->stream_stats.mode = st.mode;
-    g->stream_stats_total_ms = st.total_ms;
-    g->counted_items = st.items;
-  } else {
-    if (by_task)
-      BBTC_TRY(run_count(g, pl, vertex_count, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5],
-                         task_cycles, edge_sup, task_mask));
-    else if (detail)
-      BBTC_TRY(run_detail(g, pl, tasks, per_graph, vertex_count, edge_sup, opts.timeout_ms, s,
-                          g->ev[4], g->ev[5]));
-    else
-      BBTC_TRY(run_flat(g, pl, tasks, per_graph, opts.timeout_ms, s, g->ev[4], g->ev[5]));
-    g->stream_stats_total_ms = -1.0;
-    g->counted_items = by_task ? pl.nitems
-                               : (resident ? pl.core.nitems + pl.flat.nitems : 0) +
-                                     (detail ? detail_flat(pl).nitems : 0);
-  }
-  unsigned long long head[SCR_TASKS] = {0};
-  BBTC_CUDA(cudaMemcpyAsync(head, pl.scratch, sizeof(head), cudaMemcpyDeviceToHost, s));
-  BBTC_CUDA(cudaStreamSynchronize(s));
-  if ((int32_t)head[SCR_STATUS] != 0) return count_status_error("bbtc_count", (int32_t)head[SCR_STATUS], opts.timeout_ms);
-  if (!opts.per_task_out && !per_graph && !task_cycles && !edge_sup && !opts.per_vertex_out) {
-    *count = head[SCR_TOTAL];
-    return BBTC_OK;
-  }
-  const bool out_dev = (opts.flags & BBTC_OUT_DEVICE) != 0;
-  const cudaMemcpyKind kind = out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  if (opts.per_task_out)
-    BBTC_CUDA(cudaMemcpyAsync(opts.per_task_out, pl.scratch + SCR_TASKS,
-                              sizeof(uint64_t) * (size_t)pl.ntasks, kind, s));
-  if (per_graph)
-    BBTC_CUDA(cudaMemcpyAsync(opts.per_graph_out, pl.scratch + SCR_TASKS + pl.ntasks,
-                              sizeof(uint64_t) * (size_t)g->ng, kind, s));
-  if (task_cycles)
-    BBTC_CUDA(cudaMemcpyAsync(opts.per_task_cycles_out, task_cycles,
-                              sizeof(uint64_t) * (size_t)pl.ntasks, kind, s));
-  if (edge_sup && g->m > 0)  // resident plans index the oriented CSR directly
-    BBTC_CUDA(cudaMemcpyAsync(opts.per_edge_out, edge_sup, sizeof(uint32_t) * (size_t)g->m, kind,
-                              s));
-  if (opts.per_vertex_out && g->n > 0) {
-    unsigned long long *by_id = nullptr;
-    BBTC_TRY(scratch.get(&by_id, g->n));
-    k_scatter_by_perm<<<grid_for(g->n, 256, 16), 256, 0, s>>>(vertex_count, g->perm, g->n,
-                                                              by_id);
-    BBTC_LAUNCH_CHECK();
-    BBTC_CUDA(cudaMemcpyAsync(opts.per_vertex_out, by_id, sizeof(uint64_t) * (size_t)g->n, kind,
-                              s));
-  }
-  BBTC_CUDA(cudaStreamSynchronize(s));
-  *count = head[SCR_TOTAL];
-  return BBTC_OK;
+  // What a plan holds from earlier calls (up to three forms of the in-edges) must not
+  // keep a call from running: out of memory, it starts over with a plan of its own
+  // need alone.
+  const bool more = g->plan.p != 0 || ((opts.per_vertex_out || opts.per_edge_out) &&
+                                       (opts.per_task_out || opts.per_graph_out));
+  bool refused = false;
+  const bbtc_status st = count_once(g, opts, false, &refused, count);
+  if (st != BBTC_ENOMEM || refused || !more) return st;
+  clear_error();
+  free_plan(&g->plan, opts.stream ? (cudaStream_t)opts.stream : g->stream);
+  return count_once(g, opts, true, &refused, count);
 }
 
 bbtc_status bbtc_count_async(bbtc_graph_t g, const bbtc_opts *opts_in, uint64_t *total_dev) {
@@ -645,7 +668,18 @@ bbtc_status bbtc_graph_plan(bbtc_graph_t g, const bbtc_opts *opts_in) {
   const bool by_task = opts.per_task_cycles_out || opts.task_mask;
   BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
                       !by_task));
-  if (by_task) BBTC_TRY(build_tasks(g, s));
+  if (by_task && !g->plan.tasks_ready) {
+    const bool held = plan_countable(g->plan);
+    bbtc_status st = build_tasks(g, s);
+    if (st == BBTC_ENOMEM && held) {  // without the forms that were there
+      clear_error();
+      free_plan(&g->plan, s);
+      BBTC_TRY(build_plan(g, p, opts.kernel, opts.hash_threshold, opts.chunk, s, opts.partition,
+                          false));
+      st = build_tasks(g, s);
+    }
+    BBTC_TRY(st);
+  }
   BBTC_CUDA(cudaStreamSynchronize(s));
   return BBTC_OK;
 }

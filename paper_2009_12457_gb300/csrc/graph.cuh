@@ -369,6 +369,7 @@ struct StreamStats {
   uint64_t device_peak = 0;  // pool high-water mark during the count
   int32_t mode = 0;          // 1: block CSRs resident, in-edge blocks once; 2: general
   int64_t items = 0;         // work items drained
+  bool refused = false;      // the budget cannot hold what it has to
 };
 bbtc_status run_count_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
                                unsigned long long *vertex_count, bool per_graph,

@@ -662,8 +662,12 @@ bbtc_status build_plan(bbtc_graph *g, int p, int kernel_mode, int hash_threshold
   if (plan_matches(g->plan, p, kernel_mode, hash_threshold, chunk_req, partition)) {
     if (!resident || g->plan.flat.ready) return BBTC_OK;
     const bbtc_status st = add_resident(g, g->plan, s);
-    if (st != BBTC_OK) free_plan(&g->plan, s);
-    return st;
+    if (st == BBTC_OK) return BBTC_OK;
+    if (st != BBTC_ENOMEM) {
+      free_plan(&g->plan, s);
+      return st;
+    }
+    clear_error();  // once more, without the forms that the plan holds
   }
   free_plan(&g->plan, s);
   Plan pl;

@@ -476,6 +476,7 @@ bbtc_status run_count_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
         set_error("streamed count: the blocks of task (%d,%d,%d) do not fit in a %llu-byte "
                   "device budget", ti[t], tj[t], tk[t], (unsigned long long)budget);
         st = BBTC_ENOMEM;
+        stats->refused = true;
         break;
       }
       for (const auto &f : fresh) placed[f.first] = f.second;
@@ -651,6 +652,7 @@ bbtc_status run_flat_streamed(bbtc_graph *g, Plan &pl, uint64_t budget,
     set_error("streamed count: the blocks of task (%d,%d,%d) do not fit in a %llu-byte "
               "device budget", pl.need_task[0], pl.need_task[1], pl.need_task[2],
               (unsigned long long)budget);
+    stats->refused = true;
     return BBTC_ENOMEM;
   }
   // (any task's blocks take more than 512 bytes, so each half of the pool holds a record)
