@@ -55,10 +55,12 @@ static_assert((BK_CAP & (BK_CAP - 1)) == 0, "the table holds any bucket twice ov
 // a1 + a2: one CTA per bucket inserts its keys into a table of at least twice their
 // number; the first of equal keys goes to ukeys and counts towards its endpoints'
 // degrees, lanes that add to one vertex (a hub's edges) adding once. *nunique gets
-// HASH_FAILED when a bucket has overflowed; the results are then void.
+// HASH_FAILED when a bucket has overflowed, or when there are more than `room` keys
+// (input that lists edges under one endpoint only though said to be symmetric); the
+// results are then void.
 __global__ void __launch_bounds__(BK_NT) k_bucket_unique(const uint64_t *__restrict__ keys,
                                                          const unsigned *__restrict__ fill,
-                                                         int lb, int nb,
+                                                         int lb, int nb, int64_t room,
                                                          uint64_t *__restrict__ ukeys,
                                                          unsigned long long *__restrict__ nunique,
                                                          int32_t *__restrict__ deg) {
@@ -113,8 +115,13 @@ __global__ void __launch_bounds__(BK_NT) k_bucket_unique(const uint64_t *__restr
       total += c;
     }
     base_s = atomicAdd(nunique, (unsigned long long)total) & (HASH_FAILED - 1);
+    if ((int64_t)base_s + total > room) {
+      atomicOr(nunique, HASH_FAILED);
+      base_s = HASH_FAILED;
+    }
   }
   __syncthreads();
+  if (base_s == HASH_FAILED) return;
   int64_t at = (int64_t)base_s + fresh_of[warp];
   const uint64_t mask = (1ull << nb) - 1ull;
 #pragma unroll
@@ -427,19 +434,23 @@ __device__ __forceinline__ void load_entries(const int32_t *__restrict__ colidx,
 
 // a1: one 64-bit key (min << nb) | max per input entry that joins two different
 // vertices; the others (and, for symmetric input, entries with u > v) get the
-// sentinel, which sorts last. With BUCKETS, keys times the hash factor go to their
-// buckets (see above), whose cursors are `fill`, and the others nowhere.
-template <bool BUCKETS>
+// sentinel, which sorts last. EMIT_BUCKETS: keys times the hash factor go to their
+// buckets (see above), whose cursors are `fill`, and the others nowhere. EMIT_COUNT and
+// EMIT_PACKED (symmetric input, of which half gives no key): the keys are only counted
+// in *cursor, or written one after the other from it, a warp's in one piece.
+constexpr int EMIT_ALL = 0, EMIT_BUCKETS = 1, EMIT_COUNT = 2, EMIT_PACKED = 3;
+template <int FORM>
 __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__ rowptr,
                                                      const int32_t *__restrict__ colidx, int64_t n,
                                                      int64_t nnz, int nb, bool symmetric,
                                                      bool aligned, uint64_t sentinel,
                                                      int lb, unsigned *__restrict__ fill,
-                                                     unsigned long long *__restrict__ nunique,
+                                                     unsigned long long *__restrict__ cursor,
                                                      const int64_t *__restrict__ tile_rows,
                                                      const int64_t *__restrict__ voff, int ng,
                                                      uint64_t *__restrict__ keys,
                                                      int32_t *__restrict__ err) {
+  constexpr bool BUCKETS = FORM == EMIT_BUCKETS, WARP = FORM == EMIT_COUNT || FORM == EMIT_PACKED;
   __shared__ TileRows tr;
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
   TileAhead next, after;
@@ -456,10 +467,10 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
     const int64_t first = t0 + (int64_t)threadIdx.x * SP_ITEMS;
     const int32_t(&w)[SP_ITEMS] = here.w;
     tile_rows_mark(tr, rowptr, t0, t1, here);
-    if (first >= t1) continue;
+    if (!WARP && first >= t1) continue;
     // (a bucket has overflowed: only the checks go on)
     const bool given_up =
-        BUCKETS && (*reinterpret_cast<volatile unsigned long long *>(nunique) & HASH_FAILED) != 0;
+        BUCKETS && (*reinterpret_cast<volatile unsigned long long *>(cursor) & HASH_FAILED) != 0;
     unsigned marks = 0;
     int32_t u = tile_row_at(tr, (int)threadIdx.x * SP_ITEMS, &marks);
     int gi = 0;
@@ -509,8 +520,23 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
 #pragma unroll
       for (int i = 0; i < SP_ITEMS; ++i) {
         if (pos[i] < (unsigned)BK_CAP) keys[(key[i] >> (64 - lb)) * BK_CAP + pos[i]] = key[i];
-        else if (pos[i] == (unsigned)BK_CAP) atomicOr(nunique, HASH_FAILED);
+        else if (pos[i] == (unsigned)BK_CAP) atomicOr(cursor, HASH_FAILED);
       }
+      continue;
+    }
+    if (WARP) {
+      unsigned mine = 0;
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i) mine += key[i] != sentinel ? 1u : 0u;
+      const unsigned incl = warp_inclusive_scan(mine);
+      const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+      unsigned long long at = 0;
+      if (lane_id() == 0 && total) at = atomicAdd(cursor, (unsigned long long)total);
+      if (FORM == EMIT_COUNT) continue;
+      at = __shfl_sync(0xffffffffu, at, 0) + (incl - mine);
+#pragma unroll
+      for (int i = 0; i < SP_ITEMS; ++i)
+        if (key[i] != sentinel) keys[at++] = key[i];
       continue;
     }
     if (first + SP_ITEMS <= t1) {  // keys + first is 64-byte aligned
@@ -1399,97 +1425,116 @@ static bbtc_status prepare_small(bbtc_graph *g, const int64_t *d_rowptr, const i
   return BBTC_OK;
 }
 
-bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t *d_colidx,
-                          int64_t nnz, bool symmetric) {
+// a1-a4 for any input: distinct keys by hashing (by_hash) or by sorting. *again: the
+// keys did not go into their buckets, and nothing has been kept but g->deg.
+static bbtc_status prepare_general(bbtc_graph *g, const int64_t *d_rowptr, const int32_t *d_colidx,
+                                   int64_t nnz, bool symmetric, bool by_hash, bool *again) {
   cudaStream_t s = g->stream;
   const int64_t n = g->n;
-  const int nb = ceil_log2_u64((uint64_t)n) < 1 ? 1 : ceil_log2_u64((uint64_t)n);
-  g->nb = nb;
-  if (n > 0 && n <= SG_N && nnz > 0 && nnz <= SG_ENTRIES && !g->voff)
-    return prepare_small(g, d_rowptr, d_colidx, nnz, symmetric);
+  const int nb = g->nb;
   Scratch scratch(s);
   int32_t *err = nullptr;
-  int64_t *hstats = nullptr;  // device: [0]=m, [1]=deg_max, [2]=err
+  int64_t *hstats = nullptr;  // device: [0]=m, [1]=deg_max
   BBTC_TRY(scratch.get(&err, 1));
   BBTC_TRY(scratch.get(&hstats, 3));
   BBTC_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
-
-  // ---- symmetric input with sorted rows: per-row path, no global sort
-  if (symmetric && nnz > 0 && n > 0) {
-    bool applied = false;
-    BBTC_TRY(prepare_sym_sorted(g, d_rowptr, d_colidx, nnz, err, &applied));
-    if (applied) return BBTC_OK;
-    BBTC_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));  // fall through: general path
-  }
 
   // ---- validation of rowptr (colidx range is checked while emitting keys)
   if (n > 0) {
     k_validate_rowptr<<<grid_for(n, 256, 8), 256, 0, s>>>(d_rowptr, n, nullptr, err);
     BBTC_LAUNCH_CHECK();
   }
+  auto check = [&](int32_t herr) -> bbtc_status {
+    if (herr & 1) {
+      set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
+      return BBTC_EINVAL;
+    }
+    if (herr & 2) {
+      set_error("bbtc_graph_create: colidx entry outside [0, n)");
+      return BBTC_EINVAL;
+    }
+    return herr & SORT_FAILED ? sort_failed("bbtc_graph_create") : BBTC_OK;
+  };
 
   // ---- a1: canonical keys, the distinct ones; a2: degree
   // (no key equals the all-ones value: it would need min == max)
-  uint64_t *ka = nullptr, *kb = nullptr;
-  unsigned *fill = nullptr;  // set: by hashing
-  const int64_t nkeys = nnz;
-  const int64_t kcap = nkeys > n ? nkeys : n;  // the buffers also take the n rank keys
-  BBTC_TRY(scratch.get(&kb, kcap));
-  int lb = 1;
-  while ((nkeys >> lb) > BK_MEAN) ++lb;
-  if (nkeys > 0 && nkeys <= HASH_MAX) {
-    const int64_t cap = (int64_t)BK_CAP << lb;
-    if (scratch.get(&fill, (int64_t)BK_PAD << lb) != BBTC_OK ||
-        scratch.get(&ka, cap > kcap ? cap : kcap) != BBTC_OK) {
-      clear_error();
-      fill = nullptr;
-      ka = nullptr;
-    }
-  }
-  if (!ka) BBTC_TRY(scratch.get(&ka, kcap));
+  const uint64_t sentinel =
+      by_hash ? HASH_EMPTY : (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
+  const bool aligned = (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0;
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
+  const unsigned grid = grid_for(ntiles, 1, 32);
   int64_t *tile_rows = nullptr;
   if (nnz > 0) {
     BBTC_TRY(scratch.get(&tile_rows, ntiles + 1));
     k_tile_rows<<<grid_for(ntiles + 1, 256, 16), 256, 0, s>>>(d_rowptr, n, nnz, ntiles, tile_rows);
     BBTC_LAUNCH_CHECK();
   }
+  unsigned long long *nunique = reinterpret_cast<unsigned long long *>(&hstats[0]);
+  BBTC_CUDA(cudaMemsetAsync(nunique, 0, sizeof(*nunique), s));
+  // Keys that are expected: every entry gives one, of symmetric input every second. The
+  // buckets find out whether that holds; a sort has them counted first, since it would
+  // sort (and hold, twice) as many again as there are.
+  int64_t nkeys = symmetric ? nnz / 2 : nnz;
+  int32_t herr = 0;
+  if (!by_hash && symmetric && nnz > 0) {
+    k_emit_keys<EMIT_COUNT><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, nb, symmetric,
+                                                   aligned, sentinel, 0, nullptr, nunique,
+                                                   tile_rows, g->voff, g->ng, nullptr, err);
+    BBTC_LAUNCH_CHECK();
+    BBTC_CUDA(cudaMemcpyAsync(&nkeys, nunique, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BBTC_CUDA(cudaStreamSynchronize(s));
+    BBTC_TRY(check(herr));
+    BBTC_CUDA(cudaMemsetAsync(nunique, 0, sizeof(*nunique), s));
+  }
+  const int64_t kcap = nkeys > n ? nkeys : n;  // the buffers also take the n rank keys
+  uint64_t *ka = nullptr, *kb = nullptr, *sorted = nullptr, *ukeys = nullptr;
+  bool in_alt = false;
+  BBTC_TRY(scratch.get(&kb, kcap));
+  int lb = 1;
+  unsigned *fill = nullptr;
+  if (by_hash) {
+    while ((nkeys >> lb) > BK_MEAN) ++lb;
+    const int64_t cap = (int64_t)BK_CAP << lb;
+    BBTC_TRY(scratch.get(&fill, (int64_t)BK_PAD << lb));
+    BBTC_TRY(scratch.get(&ka, cap > kcap ? cap : kcap));
+  } else {
+    BBTC_TRY(scratch.get(&ka, kcap));
+  }
+  // (allocated after the key buffers: in front of them, among the small blocks, the
+  // additions to the degrees made k_bucket_unique take 432 us instead of 389 for R-MAT
+  // scale 20)
   if (!g->deg) {
     BBTC_TRY(dalloc_n(&g->deg, n, s));
     g->bytes += (uint64_t)(n > 0 ? n : 1) * sizeof(int32_t);
   }
-  int32_t *dmax = nullptr;
-  BBTC_TRY(scratch.get(&dmax, 1));
-  uint64_t *sorted = nullptr, *ukeys = nullptr;
-  unsigned long long *nunique = reinterpret_cast<unsigned long long *>(&hstats[0]);
-  bool in_alt = false;
-  int64_t stats[2] = {0, 0};
-  int32_t hdmax = 0, herr = 0;
-  for (;;) {  // once, or again by sorting when a bucket overflows
-    BBTC_CUDA(cudaMemsetAsync(g->deg, 0, sizeof(int32_t) * (size_t)(n > 0 ? n : 1), s));
+  BBTC_CUDA(cudaMemsetAsync(g->deg, 0, sizeof(int32_t) * (size_t)(n > 0 ? n : 1), s));
+  if (by_hash) {
+    BBTC_CUDA(cudaMemsetAsync(fill, 0, (sizeof(unsigned) * BK_PAD) << lb, s));
+    k_emit_keys<EMIT_BUCKETS><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, nb, symmetric,
+                                                     aligned, sentinel, lb, fill, nunique,
+                                                     tile_rows, g->voff, g->ng, ka, err);
+    BBTC_LAUNCH_CHECK();
+    k_bucket_unique<<<1u << lb, BK_NT, 0, s>>>(ka, fill, lb, nb, kcap, kb, nunique, g->deg);
+    BBTC_LAUNCH_CHECK();
+  } else {
+    if (symmetric && nkeys > 0)
+      k_emit_keys<EMIT_PACKED><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, nb, symmetric,
+                                                      aligned, sentinel, 0, nullptr, nunique,
+                                                      tile_rows, g->voff, g->ng, ka, err);
+    else if (nkeys > 0)
+      k_emit_keys<EMIT_ALL><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, nb, symmetric,
+                                                   aligned, sentinel, 0, nullptr, nullptr,
+                                                   tile_rows, g->voff, g->ng, ka, err);
+    if (nkeys > 0) BBTC_LAUNCH_CHECK();
+    BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
+  }
+  sorted = in_alt ? kb : ka;
+  ukeys = in_alt ? ka : kb;
+  if (!by_hash) {
     BBTC_CUDA(cudaMemsetAsync(nunique, 0, sizeof(*nunique), s));
-    const bool aligned = (reinterpret_cast<uintptr_t>(d_colidx) & 15u) == 0;
-    if (fill) {
-      BBTC_CUDA(cudaMemsetAsync(fill, 0, (sizeof(unsigned) * BK_PAD) << lb, s));
-      k_emit_keys<true><<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
-          d_rowptr, d_colidx, n, nnz, nb, symmetric, aligned, HASH_EMPTY, lb, fill, nunique,
-          tile_rows, g->voff, g->ng, ka, err);
-      BBTC_LAUNCH_CHECK();
-      k_bucket_unique<<<1u << lb, BK_NT, 0, s>>>(ka, fill, lb, nb, kb, nunique, g->deg);
-      BBTC_LAUNCH_CHECK();
-    } else if (nkeys > 0) {
-      const uint64_t sentinel = (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
-      k_emit_keys<false><<<grid_for(ntiles, 1, 32), SP_NT, 0, s>>>(
-          d_rowptr, d_colidx, n, nnz, nb, symmetric, aligned, sentinel, 0, nullptr, nullptr,
-          tile_rows, g->voff, g->ng, ka, err);
-      BBTC_LAUNCH_CHECK();
-      BBTC_TRY(radix_sort(ka, kb, nullptr, nullptr, nkeys, 0, 2 * nb, s, err, &in_alt));
-    }
-    sorted = in_alt ? kb : ka;
-    ukeys = in_alt ? ka : kb;
-    if (!fill && nkeys > 0) {
+    if (nkeys > 0) {
       const int64_t nblk = (nkeys + UQ_TILE - 1) / UQ_TILE;
-      const uint64_t sentinel = (nb * 2 >= 64) ? ~0ull : ((1ull << (2 * nb)) - 1ull);
       uint64_t *boff = nullptr;
       BBTC_TRY(scratch.get(&boff, nblk + 1));
       k_unique_count<<<(unsigned)nblk, UQ_NT, 0, s>>>(sorted, nkeys, sentinel, err, boff);
@@ -1501,22 +1546,20 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
       BBTC_CUDA(
           cudaMemcpyAsync(nunique, &boff[nblk], sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
     }
-    BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
-    BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    BBTC_CUDA(cudaMemcpyAsync(&stats[0], nunique, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    BBTC_CUDA(cudaStreamSynchronize(s));
-    if (herr & 1) {
-      set_error("bbtc_graph_create: rowptr[0] != 0 or rowptr decreases");
-      return BBTC_EINVAL;
-    }
-    if (herr & 2) {
-      set_error("bbtc_graph_create: colidx entry outside [0, n)");
-      return BBTC_EINVAL;
-    }
-    if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
-    if (!((unsigned long long)stats[0] & HASH_FAILED)) break;
-    fill = nullptr;
+  }
+  int32_t *dmax = nullptr;
+  int32_t hdmax = 0;
+  int64_t stats[2] = {0, 0};
+  BBTC_TRY(scratch.get(&dmax, 1));
+  BBTC_TRY(reduce_max_i32(g->deg, n, dmax, s));
+  BBTC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaMemcpyAsync(&stats[0], nunique, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaMemcpyAsync(&hdmax, dmax, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  BBTC_CUDA(cudaStreamSynchronize(s));
+  BBTC_TRY(check(herr));
+  if ((unsigned long long)stats[0] & HASH_FAILED) {
+    *again = true;
+    return BBTC_OK;
   }
   const int64_t m = stats[0];
   if (m > 0xFFFFFFFFLL) {
@@ -1561,9 +1604,8 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
   g->bytes += (uint64_t)(n + 1) * 8 + (uint64_t)(m > 0 ? m : 1) * 8;
   BBTC_CUDA(cudaMemsetAsync(g->rowptr, 0, sizeof(int64_t) * (size_t)(n + 1), s));
   uint64_t *ok = sorted;  // rank keys are consumed; reuse
-  unsigned *slot = nullptr;
+  unsigned *slot = reinterpret_cast<unsigned *>(g->esrc);  // (its rows are written last)
   if (m > 0) {
-    BBTC_TRY(scratch.get(&slot, m));
     k_orient_count<<<grid_for(m, 256, 32), 256, 0, s>>>(
         ukeys, m, nb, rank, ok, slot, reinterpret_cast<unsigned long long *>(g->rowptr));
     BBTC_LAUNCH_CHECK();
@@ -1595,6 +1637,31 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
     if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
   }
   return BBTC_OK;
+}
+
+bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t *d_colidx,
+                          int64_t nnz, bool symmetric) {
+  cudaStream_t s = g->stream;
+  const int64_t n = g->n;
+  g->nb = ceil_log2_u64((uint64_t)n) < 1 ? 1 : ceil_log2_u64((uint64_t)n);
+  if (n > 0 && n <= SG_N && nnz > 0 && nnz <= SG_ENTRIES && !g->voff)
+    return prepare_small(g, d_rowptr, d_colidx, nnz, symmetric);
+  // symmetric input with sorted rows: per-row path, no global sort
+  if (symmetric && nnz > 0 && n > 0) {
+    Scratch scratch(s);
+    int32_t *err = nullptr;
+    bool applied = false;
+    BBTC_TRY(scratch.get(&err, 1));
+    BBTC_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
+    BBTC_TRY(prepare_sym_sorted(g, d_rowptr, d_colidx, nnz, err, &applied));
+    if (applied) return BBTC_OK;
+  }
+  bool again = false;
+  if (nnz > 0 && nnz <= HASH_MAX) {
+    BBTC_TRY(prepare_general(g, d_rowptr, d_colidx, nnz, symmetric, true, &again));
+    if (!again) return BBTC_OK;
+  }
+  return prepare_general(g, d_rowptr, d_colidx, nnz, symmetric, false, &again);
 }
 
 }  // namespace bbtc

@@ -69,3 +69,17 @@ got += [int(out["per_task"].sum()), int(out["per_vertex"].sum()) // 3, g.count(p
 print(*got)
 """)
     assert len(got) == 9 and len(set(got)) == 1
+
+
+@pytest.mark.parametrize("n", [4000, 16_400])
+def test_symmetric_unsorted_rows_reserve_for_one_key_an_edge(n):
+    # half of the entries give keys: by buckets up to 2^28 entries, beyond by sorting.
+    # An entry's share: buckets 8 to 11 bytes or two sort buffers 8, distinct keys 4,
+    # upward entries of the sorted attempt 4, columns and sources 4
+    reserved, nnz, count, want = map(int, run(f"""
+n, rp, ci = complete({n}, upward=False)
+g = bb.Graph(n, rp, ci, symmetric=True)
+print(bb.bbtc_device_memory()["pool_reserved"], ci.numel(), g.count(), math.comb(n, 3))
+"""))
+    assert count == want
+    assert reserved < 24 * nnz

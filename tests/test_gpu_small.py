@@ -107,3 +107,37 @@ def test_interior_row_pointers_out_of_range_are_refused(row, value):
         assert e.value.status == 1
     with bb.Graph(*graphgen.gnm(2048, 30_000, 5), symmetric=True) as g:  # all is well after
         assert g.count() == oracle.bbtc(*graphgen.gnm(2048, 30_000, 5), p=1)["total"]
+
+
+def descending(graph):
+    n, rp, ci = graph
+    row = np.repeat(np.arange(n), np.diff(rp))
+    return n, rp, ci[np.lexsort((-ci.astype(np.int64), row))]
+
+
+@pytest.mark.parametrize("n,pairs", [(1100, 1500), (1100, 3000), (20_000, 300_000)])
+@pytest.mark.parametrize("form", ["both", "repeated", "upward"])
+def test_symmetric_input_with_unsorted_rows(n, pairs, form):
+    # "repeated": one edge overflows its bucket; "upward": every edge under its lower
+    # endpoint only, twice the keys that symmetric input gives (more than room, at 1,100
+    # vertices, or more than the buckets hold)
+    _, src, dst = graphgen.gnm_pairs(n, pairs, n + pairs)
+    if form == "repeated":
+        src, dst = np.append(src, np.full(50_000, 3)), np.append(dst, np.full(50_000, 5))
+    sym = graphgen.pairs_to_csr(n, src.astype(np.int32), dst.astype(np.int32))
+    ref = oracle.bbtc(*sym, p=1)
+    if form == "upward":
+        sym = one_sided(n, np.minimum(src, dst), np.maximum(src, dst))
+    with bb.Graph(*descending(sym), symmetric=True) as g:
+        o = g.oriented()
+        assert np.array_equal(o["rowptr"], ref["rowptr"])
+        assert np.array_equal(o["colidx"], ref["colidx"])
+        assert np.array_equal(o["perm"], ref["perm"])
+        assert g.count() == ref["total"]
+
+
+def test_symmetric_batch_with_unsorted_rows():
+    graphs = [graphgen.rmat(11, 12, 61), graphgen.gnm(3000, 9000, 62), graphgen.gnm(7, 4, 63)]
+    want = [oracle.bbtc(*g, p=1)["total"] for g in graphs]
+    with bb.BatchGraph([descending(g) for g in graphs], symmetric=True) as u:
+        assert u.count(p=1, per_graph=True)["per_graph"].tolist() == want
