@@ -1643,6 +1643,7 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
                           int64_t nnz, bool symmetric) {
   cudaStream_t s = g->stream;
   const int64_t n = g->n;
+  const uint64_t bytes0 = g->bytes;
   g->nb = ceil_log2_u64((uint64_t)n) < 1 ? 1 : ceil_log2_u64((uint64_t)n);
   if (n > 0 && n <= SG_N && nnz > 0 && nnz <= SG_ENTRIES && !g->voff)
     return prepare_small(g, d_rowptr, d_colidx, nnz, symmetric);
@@ -1658,8 +1659,19 @@ bbtc_status prepare_graph(bbtc_graph *g, const int64_t *d_rowptr, const int32_t 
   }
   bool again = false;
   if (nnz > 0 && nnz <= HASH_MAX) {
-    BBTC_TRY(prepare_general(g, d_rowptr, d_colidx, nnz, symmetric, true, &again));
-    if (!again) return BBTC_OK;
+    const bbtc_status st = prepare_general(g, d_rowptr, d_colidx, nnz, symmetric, true, &again);
+    if (st != BBTC_ENOMEM) {
+      if (st != BBTC_OK || !again) return st;
+    } else {  // sorting takes less memory: 16 bytes a key where buckets take up to 29
+      clear_error();
+      for (int32_t **a : {&g->deg, &g->perm, &g->colidx, &g->esrc, &g->gid}) {
+        dfree(*a, s);
+        *a = nullptr;
+      }
+      dfree(g->rowptr, s);
+      g->rowptr = nullptr;
+      g->bytes = bytes0;
+    }
   }
   return prepare_general(g, d_rowptr, d_colidx, nnz, symmetric, false, &again);
 }

@@ -100,9 +100,10 @@ class Server:
     # ------------------------------------------------------------ cache
     @staticmethod
     def _estimate_bytes(n, nnz):
-        # oriented CSR (rowptr, colidx, esrc, perm, degree), the plan (16-byte
-        # in-edge records, split table, tasks) and the preparation's temporaries,
-        # from the input size
+        # what preparation holds at its peak when it sorts the input's keys (48 bytes an
+        # edge listed in both directions: 8 of input, 32 of keys, 8 of columns and sources;
+        # the faster way by buckets takes up to 75 and is left when it finds no room);
+        # the oriented CSR and the plan (8-byte in-edge records, core) take less
         m = nnz // 2 + 1
         return 44 * n + 48 * m
 

@@ -83,3 +83,16 @@ print(bb.bbtc_device_memory()["pool_reserved"], ci.numel(), g.count(), math.comb
 """))
     assert count == want
     assert reserved < 24 * nnz
+
+
+def test_general_input_that_only_fits_by_sorting():
+    # 16 M entries: buckets of 268 MB, two sort buffers of 128 MB each
+    count, want = map(int, run("""
+n, rp, ci = complete(5657, upward=True)
+held = leave(480 << 20)
+h = bb.bbtc_graph_create(n, rp, ci)
+del held
+torch.cuda.empty_cache()
+print(bb.bbtc_count(h), math.comb(n, 3))
+"""))
+    assert count == want
