@@ -125,6 +125,12 @@ def kernel_source_hash() -> str:
     return h.hexdigest()
 
 
+def roofline_bytes(own, traffic):
+    """The bytes a count's HBM fraction is taken on: its algorithmic bytes, but no more
+    than it is known to move (on a skewed graph most list bytes are never read)."""
+    return own if traffic is None else min(own, traffic)
+
+
 def recorded_traffic(workload: str, p: int, kernel: str):
     """DRAM bytes of one count (the launches of its counting kernels) from the
     committed ncu record, when it was taken on these kernels' sources and this
@@ -688,7 +694,8 @@ def measure(args, workload: str, p: int, budget_gb: float, env, with_cpu: bool):
     # v (sum over u of d+(u)(d+(u)-1)/2 elements, 4 B each; the hubs' share is read
     # as bits instead)
     own = 4 * (3 * m + info["wedges_out"])
-    achieved = own / (kms / 1000.0) / 1e9
+    traffic = recorded_traffic(workload, p, args.kernel) if not budget else None
+    achieved = roofline_bytes(own, traffic) / (kms / 1000.0) / 1e9
     # W_min: every edge's N(v) read once per in-edge of v; these kernels
     # never make those reads, so it is reported for context, not as its roofline
     wmin = 4 * (m + info["wedges_in"])
@@ -697,7 +704,6 @@ def measure(args, workload: str, p: int, budget_gb: float, env, with_cpu: bool):
     # = 2 * sum_u C(d+(u), 2) + m
     wmerge = 4 * (2 * info["wedges_out"] + m + info["wedges_in"])
     h2d = (n + 1) * 8 + input_entries * 4
-    traffic = recorded_traffic(workload, p, args.kernel) if not budget else None
     line = {
         "metric": METRIC,
         "value": (m / (ms / 1000.0)) if shard_tasks else replica_throughput(m, world, ms),
@@ -751,9 +757,10 @@ def measure(args, workload: str, p: int, budget_gb: float, env, with_cpu: bool):
                      "algorithmic_bytes": own,
                      "bytes_formula": "4*(3m + sum over u of d+(u)(d+(u)-1)/2): 8-byte "
                                       "in-edge records, each N(v) staged once, the probed "
-                                      "part of each N(u) above v (the hubs' share is read "
-                                      "as fewer bytes of bitmap rows, so that a skewed "
-                                      "graph can come out above 1)",
+                                      "part of each N(u) above v. achieved and frac count "
+                                      "no more than traffic: the hubs' share is read as "
+                                      "fewer bytes of bitmap rows, and lists again from L2; "
+                                      "without a traffic record frac can pass 1",
                      "w_min_bytes": wmin,
                      "w_min_formula": "4*(m + sum over oriented edges (u,v) of d+(v)); reads "
                                       "N(v) once per in-edge, which these kernels do not do",

@@ -49,3 +49,9 @@ def test_clock_summary_flags_throttle_reasons(tmp_path):
     with open(s2.path, "w") as f:
         f.write("0, 1500, 2070, 800.0, 0x8, Active, Not Active, Not Active, Not Active\n")
     assert s2.summary()["reasons"] == ["hw_slowdown"]
+
+
+def test_roofline_counts_no_more_bytes_than_are_moved():
+    assert bench.roofline_bytes(311, 534) == 311
+    assert bench.roofline_bytes(71, 28) == 28
+    assert bench.roofline_bytes(71, None) == 71
