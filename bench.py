@@ -119,7 +119,7 @@ def kernel_source_hash() -> str:
     """sha256 of the counting kernels' sources (a changed kernel voids old counters)."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("core.cu", "flat.cu", "flat.cuh", "stage.cuh"):
+    for name in ("core.cu", "flat.cu", "flat.cuh", "stage.cuh", "bounds.cuh"):
         with open(os.path.join(ROOT, "paper_2009_12457_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()

@@ -34,8 +34,13 @@ namespace {
 constexpr int CORE_NT = 256;
 constexpr int CORE_WARPS = CORE_NT / 32;
 constexpr int CORE_MAX_COLS = 12288;  // columns of the core at most
-// a graph of at most so many vertices is all core, and no list is probed: R-MAT
-// scale 14 counts in 27 us where the lists took 117 (latency, not work)
+// a graph of at most so many vertices is all core, and no list is probed. Against
+// 8,192 columns and lists, graphs of 16,384 vertices count in 16.5 us instead of 37
+// (R-MAT scale 14), 38 instead of 61 (G(n, m), 262 K pairs), 136 instead of 453 (2 M
+// pairs) and 32 instead of 59 (Chung-Lu, 500 K pairs). With twice as many columns, 24,000
+// vertices gain (1 M pairs of a G(n, m): 158 us to 121, 2 M of a Chung-Lu: 148 to 80) and
+// 32,000 lose (G(n, m), 2 M pairs: 270 to 286): where all core stops paying depends on
+// the density, and lies above this bound for the graphs tried
 constexpr int CORE_ALL_COLS = 16384;
 constexpr int CORE_TABLE = 816;       // task counters kept in shared memory (p <= 16)
 constexpr int64_t CORE_WIDE_EDGES = 1 << 23;  // fewer edges: 8,192 columns
@@ -453,8 +458,9 @@ void free_core(Plan *pl, cudaStream_t s) {
 
 // Sources with fewer core neighbours stay with the lists: a row costs about
 // 500 instructions of set-up and 10 per core edge, the lists about one per
-// probe. On R-MAT scale 20 (p = 2) a bound of 48, 80 and 128 gave 1.26, 1.32
-// and 1.30 ms, on scale 21 (p = 4) 5.66, 5.64 and 5.47 ms.
+// probe. Counts with bounds of 48, 64, 80 and 128: R-MAT scale 20 739, 735, 729 and
+// 716 us, scale 21 1.60, 1.60, 1.59 and 1.61 ms, scale 22 3.96, 3.92, 3.92 and 3.99 ms, a
+// Chung-Lu graph of 28 M pairs 1.33, 1.31, 1.32 and 1.31 ms: flat around the bound.
 constexpr int CORE_MIN_ROW = 64;
 
 bbtc_status build_core(const bbtc_graph *g, Plan &pl, cudaStream_t s) {

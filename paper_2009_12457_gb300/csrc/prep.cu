@@ -27,8 +27,8 @@ __global__ void k_validate_rowptr(const int64_t *__restrict__ rowptr, int64_t n,
 }
 
 // Distinct edges by hashing instead of sorting: the steps after need the distinct
-// keys in no particular order. A key is stored times an odd factor, a bijection of
-// 64-bit words: its top bits choose one of 2^lb buckets of at most BK_CAP keys (half
+// keys in no particular order. A key is stored times an odd factor (the first
+// multiplier of SplitMix64's finaliser), a bijection of 64-bit words: its top bits choose one of 2^lb buckets of at most BK_CAP keys (half
 // to three quarters full on average), the next ones its slot in a table in shared
 // memory. EMPTY, all ones, is the image of no key (its preimage is above 2^62). A
 // bucket overflows only when an edge is listed some hundred times or the keys were
