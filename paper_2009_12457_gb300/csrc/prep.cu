@@ -551,6 +551,16 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
   }
 }
 
+// In-degrees are later taken to be the degree less the out-degree (flat.cu), which
+// holds when every edge is listed under both endpoints. Whether it does is tested by a
+// sum mod 2^32 over the upward entries of a term of the rank they point to, less the
+// same term times the in-degree for every vertex: 0 when the in-degrees agree, and not
+// else but for accidents of 2^-32.
+__device__ __forceinline__ uint32_t rank_term(int32_t r) {
+  const uint32_t x = (uint32_t)r + 0x9E3779B9u;  // (keeps small ranks from vanishing)
+  return x * x;
+}
+
 // Passes over the entries of a symmetric CSR, thread t of a tile owning entries
 // [8t, 8t + 8). An entry is an edge's first copy when it differs from its row's
 // vertex and from the entry before it in the row. The next tile's entries are
@@ -563,7 +573,8 @@ __global__ void __launch_bounds__(SP_NT) k_emit_keys(const int64_t *__restrict__
 // no second pass over the entries scatters them (it read every entry's stored
 // rank and took 0.32 ms on R-MAT scale 21). When there is no room for `up` (null),
 // the pass only counts, and a second one with `place` (the rows' offsets by rank)
-// writes into the oriented rows themselves.
+// writes into the oriented rows themselves. *mirror (nullable) receives the sum of the
+// upward entries' rank_term.
 // For a batch (voff != nullptr), the entries of a row of graph g are local ids
 // in [0, voff[g+1] - voff[g]), shifted here by voff[g].
 template <int MODE>
@@ -576,9 +587,13 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
                                                     unsigned *__restrict__ dplus,
                                                     int32_t *__restrict__ up,
                                                     const int64_t *__restrict__ place,
+                                                    unsigned *__restrict__ mirror,
                                                     int32_t *__restrict__ err,
                                                     const int64_t *__restrict__ voff, int ng) {
   __shared__ TileRows tr;
+  __shared__ unsigned mirror_s;
+  if (MODE == 1 && threadIdx.x == 0) mirror_s = 0;  // (added to after the tiles' barriers)
+  uint32_t terms = 0;
   const unsigned lane = threadIdx.x & 31u;
   const int64_t ntiles = (nnz + SP_TILE - 1) / SP_TILE;
   TileAhead next, after;
@@ -680,7 +695,10 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
 #pragma unroll
     for (int i = 0; i < SP_ITEMS; ++i) {
       if (i > 0 && ((marks >> i) & 1u)) ru = rank[tr.row[(int)threadIdx.x * SP_ITEMS + i]];
-      if (val[i] > ru) ups |= 1u << i;
+      if (val[i] > ru) {
+        ups |= 1u << i;
+        terms += rank_term(val[i]);
+      }
     }
     const unsigned later0 = marks & ~1u;  // rows that start after the thread's first entry
     // a warp inside one long row (a hub's) reserves once for all its lanes
@@ -721,26 +739,43 @@ __global__ void __launch_bounds__(SP_NT) k_sym_pass(const int64_t *__restrict__ 
       }
     }
   }
+  if (MODE == 1 && mirror) {
+    terms = __reduce_add_sync(0xffffffffu, terms);
+    __syncthreads();
+    if (lane == 0) atomicAdd(&mirror_s, terms);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(mirror, mirror_s);
+  }
 }
 
-// out-degree by position from the out-degree by vertex, and its maximum
+// out-degree by position from the out-degree by vertex, and its maximum; the vertices'
+// terms are taken off *mirror
 __global__ void k_rowlen_by_rank(const unsigned *__restrict__ dplus,
-                                 const int32_t *__restrict__ perm, int64_t n,
+                                 const int32_t *__restrict__ deg,
+                                 const int32_t *__restrict__ perm,
+                                 const int32_t *__restrict__ rank, int64_t n,
                                  uint64_t *__restrict__ rowlen,
-                                 unsigned long long *__restrict__ longest) {
+                                 unsigned long long *__restrict__ longest,
+                                 unsigned *__restrict__ mirror) {
   unsigned best = 0;
+  uint32_t terms = 0;
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r <= n;
        r += (int64_t)gridDim.x * blockDim.x) {
     const unsigned d = r < n ? dplus[perm[r]] : 0u;
     rowlen[r] = d;
     best = d > best ? d : best;
+    if (r < n) terms += rank_term(rank[r]) * ((unsigned)deg[r] - dplus[r]);  // (r as a vertex)
   }
   best = __reduce_max_sync(0xffffffffu, best);
+  terms = __reduce_add_sync(0xffffffffu, terms);
   if ((threadIdx.x & 31) == 0 && best > 0) atomicMax(longest, (unsigned long long)best);
+  if ((threadIdx.x & 31) == 0 && terms) atomicSub(mirror, terms);
 }
 
-// {largest out-degree, edges, largest degree (that of the last position), error bits}
+// {largest out-degree, edges, largest degree (that of the last position), error bits,
+// what *mirror holds}
 __global__ void k_sym_stats(const unsigned long long *__restrict__ longest,
+                            const unsigned *__restrict__ mirror,
                             const int64_t *__restrict__ rowptr, const int32_t *__restrict__ deg,
                             const int32_t *__restrict__ perm, int64_t n,
                             const int32_t *__restrict__ err, int64_t *__restrict__ stats) {
@@ -748,6 +783,7 @@ __global__ void k_sym_stats(const unsigned long long *__restrict__ longest,
   stats[1] = rowptr[n];
   stats[2] = deg[perm[n - 1]];
   stats[3] = *err;
+  stats[4] = (int64_t)*mirror;
 }
 
 // esrc[x] = the row of position x, for every position of the oriented CSR.
@@ -1218,7 +1254,8 @@ static bbtc_status sort_rows(const int64_t *rowptr, int64_t n, const RowSource &
 }
 
 // a1-a4 for symmetric input with sorted rows. Sets *applied = false (and does
-// nothing lasting) when some row turns out unsorted.
+// nothing lasting) when some row turns out unsorted, or some edge turns out to be
+// listed under one endpoint only.
 static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
                                       const int32_t *d_colidx, int64_t nnz, int32_t *err,
                                       bool *applied) {
@@ -1239,7 +1276,8 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   BBTC_LAUNCH_CHECK();
   const unsigned grid = grid_for(ntiles, 1, 32);
   k_sym_pass<0><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, g->deg,
-                                       nullptr, nullptr, nullptr, nullptr, err, g->voff, g->ng);
+                                       nullptr, nullptr, nullptr, nullptr, nullptr, err, g->voff,
+                                       g->ng);
   BBTC_LAUNCH_CHECK();
   int32_t herr = 0, hdmax = 0;
   // what pass 0 found in the input: BBTC_OK and *sorted, or the error
@@ -1304,7 +1342,8 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   unsigned *dplus = nullptr;
   unsigned long long *longest = nullptr;
   BBTC_TRY(scratch.get(&dplus, n));
-  BBTC_TRY(scratch.get(&longest, 1));
+  BBTC_TRY(scratch.get(&longest, 2));
+  unsigned *mirror = reinterpret_cast<unsigned *>(longest + 1);
   if (dalloc_n(&up, nnz, s) != BBTC_OK) {  // no room: the rows are written in a second pass
     clear_error();
     up = nullptr;
@@ -1315,26 +1354,27 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
     ~FreeUp() { dfree(p, s); }
   } free_up{up, s};
   BBTC_CUDA(cudaMemsetAsync(dplus, 0, sizeof(unsigned) * (size_t)n, s));
-  BBTC_CUDA(cudaMemsetAsync(longest, 0, sizeof(unsigned long long), s));
+  BBTC_CUDA(cudaMemsetAsync(longest, 0, 2 * sizeof(unsigned long long), s));
   k_sym_pass<1><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, nullptr, rank,
-                                       dplus, up, nullptr, err, g->voff, g->ng);
+                                       dplus, up, nullptr, mirror, err, g->voff, g->ng);
   BBTC_LAUNCH_CHECK();
   k_rowlen_by_rank<<<grid_for(n + 1, 256, 16), 256, 0, s>>>(
-      dplus, g->perm, n, reinterpret_cast<uint64_t *>(g->rowptr), longest);
+      dplus, g->deg, g->perm, rank, n, reinterpret_cast<uint64_t *>(g->rowptr), longest, mirror);
   BBTC_LAUNCH_CHECK();
   BBTC_TRY(exclusive_scan_u64(reinterpret_cast<uint64_t *>(g->rowptr),
                               reinterpret_cast<uint64_t *>(g->rowptr), n + 1, s));
   int64_t *stats = nullptr;
-  BBTC_TRY(scratch.get(&stats, 4));
-  k_sym_stats<<<1, 1, 0, s>>>(longest, g->rowptr, g->deg, g->perm, n, err, stats);
+  BBTC_TRY(scratch.get(&stats, 5));
+  k_sym_stats<<<1, 1, 0, s>>>(longest, mirror, g->rowptr, g->deg, g->perm, n, err, stats);
   BBTC_LAUNCH_CHECK();
-  int64_t h[4] = {0, 0, 0, 0};
+  int64_t h[5] = {0, 0, 0, 0, 0};
   BBTC_CUDA(cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, s));
   BBTC_CUDA(cudaStreamSynchronize(s));
   herr = (int32_t)h[3];
   BBTC_TRY(check(&sorted_rows));
   if (herr & SORT_FAILED) return sort_failed("bbtc_graph_create");
-  if (!sorted_rows) {  // the general path takes over
+  // the general path takes over: it reads the entries u < v whatever the others say
+  if (!sorted_rows || h[4] != 0) {
     dfree(g->perm, s);
     dfree(g->rowptr, s);
     dfree(g->gid, s);
@@ -1360,7 +1400,8 @@ static bbtc_status prepare_sym_sorted(bbtc_graph *g, const int64_t *d_rowptr,
   if (!up && m > 0) {
     BBTC_CUDA(cudaMemsetAsync(dplus, 0, sizeof(unsigned) * (size_t)n, s));
     k_sym_pass<1><<<grid, SP_NT, 0, s>>>(d_rowptr, d_colidx, n, nnz, aligned, tile_rows, nullptr,
-                                         rank, dplus, g->colidx, g->rowptr, err, g->voff, g->ng);
+                                         rank, dplus, g->colidx, g->rowptr, nullptr, err, g->voff,
+                                         g->ng);
     BBTC_LAUNCH_CHECK();
   }
   const RowSource from = up ? RowSource{up, d_rowptr, g->perm}

@@ -141,3 +141,30 @@ def test_symmetric_batch_with_unsorted_rows():
     want = [oracle.bbtc(*g, p=1)["total"] for g in graphs]
     with bb.BatchGraph([descending(g) for g in graphs], symmetric=True) as u:
         assert u.count(p=1, per_graph=True)["per_graph"].tolist() == want
+
+
+@pytest.mark.parametrize("n,pairs", [(1500, 20_000), (20_000, 400_000), (300_000, 900_000)])
+@pytest.mark.parametrize("form", ["upward", "less_one_up", "less_one_down", "less_half"])
+def test_edges_listed_under_one_endpoint_though_said_to_be_symmetric(n, pairs, form):
+    # rows sorted: the entries u < v are the edges, whatever the others say, and no
+    # in-degree may be taken from a degree that misses some
+    sym = graphgen.gnm(n, pairs, n)
+    rp, ci = sym[1], sym[2]
+    row, rng = np.repeat(np.arange(n), np.diff(rp)), np.random.default_rng(n)
+    keep = np.ones(len(ci), dtype=bool)
+    if form == "upward":
+        keep = row <= ci
+    elif form == "less_half":
+        keep = (row <= ci) | (rng.random(len(ci)) < 0.5)
+    else:
+        u, v = (min, max) if form == "less_one_up" else (max, min)
+        e = int(np.flatnonzero(row != ci)[len(ci) // 2])
+        a, b = u(row[e], ci[e]), v(row[e], ci[e])
+        keep = ~((row == a) & (ci == b))
+    src, dst = row[keep], ci[keep]
+    up = src < dst
+    ref = oracle.bbtc(*graphgen.pairs_to_csr(n, src[up].astype(np.int32), dst[up].astype(np.int32)), p=1)
+    with bb.Graph(*one_sided(n, src, dst), symmetric=True) as g:
+        assert np.array_equal(g.oriented()["colidx"], ref["colidx"])
+        for p in (1, 2):
+            assert g.count(p=p) == ref["total"], p
