@@ -3,7 +3,7 @@
 Requests name a graph (any hashable key); a `source(key)` callable returns its
 host CSR. The server keeps prepared graphs resident: a cache entry is the
 handle that bbtc_graph_create built (the oriented CSR) together with the plan
-that bbtc_graph_plan built on it (blocks, tasks, work items).
+that bbtc_graph_plan built on it (cuts, dense core, in-edges in work items).
 
 Three kinds of threads share the device, each on its own CUDA stream:
 
